@@ -255,6 +255,7 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   L->spec = take(8 * (2 * (size_t)p->spec_np + 1));  // edges [np + 1], counts [np]
   // profiles: n [nxn], dB^2 [nx], B [nx][3], B-perp spectrum [nx/2 + 1]
   L->prof = take(8 * ((size_t)g->nxn + p->nx + 3 * (size_t)p->nx + (size_t)p->nx / 2 + 1));
+  L->twiddle = take(16 * (size_t)p->nx);  // exp(-2 pi i j / nx) of the spectrum's FFT
   L->total = up(o, kAlign);
   return FS_OK;
 }
@@ -897,7 +898,7 @@ int fs_moments(fs_handle* h, int what, void* dst, size_t dst_bytes, int dst_on_d
   if (what == FS_PROFILE_N || what == FS_PROFILE_DB2) {
     const size_t cnt = (what == FS_PROFILE_N) ? g.nxn : g.nx;
     if (dst_bytes < 8 * cnt) return FS_EINVAL;
-    if (s->ops->profiles(s) != cudaSuccess) return s->sticky = FS_ECUDA;
+    if (s->ops->profiles(s, what) != cudaSuccess) return s->sticky = FS_ECUDA;
     const size_t off = s->L.prof + (what == FS_PROFILE_N ? 0 : 8 * (size_t)g.nxn);
     if (cudaMemcpyAsync(dst, s->base + off, 8 * cnt,
                         dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,

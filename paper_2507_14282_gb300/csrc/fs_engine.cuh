@@ -1506,31 +1506,74 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// A value as FP32, correct to one unit in the last place: FP64 values are cut
+// by integer operations (the conversion instruction runs on GB300's narrow
+// FP64 pipe); below FP32's range 0, above it an infinity.
+__device__ __forceinline__ float near_float(float x) { return x; }
+__device__ __forceinline__ float near_float(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7FFu) - 896;
+  const unsigned m = e <= 0 ? 0u
+                     : e >= 255 ? 0x7F800000u
+                                : ((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+  return __uint_as_float((hi & 0x80000000u) | m);
+}
+// An FP32 value as FP64 (exact) by integer operations, for the same reason;
+// zero and subnormals give zero, infinities and NaN stay so.
+__device__ __forceinline__ double wide_double(double x) { return x; }
+__device__ __forceinline__ double wide_double(float x) {
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xFFu;
+  const unsigned hi = (b & 0x80000000u) |
+                      (e == 0 ? 0u : (((e == 0xFFu ? 0x7FFu : e + 896u) << 20) | ((b & 0x7FFFFFu) >> 3)));
+  return __hiloint2double((int)hi, e == 0 ? 0 : (int)((b & 7u) << 29));
+}
+
+constexpr int kWarpsPerBlock = kBlock / 32;
+
+// Kinetic energy and momentum sums of buffer buf. One warp per tile, a grid
+// of a few CTAs per SM that strides over the tiles. Bound by the FP64 pipe:
+// without relativistic terms a particle adds its velocity and square (6
+// operations) to its species' sums, which take the weight and cell volume
+// once at the end, not per particle (19 operations and a block reduction per
+// tile before: 17.8 M particles FP64 990 us).
 template <typename T, int DIM>
-__global__ void k_diag_particles(DevPtrs<T> d, Geo g, Phys ph, int buf) {
-  const int t = blockIdx.x;
-  const int cnt = min(d.cnt[buf][t], g.tile_cap), base = d.tile_base[t];
+__global__ void __launch_bounds__(kBlock) k_diag_particles(DevPtrs<T> d, Geo g, Phys ph, int buf) {
   const Parts<T> P = d.P[buf];
-  double s[4] = {0, 0, 0, 0};
-  for (int p = threadIdx.x; p < cnt; p += blockDim.x) {
-    const int gi = base + p;
-    const double wp = (P.id[gi] & kIdCR) ? ph.w_cr : ph.w_th;
-    const double vx = P.vx[gi], vy = P.vy[gi], vz = P.vz[gi];
-    s[0] += kinetic(wp, vx, vy, vz, ph.cellvol, ph.c2inv);
-    s[1] += (wp * vx) * ph.cellvol;
-    s[2] += (wp * vy) * ph.cellvol;
-    s[3] += (wp * vz) * ph.cellvol;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double s[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};  // per species: v.v or energy, v
+  const bool rel = ph.c2inv > 0.0;
+  for (int t = blockIdx.x * kWarpsPerBlock + warp; t < g.ntiles;
+       t += gridDim.x * kWarpsPerBlock) {
+    const int cnt = min(d.cnt[buf][t], g.tile_cap), base = t * g.tile_cap;
+#pragma unroll 4
+    for (int p = lane; p < cnt; p += 32) {
+      const int gi = base + p;
+      const bool cr = (P.id[gi] & kIdCR) != 0;
+      const double vx = wide_double(P.vx[gi]), vy = wide_double(P.vy[gi]),
+                   vz = wide_double(P.vz[gi]);
+      auto add = [&](double (&a)[4]) {
+        if (rel) a[0] += kinetic(1.0, vx, vy, vz, 1.0, ph.c2inv);
+        else a[0] = __fma_rn(vz, vz, __fma_rn(vy, vy, __fma_rn(vx, vx, a[0])));
+        a[1] += vx;
+        a[2] += vy;
+        a[3] += vz;
+      };
+      if (cr) add(s[1]);
+      else add(s[0]);
+    }
   }
-  __shared__ double red[4][kBlock / 32];
+  __shared__ double red[4][kWarpsPerBlock];
+  const double wt = ph.w_th * ph.cellvol, wc = ph.w_cr * ph.cellvol;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const double v = warp_sum(s[q]);
-    if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = v;
+    const double half = (q == 0 && !rel) ? 0.5 : 1.0;
+    const double v = warp_sum(half * (wt * s[0][q] + wc * s[1][q]));
+    if (lane == 0) red[q][warp] = v;
   }
   __syncthreads();
   if (threadIdx.x < 4) {
     double v = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
+    for (int w = 0; w < kWarpsPerBlock; ++w) v += red[threadIdx.x][w];
     atomicAdd(&d.ctr->sums[threadIdx.x], v);
   }
 }
@@ -1552,12 +1595,38 @@ __global__ void k_diag_field(DevPtrs<T> d, Geo g, Phys ph) {
   // differences, plus advection, k |u| with k <= 2/dx + 2/dy. Kept as the
   // maximum over nodes in sums[5] (non-negative doubles order like their
   // bit patterns).
+  // Two square roots and a division per node in FP64 would bind this kernel to
+  // the FP64 pipe, so a node's z is first formed in FP32 and only nodes
+  // within 1e-4 of the block's largest take the FP64 expression.
   const double kk = 16.0 * (ph.hdx * ph.hdx + ph.hdy * ph.hdy);
   const double ka = 4.0 * (ph.hdx + ph.hdy);
   const int nn = g.nxn * g.ny;
+  const float kkf = (float)kk, kaf = (float)ka;
+  auto approx = [&](int c) {
+    const float bx = near_float(d.Bb[c]), by = near_float(d.Bb[nn + c]),
+                bz = near_float(d.Bb[2 * nn + c]);
+    const float ux = near_float(d.u[c]), uy = near_float(d.u[nn + c]),
+                uz = near_float(d.u[2 * nn + c]);
+    return kkf * sqrtf(bx * bx + by * by + bz * bz) / near_float(d.n[c]) +
+           kaf * sqrtf(ux * ux + uy * uy + uz * uz);
+  };
+  float zf = 0.0f;
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nn; c += gridDim.x * blockDim.x) {
+    const float z = approx(c);
+    // beyond FP32's range (or NaN): every node takes the FP64 expression
+    zf = (z < 1e30f) ? fmaxf(zf, z) : INFINITY;
+  }
+  __shared__ unsigned zblk;
+  if (threadIdx.x == 0) zblk = 0u;
+  __syncthreads();
+  atomicMax(&zblk, __reduce_max_sync(0xffffffffu, __float_as_uint(zf)));
+  __syncthreads();
+  const float lim = __uint_as_float(zblk);
+  const float from = (lim < 1e30f && lim > 1e-30f) ? lim * (1.0f - 1e-4f) : -1.0f;
   double zmax = 0.0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nn;
        c += gridDim.x * blockDim.x) {
+    if (from >= 0.0f && !(approx(c) >= from)) continue;
     const double bx = d.Bb[c], by = d.Bb[nn + c], bz = d.Bb[2 * nn + c];
     const double ux = d.u[c], uy = d.u[nn + c], uz = d.u[2 * nn + c];
     const double b = sqrt(bx * bx + by * by + bz * bz);
@@ -1565,56 +1634,71 @@ __global__ void k_diag_field(DevPtrs<T> d, Geo g, Phys ph) {
     const double z = ph.h * (kk * b / (double)d.n[c] + ka * um);
     zmax = z > zmax ? z : zmax;  // a NaN z leaves zmax; NaN is caught elsewhere
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const double w = __shfl_xor_sync(0xffffffffu, zmax, o);
-    zmax = w > zmax ? w : zmax;
-  }
-  if ((threadIdx.x & 31) == 0 && zmax > 0.0)
+  if (zmax > 0.0)
     atomicMax((unsigned long long*)&d.ctr->sums[5], (unsigned long long)__double_as_longlong(zmax));
 }
 
+// x - p_x histogram of buffer buf. A CTA takes gx x gy tiles (a warp per
+// tile); their particles reach only a few x bins, so the counts are kept in
+// shared memory (nbx x hist_np counters; nbx = 0: too many, straight to
+// global memory) and added to the histogram once. The bins are formed in FP32
+// relative to the CTA's first cell; only values within eps of a bin edge
+// take the written FP64 expressions (GB300's FP64 pipe is narrow).
+// 17.8 M particles FP64: 505 us before.
+constexpr int kHistShared = 8192;  // counters
 template <typename T, int DIM>
-__global__ void k_hist(DevPtrs<T> d, Geo g, Phys ph, int buf, int species) {
-  const int t = blockIdx.x;
-  const int cnt = min(d.cnt[buf][t], g.tile_cap), base = d.tile_base[t];
+__global__ void __launch_bounds__(kBlock)
+    k_hist(DevPtrs<T> d, Geo g, Phys ph, int buf, int species, int gx, int gy, int nbx) {
+  extern __shared__ unsigned sh[];
   const Parts<T> P = d.P[buf];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double hsx = (double)ph.hist_nx / (double)g.nx;
   const double hsp = (double)ph.hist_np / (ph.hist_pmax - ph.hist_pmin);
-  for (int p = threadIdx.x; p < cnt; p += blockDim.x) {
-    const int gi = base + p;
-    const int cr = (P.id[gi] & kIdCR) ? 1 : 0;
-    if (species >= 0 && cr != species) continue;
-    const int cell = P.cell[gi];
-    int bx = (int)floor(((double)(cell & 0xFFFF) + (double)P.ox[gi]) * hsx);
-    bx = min(max(bx, 0), ph.hist_nx - 1);
-    const double bpd = floor(((double)P.vx[gi] - ph.hist_pmin) * hsp);
-    if (!(bpd >= 0.0 && bpd < (double)ph.hist_np)) continue;
-    atomicAdd(&d.hist[(size_t)bx * ph.hist_np + (int)bpd], 1ull);
-  }
-}
-
-// y-averaged n at nodes and |B - B0|^2 at centres (rows summed in order)
-template <typename T>
-__global__ void k_profiles(DevPtrs<T> d, Geo g, Phys ph) {
-  const int nc = g.nx * g.ny, nn = g.nxn * g.ny;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.nxn;
-       i += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int j = 0; j < g.ny; ++j) acc = acc + (double)d.n[j * g.nxn + i];
-    d.prof[i] = acc / (double)g.ny;
-    if (i < g.nx) {
-      double a2 = 0.0;
-      for (int j = 0; j < g.ny; ++j) {
-        const int c = j * g.nx + i;
-        const double dbx = (double)d.B[c] - ph.b0x;
-        const double dby = (double)d.B[nc + c] - ph.b0y;
-        const double dbz = (double)d.B[2 * nc + c] - ph.b0z;
-        a2 = a2 + ((dbx * dbx + dby * dby) + dbz * dbz);
+  const int tx0 = blockIdx.x * gx, ty0 = blockIdx.y * gy;
+  const int ntx = min(gx, g.ntx - tx0), nty = min(gy, g.nty - ty0);
+  const int i0 = tx0 * g.TX, np = ph.hist_np;
+  const double xb = (double)i0 * hsx;
+  const int bx0 = min((int)floor(xb), ph.hist_nx - 1);
+  for (int k = threadIdx.x; k < nbx * np; k += kBlock) sh[k] = 0u;
+  __syncthreads();
+  const float fsx = (float)hsx, fsp = (float)hsp, fx0 = (float)(xb - (double)bx0);
+  const float pmin = (float)ph.hist_pmin;
+  const float epx = 2e-6f * ((float)(gx * g.TX) * fsx + 2.0f);
+  const float epp = 2e-6f * ((fabsf(pmin) + fabsf((float)ph.hist_pmax)) * fsp + (float)np);
+  const bool fast = epx < 0.25f && epp < 0.25f;
+  for (int w = warp; w < ntx * nty; w += kWarpsPerBlock) {
+    const int t = (ty0 + w / ntx) * g.ntx + tx0 + w % ntx;
+    const int cnt = min(d.cnt[buf][t], g.tile_cap), base = t * g.tile_cap;
+#pragma unroll 4
+    for (int p = lane; p < cnt; p += 32) {
+      const int gi = base + p;
+      const int cr = (P.id[gi] & kIdCR) ? 1 : 0;
+      if (species >= 0 && cr != species) continue;
+      const int i = P.cell[gi] & 0xFFFF;
+      const T ox = P.ox[gi], vx = P.vx[gi];
+      const float tx = fmaf((float)(i - i0) + near_float(ox), fsx, fx0);
+      const float tp = (near_float(vx) - pmin) * fsp;
+      const float bxf = floorf(tx), bpf = floorf(tp);
+      const float rx = tx - bxf, rp = tp - bpf;
+      int bx, bp;
+      if (fast && fabsf(tp) < 1e6f && rx > epx && rx < 1.0f - epx && rp > epp && rp < 1.0f - epp) {
+        bp = (int)bpf;
+        if (bp < 0 || bp >= np) continue;
+        bx = min(max(bx0 + (int)bxf, 0), ph.hist_nx - 1);
+      } else {
+        bx = (int)floor(((double)i + (double)ox) * hsx);
+        bx = min(max(bx, 0), ph.hist_nx - 1);
+        const double bpd = floor(((double)vx - ph.hist_pmin) * hsp);
+        if (!(bpd >= 0.0 && bpd < (double)np)) continue;
+        bp = (int)bpd;
       }
-      d.prof[g.nxn + i] = a2 / (double)g.ny;
+      if ((unsigned)(bx - bx0) < (unsigned)nbx) atomicAdd(&sh[(bx - bx0) * np + bp], 1u);
+      else atomicAdd(&d.hist[(size_t)bx * np + bp], 1ull);
     }
   }
-  (void)nn;
+  __syncthreads();
+  for (int k = threadIdx.x; k < nbx * np; k += kBlock)
+    if (sh[k]) atomicAdd(&d.hist[(size_t)(bx0 + k / np) * np + k % np], (unsigned long long)sh[k]);
 }
 
 // Grid export / import in FP64 host layout ([row][col][component]).

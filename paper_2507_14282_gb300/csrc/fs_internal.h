@@ -83,7 +83,7 @@ struct Layout {
   size_t part[2][7], mov[7], stg[7];
   size_t tile_base, cnt[2], mcnt;
   size_t B, Bs, Bsum, E, Es, Bb, G, n, u, J, pre;
-  size_t partial, far, acc, inj, ctr, hist, prof, spec;
+  size_t partial, far, acc, inj, ctr, hist, prof, spec, twiddle;
   size_t total;
 };
 
@@ -185,7 +185,7 @@ struct Ops {
   cudaError_t (*insert_staged)(Sim*, int buf, int n, bool from_movers);
   cudaError_t (*diag)(Sim*, int buf);
   cudaError_t (*hist)(Sim*, int buf, int species);
-  cudaError_t (*profiles)(Sim*);
+  cudaError_t (*profiles)(Sim*, int which);  // FS_PROFILE_N or FS_PROFILE_DB2
   cudaError_t (*profile_B)(Sim*);       // y-averaged B into the profile region
   cudaError_t (*spectrum_bperp)(Sim*);  // B-perp power spectrum into the profile region
   cudaError_t (*spectrum_p)(Sim*, int buf, int species);  // n(p) counts

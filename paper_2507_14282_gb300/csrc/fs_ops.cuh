@@ -506,37 +506,54 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
+  // CTAs of a kernel whose warps stride over the tiles
+  static int tile_warps_grid(Sim* s) {
+    return std::max(1, std::min((s->g.ntiles + kWarpsPerBlock - 1) / kWarpsPerBlock, 152 * 8));
+  }
+
   static cudaError_t diag(Sim* s, int buf) {
     DevPtrs<T> d = P(s);
     cudaError_t e = cudaMemsetAsync(d.ctr->sums, 0, sizeof(d.ctr->sums), s->stream);
     if (e != cudaSuccess) return e;
     if (s->g.dim == 1)
-      k_diag_particles<T, 1><<<s->g.ntiles, kBlock, 0, s->stream>>>(d, s->g, s->ph, buf);
+      k_diag_particles<T, 1><<<tile_warps_grid(s), kBlock, 0, s->stream>>>(d, s->g, s->ph, buf);
     else
-      k_diag_particles<T, 2><<<s->g.ntiles, kBlock, 0, s->stream>>>(d, s->g, s->ph, buf);
-    k_diag_field<T><<<grid_for((long long)s->g.nx * s->g.ny), kBlock, 0, s->stream>>>(d, s->g, s->ph);
+      k_diag_particles<T, 2><<<tile_warps_grid(s), kBlock, 0, s->stream>>>(d, s->g, s->ph, buf);
+    // several nodes per thread, so that few of them take the FP64 expression
+    const int grid = std::min(grid_for((long long)s->g.nx * s->g.ny), 152 * 4);
+    k_diag_field<T><<<grid, kBlock, 0, s->stream>>>(d, s->g, s->ph);
     return cudaGetLastError();
   }
 
   static cudaError_t hist(Sim* s, int buf, int species) {
     DevPtrs<T> d = P(s);
+    const Geo& g = s->g;
     cudaError_t e = cudaMemsetAsync(d.hist, 0,
                                     sizeof(unsigned long long) * s->ph.hist_nx * s->ph.hist_np,
                                     s->stream);
     if (e != cudaSuccess) return e;
-    if (s->g.dim == 1)
-      k_hist<T, 1><<<s->g.ntiles, kBlock, 0, s->stream>>>(d, s->g, s->ph, buf, species);
+    const int gx = g.dim == 1 ? kWarpsPerBlock : 1, gy = g.dim == 1 ? 1 : 4 * kWarpsPerBlock;
+    const dim3 grid((g.ntx + gx - 1) / gx, (g.nty + gy - 1) / gy);
+    // x bins a CTA's cells can reach: a span of gx TX cells anywhere in the box
+    const long long span =
+        (long long)ceil((double)gx * g.TX * s->ph.hist_nx / (double)g.nx) + 2;
+    const int nbx = span * s->ph.hist_np <= kHistShared ? (int)span : 0;
+    const size_t smem = sizeof(unsigned) * (size_t)nbx * s->ph.hist_np;
+    if (g.dim == 1)
+      k_hist<T, 1><<<grid, kBlock, smem, s->stream>>>(d, g, s->ph, buf, species, gx, gy, nbx);
     else
-      k_hist<T, 2><<<s->g.ntiles, kBlock, 0, s->stream>>>(d, s->g, s->ph, buf, species);
+      k_hist<T, 2><<<grid, kBlock, smem, s->stream>>>(d, g, s->ph, buf, species, gx, gy, nbx);
     return cudaGetLastError();
   }
 
   static double* profile_region(Sim* s) { return (double*)(s->base + s->L.prof); }
 
+  static int prof_grid(long long n) { return (int)((n + kProfThreads - 1) / kProfThreads); }
+
   static cudaError_t profile_B(Sim* s) {
     const int nx = s->g.nx;
     double* out = profile_region(s) + s->g.nxn + nx;
-    k_profile_B<T><<<grid_for(nx), kBlock, 0, s->stream>>>(P(s).B, nx, s->g.ny, out);
+    k_profile_B<T><<<prof_grid(3LL * nx), kProfThreads, 0, s->stream>>>(P(s).B, nx, s->g.ny, out);
     return cudaGetLastError();
   }
 
@@ -545,15 +562,16 @@ struct OpsImpl {
     double* out = profile_region(s) + s->g.nxn + 4 * (size_t)nx;
     cudaError_t e = cudaMemsetAsync(out, 0, 8 * ((size_t)nx / 2 + 1), s->stream);
     if (e != cudaSuccess) return e;
-    const bool pow2 = (nx & (nx - 1)) == 0;
-    if (pow2 && nx <= kFftMax) {
-      int logn = 0;
-      while ((1 << logn) < nx) ++logn;
+    FftPlan f;
+    if (fft_plan(nx, ny, &f)) {
+      double2* W = (double2*)(s->base + s->L.twiddle);
       const size_t smem = sizeof(double2) * (size_t)nx;
       e = cudaFuncSetAttribute(k_bperp_fft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
+                               (int)(sizeof(double2) * (size_t)kFftMax));
       if (e != cudaSuccess) return e;
-      k_bperp_fft<T><<<ny, kFftThreads, smem, s->stream>>>(P(s).B, nx, ny, logn, out);
+      k_fft_twiddles<<<(nx + 127) / 128, 128, 0, s->stream>>>(W, nx);
+      const int threads = nx >= 2048 ? kFftThreads : nx >= 512 ? 256 : 64;
+      k_bperp_fft<T><<<ny, threads, smem, s->stream>>>(P(s).B, ny, f, W, out);
     } else {
       const long long work = (long long)(nx / 2 + 1) * ny;
       k_bperp_dft<T><<<grid_for(work), kBlock, 0, s->stream>>>(P(s).B, nx, ny, out);
@@ -567,12 +585,28 @@ struct OpsImpl {
     unsigned long long* out = (unsigned long long*)(s->base + s->L.spec + 8 * ((size_t)np + 1));
     cudaError_t err = cudaMemsetAsync(out, 0, 8 * (size_t)np, s->stream);
     if (err != cudaSuccess) return err;
-    k_spectrum_p<T><<<s->g.ntiles, kBlock, 0, s->stream>>>(P(s), s->g, buf, species, np, e, out);
+    const int copies = (long long)np * kWarpsPerBlock <= kSpecShared ? kWarpsPerBlock
+                       : np <= kSpecShared                           ? 1
+                                                                     : 0;
+    // the FP32 bin: log2 of u.u is within about 1e-5 of the exact value
+    const double per = (double)np / log2(s->p.spec_pmax / s->p.spec_pmin);
+    const double eps = 1e-5 * per * (1.0 + 0.05 * fabs(log2(s->p.spec_pmin))) + 1e-6 * np;
+    const size_t smem = sizeof(unsigned) * (size_t)np * copies;
+    k_spectrum_p<T><<<tile_warps_grid(s), kBlock, smem, s->stream>>>(
+        P(s), s->g, buf, species, np, copies, (float)log2(s->p.spec_pmin), (float)per,
+        (float)std::min(eps, 1.0), e, out);
     return cudaGetLastError();
   }
 
-  static cudaError_t profiles(Sim* s) {
-    k_profiles<T><<<grid_for(s->g.nxn), kBlock, 0, s->stream>>>(P(s), s->g, s->ph);
+  // which: FS_PROFILE_N or FS_PROFILE_DB2
+  static cudaError_t profiles(Sim* s, int which) {
+    const Geo& g = s->g;
+    double* out = profile_region(s);
+    if (which == FS_PROFILE_N)
+      k_profile_n<T><<<prof_grid(g.nxn), kProfThreads, 0, s->stream>>>(P(s).n, g.nxn, g.ny, out);
+    else
+      k_profile_db2<T><<<prof_grid(g.nx), kProfThreads, 0, s->stream>>>(
+          P(s).B, g.nx, g.ny, s->ph.b0x, s->ph.b0y, s->ph.b0z, out + g.nxn);
     return cudaGetLastError();
   }
 
