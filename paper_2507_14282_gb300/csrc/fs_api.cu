@@ -154,7 +154,6 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   if (mpt * g->ntiles >= (1LL << 31) - 1) return FS_EINVAL;
   g->mover_per_tile = (int)mpt;
   g->mover_cap = (int)(mpt * g->ntiles);
-  g->staging_cap = 1 << 16;
   g->chunk = push_chunk_of(p, tx, ty);
   g->push_ctas = p->push_ctas_per_sm;
   g->na = (tx + 3) * (p->dim == 2 ? ty + 3 : 1);
@@ -228,7 +227,6 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   parts(L->part[0], g->cap_total);
   parts(L->part[1], g->cap_total);
   parts(L->mov, g->mover_cap);
-  parts(L->stg, g->staging_cap);
   L->tile_base = take(4 * (size_t)g->ntiles);
   L->cnt[0] = take(4 * (size_t)g->ntiles);
   L->cnt[1] = take(4 * (size_t)g->ntiles);
@@ -287,18 +285,50 @@ __global__ void k_fill_B(T* B, int nc, double bx, double by, double bz) {
   }
 }
 
-// Synchronise the stream, then fold the device status word into the handle.
-int sync_and_check(Sim* s) {
+// Copies the counters out behind everything on the stream, waits for it, and
+// folds the device status word into the handle.
+int read_counters(Sim* s, Counters* c) {
   if (s->sticky) return s->sticky;
-  cudaError_t e = cudaStreamSynchronize(s->stream);
-  if (e != cudaSuccess) return s->sticky = FS_ECUDA;
-  int st = 0;
-  e = cudaMemcpy(&st, s->base + s->L.ctr + offsetof(Counters, status), sizeof(int),
-                 cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return s->sticky = FS_ECUDA;
-  const int code = status_to_code(st);
+  if (cudaMemcpyAsync(c, s->base + s->L.ctr, sizeof(*c), cudaMemcpyDeviceToHost, s->stream) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(s->stream) != cudaSuccess)
+    return s->sticky = FS_ECUDA;
+  const int code = status_to_code(c->status);
   if (code) s->sticky = code;
   return code;
+}
+int sync_and_check(Sim* s) {
+  Counters c;
+  return read_counters(s, &c);
+}
+
+// Device scratch of the host transfers: the particle buffer that holds no
+// current particles (the next step's output, which the push overwrites).
+struct Scratch {
+  char* p;
+  size_t bytes;
+};
+Scratch transfer_scratch(const Sim* s) {
+  const size_t* off = s->L.part[1 - s->cur];
+  return {s->base + off[0], off[6] + 4 * (size_t)s->g.cap_total - off[0]};
+}
+// particles whose columns fit it
+long long scratch_particles(const Sim* s) {
+  return (long long)((transfer_scratch(s).bytes - 8 * kAlign) / kColumnBytes);
+}
+Columns scratch_columns(const Sim* s, size_t m) {
+  char* b = transfer_scratch(s).p;
+  auto take = [&](size_t bytes) {
+    char* r = b;
+    b += up(bytes, kAlign);
+    return r;
+  };
+  Columns c;
+  for (double*& q : c.col) q = (double*)take(8 * m);
+  c.ci = (int*)take(4 * m);
+  c.cj = (int*)take(4 * m);
+  c.id = (uint32_t*)take(4 * m);
+  return c;
 }
 
 int grid_blocks(long long n) {
@@ -468,17 +498,6 @@ void parallel_slices(long long n, F f) {
   for (auto& x : th) x.join();
 }
 
-// Staged copies of the caller's columns: cell = (j << 16) | i from the i
-// column (in `cell`) and the j column (in `id`, 2D), then the ids first,
-// first + 1, ... in input order.
-__global__ void k_pack_staged(int* cell, uint32_t* id, int m, int dim,
-                              unsigned long long first) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    const int j = (dim == 2) ? (int)id[k] : 0;
-    cell[k] = (j << 16) | cell[k];
-    id[k] = (uint32_t)(first + (unsigned long long)k);
-  }
-}
 }  // namespace
 
 namespace {
@@ -709,106 +728,49 @@ int fs_inject(fs_handle* h, long long n, const int* ci, const int* cj,
   // every input is checked before anything reaches the device
   const int dim = s->g.dim, nx = s->g.nx, ny = s->g.ny;
   std::atomic<bool> bad(false);
+  std::atomic<unsigned long long> top(0);  // one past the largest caller-given number
   parallel_slices(n, [&](long long lo, long long hi) {
+    unsigned long long mx = 0;
     for (long long k = lo; k < hi && !bad.load(std::memory_order_relaxed); ++k) {
       const int j = (dim == 2) ? cj[k] : 0;
       if (ci[k] < 0 || ci[k] >= nx || j < 0 || j >= ny || !(fx[k] >= 0.0 && fx[k] < 1.0) ||
           (dim == 2 && !(fy[k] >= 0.0 && fy[k] < 1.0)) || !isfinite(vx[k]) ||
           !isfinite(vy[k]) || !isfinite(vz[k]))
         bad.store(true, std::memory_order_relaxed);
+      if (ids) mx = std::max<unsigned long long>(mx, (ids[k] & kIdMask) + 1ull);
+    }
+    unsigned long long cur = top.load();
+    while (mx > cur && !top.compare_exchange_weak(cur, mx)) {
     }
   });
   if (bad.load()) return FS_EINVAL;
-  int r = sync_and_check(s);
+  Counters c;
+  int r = read_counters(s, &c);
   if (r) return r;
-  unsigned long long next = 0;
-  if (cudaMemcpy(&next, s->base + s->L.ctr + offsetof(Counters, next_id), 8,
-                 cudaMemcpyDeviceToHost) != cudaSuccess)
-    return s->sticky = FS_ECUDA;
+  unsigned long long next = c.next_id;
   if (!ids && next + (unsigned long long)n - 1 > kIdMask) return s->sticky = FS_EIDOVERFLOW;
-  const bool dbl = (s->p.precision == FS_FP64);
-  const size_t Tsz = dbl ? 8 : 4;
-  // stage through the mover list (unused between steps) in large chunks
-  const int chunk = s->g.mover_cap > s->g.staging_cap ? s->g.mover_cap : s->g.staging_cap;
-  const size_t* stg = s->g.mover_cap > s->g.staging_cap ? s->L.mov : s->L.stg;
-  char* base = s->base;
-  auto h2d = [&](size_t off, const void* src, size_t bytes) {
-    return cudaMemcpyAsync(base + off, src, bytes, cudaMemcpyHostToDevice, s->stream);
-  };
-  if (dbl && !ids) {
-    // FP64 without caller ids: the caller's columns go to the staging area as
-    // they are (a pinned caller's arrays take the DMA path), the cell index
-    // and the ids are formed on the device; the stream orders the chunks
-    for (long long k0 = 0; k0 < n; k0 += chunk) {
-      const int m = (int)((n - k0) < chunk ? (n - k0) : chunk);
-      cudaError_t e = h2d(stg[0], ci + k0, 4 * (size_t)m);
-      if (e == cudaSuccess && dim == 2) e = h2d(stg[6], cj + k0, 4 * (size_t)m);
-      if (e == cudaSuccess) e = h2d(stg[1], fx + k0, 8 * (size_t)m);
-      if (e == cudaSuccess && dim == 2) e = h2d(stg[2], fy + k0, 8 * (size_t)m);
-      if (e == cudaSuccess) e = h2d(stg[3], vx + k0, 8 * (size_t)m);
-      if (e == cudaSuccess) e = h2d(stg[4], vy + k0, 8 * (size_t)m);
-      if (e == cudaSuccess) e = h2d(stg[5], vz + k0, 8 * (size_t)m);
-      if (e == cudaSuccess) {
-        k_pack_staged<<<std::min(1024, (m + 255) / 256), 256, 0, s->stream>>>(
-            (int*)(base + stg[0]), (uint32_t*)(base + stg[6]), m, dim, next + (unsigned long long)k0);
-        e = cudaGetLastError();
-      }
-      if (e == cudaSuccess) e = s->ops->insert_staged(s, s->cur, m, stg == s->L.mov);
-      if (e != cudaSuccess) return s->sticky = FS_ECUDA;
-    }
-    next += (unsigned long long)n;
-  } else {
-    std::vector<int> cell(chunk);
-    std::vector<uint32_t> id(chunk);
-    std::vector<char> buf(5 * Tsz * (size_t)chunk);
-    for (long long k0 = 0; k0 < n; k0 += chunk) {
-      const int m = (int)((n - k0) < chunk ? (n - k0) : chunk);
-      char* cols[5];
-      for (int c = 0; c < 5; ++c) cols[c] = buf.data() + (size_t)c * Tsz * chunk;
-      std::atomic<unsigned long long> top(next);
-      parallel_slices(m, [&](long long lo, long long hi) {
-        unsigned long long mx = 0;
-        for (long long k = lo; k < hi; ++k) {
-          const long long q = k0 + k;
-          const int j = (dim == 2) ? cj[q] : 0;
-          cell[k] = (j << 16) | ci[q];
-          uint32_t w;
-          if (ids) {
-            w = ids[q];
-            const unsigned long long num = w & kIdMask;
-            if (num + 1 > mx) mx = num + 1;
-          } else {
-            w = (uint32_t)(next + (unsigned long long)q);
-          }
-          id[k] = w;
-          const double vals[5] = {fx[q], dim == 2 ? fy[q] : 0.0, vx[q], vy[q], vz[q]};
-          for (int c = 0; c < 5; ++c) {
-            if (dbl) {
-              ((double*)cols[c])[k] = vals[c];
-            } else {
-              float f = (float)vals[c];
-              if (c < 2 && f >= 1.0f) f = 0x1.fffffep-1f;
-              ((float*)cols[c])[k] = f;
-            }
-          }
-        }
-        unsigned long long cur = top.load();
-        while (mx > cur && !top.compare_exchange_weak(cur, mx)) {
-        }
-      });
-      cudaError_t e = h2d(stg[0], cell.data(), 4 * (size_t)m);
-      for (int c = 0; c < 5 && e == cudaSuccess; ++c) {
-        if (c == 1 && dim == 1) continue;
-        e = h2d(stg[1 + c], cols[c], Tsz * (size_t)m);
-      }
-      if (e == cudaSuccess) e = h2d(stg[6], id.data(), 4 * (size_t)m);
-      if (e == cudaSuccess) e = s->ops->insert_staged(s, s->cur, m, stg == s->L.mov);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // host buffers reused
-      if (e != cudaSuccess) return s->sticky = FS_ECUDA;
-      next = ids ? top.load() : next;
-    }
-    if (!ids) next += (unsigned long long)n;
+  // the caller's columns go to the device as they are (a pinned caller's
+  // arrays take the DMA path); the insertion rounds them to the run's
+  // precision and forms the cell and the ids. The stream orders the chunks.
+  const long long chunk = std::min(n, scratch_particles(s));
+  const Columns col = scratch_columns(s, (size_t)chunk);
+  const double* src[5] = {fx, fy, vx, vy, vz};
+  for (long long k0 = 0; k0 < n; k0 += chunk) {
+    const int m = (int)std::min(chunk, n - k0);
+    auto h2d = [&](void* dst, const void* from, size_t bytes) {
+      return cudaMemcpyAsync(dst, from, bytes, cudaMemcpyHostToDevice, s->stream);
+    };
+    cudaError_t e = h2d(col.ci, ci + k0, 4 * (size_t)m);
+    if (e == cudaSuccess && dim == 2) e = h2d(col.cj, cj + k0, 4 * (size_t)m);
+    for (int q = 0; q < 5 && e == cudaSuccess; ++q)
+      if (q != 1 || dim == 2) e = h2d(col.col[q], src[q] + k0, 8 * (size_t)m);
+    if (e == cudaSuccess && ids) e = h2d(col.id, ids + k0, 4 * (size_t)m);
+    if (e == cudaSuccess)
+      e = s->ops->insert_columns(s, s->cur, col, m, ids ? col.id : nullptr,
+                                 next + (unsigned long long)k0);
+    if (e != cudaSuccess) return s->sticky = FS_ECUDA;
   }
+  next = ids ? std::max(next, top.load()) : next + (unsigned long long)n;
   if (cudaMemcpyAsync(s->base + s->L.ctr + offsetof(Counters, next_id), &next, 8,
                       cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
       cudaStreamSynchronize(s->stream) != cudaSuccess)
@@ -825,17 +787,16 @@ int fs_load_fields(fs_handle* h, const double* B_host) {
   Sim* s = &h->sim;
   int r = sync_and_check(s);
   if (r) return r;
-  const size_t nc = (size_t)s->g.nx * s->g.ny;
-  const bool dbl = (s->p.precision == FS_FP64);
-  std::vector<char> tmp(3 * nc * (dbl ? 8 : 4));
-  for (size_t q = 0; q < nc; ++q)
-    for (int c = 0; c < 3; ++c) {
-      if (dbl) ((double*)tmp.data())[c * nc + q] = B_host[q * 3 + c];
-      else ((float*)tmp.data())[c * nc + q] = (float)B_host[q * 3 + c];
-    }
-  if (cudaMemcpyAsync(s->base + s->L.B, tmp.data(), tmp.size(), cudaMemcpyHostToDevice,
-                      s->stream) != cudaSuccess)
-    return s->sticky = FS_ECUDA;
+  const long long nc = (long long)s->g.nx * s->g.ny;
+  const Scratch scr = transfer_scratch(s);
+  const long long chunk = std::min<long long>(nc, (long long)(scr.bytes / 24));
+  for (long long q0 = 0; q0 < nc; q0 += chunk) {
+    const int m = (int)std::min(chunk, nc - q0);
+    if (cudaMemcpyAsync(scr.p, B_host + 3 * q0, 24 * (size_t)m, cudaMemcpyHostToDevice,
+                        s->stream) != cudaSuccess ||
+        s->ops->import_B(s, (const double*)scr.p, (int)q0, m) != cudaSuccess)
+      return s->sticky = FS_ECUDA;
+  }
   if (s->ops->ohm_final(s) != cudaSuccess) return s->sticky = FS_ECUDA;
   return sync_and_check(s);
   FS_GUARD_END
@@ -845,22 +806,17 @@ int fs_moments(fs_handle* h, int what, void* dst, size_t dst_bytes, int dst_on_d
   FS_GUARD_BEGIN
   if (!h || !dst) return FS_EINVAL;
   Sim* s = &h->sim;
-  int r = sync_and_check(s);
-  if (r) return r;
+  if (s->sticky) return s->sticky;
   const Geo& g = s->g;
-  const bool dbl = (s->p.precision == FS_FP64);
-  const size_t Tsz = dbl ? 8 : 4;
   if (what == FS_STATE) {
     const size_t need = sizeof(fs_run_state) + 8 * (size_t)g.ny;
     if (dst_bytes < need) return FS_EINVAL;
     Counters c;
     std::vector<char> blob(need);
-    if (cudaMemcpyAsync(&c, s->base + s->L.ctr, sizeof(c), cudaMemcpyDeviceToHost,
-                        s->stream) != cudaSuccess ||
-        cudaMemcpyAsync(blob.data() + sizeof(fs_run_state), s->base + s->L.acc,
+    if (cudaMemcpyAsync(blob.data() + sizeof(fs_run_state), s->base + s->L.acc,
                         8 * (size_t)g.ny, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
       return s->sticky = FS_ECUDA;
-    r = sync_and_check(s);
+    const int r = read_counters(s, &c);
     if (r) return r;
     fs_run_state st;
     memset(&st, 0, sizeof st);
@@ -930,34 +886,31 @@ int fs_moments(fs_handle* h, int what, void* dst, size_t dst_bytes, int dst_on_d
       return s->sticky = FS_ECUDA;
     return sync_and_check(s);
   }
-  size_t planes = 3, cols = g.nxn, src = 0;
+  size_t planes = 3, cols = g.nxn;
   switch (what) {
-    case FS_B: src = s->L.B; cols = g.nx; break;
-    case FS_E: src = s->L.E; break;
-    case FS_BBAR: src = s->L.Bb; break;
-    case FS_N: src = s->L.n; planes = 1; break;
-    case FS_J: src = s->L.J; break;
-    case FS_U: src = s->L.u; break;
+    case FS_B: cols = g.nx; break;
+    case FS_N: planes = 1; break;
+    case FS_E: case FS_BBAR: case FS_J: case FS_U: break;
     default: return FS_EINVAL;
   }
-  const size_t npts = cols * g.ny;
-  if (dst_bytes < 8 * planes * npts) return FS_EINVAL;
+  const long long npts = (long long)cols * g.ny;
+  if (dst_bytes < 8 * planes * (size_t)npts) return FS_EINVAL;
   if (dst_on_device) {
-    if (s->ops->export_grid(s, what, (double*)dst) != cudaSuccess) return s->sticky = FS_ECUDA;
+    if (s->ops->export_grid(s, what, 0, (int)npts, (double*)dst) != cudaSuccess)
+      return s->sticky = FS_ECUDA;
     return sync_and_check(s);
   }
-  std::vector<char> tmp(planes * npts * Tsz);
-  if (cudaMemcpyAsync(tmp.data(), s->base + src, tmp.size(), cudaMemcpyDeviceToHost,
-                      s->stream) != cudaSuccess)
-    return s->sticky = FS_ECUDA;
-  r = sync_and_check(s);
-  if (r) return r;
-  double* o = (double*)dst;
-  for (size_t q = 0; q < npts; ++q)
-    for (size_t c = 0; c < planes; ++c)
-      o[q * planes + c] = dbl ? ((double*)tmp.data())[c * npts + q]
-                              : (double)((float*)tmp.data())[c * npts + q];
-  return FS_OK;
+  // to the host through the device scratch, in the layout the caller gets
+  const Scratch scr = transfer_scratch(s);
+  const long long chunk = std::min<long long>(npts, (long long)(scr.bytes / (8 * planes)));
+  for (long long q0 = 0; q0 < npts; q0 += chunk) {
+    const int m = (int)std::min(chunk, npts - q0);
+    if (s->ops->export_grid(s, what, (int)q0, m, (double*)scr.p) != cudaSuccess ||
+        cudaMemcpyAsync((double*)dst + planes * q0, scr.p, 8 * planes * (size_t)m,
+                        cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+      return s->sticky = FS_ECUDA;
+  }
+  return sync_and_check(s);
   FS_GUARD_END
 }
 
@@ -1005,15 +958,12 @@ int fs_num_particles(fs_handle* h, long long* n) {
   FS_GUARD_BEGIN
   if (!h || !n) return FS_EINVAL;
   Sim* s = &h->sim;
-  int r = sync_and_check(s);
+  if (s->sticky) return s->sticky;
+  if (s->ops->scan_counts(s, s->cur) != cudaSuccess) return s->sticky = FS_ECUDA;
+  Counters c;
+  const int r = read_counters(s, &c);
   if (r) return r;
-  std::vector<int> cnt(s->g.ntiles);
-  if (cudaMemcpy(cnt.data(), s->base + s->L.cnt[s->cur], 4 * (size_t)s->g.ntiles,
-                 cudaMemcpyDeviceToHost) != cudaSuccess)
-    return s->sticky = FS_ECUDA;
-  long long tot = 0;
-  for (int c : cnt) tot += (c < s->g.tile_cap ? c : s->g.tile_cap);
-  *n = tot;
+  *n = (long long)c.live;
   return FS_OK;
   FS_GUARD_END
 }
@@ -1025,50 +975,28 @@ int fs_get_particles(fs_handle* h, long long cap, int* ci, int* cj, double* fx,
   if (!h || !n) return FS_EINVAL;
   Sim* s = &h->sim;
   long long tot = 0;
-  int r = fs_num_particles(h, &tot);
+  int r = fs_num_particles(h, &tot);  // leaves the tiles' first numbers on the device
   if (r) return r;
   *n = tot;
   if (cap < tot) return FS_EINVAL;
   if (tot > 0 && (!ci || !cj || !fx || !fy || !vx || !vy || !vz || !id)) return FS_EINVAL;
-  const Geo& g = s->g;
-  const bool dbl = (s->p.precision == FS_FP64);
-  const size_t Tsz = dbl ? 8 : 4;
-  std::vector<int> cnt(g.ntiles), base(g.ntiles);
-  cudaMemcpy(cnt.data(), s->base + s->L.cnt[s->cur], 4 * (size_t)g.ntiles, cudaMemcpyDeviceToHost);
-  cudaMemcpy(base.data(), s->base + s->L.tile_base, 4 * (size_t)g.ntiles, cudaMemcpyDeviceToHost);
-  const size_t* off = s->L.part[s->cur];
-  long long o = 0;
-  std::vector<char> tb(7 * 8 * (size_t)g.tile_cap);
-  for (int t = 0; t < g.ntiles; ++t) {
-    const int c = cnt[t] < g.tile_cap ? cnt[t] : g.tile_cap;
-    if (c <= 0) continue;
-    const size_t b = (size_t)base[t];
-    cudaError_t e = cudaSuccess;
-    char* p[7];
-    for (int k = 0; k < 7; ++k) p[k] = tb.data() + (size_t)k * 8 * g.tile_cap;
-    e = cudaMemcpy(p[0], s->base + off[0] + 4 * b, 4 * (size_t)c, cudaMemcpyDeviceToHost);
-    for (int k = 1; k <= 5 && e == cudaSuccess; ++k) {
-      if (k == 2 && g.dim == 1) continue;
-      e = cudaMemcpy(p[k], s->base + off[k] + Tsz * b, Tsz * (size_t)c, cudaMemcpyDeviceToHost);
-    }
-    if (e == cudaSuccess)
-      e = cudaMemcpy(p[6], s->base + off[6] + 4 * b, 4 * (size_t)c, cudaMemcpyDeviceToHost);
+  const long long chunk = std::min(tot, scratch_particles(s));
+  const Columns col = scratch_columns(s, (size_t)chunk);
+  double* dst[5] = {fx, fy, vx, vy, vz};
+  for (long long k0 = 0; k0 < tot; k0 += chunk) {
+    const int m = (int)std::min(chunk, tot - k0);
+    auto d2h = [&](void* to, const void* from, size_t bytes) {
+      return cudaMemcpyAsync(to, from, bytes, cudaMemcpyDeviceToHost, s->stream);
+    };
+    cudaError_t e = s->ops->pack_columns(s, s->cur, (int)k0, m, col);
+    if (e == cudaSuccess) e = d2h(ci + k0, col.ci, 4 * (size_t)m);
+    if (e == cudaSuccess) e = d2h(cj + k0, col.cj, 4 * (size_t)m);
+    if (e == cudaSuccess) e = d2h(id + k0, col.id, 4 * (size_t)m);
+    for (int q = 0; q < 5 && e == cudaSuccess; ++q)
+      e = d2h(dst[q] + k0, col.col[q], 8 * (size_t)m);
     if (e != cudaSuccess) return s->sticky = FS_ECUDA;
-    for (int k = 0; k < c; ++k, ++o) {
-      const int cell = ((int*)p[0])[k];
-      ci[o] = cell & 0xFFFF;
-      cj[o] = cell >> 16;
-      auto getT = [&](int col) {
-        return dbl ? ((double*)p[col])[k] : (double)((float*)p[col])[k];
-      };
-      fx[o] = getT(1);
-      fy[o] = (g.dim == 2) ? getT(2) : 0.0;
-      vx[o] = getT(3);
-      vy[o] = getT(4);
-      vz[o] = getT(5);
-      id[o] = ((uint32_t*)p[6])[k];
-    }
   }
+  if (cudaStreamSynchronize(s->stream) != cudaSuccess) return s->sticky = FS_ECUDA;
   return FS_OK;
   FS_GUARD_END
 }
@@ -1077,21 +1005,14 @@ int fs_diag(fs_handle* h, fs_diag_t* out) {
   FS_GUARD_BEGIN
   if (!h || !out) return FS_EINVAL;
   Sim* s = &h->sim;
-  int r = sync_and_check(s);
-  if (r) return r;
+  if (s->sticky) return s->sticky;
   if (s->ops->diag(s, s->cur) != cudaSuccess) return s->sticky = FS_ECUDA;
   Counters c;
-  if (cudaMemcpyAsync(&c, s->base + s->L.ctr, sizeof(c), cudaMemcpyDeviceToHost,
-                      s->stream) != cudaSuccess)
-    return s->sticky = FS_ECUDA;
-  r = sync_and_check(s);
-  if (r) return r;
-  long long np = 0;
-  r = fs_num_particles(h, &np);
+  const int r = read_counters(s, &c);
   if (r) return r;
   memset(out, 0, sizeof(*out));
   out->step = s->step;
-  out->n_particles = np;
+  out->n_particles = (long long)c.live;
   out->next_id = (long long)c.next_id;
   out->incident = (long long)c.incident;
   out->transmitted = (long long)c.transmitted;

@@ -32,7 +32,8 @@ struct Counters {
   double fs_energy, injected_energy, removed_energy;
   double sums[8];        // diagnostics: kinetic, px, py, pz, magnetic
   int status;            // kStatus* bits
-  int mover_count;       // unused
+  int reserved;
+  unsigned long long live;  // particles counted by the last k_diag_particles / k_scan_counts
   long long step;        // step being taken (the Philox step counter)
 };
 
@@ -48,6 +49,15 @@ struct Parts {
   uint32_t* id;
 };
 
+// Particles as host-layout columns on the device: cell indices, {fx, fy, vx,
+// vy, vz} in FP64, id words.
+struct Columns {
+  int *ci, *cj;
+  double* col[5];
+  uint32_t* id;
+};
+constexpr size_t kColumnBytes = 3 * 4 + 5 * 8;  // per particle
+
 // Geometry of the grid and of the tile decomposition.
 struct Geo {
   int dim, nx, ny, nxn;     // nxn node columns: nx + 1, or nx when periodic
@@ -58,7 +68,6 @@ struct Geo {
   long long cap_total;      // ntiles * tile_cap
   int mover_per_tile;       // mover-list slots of each tile
   int mover_cap;            // mover-list slots: ntiles * mover_per_tile
-  int staging_cap;          // host-injection staging slots
   int na;                   // accumulator nodes per tile: (TX+3)*(TY+3) or TX+3
   int nk;                   // sort keys per tile
   int push_ctas;            // cap on the push's persistent CTAs per SM (0: none)
@@ -80,7 +89,7 @@ struct Phys {
 
 // Byte offsets of every region inside the caller's device buffer.
 struct Layout {
-  size_t part[2][7], mov[7], stg[7];
+  size_t part[2][7], mov[7];
   size_t tile_base, cnt[2], mcnt;
   size_t B, Bs, Bsum, E, Es, Bb, G, n, u, J, pre;
   size_t partial, far, acc, inj, ctr, hist, prof, spec, twiddle;
@@ -90,7 +99,7 @@ struct Layout {
 // Typed device pointers (resolved from the layout).
 template <typename T>
 struct DevPtrs {
-  Parts<T> P[2], M, S;
+  Parts<T> P[2], M;
   int* tile_base;
   int* cnt[2];
   int* mcnt;      // movers written by each tile this step
@@ -182,17 +191,22 @@ struct Ops {
                             int n_sub_max, cudaStream_t st, cudaStream_t side,
                             cudaEvent_t fork, cudaEvent_t join);
   cudaError_t (*fields)(Sim*);
-  cudaError_t (*insert_staged)(Sim*, int buf, int n, bool from_movers);
+  // ids NULL: first, first + 1, ...
+  cudaError_t (*insert_columns)(Sim*, int buf, const Columns& src, int n, const uint32_t* ids,
+                                unsigned long long first);
+  // exclusive prefix of the tiles' counts into the movers' counts (free between
+  // steps), the total into Counters::live
+  cudaError_t (*scan_counts)(Sim*, int buf);
+  cudaError_t (*pack_columns)(Sim*, int buf, int k0, int m, const Columns& dst);
   cudaError_t (*diag)(Sim*, int buf);
   cudaError_t (*hist)(Sim*, int buf, int species);
   cudaError_t (*profiles)(Sim*, int which);  // FS_PROFILE_N or FS_PROFILE_DB2
   cudaError_t (*profile_B)(Sim*);       // y-averaged B into the profile region
   cudaError_t (*spectrum_bperp)(Sim*);  // B-perp power spectrum into the profile region
   cudaError_t (*spectrum_p)(Sim*, int buf, int species);  // n(p) counts
-  cudaError_t (*export_grid)(Sim*, int what, double* dst_dev);
-  cudaError_t (*import_B)(Sim*, const double* src_dev);
-  cudaError_t (*export_particles)(Sim*, int buf, double* dst_dev, int* cell_dev,
-                                  uint32_t* id_dev, int* count_dev);
+  // points q0 .. q0 + n - 1 of the grid
+  cudaError_t (*export_grid)(Sim*, int what, int q0, int n, double* dst_dev);
+  cudaError_t (*import_B)(Sim*, const double* src_dev, int q0, int n);
 };
 
 const Ops& ops_f32();
@@ -251,7 +265,6 @@ inline DevPtrs<T> Sim::ptrs(int) const {
   d.P[0] = parts_at<T>(base, L.part[0]);
   d.P[1] = parts_at<T>(base, L.part[1]);
   d.M = parts_at<T>(base, L.mov);
-  d.S = parts_at<T>(base, L.stg);
   d.tile_base = (int*)(base + L.tile_base);
   d.cnt[0] = (int*)(base + L.cnt[0]);
   d.cnt[1] = (int*)(base + L.cnt[1]);

@@ -496,13 +496,31 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  static cudaError_t insert_staged(Sim* s, int buf, int n, bool from_movers) {
+  static cudaError_t insert_columns(Sim* s, int buf, const Columns& src, int n,
+                                    const uint32_t* ids, unsigned long long first) {
     DevPtrs<T> d = P(s);
-    const Parts<T> src = from_movers ? d.M : d.S;
     if (s->g.dim == 1)
-      k_insert_staged<T, 1><<<grid_for(n), kBlock, 0, s->stream>>>(d, src, s->g, buf, n);
+      k_insert_columns<T, 1><<<grid_for(n), kBlock, 0, s->stream>>>(d, src, s->g, buf, n, ids, first);
     else
-      k_insert_staged<T, 2><<<grid_for(n), kBlock, 0, s->stream>>>(d, src, s->g, buf, n);
+      k_insert_columns<T, 2><<<grid_for(n), kBlock, 0, s->stream>>>(d, src, s->g, buf, n, ids, first);
+    return cudaGetLastError();
+  }
+
+  static cudaError_t scan_counts(Sim* s, int buf) {
+    DevPtrs<T> d = P(s);
+    k_scan_counts<<<1, 1024, 0, s->stream>>>(d.cnt[buf], s->g.ntiles, s->g.tile_cap, d.mcnt,
+                                             &d.ctr->live);
+    return cudaGetLastError();
+  }
+
+  static cudaError_t pack_columns(Sim* s, int buf, int k0, int m, const Columns& dst) {
+    DevPtrs<T> d = P(s);
+    if (s->g.dim == 1)
+      k_pack_columns<T, 1><<<tile_warps_grid(s), kBlock, 0, s->stream>>>(d, s->g, buf, d.mcnt, k0,
+                                                                         m, dst);
+    else
+      k_pack_columns<T, 2><<<tile_warps_grid(s), kBlock, 0, s->stream>>>(d, s->g, buf, d.mcnt, k0,
+                                                                         m, dst);
     return cudaGetLastError();
   }
 
@@ -514,6 +532,7 @@ struct OpsImpl {
   static cudaError_t diag(Sim* s, int buf) {
     DevPtrs<T> d = P(s);
     cudaError_t e = cudaMemsetAsync(d.ctr->sums, 0, sizeof(d.ctr->sums), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&d.ctr->live, 0, sizeof(d.ctr->live), s->stream);
     if (e != cudaSuccess) return e;
     if (s->g.dim == 1)
       k_diag_particles<T, 1><<<tile_warps_grid(s), kBlock, 0, s->stream>>>(d, s->g, s->ph, buf);
@@ -610,7 +629,7 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  static cudaError_t export_grid(Sim* s, int what, double* dst) {
+  static cudaError_t export_grid(Sim* s, int what, int q0, int n, double* dst) {
     DevPtrs<T> d = P(s);
     const T* src = nullptr;
     int planes = 3, cols = s->g.nxn;
@@ -623,23 +642,12 @@ struct OpsImpl {
       case FS_U: src = d.u; break;
       default: return cudaErrorInvalidValue;
     }
-    const long long n = (long long)cols * s->g.ny;
-    k_export_grid<T><<<grid_for(n), kBlock, 0, s->stream>>>(src, planes, cols, s->g.ny, dst);
+    k_export_grid<T><<<grid_for(n), kBlock, 0, s->stream>>>(src, planes, cols * s->g.ny, q0, n, dst);
     return cudaGetLastError();
   }
 
-  static cudaError_t import_B(Sim* s, const double* src) {
-    const int nc = s->g.nx * s->g.ny;
-    k_import_B<T><<<grid_for(nc), kBlock, 0, s->stream>>>(P(s).B, src, nc);
-    return cudaGetLastError();
-  }
-
-  static cudaError_t export_particles(Sim* s, int buf, double* dst, int* cell,
-                                      uint32_t* id, int* count) {
-    if (s->g.dim == 1)
-      k_export_particles<T, 1><<<s->g.ntiles, kBlock, 0, s->stream>>>(P(s), s->g, buf, dst, cell, id, count);
-    else
-      k_export_particles<T, 2><<<s->g.ntiles, kBlock, 0, s->stream>>>(P(s), s->g, buf, dst, cell, id, count);
+  static cudaError_t import_B(Sim* s, const double* src, int q0, int n) {
+    k_import_B<T><<<grid_for(n), kBlock, 0, s->stream>>>(P(s).B, src, s->g.nx * s->g.ny, q0, n);
     return cudaGetLastError();
   }
 
@@ -651,7 +659,9 @@ struct OpsImpl {
     o.ohm_final = ohm_final;
     o.step = step;
     o.fields = fields;
-    o.insert_staged = insert_staged;
+    o.insert_columns = insert_columns;
+    o.scan_counts = scan_counts;
+    o.pack_columns = pack_columns;
     o.diag = diag;
     o.hist = hist;
     o.profiles = profiles;
@@ -667,7 +677,6 @@ struct OpsImpl {
     o.profile_B = profile_B;
     o.spectrum_bperp = spectrum_bperp;
     o.spectrum_p = spectrum_p;
-    o.export_particles = export_particles;
     return o;
   }
 };

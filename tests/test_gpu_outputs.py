@@ -98,3 +98,36 @@ def test_counts_equal_numpy(fs, prec, dim, nx, ny, hist, spec):
     for k in ("vx", "vy", "vz"):
         assert abs(d["p" + k[1]] - (w * p[k]).sum()) <= 1e-12 * (w * np.abs(p[k])).sum()
     sim.close()
+
+
+@pytest.mark.parametrize("dim,nx,ny,prec", [(1, 4000, 1, 1), (1, 640, 1, 0), (2, 96, 50, 1)])
+def test_particles_round_trip_in_chunks(fs, dim, nx, ny, prec):
+    """More particles than the transfer scratch holds at once (no spare slots:
+    capacity factor 1): what goes in comes out, values in the run's precision,
+    and the fields with it; counts agree."""
+    ppc = 40
+    kw = dict(dim=dim, nx=nx, ny=ny, ppc=ppc, precision=prec, capacity_factor=1.0, init_plasma=0)
+    rng = np.random.default_rng(nx)
+    n = nx * ny * ppc
+    T = np.float32 if prec else np.float64
+    cell = np.arange(n) % (nx * ny)
+    f = rng.random((2, n)).astype(T).astype(float)
+    f[:, :3] = [0.0, 1.0 - 2.0 ** -24, 0.5]
+    if dim == 1:
+        f[1] = 0.0
+    v = rng.normal(size=(3, n)).astype(T).astype(float)
+    ids = (rng.permutation(n).astype(np.uint32) | np.where(rng.random(n) < 0.1, fs.ID_CR, 0)
+           .astype(np.uint32))
+    sim = fs.FauxShock(**kw)
+    sim.inject(cell % nx, cell // nx, f[0], f[1], v[0], v[1], v[2], ids=ids)
+    assert sim.num_particles() == n == sim.diag()["n_particles"]
+    p = sim.particles()
+    a, b = np.argsort(p["id"] & fs.ID_MASK), np.argsort(ids & fs.ID_MASK)
+    for got, want in ((p["ci"], cell % nx), (p["cj"], cell // nx), (p["fx"], f[0]),
+                      (p["fy"], f[1]), (p["vx"], v[0]), (p["vy"], v[1]), (p["vz"], v[2]),
+                      (p["id"], ids)):
+        np.testing.assert_array_equal(got[a], want[b])
+    B = rng.normal(size=(ny, nx, 3)).astype(T).astype(float)
+    sim.load_fields(B)
+    np.testing.assert_array_equal(sim.grid(fs.FS_B), B)
+    sim.close()
