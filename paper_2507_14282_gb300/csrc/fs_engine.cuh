@@ -1055,10 +1055,83 @@ __device__ __forceinline__ FieldConst<T> field_const_dev(const Phys& ph) {
                        (T)ph.eta, (T)ph.h,   (T)ph.hh,  (T)ph.h6, ph.eta != 0.0 ? 1 : 0};
 }
 
+// E_y (comp 0) or E_z (comp 1) at a node of a 1D grid: the values ohm_e gives
+// there (no y differences; with j_ext = 0 its zero products drop out). bm, bp:
+// B_y, B_z of the node's left and right cells; bbx: B_x at the node. E_x is
+// not needed within a step: Faraday's law has no use for it in 1D and B_x
+// stays as it is.
+template <typename T>
+__device__ __forceinline__ T ohm1_comp(int comp, T bmy, T bpy, T bmz, T bpz, T bbx, T inv_n, T ux,
+                                       T uy, T uz, const FieldConst<T>& fc) {
+  const T ax = (T)0 - fc.jcr;
+  if (comp == 0) {
+    const T dby = (bpy - bmy) * fc.idx;
+    const T bbz = (T)0.5 * (bmz + bpz);
+    const T cay = fc.jcr != (T)0 ? fmaT(dby, bbx, -(ax * bbz)) : dby * bbx;
+    const T cuy = fmaT(uz, bbx, -(ux * bbz));
+    T ey = fmaT(cay, inv_n, -cuy);
+    if (fc.resist) {
+      const T cyv = -((bpz - bmz) * fc.idx);
+      ey = ey + fc.eta * cyv;
+    }
+    return ey;
+  }
+  const T dbz = (bpz - bmz) * fc.idx;
+  const T bby = (T)0.5 * (bmy + bpy);
+  const T caz = fc.jcr != (T)0 ? fmaT(ax, bby, dbz * bbx) : dbz * bbx;
+  const T cuz = fmaT(ux, bby, -(uy * bbx));
+  T ez = fmaT(caz, inv_n, -cuz);
+  if (fc.resist) {
+    const T czv = (bpy - bmy) * fc.idx;
+    ez = ez + fc.eta * czv;
+  }
+  return ez;
+}
+
+// A 1D tile in shared memory: L cells, L + 1 nodes. The block's two halves
+// (half threads each, a multiple of the warp) take one component each.
+template <typename T>
+struct Tile1 {
+  int L, half, comp, l0;  // this thread's component and first element
+  T *Bx, *B, *Bs, *K;     // B_x [L]; B, stage B, RK4 sum of (y, z) [2][L]
+  T *E;                   // E_y, E_z [2][L + 1]
+  T *inv, *bbx, *u;       // per node: 1/n, B_x, u [3][L + 1]
+};
+
+// One RK4 substep (four stages of Ohm and Faraday) of a tile with n, u
+// frozen. At the tile's ends the node reads its end cell on both sides. Stage
+// s's input field is kept in keep[s] ([2][L] doubles each) if given.
+template <typename T>
+__device__ __forceinline__ void tile1_substep(const Tile1<T>& t, const FieldConst<T>& fc,
+                                              double* keep) {
+  const int L = t.L, Ln = L + 1;
+  for (int stage = 1; stage <= 4; ++stage) {
+    const T* By = (stage == 1) ? t.B : t.Bs;
+    const T* Bz = By + L;
+    if (keep)
+      for (int a = t.l0; a < L; a += t.half)
+        keep[(size_t)(2 * (stage - 1) + t.comp) * L + a] = (double)By[t.comp * L + a];
+    for (int a = t.l0; a < Ln; a += t.half) {
+      const int m = max(a - 1, 0), p = min(a, L - 1);
+      t.E[t.comp * Ln + a] = ohm1_comp<T>(t.comp, By[m], By[p], Bz[m], Bz[p], t.bbx[a], t.inv[a],
+                                          t.u[a], t.u[Ln + a], t.u[2 * Ln + a], fc);
+    }
+    __syncthreads();
+    // K_y = dE_z/dx, K_z = -dE_y/dx
+    const T* Eo = t.E + (t.comp ? 0 : Ln);
+    for (int a = t.l0; a < L; a += t.half) {
+      const T dx = (Eo[a + 1] - Eo[a]) * fc.idx;
+      const int k = t.comp * L + a;
+      rk4_stage<T>(stage, t.comp ? -dx : dx, t.K[k], t.Bs[k], t.B[k], fc.h, fc.hh, fc.h6);
+    }
+    __syncthreads();
+  }
+}
+
 // ------------------------------------------------------------------------
 // The whole field advance of a 1D step with x walls (n_sub RK4 substeps,
 // then Ohm's E and Bbar for the next gather) in one launch: on a 1D grid
-// the separate passes are tens of tiny launches per step. A CTA owns kF1
+// the separate passes are tens of tiny launches per step. A CTA owns TILE
 // cells (and their left nodes; the last tile also node nx) and runs every
 // pass in shared memory over its cells plus field1_halo(n_sub) cells around
 // them, which it recomputes: each pass's stencil reaches one cell, so
@@ -1069,17 +1142,28 @@ __device__ __forceinline__ FieldConst<T> field_const_dev(const Phys& ph) {
 // Bout (neighbouring tiles read Bin's cells), E, Bbar and the packed gather
 // block G at the owned nodes. Same per-element arithmetic as ohm_node /
 // faraday_cell (1D), so FP64 results are those of the separate passes.
-constexpr int kF1 = 64, kF1Threads = 128;
+// A chain of 16 dependent passes: in FP64 each instruction holds an SM
+// quarter's pipe for some 64 cycles, so a pass costs its instruction count.
+// 1/n and the pressure term are formed once, B_x and E_x are left out of the
+// stages, and the y and z components go to different warps (8 + 4
+// operations per stage and thread instead of about 70 and a division).
+// TILE 32 while that leaves SMs free (tile and halo fill two warps a
+// component), 64 beyond (less halo to recompute).
 __host__ __device__ inline int field1_halo(int n_sub) { return 4 * n_sub + 2; }
+constexpr int kF1 = 64, kF1Small = 32;
+// threads of a component: the nodes of a TILE with the halo of two substeps
+constexpr int field1_threads(int tile) { return 2 * ((tile + 2 * 10 + 1 + 31) / 32 * 32); }
+constexpr int kF1Threads = field1_threads(kF1);
+inline int field1_tile(int nx) { return nx <= 152 * kF1 ? kF1Small : kF1; }
 template <typename T>
-inline size_t field1_smem(int n_sub) {
-  const size_t L = kF1 + 2 * (size_t)field1_halo(n_sub);
-  return sizeof(T) * (9 * L + 7 * (L + 1));
+inline size_t field1_smem(int n_sub, int tile) {
+  const size_t L = tile + 2 * (size_t)field1_halo(n_sub);
+  return sizeof(T) * (7 * L + 8 * (L + 1));
 }
 
 // Tile blk of the 1D field advance (the body of k_field_step1); smem is the
-// block's dynamic shared memory (field1_smem(n_sub) bytes).
-template <typename T>
+// block's dynamic shared memory (field1_smem(n_sub, TILE) bytes).
+template <typename T, int TILE>
 __device__ __forceinline__ void field_step1_body(const T* __restrict__ Bin, T* __restrict__ Bout,
                                                  const T* __restrict__ nN,
                                                  const T* __restrict__ uN, T* __restrict__ Eo,
@@ -1088,76 +1172,62 @@ __device__ __forceinline__ void field_step1_body(const T* __restrict__ Bin, T* _
                                                  int n_sub, int blk, unsigned char* smem) {
   const int nx = g.nx, nxn = g.nxn, t0 = threadIdx.x, nt = blockDim.x;
   const int H = field1_halo(n_sub);
-  const int c0 = blk * kF1, c1 = min(nx, c0 + kF1);
+  const int c0 = blk * TILE, c1 = min(nx, c0 + TILE);
   const int lo = max(0, c0 - H), L = min(nx, c1 + H) - lo, Ln = L + 1;
-  T* sB = (T*)smem;
-  T* sBs = sB + 3 * L;
-  T* sK = sBs + 3 * L;
-  T* sE = sK + 3 * L;  // [3][Ln]
-  T* sn = sE + 3 * Ln;
-  T* su = sn + Ln;     // [3][Ln]
+  Tile1<T> t;
+  t.L = L;
+  t.half = nt / 2;
+  t.comp = t0 >= t.half;
+  t.l0 = t0 - t.comp * t.half;
+  t.Bx = (T*)smem;
+  t.B = t.Bx + L;
+  t.Bs = t.B + 2 * L;
+  t.K = t.Bs + 2 * L;
+  t.E = t.K + 2 * L;
+  t.inv = t.E + 2 * Ln;
+  t.bbx = t.inv + Ln;
+  t.u = t.bbx + Ln;
+  T* pg = t.u + 3 * Ln;  // the pressure term -(T_e dn/dx)
+  T* sn = t.E;           // the density, until the first stage writes E
 #pragma unroll
   for (int c = 0; c < 3; ++c)
-    for (int a = t0; a < L; a += nt) sB[c * L + a] = Bin[c * nx + lo + a];
+    for (int a = t0; a < L; a += nt) t.Bx[c * L + a] = Bin[c * nx + lo + a];
   for (int a = t0; a < Ln; a += nt) {
     sn[a] = nN[lo + a];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) su[c * Ln + a] = uN[c * nxn + lo + a];
+    for (int c = 0; c < 3; ++c) t.u[c * Ln + a] = uN[c * nxn + lo + a];
   }
   __syncthreads();
-  const T idx = fc.idx, hdx = fc.hdx, te = fc.te, jcr = fc.jcr, eta = fc.eta;
-  const T h = fc.h, hh = fc.hh, h6 = fc.h6;
-  const bool resist = fc.resist != 0;
-  // Ohm at local node a from the centre field Bc (local layout)
-  auto ohm = [&](const T* Bc, int a, T E[3], T Bb[3]) {
-    const int im = min(max(a - 1, 0), L - 1), ip = min(a, L - 1);
-    const T bmy = Bc[L + im], bpy = Bc[L + ip], bmz = Bc[2 * L + im], bpz = Bc[2 * L + ip];
-    Bb[0] = (T)0.5 * (Bc[im] + Bc[ip]);
-    Bb[1] = (T)0.5 * (bmy + bpy);
-    Bb[2] = (T)0.5 * (bmz + bpz);
-    const T dby = (bpy - bmy) * idx;
-    const T dbz = (bpz - bmz) * idx;
-    const int gi = lo + a;
-    const int xp = ((gi + 1 > nx) ? 2 * nx - (gi + 1) : gi + 1) - lo;
-    const int xm = ((gi - 1 < 0) ? -(gi - 1) : gi - 1) - lo;
-    const T dnx = (sn[min(max(xp, 0), L)] - sn[min(max(xm, 0), L)]) * hdx;
-    const T inv_n = (T)1 / sn[a];
-    ohm_e<T>((T)0, -dbz, dby, Bb[0], Bb[1], Bb[2], inv_n, -(te * dnx), -(te * (T)0), su[a],
-             su[Ln + a], su[2 * Ln + a], jcr, eta, resist, E[0], E[1], E[2]);
-  };
-  for (int sub = 0; sub < n_sub; ++sub) {
-    for (int stage = 1; stage <= 4; ++stage) {
-      const T* Bc = (stage == 1) ? sB : sBs;
-      for (int a = t0; a < Ln; a += nt) {
-        T E[3], Bb[3];
-        ohm(Bc, a, E, Bb);
-        sE[a] = E[0];
-        sE[Ln + a] = E[1];
-        sE[2 * Ln + a] = E[2];
-      }
-      __syncthreads();
-      for (int a = t0; a < L; a += nt) {
-        const T dxey = (sE[Ln + a + 1] - sE[Ln + a]) * idx;
-        const T dxez = (sE[2 * Ln + a + 1] - sE[2 * Ln + a]) * idx;
-        const T K[3] = {(T)0, dxez, -dxey};
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          rk4_stage<T>(stage, K[c], sK[c * L + a], sBs[c * L + a], sB[c * L + a], h, hh, h6);
-      }
-      __syncthreads();
+  for (int a = t.l0; a < Ln; a += t.half) {
+    if (t.comp == 0) {
+      t.inv[a] = (T)1 / sn[a];
+    } else {
+      const int gi = lo + a;
+      const int xp = ((gi + 1 > nx) ? 2 * nx - (gi + 1) : gi + 1) - lo;
+      const int xm = ((gi - 1 < 0) ? -(gi - 1) : gi - 1) - lo;
+      const T dnx = (sn[min(max(xp, 0), L)] - sn[min(max(xm, 0), L)]) * fc.hdx;
+      pg[a] = -(fc.te * dnx);
+      t.bbx[a] = (T)0.5 * (t.Bx[max(a - 1, 0)] + t.Bx[min(a, L - 1)]);
     }
   }
+  __syncthreads();
+  for (int sub = 0; sub < n_sub; ++sub) tile1_substep<T>(t, fc, nullptr);
   for (int a = t0; a < Ln; a += nt) {
     const int gi = lo + a;
     if (gi < c0 || (gi >= c1 && !(gi == nx && c1 == nx))) continue;
-    T E[3], Bb[3];
-    ohm(sB, a, E, Bb);
+    const int im = max(a - 1, 0), ip = min(a, L - 1);
+    const T bmy = t.B[im], bpy = t.B[ip], bmz = t.B[L + im], bpz = t.B[L + ip];
+    const T bby = (T)0.5 * (bmy + bpy), bbz = (T)0.5 * (bmz + bpz);
+    const T dby = (bpy - bmy) * fc.idx, dbz = (bpz - bmz) * fc.idx;
+    T ex, ey, ez;
+    ohm_e<T>((T)0, -dbz, dby, t.bbx[a], bby, bbz, t.inv[a], pg[a], -(fc.te * (T)0), t.u[a],
+             t.u[Ln + a], t.u[2 * Ln + a], fc.jcr, fc.eta, fc.resist != 0, ex, ey, ez);
+    const T v[8] = {ex, ey, ez, t.bbx[a], bby, bbz, (T)0, (T)0};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      Eo[c * nxn + gi] = E[c];
-      Bbo[c * nxn + gi] = Bb[c];
+      Eo[c * nxn + gi] = v[c];
+      Bbo[c * nxn + gi] = v[3 + c];
     }
-    const T v[8] = {E[0], E[1], E[2], Bb[0], Bb[1], Bb[2], (T)0, (T)0};
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       G[(size_t)gi * 8 + c] = v[c];                  // row 0
@@ -1168,17 +1238,17 @@ __device__ __forceinline__ void field_step1_body(const T* __restrict__ Bin, T* _
   for (int c = 0; c < 3; ++c)
     for (int a = t0; a < L; a += nt) {
       const int gi = lo + a;
-      if (gi >= c0 && gi < c1) Bout[c * nx + gi] = sB[c * L + a];
+      if (gi >= c0 && gi < c1) Bout[c * nx + gi] = t.Bx[c * L + a];
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kF1Threads)
+template <typename T, int TILE>
+__global__ void __launch_bounds__(field1_threads(TILE))
     k_field_step1(const T* __restrict__ Bin, T* __restrict__ Bout, const T* __restrict__ nN,
                   const T* __restrict__ uN, T* __restrict__ Eo, T* __restrict__ Bbo,
-                  T* __restrict__ G, Geo g, Phys ph, FieldConst<T> fc, int n_sub) {
+                  T* __restrict__ G, Geo g, FieldConst<T> fc, int n_sub) {
   extern __shared__ __align__(16) unsigned char smem[];
-  field_step1_body<T>(Bin, Bout, nN, uN, Eo, Bbo, G, g, fc, n_sub, blockIdx.x, smem);
+  field_step1_body<T, TILE>(Bin, Bout, nN, uN, Eo, Bbo, G, g, fc, n_sub, blockIdx.x, smem);
 }
 
 // ------------------------------------------------------------------------
@@ -1571,19 +1641,40 @@ __device__ __forceinline__ double wide_double(float x) {
 
 constexpr int kWarpsPerBlock = kBlock / 32;
 
+// Adds 1 to cnt[k] for every lane of the warp with k >= 0 (all lanes call).
+// Lanes on the counter of the lowest remaining lane are added as one, twice
+// over; the rest add their own: a drifting thermal plasma puts most lanes
+// on one or two counters, and shared atomics on one word are serialised lane
+// by lane.
+__device__ __forceinline__ void count_shared(unsigned* cnt, int k) {
+  unsigned todo = __ballot_sync(0xffffffffu, k >= 0);
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    if (!todo) return;
+    const int l = __ffs(todo) - 1;
+    const int k0 = __shfl_sync(0xffffffffu, k, l);
+    const unsigned same = __ballot_sync(0xffffffffu, k == k0);
+    if (lane == l) atomicAdd(&cnt[k0], (unsigned)__popc(same));
+    todo &= ~same;
+  }
+  if ((todo >> lane) & 1u) atomicAdd(&cnt[k], 1u);
+}
+
 // Kinetic energy and momentum sums of buffer buf. One warp per tile, a grid
-// of a few CTAs per SM that strides over the tiles. Bound by the FP64 pipe:
-// without relativistic terms a particle adds its velocity and square (6
-// operations) to its species' sums, which take the weight and cell volume
-// once at the end, not per particle (19 operations and a block reduction per
-// tile before: 17.8 M particles FP64 990 us).
+// of a few CTAs per SM that strides over the tiles. Bound by the FP64 pipe: 7
+// operations per particle without relativistic terms (its weight and the cell
+// volume come as one factor), against 19 and a block reduction per tile
+// before; one set of sums for both species (two, chosen per lane, ran both
+// sides of the choice: 449 us). 17.8 M particles FP64: 990 us before.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kBlock) k_diag_particles(DevPtrs<T> d, Geo g, Phys ph, int buf) {
   const Parts<T> P = d.P[buf];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double s[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};  // per species: v.v or energy, v
+  double s[4] = {0, 0, 0, 0};  // w v.v / 2 (or energy), w v
   unsigned long long live = 0;
   const bool rel = ph.c2inv > 0.0;
+  const double wt = ph.w_th * ph.cellvol, wc = ph.w_cr * ph.cellvol;
   for (int t = blockIdx.x * kWarpsPerBlock + warp; t < g.ntiles;
        t += gridDim.x * kWarpsPerBlock) {
     const int cnt = min(d.cnt[buf][t], g.tile_cap), base = t * g.tile_cap;
@@ -1591,27 +1682,21 @@ __global__ void __launch_bounds__(kBlock) k_diag_particles(DevPtrs<T> d, Geo g, 
 #pragma unroll 4
     for (int p = lane; p < cnt; p += 32) {
       const int gi = base + p;
-      const bool cr = (P.id[gi] & kIdCR) != 0;
+      const double w = (P.id[gi] & kIdCR) ? wc : wt;
       const double vx = wide_double(P.vx[gi]), vy = wide_double(P.vy[gi]),
                    vz = wide_double(P.vz[gi]);
-      auto add = [&](double (&a)[4]) {
-        if (rel) a[0] += kinetic(1.0, vx, vy, vz, 1.0, ph.c2inv);
-        else a[0] = __fma_rn(vz, vz, __fma_rn(vy, vy, __fma_rn(vx, vx, a[0])));
-        a[1] += vx;
-        a[2] += vy;
-        a[3] += vz;
-      };
-      if (cr) add(s[1]);
-      else add(s[0]);
+      if (rel) s[0] += kinetic(w, vx, vy, vz, 1.0, ph.c2inv);
+      else s[0] = __fma_rn(w, __fma_rn(vz, vz, __fma_rn(vy, vy, __dmul_rn(vx, vx))), s[0]);
+      s[1] = __fma_rn(w, vx, s[1]);
+      s[2] = __fma_rn(w, vy, s[2]);
+      s[3] = __fma_rn(w, vz, s[3]);
     }
   }
   if (lane == 0 && live) atomicAdd(&d.ctr->live, live);
   __shared__ double red[4][kWarpsPerBlock];
-  const double wt = ph.w_th * ph.cellvol, wc = ph.w_cr * ph.cellvol;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const double half = (q == 0 && !rel) ? 0.5 : 1.0;
-    const double v = warp_sum(half * (wt * s[0][q] + wc * s[1][q]));
+    const double v = warp_sum((q == 0 && !rel) ? 0.5 * s[q] : s[q]);
     if (lane == 0) red[q][warp] = v;
   }
   __syncthreads();
@@ -1710,34 +1795,46 @@ __global__ void __launch_bounds__(kBlock)
   const float epx = 2e-6f * ((float)(gx * g.TX) * fsx + 2.0f);
   const float epp = 2e-6f * ((fabsf(pmin) + fabsf((float)ph.hist_pmax)) * fsp + (float)np);
   const bool fast = epx < 0.25f && epp < 0.25f;
+  constexpr int U = 4;  // particles of a lane whose loads are in flight together
   for (int w = warp; w < ntx * nty; w += kWarpsPerBlock) {
     const int t = (ty0 + w / ntx) * g.ntx + tx0 + w % ntx;
     const int cnt = min(d.cnt[buf][t], g.tile_cap), base = t * g.tile_cap;
-#pragma unroll 4
-    for (int p = lane; p < cnt; p += 32) {
-      const int gi = base + p;
-      const int cr = (P.id[gi] & kIdCR) ? 1 : 0;
-      if (species >= 0 && cr != species) continue;
-      const int i = P.cell[gi] & 0xFFFF;
-      const T ox = P.ox[gi], vx = P.vx[gi];
-      const float tx = fmaf((float)(i - i0) + near_float(ox), fsx, fx0);
-      const float tp = (near_float(vx) - pmin) * fsp;
-      const float bxf = floorf(tx), bpf = floorf(tp);
-      const float rx = tx - bxf, rp = tp - bpf;
-      int bx, bp;
-      if (fast && fabsf(tp) < 1e6f && rx > epx && rx < 1.0f - epx && rp > epp && rp < 1.0f - epp) {
-        bp = (int)bpf;
-        if (bp < 0 || bp >= np) continue;
-        bx = min(max(bx0 + (int)bxf, 0), ph.hist_nx - 1);
-      } else {
-        bx = (int)floor(((double)i + (double)ox) * hsx);
-        bx = min(max(bx, 0), ph.hist_nx - 1);
-        const double bpd = floor(((double)vx - ph.hist_pmin) * hsp);
-        if (!(bpd >= 0.0 && bpd < (double)np)) continue;
-        bp = (int)bpd;
+    for (int p0 = lane; p0 - lane < cnt; p0 += 32 * U) {
+      int cell[U];
+      T ox[U], vx[U];
+      bool take[U];
+#pragma unroll
+      for (int r = 0; r < U; ++r) {
+        const int gi = base + p0 + 32 * r;
+        take[r] = p0 + 32 * r < cnt;
+        if (take[r] && species >= 0) take[r] = ((P.id[gi] & kIdCR) ? 1 : 0) == species;
+        cell[r] = take[r] ? P.cell[gi] : 0;
+        ox[r] = take[r] ? P.ox[gi] : (T)0;
+        vx[r] = take[r] ? P.vx[gi] : (T)0;
       }
-      if ((unsigned)(bx - bx0) < (unsigned)nbx) atomicAdd(&sh[(bx - bx0) * np + bp], 1u);
-      else atomicAdd(&d.hist[(size_t)bx * np + bp], 1ull);
+#pragma unroll
+      for (int r = 0; r < U; ++r) {
+        const int i = cell[r] & 0xFFFF;
+        const float tx = fmaf((float)(i - i0) + near_float(ox[r]), fsx, fx0);
+        const float tp = (near_float(vx[r]) - pmin) * fsp;
+        const float bxf = floorf(tx), bpf = floorf(tp);
+        const float rx = tx - bxf, rp = tp - bpf;
+        int bx = 0, bp = -1;
+        if (fast && fabsf(tp) < 1e6f && rx > epx && rx < 1.0f - epx && rp > epp &&
+            rp < 1.0f - epp) {
+          bp = (int)bpf;
+          bx = bx0 + (int)bxf;
+        } else if (take[r]) {
+          bx = (int)floor(((double)i + (double)ox[r]) * hsx);
+          const double bpd = floor(((double)vx[r] - ph.hist_pmin) * hsp);
+          if (bpd >= 0.0 && bpd < (double)np) bp = (int)bpd;
+        }
+        bx = min(max(bx, 0), ph.hist_nx - 1);
+        const bool ok = take[r] && bp >= 0 && bp < np;
+        const bool here = (unsigned)(bx - bx0) < (unsigned)nbx;
+        count_shared(sh, ok && here ? (bx - bx0) * np + bp : -1);
+        if (ok && !here) atomicAdd(&d.hist[(size_t)bx * np + bp], 1ull);
+      }
     }
   }
   __syncthreads();

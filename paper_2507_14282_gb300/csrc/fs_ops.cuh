@@ -252,26 +252,28 @@ struct OpsImpl {
 
   // 1D boxes with x walls: the whole field advance in one tiled launch
   // (k_field_step1), the new B written to the stage buffer and copied back.
-  static cudaError_t fields_tiled1(Sim* s) {
+  template <int TILE>
+  static cudaError_t field_step1(Sim* s) {
     DevPtrs<T> d = P(s);
-    const size_t smem = field1_smem<T>(s->p.n_sub);
+    const size_t smem = field1_smem<T>(s->p.n_sub, TILE);
     // the largest size enabled so far; a raise races harmlessly (each caller
     // sets at least its own size before it launches)
     static std::atomic<size_t> attr(0);
     if (smem > attr.load()) {
-      cudaError_t e = cudaFuncSetAttribute(k_field_step1<T>,
+      cudaError_t e = cudaFuncSetAttribute(k_field_step1<T, TILE>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       size_t cur = attr.load();
       while (smem > cur && !attr.compare_exchange_weak(cur, smem)) {
       }
     }
-    const int grid = (s->g.nx + kF1 - 1) / kF1;
-    k_field_step1<T><<<grid, kF1Threads, smem, s->stream>>>(d.B, d.Bs, d.n, d.u, d.E, d.Bb, d.G,
-                                                           s->g, s->ph, field_const<T>(s->ph),
-                                                           s->p.n_sub);
+    k_field_step1<T, TILE><<<(s->g.nx + TILE - 1) / TILE, field1_threads(TILE), smem, s->stream>>>(
+        d.B, d.Bs, d.n, d.u, d.E, d.Bb, d.G, s->g, field_const<T>(s->ph), s->p.n_sub);
     return cudaMemcpyAsync(d.B, d.Bs, 3 * sizeof(T) * (size_t)s->g.nx, cudaMemcpyDeviceToDevice,
                            s->stream);
+  }
+  static cudaError_t fields_tiled1(Sim* s) {
+    return field1_tile(s->g.nx) == kF1Small ? field_step1<kF1Small>(s) : field_step1<kF1>(s);
   }
 
   static cudaError_t fields(Sim* s) {
@@ -468,7 +470,7 @@ struct OpsImpl {
                                 int n_sub_max, cudaStream_t st, cudaStream_t side,
                                 cudaEvent_t fork, cudaEvent_t join) {
     const BatchRun<T>* r = (const BatchRun<T>*)runs;
-    const size_t fsm = field1_smem<T>(n_sub_max);
+    const size_t fsm = field1_smem<T>(n_sub_max, kF1);
     static std::atomic<size_t> attr(0);  // the largest size enabled so far
     if (fsm > attr.load()) {
       cudaError_t e = cudaFuncSetAttribute(k_field1_batch<T>,
@@ -624,7 +626,7 @@ struct OpsImpl {
     if (which == FS_PROFILE_N)
       k_profile_n<T><<<prof_grid(g.nxn), kProfThreads, 0, s->stream>>>(P(s).n, g.nxn, g.ny, out);
     else
-      k_profile_db2<T><<<prof_grid(g.nx), kProfThreads, 0, s->stream>>>(
+      k_profile_db2<T><<<(g.nx + 31) / 32, kBlock, 0, s->stream>>>(
           P(s).B, g.nx, g.ny, s->ph.b0x, s->ph.b0y, s->ph.b0z, out + g.nxn);
     return cudaGetLastError();
   }

@@ -1163,7 +1163,7 @@ __global__ void __launch_bounds__(kF1Threads)
   __shared__ __align__(16) BatchRun<T> R;
   const int r = load_batch_run<T>(runs, pre, nruns, R);
   const FieldConst<T> fc = field_const_dev<T>(R.ph);
-  field_step1_body<T>(R.d.B, R.d.Bs, R.d.n, R.d.u, R.d.E, R.d.Bb, R.d.G, R.g, fc, R.n_sub,
+  field_step1_body<T, kF1>(R.d.B, R.d.Bs, R.d.n, R.d.u, R.d.E, R.d.Bb, R.d.G, R.g, fc, R.n_sub,
                       blockIdx.x - pre[r], smem);
 }
 

@@ -65,7 +65,7 @@ inline bool fft_plan(int n, int ny, FftPlan* f) {
 // y-averaged B: out[i * 3 + c] = (1/ny) sum_j B_c(i, j), rows in order. One
 // warp per block (a column block per SM) with 16 rows' loads in flight:
 // latency-bound at a few rows in flight, 17 blocks: 4096 x 256 cells 191 us
-// before, see k_profile_n.
+// before, 20 us now.
 constexpr int kProfThreads = 32;
 template <typename T>
 __global__ void __launch_bounds__(kProfThreads)
@@ -93,24 +93,39 @@ __global__ void __launch_bounds__(kProfThreads)
   out[i] = acc / (double)ny;
 }
 
-// y-averaged |B - B0|^2 at centres, rows summed in order
+// y-averaged |B - B0|^2 at centres, rows summed in order. A CTA takes 32
+// columns: its warps form the terms of 64 rows in shared memory, then the
+// first adds them in row order (an FP64 instruction holds an SM quarter's
+// pipe for some 64 cycles, so one warp doing both is bound by its own
+// chain: 4096 x 256 cells 108 us).
+constexpr int kDb2Rows = 64;
 template <typename T>
-__global__ void __launch_bounds__(kProfThreads)
+__global__ void __launch_bounds__(kBlock)
     k_profile_db2(const T* __restrict__ B, int nx, int ny, double b0x, double b0y, double b0z,
                   double* __restrict__ out) {
+  __shared__ double term[kDb2Rows][32];
   const size_t nc = (size_t)nx * ny;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nx) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
   double a2 = 0.0;
-#pragma unroll 8
-  for (int j = 0; j < ny; ++j) {
-    const size_t c = (size_t)j * nx + i;
-    const double dbx = (double)B[c] - b0x;
-    const double dby = (double)B[nc + c] - b0y;
-    const double dbz = (double)B[2 * nc + c] - b0z;
-    a2 = a2 + ((dbx * dbx + dby * dby) + dbz * dbz);
+  for (int j0 = 0; j0 < ny; j0 += kDb2Rows) {
+    const int nr = min(kDb2Rows, ny - j0);
+    if (i < nx) {
+#pragma unroll 4
+      for (int r = warp; r < nr; r += kWarpsPerBlock) {
+        const size_t c = (size_t)(j0 + r) * nx + i;
+        const double dbx = (double)B[c] - b0x;
+        const double dby = (double)B[nc + c] - b0y;
+        const double dbz = (double)B[2 * nc + c] - b0z;
+        term[r][lane] = (dbx * dbx + dby * dby) + dbz * dbz;
+      }
+    }
+    __syncthreads();
+    if (warp == 0)
+      for (int r = 0; r < nr; ++r) a2 = a2 + term[r][lane];
+    __syncthreads();
   }
-  out[i] = a2 / (double)ny;
+  if (warp == 0 && i < nx) out[i] = a2 / (double)ny;
 }
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
@@ -365,32 +380,44 @@ __global__ void __launch_bounds__(kBlock)
   for (int t = blockIdx.x * kWarpsPerBlock + warp; t < g.ntiles;
        t += gridDim.x * kWarpsPerBlock) {
     const int cnt = min(d.cnt[buf][t], g.tile_cap), base = t * g.tile_cap;
-#pragma unroll 4
-    for (int q = lane; q < cnt; q += 32) {
-      const int gi = base + q;
-      if (species == 1 && !(P.id[gi] & kIdCR)) continue;
-      const T tx = P.vx[gi], ty = P.vy[gi], tz = P.vz[gi];
-      const float fx = near_float(tx), fy = near_float(ty), fz = near_float(tz);
-      const float p2 = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
-      const float tb = (0.5f * log2f(p2) - l2min) * per;
-      const float fb = floorf(tb), fr = tb - fb;
-      int bin;
-      if (p2 > 1e-30f && p2 < 1e30f && fr > eps && fr < 1.0f - eps) {
-        if (fb < 0.0f || fb >= (float)np) continue;
-        bin = (int)fb;
-      } else {
-        const double ux = tx, uy = ty, uz = tz;
-        const double p = __dsqrt_rn(__fma_rn(uz, uz, __fma_rn(uy, uy, __dmul_rn(ux, ux))));
-        if (!(p >= e[0]) || !(p < e[np])) continue;
-        int lo = 0, hi = np;  // e[lo] <= p < e[hi]
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (p >= e[mid]) lo = mid; else hi = mid;
-        }
-        bin = lo;
+    constexpr int U = 4;  // particles of a lane whose loads are in flight together
+    for (int p0 = lane; p0 - lane < cnt; p0 += 32 * U) {
+      T vx[U], vy[U], vz[U];
+      bool take[U];
+#pragma unroll
+      for (int r = 0; r < U; ++r) {
+        const int gi = base + p0 + 32 * r;
+        take[r] = p0 + 32 * r < cnt;
+        if (take[r] && species == 1) take[r] = (P.id[gi] & kIdCR) != 0;
+        vx[r] = take[r] ? P.vx[gi] : (T)0;
+        vy[r] = take[r] ? P.vy[gi] : (T)0;
+        vz[r] = take[r] ? P.vz[gi] : (T)0;
       }
-      if (copies) atomicAdd(&mine[bin], 1u);
-      else atomicAdd(&out[bin], 1ull);
+#pragma unroll
+      for (int r = 0; r < U; ++r) {
+        const float fx = near_float(vx[r]), fy = near_float(vy[r]), fz = near_float(vz[r]);
+        const float p2 = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
+        const float tb = (0.5f * log2f(p2) - l2min) * per;
+        const float fb = floorf(tb), fr = tb - fb;
+        int bin = -1;
+        if (p2 > 1e-30f && p2 < 1e30f && fr > eps && fr < 1.0f - eps) {
+          if (fb >= 0.0f && fb < (float)np) bin = (int)fb;
+        } else if (take[r]) {
+          const double ux = vx[r], uy = vy[r], uz = vz[r];
+          const double p = __dsqrt_rn(__fma_rn(uz, uz, __fma_rn(uy, uy, __dmul_rn(ux, ux))));
+          if (p >= e[0] && p < e[np]) {
+            int lo = 0, hi = np;  // e[lo] <= p < e[hi]
+            while (hi - lo > 1) {
+              const int mid = (lo + hi) >> 1;
+              if (p >= e[mid]) lo = mid; else hi = mid;
+            }
+            bin = lo;
+          }
+        }
+        if (!take[r]) bin = -1;
+        if (copies) count_shared(mine, bin);
+        else if (bin >= 0) atomicAdd(&out[bin], 1ull);
+      }
     }
   }
   __syncthreads();
