@@ -47,10 +47,9 @@ bool push_tile_fits(const fs_params* p, int tx, int ty) {
 
 // Tile shape: the most cells (then the squarest tile) whose mean particle
 // count stays within 512 and whose push fits shared memory; tile sides
-// divide the box.
-void choose_tile(const fs_params* p, int* tx, int* ty) {
+// divide the box. *ref: that tile's cells.
+void choose_full_tile(const fs_params* p, int* tx, int* ty, long long* ref) {
   if (p->dim == 1) {
-    if (p->tile_x > 0) { *tx = p->tile_x; *ty = 1; return; }
     int best = 0;
     for (int c = 2; c <= 256 && c <= p->nx; ++c) {
       if (!divides(c, p->nx)) continue;
@@ -58,9 +57,9 @@ void choose_tile(const fs_params* p, int* tx, int* ty) {
     }
     *tx = best ? best : p->nx;
     *ty = 1;
+    *ref = *tx;
     return;
   }
-  if (p->tile_x > 0 && p->tile_y > 0) { *tx = p->tile_x; *ty = p->tile_y; return; }
   int bx = 0, by = 0;
   long long bestc = -1;
   for (int cy = 1; cy <= 32 && cy <= p->ny; ++cy) {
@@ -79,6 +78,42 @@ void choose_tile(const fs_params* p, int* tx, int* ty) {
     bx = 0;
     for (int cx = 2; cx <= p->nx; ++cx) if (divides(cx, p->nx)) { bx = cx; break; }
     by = 1;
+  }
+  *tx = bx;
+  *ty = by;
+  *ref = (long long)bx * by;
+}
+
+// The tile of a run: the caller's, else the full tile; in a box whose full
+// tiles occupy at most half of the GPU's SMs, tiles cut into equal parts of at
+// least 128 particles on average until there is one per SM (a CTA works on one tile at a
+// time: 512 cells of 32 particles in 32 tiles left 120 SMs idle and gave each
+// of the rest two rounds of particles, FP64 push 24 us per step). A cut tile
+// keeps the slots of the full one (*ref cells' worth), so that a density peak
+// that fitted before still does.
+void choose_tile(const fs_params* p, int* tx, int* ty, long long* ref) {
+  if (p->tile_x > 0 && (p->dim == 1 || p->tile_y > 0)) {
+    *tx = p->tile_x;
+    *ty = p->dim == 1 ? 1 : p->tile_y;
+    *ref = (long long)*tx * *ty;
+    return;
+  }
+  choose_full_tile(p, tx, ty, ref);
+  constexpr long long kSms = 152;
+  const long long cells = (long long)p->nx * p->ny;
+  if (*tx < 2 || 2 * (cells / *ref) > kSms) return;
+  int bx = *tx, by = *ty;
+  long long best = *ref;  // the largest part with a tile per SM, else the smallest
+  for (int cy = 1; cy <= *ty; ++cy) {
+    if (!divides(cy, *ty)) continue;
+    for (int cx = 2; cx <= *tx; ++cx) {
+      if (!divides(cx, *tx)) continue;
+      const long long c = (long long)cx * cy;
+      if (c * p->ppc < 128) continue;
+      const bool enough = cells / c >= kSms, had = cells / best >= kSms;
+      const bool squarer = c == best && abs(cx - 2 * cy) < abs(bx - 2 * by);
+      if (squarer || (had ? (enough && c > best) : c < best)) { best = c; bx = cx; by = cy; }
+    }
   }
   *tx = bx;
   *ty = by;
@@ -125,7 +160,8 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   memset(ph, 0, sizeof(*ph));
   memset(L, 0, sizeof(*L));
   int tx, ty;
-  choose_tile(p, &tx, &ty);
+  long long ref = 0;
+  choose_tile(p, &tx, &ty, &ref);
   if (tx < 2 || !divides(tx, p->nx)) return FS_EINVAL;
   if (p->dim == 2) {
     if (ty < 1 || !divides(ty, p->ny)) return FS_EINVAL;
@@ -143,13 +179,14 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   g->nty = p->ny / ty;
   g->ntiles = g->ntx * g->nty;
   const long long cells_per_tile = (long long)tx * ty;
-  long long cap = (long long)ceil(p->capacity_factor * (double)(cells_per_tile * p->ppc)) + 64;
+  long long cap = (long long)ceil(p->capacity_factor * (double)(ref * p->ppc)) + 64;
   cap = (cap + 31) / 32 * 32;
   if (cap > (1LL << 30)) return FS_EINVAL;
   g->tile_cap = (int)cap;
   g->cap_total = cap * g->ntiles;
   if (g->cap_total >= (1LL << 31) - 1) return FS_EINVAL;
   long long mpt = (long long)ceil(p->mover_fraction * (double)cap) + 32;
+  if (cells_per_tile < ref) mpt = std::max(mpt, cap);  // a cut tile may empty in one step
   mpt = (mpt + 31) / 32 * 32;
   if (mpt * g->ntiles >= (1LL << 31) - 1) return FS_EINVAL;
   g->mover_per_tile = (int)mpt;
@@ -205,6 +242,13 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
                                   : p->p_iso;
   ph->spec_np = p->spec_np;
 
+  // records of a step's injected particles: a row injects at most rate + 1 of
+  // each species
+  const int kinds = p->bc_x == FS_BC_FAUXSHOCK ? ph->inject_thermal + ph->cr_enable : 0;
+  const double recs = (floor(ph->rate) + 2.0) * kinds * p->ny;
+  if (!(recs < 2147483647.0)) return FS_EINVAL;
+  g->ninj = (int)recs;
+
   // device buffer layout
   const size_t T = (p->precision == FS_FP64) ? 8 : 4;
   const size_t A = (p->precision == FS_FP64) ? 8 : 4;
@@ -227,6 +271,7 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   parts(L->part[0], g->cap_total);
   parts(L->part[1], g->cap_total);
   parts(L->mov, g->mover_cap);
+  parts(L->injp, g->ninj);
   L->tile_base = take(4 * (size_t)g->ntiles);
   L->cnt[0] = take(4 * (size_t)g->ntiles);
   L->cnt[1] = take(4 * (size_t)g->ntiles);
@@ -340,22 +385,23 @@ int grid_blocks(long long n) {
 
 // Capture one step for each ping-pong parity on a private stream (the legacy
 // default stream cannot be captured); the graphs replay on the caller's stream.
-// Kernels one step launches: push, movers, injection (3), moments, the field
-// advance, step end. The field advance is one tiled launch in 1D boxes with
-// x walls, one per substep in FP32 2D boxes with x walls, else [FP64: Ohm
-// density terms], 2 x 4 x n_sub stage passes and the final Ohm (the same
-// choice as the field launcher makes).
+// Kernels one step launches: push, movers, injection (1, or 2 with many rows),
+// moments, the field advance, step end. Moments and field advance are one
+// tiled launch in 1D boxes with x walls; else the field advance is one launch
+// per substep in FP32 2D boxes with x walls, or [FP64: Ohm density terms],
+// 2 x 4 x n_sub stage passes and the final Ohm (the same choice as the field
+// launcher makes).
 long long launches_per_step(const Sim* s) {
-  const bool inj = s->g.bc_x == FS_BC_FAUXSHOCK && (s->ph.inject_thermal || s->ph.cr_enable);
+  const long long inj = s->g.ninj == 0 ? 0 : s->g.ninj <= 256 ? 1 : 2;
   const bool walls = s->g.bc_x != FS_BC_PERIODIC;
   long long fields;
   if (s->g.dim == 1 && walls && s->p.n_sub <= 16)
-    fields = 1;
+    fields = 0;  // with the moments
   else if (s->p.precision == FS_FP32 && s->g.dim == 2 && walls)
     fields = s->p.n_sub;
   else
     fields = (s->p.precision == FS_FP64 ? 1 : 0) + 8LL * s->p.n_sub + 1;
-  return 1 + 1 + (inj ? 3 : 0) + 1 + fields + 1;
+  return 1 + 1 + inj + 1 + fields + 1;
 }
 
 int build_graphs(Sim* s) {
@@ -364,9 +410,9 @@ int build_graphs(Sim* s) {
     return FS_ECUDA;
   if (!s->side && cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess)
     return FS_ECUDA;
-  if ((!s->ev_fork && cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess) ||
-      (!s->ev_join && cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess))
-    return FS_ECUDA;
+  for (cudaEvent_t* ev : {&s->ev_fork, &s->ev_draw, &s->ev_push, &s->ev_join})
+    if (!*ev && cudaEventCreateWithFlags(ev, cudaEventDisableTiming) != cudaSuccess)
+      return FS_ECUDA;
   if (!s->side2 && cudaStreamCreateWithFlags(&s->side2, cudaStreamNonBlocking) != cudaSuccess)
     return FS_ECUDA;
   if ((!s->ev_fork2 && cudaEventCreateWithFlags(&s->ev_fork2, cudaEventDisableTiming) != cudaSuccess) ||
@@ -413,14 +459,11 @@ void release_graphs(Sim* s) {
     cudaStreamDestroy(s->side);
     s->side = nullptr;
   }
-  if (s->ev_fork) {
-    cudaEventDestroy(s->ev_fork);
-    s->ev_fork = nullptr;
-  }
-  if (s->ev_join) {
-    cudaEventDestroy(s->ev_join);
-    s->ev_join = nullptr;
-  }
+  for (cudaEvent_t* ev : {&s->ev_fork, &s->ev_draw, &s->ev_push, &s->ev_join})
+    if (*ev) {
+      cudaEventDestroy(*ev);
+      *ev = nullptr;
+    }
   if (s->side2) {
     cudaStreamDestroy(s->side2);
     s->side2 = nullptr;
@@ -1110,20 +1153,16 @@ size_t batch_rec_bytes(int precision) {
 size_t batch_map_offset(int nruns, int precision) {
   return up(2 * (size_t)nruns * batch_rec_bytes(precision), kAlign);
 }
-// the block prefixes of the batched step tail (movers, moments, field tiles)
+// the block prefixes of the batched step tail (movers, field tiles)
 size_t batch_pre_offset(int nruns, int precision) {
   return up(batch_map_offset(nruns, precision) + sizeof(int2) * (size_t)kBatchMaxCtas, kAlign);
 }
 size_t batch_table_bytes(int nruns, int precision) {
-  return batch_pre_offset(nruns, precision) + 3 * sizeof(int) * ((size_t)nruns + 1);
+  return batch_pre_offset(nruns, precision) + 2 * sizeof(int) * ((size_t)nruns + 1);
 }
 // blocks of the per-run step kernels the batched tail replaces (as step_rest
 // and the 1D field launcher size them)
 int movers_blocks(const Sim& s) { return std::min((s.g.ntiles + 7) / 8, 152 * 16); }
-int moments_blocks(const Sim& s) {
-  const long long nn = (long long)s.g.nxn * s.g.ny;
-  return (int)std::max(1LL, std::min((nn + 255) / 256, 152LL * 16));
-}
 int field1_blocks(const Sim& s) { return (s.g.nx + 63) / 64; }
 // runs whose whole step tail the batched kernels cover: 1D boxes with x
 // walls and the one-launch field advance
@@ -1140,6 +1179,8 @@ struct fs_batch {
   std::vector<cudaStream_t> branch;
   std::vector<cudaEvent_t> join;
   cudaEvent_t fork = nullptr;
+  cudaStream_t draw = nullptr;  // the batched injection draws, beside the push
+  cudaEvent_t drawn = nullptr;
   char* table = nullptr;
   size_t rec = 0;
   int2* map = nullptr;
@@ -1155,7 +1196,7 @@ struct fs_batch {
   const Ops* ops = nullptr;
   int parity = 0;  // steps taken, mod 2
   bool tail_batched = false;  // the step tail runs as one launch per kernel
-  int nblk[3] = {0, 0, 0};    // blocks of the batched movers, moments, field tiles
+  int nblk[2] = {0, 0};       // blocks of the batched movers, field tiles
   int n_sub_max = 1;
   int* pre = nullptr;         // their block prefixes in the table
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -1170,10 +1211,16 @@ cudaError_t batch_enqueue(fs_batch* b, int p, cudaStream_t st) {
   const int nr = (int)b->runs.size();
   cudaError_t e = cudaSuccess;
   const int nc = (int)b->classes.size();
+  if ((e = cudaEventRecord(b->fork, st)) != cudaSuccess) return e;
+  if (b->tail_batched) {  // the injection's draws beside the push
+    if ((e = cudaStreamWaitEvent(b->draw, b->fork, 0)) != cudaSuccess) return e;
+    if ((e = b->ops->batch_draw(b->table + (size_t)p * nr * b->rec, nr, b->draw)) != cudaSuccess)
+      return e;
+    if ((e = cudaEventRecord(b->drawn, b->draw)) != cudaSuccess) return e;
+  }
   if (nc > 1 && (int)b->branch.size() >= nc) {
     // the classes' push launches side by side (one branch each), so that one
     // launch's last CTAs overlap the others'
-    if ((e = cudaEventRecord(b->fork, st)) != cudaSuccess) return e;
     for (int k = 0; k < nc; ++k) {
       const auto& c = b->classes[k];
       cudaStream_t bs = b->branch[k];
@@ -1193,9 +1240,11 @@ cudaError_t batch_enqueue(fs_batch* b, int p, cudaStream_t st) {
       if (e != cudaSuccess) return e;
     }
   }
-  if (b->tail_batched)
+  if (b->tail_batched) {
+    if ((e = cudaStreamWaitEvent(st, b->drawn, 0)) != cudaSuccess) return e;
     return b->ops->batch_rest(b->table + (size_t)p * nr * b->rec, b->pre, nr, b->nblk,
                               b->n_sub_max, st, b->branch[0], b->fork, b->join[0]);
+  }
   if ((e = cudaEventRecord(b->fork, st)) != cudaSuccess) return e;
   const int K = (int)b->branch.size();
   for (int k = 0; k < K; ++k)
@@ -1204,7 +1253,7 @@ cudaError_t batch_enqueue(fs_batch* b, int p, cudaStream_t st) {
     Sim* s = &b->runs[r]->sim;
     cudaStream_t user = s->stream;
     s->stream = b->branch[r % K];
-    e = s->ops->step_rest(s, (b->cur0[r] + p) & 1, nullptr);
+    e = s->ops->step_rest(s, (b->cur0[r] + p) & 1, nullptr, false);
     s->stream = user;
     if (e != cudaSuccess) return e;
   }
@@ -1397,7 +1446,7 @@ int fs_batch_init(fs_handle* const* runs, int nruns, void* table_dev, size_t tab
   b->pre = (int*)(b->table + batch_pre_offset(nruns, s0.p.precision));
   std::vector<char> host(need, 0);
   std::vector<int2> map;
-  std::vector<int> pre(3 * ((size_t)nruns + 1), 0);
+  std::vector<int> pre(2 * ((size_t)nruns + 1), 0);
   b->tail_batched = true;
   for (int r = 0; r < nruns; ++r) {
     const Sim& s = runs[r]->sim;
@@ -1410,10 +1459,9 @@ int fs_batch_init(fs_handle* const* runs, int nruns, void* table_dev, size_t tab
     b->n_sub_max = std::max(b->n_sub_max, s.p.n_sub);
     const int n1 = nruns + 1;
     pre[r + 1] = pre[r] + movers_blocks(s);
-    pre[n1 + r + 1] = pre[n1 + r] + moments_blocks(s);
-    pre[2 * n1 + r + 1] = pre[2 * n1 + r] + field1_blocks(s);
+    pre[n1 + r + 1] = pre[n1 + r] + field1_blocks(s);
   }
-  for (int k = 0; k < 3; ++k) b->nblk[k] = pre[(size_t)k * (nruns + 1) + nruns];
+  for (int k = 0; k < 2; ++k) b->nblk[k] = pre[(size_t)k * (nruns + 1) + nruns];
   for (size_t c = 0; c < classes.size(); ++c)  // the map in class order
     for (int r = 0; r < nruns; ++r)
       if (cls[r] == (int)c)
@@ -1427,7 +1475,9 @@ int fs_batch_init(fs_handle* const* runs, int nruns, void* table_dev, size_t tab
                 cudaSuccess &&
             cudaStreamSynchronize(b->stream) == cudaSuccess;
   const int K = std::min(nruns, kBatchBranches);
-  ok = ok && cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+  ok = ok && cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&b->drawn, cudaEventDisableTiming) == cudaSuccess &&
+       cudaStreamCreateWithFlags(&b->draw, cudaStreamNonBlocking) == cudaSuccess;
   for (int k = 0; ok && k < K; ++k) {
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
@@ -1492,6 +1542,8 @@ int fs_batch_destroy(fs_batch* b) {
   for (cudaStream_t st : b->branch) cudaStreamDestroy(st);
   for (cudaEvent_t ev : b->join) cudaEventDestroy(ev);
   if (b->fork) cudaEventDestroy(b->fork);
+  if (b->drawn) cudaEventDestroy(b->drawn);
+  if (b->draw) cudaStreamDestroy(b->draw);
   if (b->cap) cudaStreamDestroy(b->cap);
   cudaGetLastError();
   delete b;

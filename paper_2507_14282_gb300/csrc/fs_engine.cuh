@@ -11,9 +11,10 @@
 //              stayers written back to the tile's bucket and leavers to the
 //              mover list. Deposit partials per tile, no global atomics
 //              (except rare far movers).
-//   k_movers   leavers appended to their destination tile's bucket (in the
-//              captured step, beside the next three, which read no bucket).
-//   k_inject_* thermal inflow at x = L and the cosmic-ray source at x = 0.
+//   k_inject_* thermal inflow at x = L and the cosmic-ray source at x = 0, drawn
+//              into records (in the captured step, beside the push).
+//   k_movers   leavers and new particles appended to their tile's bucket (in the
+//              captured step, beside the next two, which read no bucket).
 //   k_moments  sum of the per-tile partials in a fixed order, wall
 //              half-volume correction, density floor, u = J / n
 //              (k_moments_ct: the same with the 2D tile shape compiled in).
@@ -336,9 +337,27 @@ __device__ __forceinline__ void movers_body(const DevPtrs<T>& d, const Geo& g, i
   }
 }
 
+// The step's new particles (drawn by inject_draw into d.I, cell -1: none) into
+// their tiles' buckets.
 template <typename T, int DIM>
-__global__ void k_movers(DevPtrs<T> d, Geo g, int out) {
-  movers_body<T, DIM>(d, g, out, blockIdx.x, gridDim.x);
+__device__ __forceinline__ void place_injected(const DevPtrs<T>& d, const Geo& g, int out, int blk,
+                                               int nblk) {
+  const Parts<T> I = d.I;
+  for (int k = blk * blockDim.x + threadIdx.x; k < g.ninj; k += nblk * blockDim.x) {
+    const int cell = I.cell[k];
+    if (cell < 0) continue;
+    const MoverRec<T> r{cell, I.ox[k], DIM == 2 ? I.oy[k] : (T)0, I.vx[k], I.vy[k], I.vz[k],
+                        I.id[k]};
+    const int dt = mover_dest(g, true, r);
+    mover_store<T, DIM>(d, g, out, true, dt, atomicAdd(&d.cnt[out][dt], 1), r);
+  }
+}
+
+// what: 1 the leavers of every tile, 2 the injected particles, 3 both
+template <typename T, int DIM>
+__global__ void k_movers(DevPtrs<T> d, Geo g, int out, int what) {
+  if (what & 1) movers_body<T, DIM>(d, g, out, blockIdx.x, gridDim.x);
+  if (what & 2) place_injected<T, DIM>(d, g, out, blockIdx.x, gridDim.x);
 }
 
 // Deposit of one particle into the far accumulators (global atomics).
@@ -377,28 +396,20 @@ __device__ __forceinline__ void deposit_far(const DevPtrs<T>& d, const Geo& g,
   }
 }
 
-// Place one new particle into the bucket of its tile; deposit it.
+// One new particle as record k of d.I (placed into its tile's bucket after the
+// push, place_injected), deposited into the far accumulators now.
 template <typename T, int DIM>
-__device__ __forceinline__ void place_new(const DevPtrs<T>& d, const Geo& g,
-                                          const Phys& ph, int buf, int i, int j,
-                                          T fx, T fy, T vx, T vy, T vz,
-                                          uint32_t id) {
-  const int t = (j / g.TY) * g.ntx + i / g.TX;
-  const int slot = atomicAdd(&d.cnt[buf][t], 1);
-  if (slot >= g.tile_cap) {
-    atomicSub(&d.cnt[buf][t], 1);
-    atomicOr(&d.ctr->status, kStatusCapacity);
-    return;
-  }
-  const int gi = t * g.tile_cap + slot;  // a tile's bucket starts at tile x capacity
-  const Parts<T> P = d.P[buf];
-  P.cell[gi] = (j << 16) | i;
-  P.ox[gi] = fx;
-  if (DIM == 2) P.oy[gi] = fy;
-  P.vx[gi] = vx;
-  P.vy[gi] = vy;
-  P.vz[gi] = vz;
-  P.id[gi] = id;
+__device__ __forceinline__ void record_new(const DevPtrs<T>& d, const Geo& g, const Phys& ph,
+                                           int k, int i, int j, T fx, T fy, T vx, T vy, T vz,
+                                           uint32_t id) {
+  const Parts<T> I = d.I;
+  I.cell[k] = (j << 16) | i;
+  I.ox[k] = fx;
+  if (DIM == 2) I.oy[k] = fy;
+  I.vx[k] = vx;
+  I.vy[k] = vy;
+  I.vz[k] = vz;
+  I.id[k] = id;
   const double ws = deposit_weight_scale<T>();
   const T wp = (T)(((id & kIdCR) ? ph.w_cr : ph.w_th) * ws);
   T dvx, dvy, dvz;  // the current uses the velocity
@@ -409,8 +420,11 @@ __device__ __forceinline__ void place_new(const DevPtrs<T>& d, const Geo& g,
 // ------------------------------------------------------------------------
 // Injection (Sec. 2). k_inject_count (one CTA): per transverse row the
 // accumulator advances by ppc u_sh dt/dx, its integer part is this step's
-// count; a scan over rows gives each row's first id. k_inject_gen: one thread
-// per (row, slot) draws the particle.
+// count; a scan over rows gives each row's first id. k_inject_draw: one thread
+// per (row, slot, species) draws the particle into its record and deposits it.
+// The draws need nothing of the step's push (a long chain of FP64 operations:
+// 17 us, 35 us for both species in one thread), so the captured step runs
+// them beside it; k_movers puts the records into the buckets.
 // ------------------------------------------------------------------------
 // The whole block (any multiple of 32 threads up to 1024) counts every row.
 __device__ __forceinline__ void inject_count_body(double* acc, int* rowcnt, int* rowoff, int ny,
@@ -462,159 +476,120 @@ static __global__ void k_inject_count(double* acc, int* rowcnt, int* rowoff, int
   inject_count_body(acc, rowcnt, rowoff, ny, rate, per_row_mult);
 }
 
-// New particle k of row j (thermal at x = L, then the cosmic rays at x = 0),
-// ids from `first` (next_id before this step's injection) in (row, slot)
+// New particle k of row j of one species (cr: a cosmic ray at x = 0, else
+// thermal at x = L) into record rec (cell -1 when the row has fewer), ids from
+// `first` (next_id before this step's injection) in (row, thermal, cosmic ray)
 // order; counts and energy added to the caller's l_inj, l_e.
 template <typename T, int DIM>
-__device__ __forceinline__ void inject_one(const DevPtrs<T>& d, const Geo& g, const Phys& ph,
-                                           int buf, const int* rowcnt, const int* rowoff, int j,
-                                           int k, unsigned long long first, long long step,
-                                           long long& l_inj, double& l_e) {
-  if (j < g.ny) {
-    const int n = rowcnt[j];
-    if (k < n) {
-      const int nx = g.nx;
-      if (ph.inject_thermal) {
-        const unsigned long long num = first + rowoff[j] + k;
-        if (num > kIdMask) {
-          atomicOr(&d.ctr->status, kStatusIdOverflow);
-        } else {
-          const uint32_t pid = (uint32_t)num;
-          const Philox4 ra = draw4(ph.seed, pid, step, kPurposeInjA);
-          const Philox4 rb = draw4(ph.seed, pid, step, kPurposeInjB);
-          double g0, g1, g2, g3;
-          gauss2(u01(ra.x[0]), u01(ra.x[1]), &g0, &g1);
-          gauss2(u01(ra.x[2]), u01(ra.x[3]), &g2, &g3);
-          const double vx = __dsub_rn(__dmul_rn(ph.vth, g0), ph.mach_a);
-          const double vy = __dmul_rn(ph.vth, g1);
-          const double vz = __dmul_rn(ph.vth, g2);
-          const double X = __dsub_rn(
-              (double)nx, __dmul_rn(__dmul_rn(u01(rb.x[0]), fabs(vx)), ph.dtdx));
-          const double ix = floor(X);
-          int i = (int)ix;
-          double fx = __dsub_rn(X, ix);
-          if (i >= nx) { i = nx - 1; fx = Num<double>::offmax; }
-          if (i < 0) { i = 0; fx = 0.0; }
-          if (fx >= 1.0) fx = Num<double>::offmax;
-          const double fy = (DIM == 2) ? u01(rb.x[1]) : 0.0;
-          T ft = (T)fx;
-          if (ft >= (T)1) ft = Num<T>::offmax;
-          T fyt = (T)fy;
-          if (fyt >= (T)1) fyt = Num<T>::offmax;
-          double ux = vx, uy = vy, uz = vz;  // stored as u = gamma v
-          if (ph.c2inv > 0.0) {
-            const double gv = gamma_v(vx, vy, vz, ph.c2inv);
-            ux = __dmul_rn(vx, gv); uy = __dmul_rn(vy, gv); uz = __dmul_rn(vz, gv);
-          }
-          place_new<T, DIM>(d, g, ph, buf, i, j, ft, fyt, (T)ux, (T)uy, (T)uz, pid);
-          ++l_inj;
-          l_e = __dadd_rn(l_e, kinetic(ph.w_th, ux, uy, uz, ph.cellvol, ph.c2inv));
-        }
-      }
-      if (ph.cr_enable) {
-        const int thermal_n = ph.inject_thermal ? n : 0;
-        const unsigned long long num = first + rowoff[j] + thermal_n + k;
-        if (num > kIdMask) {
-          atomicOr(&d.ctr->status, kStatusIdOverflow);
-        } else {
-          const uint32_t pid = (uint32_t)num;
-          const Philox4 rc = draw4(ph.seed, pid, step, kPurposeInjCR);
-          // speed p_iso / gamma(p_iso) in the downstream frame (p_iso without c)
-          const double a = __ddiv_rn(ph.u_cr, ph.p_iso_v);
-          const double mu =
-              __dadd_rn(a, __dmul_rn(__dsub_rn(1.0, a), __dsqrt_rn(u01(rc.x[0]))));
-          const double sn = __dsqrt_rn(__dsub_rn(1.0, __dmul_rn(mu, mu)));
-          double c, s;
-          fs_sincos2pi(u01(rc.x[1]), &c, &s);
-          const double ws = __dmul_rn(ph.p_iso_v, sn);
-          const double vx = __dsub_rn(__dmul_rn(ph.p_iso_v, mu), ph.u_cr);
-          const double vy = __dmul_rn(ws, c);
-          const double vz = __dmul_rn(ws, s);
-          const double X = __dmul_rn(__dmul_rn(u01(rc.x[2]), vx), ph.dtdx);
-          const double ix = floor(X);
-          int i = (int)ix;
-          double fx = __dsub_rn(X, ix);
-          if (i >= nx) { i = nx - 1; fx = Num<double>::offmax; }
-          if (i < 0) { i = 0; fx = 0.0; }
-          if (fx >= 1.0) fx = Num<double>::offmax;
-          const double fy = (DIM == 2) ? u01(rc.x[3]) : 0.0;
-          T ft = (T)fx;
-          if (ft >= (T)1) ft = Num<T>::offmax;
-          T fyt = (T)fy;
-          if (fyt >= (T)1) fyt = Num<T>::offmax;
-          double ux = vx, uy = vy, uz = vz;  // stored as u = gamma v
-          if (ph.c2inv > 0.0) {
-            const double gv = gamma_v(vx, vy, vz, ph.c2inv);
-            ux = __dmul_rn(vx, gv); uy = __dmul_rn(vy, gv); uz = __dmul_rn(vz, gv);
-          }
-          place_new<T, DIM>(d, g, ph, buf, i, j, ft, fyt, (T)ux, (T)uy, (T)uz,
-                            pid | kIdCR);
-          ++l_inj;
-          l_e = __dadd_rn(l_e, kinetic(ph.w_cr, ux, uy, uz, ph.cellvol, ph.c2inv));
-        }
-      }
-    }
+__device__ __forceinline__ void inject_draw(const DevPtrs<T>& d, const Geo& g, const Phys& ph,
+                                            const int* rowcnt, const int* rowoff, int j, int k,
+                                            bool cr, int rec, unsigned long long first,
+                                            long long step, long long& l_inj, double& l_e) {
+  const int n = rowcnt[j], nx = g.nx;
+  const unsigned long long num = first + rowoff[j] + k + (cr && ph.inject_thermal ? n : 0);
+  if (k >= n || num > kIdMask) {
+    if (k < n) atomicOr(&d.ctr->status, kStatusIdOverflow);
+    d.I.cell[rec] = -1;
+    return;
   }
+  const uint32_t pid = (uint32_t)num;
+  double vx, vy, vz, X, fy;
+  if (!cr) {
+    const Philox4 ra = draw4(ph.seed, pid, step, kPurposeInjA);
+    const Philox4 rb = draw4(ph.seed, pid, step, kPurposeInjB);
+    double g0, g1, g2, g3;
+    gauss2(u01(ra.x[0]), u01(ra.x[1]), &g0, &g1);
+    gauss2(u01(ra.x[2]), u01(ra.x[3]), &g2, &g3);
+    vx = __dsub_rn(__dmul_rn(ph.vth, g0), ph.mach_a);
+    vy = __dmul_rn(ph.vth, g1);
+    vz = __dmul_rn(ph.vth, g2);
+    X = __dsub_rn((double)nx, __dmul_rn(__dmul_rn(u01(rb.x[0]), fabs(vx)), ph.dtdx));
+    fy = u01(rb.x[1]);
+  } else {
+    const Philox4 rc = draw4(ph.seed, pid, step, kPurposeInjCR);
+    // speed p_iso / gamma(p_iso) in the downstream frame (p_iso without c)
+    const double a = __ddiv_rn(ph.u_cr, ph.p_iso_v);
+    const double mu = __dadd_rn(a, __dmul_rn(__dsub_rn(1.0, a), __dsqrt_rn(u01(rc.x[0]))));
+    const double sn = __dsqrt_rn(__dsub_rn(1.0, __dmul_rn(mu, mu)));
+    double c, s;
+    fs_sincos2pi(u01(rc.x[1]), &c, &s);
+    const double ws = __dmul_rn(ph.p_iso_v, sn);
+    vx = __dsub_rn(__dmul_rn(ph.p_iso_v, mu), ph.u_cr);
+    vy = __dmul_rn(ws, c);
+    vz = __dmul_rn(ws, s);
+    X = __dmul_rn(__dmul_rn(u01(rc.x[2]), vx), ph.dtdx);
+    fy = u01(rc.x[3]);
+  }
+  const double ix = floor(X);
+  int i = (int)ix;
+  double fx = __dsub_rn(X, ix);
+  if (i >= nx) { i = nx - 1; fx = Num<double>::offmax; }
+  if (i < 0) { i = 0; fx = 0.0; }
+  if (fx >= 1.0) fx = Num<double>::offmax;
+  T ft = (T)fx;
+  if (ft >= (T)1) ft = Num<T>::offmax;
+  T fyt = (DIM == 2) ? (T)fy : (T)0;
+  if (fyt >= (T)1) fyt = Num<T>::offmax;
+  if (ph.c2inv > 0.0) {  // stored as u = gamma v
+    const double gv = gamma_v(vx, vy, vz, ph.c2inv);
+    vx = __dmul_rn(vx, gv); vy = __dmul_rn(vy, gv); vz = __dmul_rn(vz, gv);
+  }
+  record_new<T, DIM>(d, g, ph, rec, i, j, ft, fyt, (T)vx, (T)vy, (T)vz, cr ? pid | kIdCR : pid);
+  ++l_inj;
+  l_e = __dadd_rn(l_e, kinetic(cr ? ph.w_cr : ph.w_th, vx, vy, vz, ph.cellvol, ph.c2inv));
 }
 
+// Draws of thread `id` of `nthreads`: record rec = (row j, slot k, species)
 template <typename T, int DIM>
-__global__ void k_inject_gen(DevPtrs<T> d, Geo g, Phys ph, int buf,
-                             const int* rowcnt, const int* rowoff, int maxk) {
+__device__ __forceinline__ void inject_draws(const DevPtrs<T>& d, const Geo& g, const Phys& ph,
+                                             int id, int nthreads) {
   const long long step = d.ctr->step;
-  const int gidx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = gidx / maxk, k = gidx % maxk;
-  __shared__ unsigned long long s_first;
-  if (threadIdx.x == 0) s_first = d.ctr->next_id;
-  __syncthreads();
-  const unsigned long long first = s_first;
+  const unsigned long long first = d.ctr->next_id;
+  const int* rowcnt = d.inj;
+  const int* rowoff = rowcnt + g.ny;
+  const int both = ph.inject_thermal && ph.cr_enable;
+  const int per = g.ninj / g.ny, maxk = both ? per / 2 : per;
   long long l_inj = 0;
   double l_e = 0.0;
-  inject_one<T, DIM>(d, g, ph, buf, rowcnt, rowoff, j, k, first, step, l_inj, l_e);
+  for (int r = id; r < g.ninj; r += nthreads) {
+    const int j = r / per, q = r - j * per;
+    const bool cr = both ? q >= maxk : !ph.inject_thermal;
+    inject_draw<T, DIM>(d, g, ph, rowcnt, rowoff, j, both && cr ? q - maxk : q, cr, r, first, step,
+                        l_inj, l_e);
+  }
   if (l_inj) {
     atomicAdd(&d.ctr->injected, (unsigned long long)l_inj);
     atomicAdd(&d.ctr->injected_energy, l_e);
   }
 }
 
-// The injection of one run by one whole block: the row counts (as
-// k_inject_count), every (row, slot) draw (as k_inject_gen) and the id
-// commit (as k_inject_commit), with block barriers between them.
+template <typename T, int DIM>
+__global__ void __launch_bounds__(64) k_inject_draw(DevPtrs<T> d, Geo g, Phys ph) {
+  inject_draws<T, DIM>(d, g, ph, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// The row counts and the draws of one run by one block.
 template <typename T, int DIM>
 __device__ __forceinline__ void inject_run_block(const DevPtrs<T>& d, const Geo& g,
-                                                 const Phys& ph, int buf) {
-  const int mult = (ph.inject_thermal ? 1 : 0) + (ph.cr_enable ? 1 : 0);
-  int* rowcnt = d.inj;
-  int* rowoff = rowcnt + g.ny;
-  inject_count_body(d.acc, rowcnt, rowoff, g.ny, ph.rate, mult);
-  __shared__ unsigned long long s_first;
-  __shared__ long long s_step;
-  if (threadIdx.x == 0) {
-    s_first = d.ctr->next_id;
-    s_step = d.ctr->step;
-  }
+                                                 const Phys& ph) {
+  inject_count_body(d.acc, d.inj, d.inj + g.ny, g.ny, ph.rate,
+                    (ph.inject_thermal ? 1 : 0) + (ph.cr_enable ? 1 : 0));
   __syncthreads();
-  const int maxk = (int)ph.rate + 2;
-  long long l_inj = 0;
-  double l_e = 0.0;
-  for (int gidx = threadIdx.x; gidx < g.ny * maxk; gidx += blockDim.x)
-    inject_one<T, DIM>(d, g, ph, buf, rowcnt, rowoff, gidx / maxk, gidx % maxk, s_first,
-                       s_step, l_inj, l_e);
-  if (l_inj) {
-    atomicAdd(&d.ctr->injected, (unsigned long long)l_inj);
-    atomicAdd(&d.ctr->injected_energy, l_e);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) d.ctr->next_id += rowoff[g.ny];
+  inject_draws<T, DIM>(d, g, ph, threadIdx.x, blockDim.x);
+}
+template <typename T, int DIM>
+__global__ void __launch_bounds__(kBlock) k_inject_run(DevPtrs<T> d, Geo g, Phys ph) {
+  inject_run_block<T, DIM>(d, g, ph);
 }
 
-// end of a step: advance the device step counter
-static __global__ void k_step_end(Counters* ctr) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) ctr->step += 1;
+// end of a step: advance the device step counter and next_id (past the step's
+// injected particles)
+__device__ __forceinline__ void step_end(Counters* ctr, const int* inj, const Geo& g) {
+  ctr->step += 1;
+  if (g.ninj) ctr->next_id += inj[2 * g.ny];
 }
-
-// advance next_id by this step's total (after k_inject_gen has read it)
-static __global__ void k_inject_commit(Counters* ctr, const int* rowoff, int ny) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) ctr->next_id += rowoff[ny];
+static __global__ void k_step_end(Counters* ctr, const int* inj, Geo g) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) step_end(ctr, inj, g);
 }
 
 // ------------------------------------------------------------------------
@@ -1055,6 +1030,23 @@ __device__ __forceinline__ FieldConst<T> field_const_dev(const Phys& ph) {
                        (T)ph.eta, (T)ph.h,   (T)ph.hh,  (T)ph.h6, ph.eta != 0.0 ? 1 : 0};
 }
 
+// Quantity c (n, Jx, Jy, Jz) at node i of a 1D box with x walls: the far sum,
+// then the partials of the tiles whose accumulators cover the node (tile tx:
+// nodes tx TX - 1 .. tx TX + TX + 1) in increasing order, wall nodes x2: the
+// sums of moments_body.
+template <typename T>
+__device__ __forceinline__ T moment1(const DevPtrs<T>& d, const Geo& g, int i, int c) {
+  using A = typename Num<T>::acc;
+  const int TX = g.TX, NA = TX + 3;
+  A s = ((const A*)d.far)[(size_t)c * g.nxn + i];
+  const int hi = min((i + 1) / TX, g.ntx - 1);
+  for (int tx = i >= 2 ? (i - 2) / TX : 0; tx <= hi; ++tx)
+    s += ((const A*)d.partial)[((size_t)tx * 4 + c) * NA + i - (tx * TX - 1)];
+  T v = acc_value(s);
+  if (i == 0 || i == g.nx) v = v * (T)2;
+  return v;
+}
+
 // E_y (comp 0) or E_z (comp 1) at a node of a 1D grid: the values ohm_e gives
 // there (no y differences; with j_ext = 0 its zero products drop out). bm, bp:
 // B_y, B_z of the node's left and right cells; bbx: B_x at the node. E_x is
@@ -1088,50 +1080,106 @@ __device__ __forceinline__ T ohm1_comp(int comp, T bmy, T bpy, T bmz, T bpz, T b
   return ez;
 }
 
-// A 1D tile in shared memory: L cells, L + 1 nodes. The block's two halves
-// (half threads each, a multiple of the warp) take one component each.
+// A 1D tile: L cells, L + 1 nodes; the block's two halves (half >= L + 1
+// threads each, a multiple of the warp) take one transverse component each,
+// a thread one cell and one node. What stays fixed over the stages and the
+// thread's own B and RK4 sum are in registers; the stage field S and, in FP64,
+// E_y and E_z at the nodes are in shared memory.
+template <typename T>
+struct Node1 {  // 1/n, B_x and u at a node
+  T inv, bbx, ux, uy, uz;
+};
 template <typename T>
 struct Tile1 {
-  int L, half, comp, l0;  // this thread's component and first element
-  T *Bx, *B, *Bs, *K;     // B_x [L]; B, stage B, RK4 sum of (y, z) [2][L]
-  T *E;                   // E_y, E_z [2][L + 1]
-  T *inv, *bbx, *u;       // per node: 1/n, B_x, u [3][L + 1]
+  int L, half, comp, a;
+  T* S;  // stage field: FP32 [2 buffers][2][L], FP64 [2][L]
+  T* E;  // FP64 only: E_y, E_z [2][L + 1]
+  Node1<T> n0, n1;  // the thread's node a, and (FP32) node a + 1
+  T b, k;           // B of the thread's component at cell a, the RK4 sum
+  __device__ __forceinline__ T* field() { return S; }  // [2][L] between substeps
 };
+// values of T a tile keeps in shared memory
+__host__ __device__ constexpr size_t tile1_words(size_t L, size_t tsz) {
+  return tsz == 4 ? 4 * L : 2 * L + 2 * (L + 1);
+}
+// threads of a block of two halves for a tile of L cells
+__host__ __device__ constexpr int tile1_threads(int L) { return 2 * ((L + 1 + 31) / 32 * 32); }
 
 // One RK4 substep (four stages of Ohm and Faraday) of a tile with n, u
-// frozen. At the tile's ends the node reads its end cell on both sides. Stage
-// s's input field is kept in keep[s] ([2][L] doubles each) if given.
+// frozen, K_y = dE_z/dx, K_z = -dE_y/dx. At the tile's ends a node reads its
+// end cell on both sides. Stage s's input field goes to keep[s] ([2][L]) if
+// given. FP32, latency-bound: a thread forms the E of both nodes of its cell,
+// so that a stage is one pass and one barrier on alternating buffers. FP64,
+// bound by its instruction count (an FP64 instruction holds an SM quarter's
+// pipe for 64 cycles): E once per node, in a pass of its own.
 template <typename T>
-__device__ __forceinline__ void tile1_substep(const Tile1<T>& t, const FieldConst<T>& fc,
-                                              double* keep) {
-  const int L = t.L, Ln = L + 1;
-  for (int stage = 1; stage <= 4; ++stage) {
-    const T* By = (stage == 1) ? t.B : t.Bs;
-    const T* Bz = By + L;
-    if (keep)
-      for (int a = t.l0; a < L; a += t.half)
-        keep[(size_t)(2 * (stage - 1) + t.comp) * L + a] = (double)By[t.comp * L + a];
-    for (int a = t.l0; a < Ln; a += t.half) {
-      const int m = max(a - 1, 0), p = min(a, L - 1);
-      t.E[t.comp * Ln + a] = ohm1_comp<T>(t.comp, By[m], By[p], Bz[m], Bz[p], t.bbx[a], t.inv[a],
-                                          t.u[a], t.u[Ln + a], t.u[2 * Ln + a], fc);
+__device__ __forceinline__ void tile1_substep(Tile1<T>& t, const FieldConst<T>& fc, T* keep) {
+  const int L = t.L, Ln = L + 1, a = t.a;
+  const bool cell = a < L;
+  T bs = t.b;
+  if constexpr (sizeof(T) == 4) {
+    const int m = max(a - 1, 0), p = min(a + 1, L - 1);
+#pragma unroll
+    for (int stage = 1; stage <= 4; ++stage) {
+      const T* y = t.S + ((stage - 1) & 1) * 2 * L;
+      T* d = t.S + (stage & 1) * 2 * L;
+      if (cell) {
+        const T ym = y[m], yc = y[a], yp = y[p];
+        const T zm = y[L + m], zc = y[L + a], zp = y[L + p];
+        if (keep) keep[(2 * (stage - 1) + t.comp) * L + a] = t.comp ? zc : yc;
+        const int oc = 1 - t.comp;  // B_y needs E_z, B_z needs E_y
+        const T e0 = ohm1_comp<T>(oc, ym, yc, zm, zc, t.n0.bbx, t.n0.inv, t.n0.ux, t.n0.uy,
+                                  t.n0.uz, fc);
+        const T e1 = ohm1_comp<T>(oc, yc, yp, zc, zp, t.n1.bbx, t.n1.inv, t.n1.ux, t.n1.uy,
+                                  t.n1.uz, fc);
+        const T dx = (e1 - e0) * fc.idx;
+        rk4_stage<T>(stage, t.comp ? -dx : dx, t.k, bs, t.b, fc.h, fc.hh, fc.h6);
+        d[t.comp * L + a] = stage == 4 ? t.b : bs;
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    // K_y = dE_z/dx, K_z = -dE_y/dx
-    const T* Eo = t.E + (t.comp ? 0 : Ln);
-    for (int a = t.l0; a < L; a += t.half) {
-      const T dx = (Eo[a + 1] - Eo[a]) * fc.idx;
-      const int k = t.comp * L + a;
-      rk4_stage<T>(stage, t.comp ? -dx : dx, t.K[k], t.Bs[k], t.B[k], fc.h, fc.hh, fc.h6);
+  } else {
+    const int m = max(a - 1, 0), p = min(a, L - 1);
+    T* own = t.S + t.comp * L + a;
+    const T* eo = t.E + (t.comp ? 0 : Ln) + a;
+#pragma unroll
+    for (int stage = 1; stage <= 4; ++stage) {
+      const T* y = t.S;
+      if (keep && cell) keep[(2 * (stage - 1) + t.comp) * L + a] = *own;
+      if (a < Ln)
+        t.E[t.comp * Ln + a] = ohm1_comp<T>(t.comp, y[m], y[p], y[L + m], y[L + p], t.n0.bbx,
+                                            t.n0.inv, t.n0.ux, t.n0.uy, t.n0.uz, fc);
+      __syncthreads();
+      if (cell) {
+        const T dx = (eo[1] - eo[0]) * fc.idx;
+        rk4_stage<T>(stage, t.comp ? -dx : dx, t.k, bs, t.b, fc.h, fc.hh, fc.h6);
+        *own = stage == 4 ? t.b : bs;
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
 }
 
+// The full Ohm's law at a tile's node from its field y ([2][L]), the node's
+// cells m and p and its pressure term.
+template <typename T>
+__device__ __forceinline__ void tile1_ohm(const T* y, int L, int m, int p, const Node1<T>& n,
+                                          T pg, const FieldConst<T>& fc, T (&E)[3], T (&Bb)[3]) {
+  const T bmy = y[m], bpy = y[p], bmz = y[L + m], bpz = y[L + p];
+  Bb[0] = n.bbx;
+  Bb[1] = (T)0.5 * (bmy + bpy);
+  Bb[2] = (T)0.5 * (bmz + bpz);
+  const T dby = (bpy - bmy) * fc.idx, dbz = (bpz - bmz) * fc.idx;
+  ohm_e<T>((T)0, -dbz, dby, Bb[0], Bb[1], Bb[2], n.inv, pg, -(fc.te * (T)0), n.ux, n.uy, n.uz,
+           fc.jcr, fc.eta, fc.resist != 0, E[0], E[1], E[2]);
+}
+
 // ------------------------------------------------------------------------
-// The whole field advance of a 1D step with x walls (n_sub RK4 substeps,
-// then Ohm's E and Bbar for the next gather) in one launch: on a 1D grid
-// the separate passes are tens of tiny launches per step. A CTA owns TILE
+// The moments and the whole field advance of a 1D step with x walls (n, J, u
+// from the deposit, n_sub RK4 substeps, then Ohm's E and Bbar for the next
+// gather) in one launch: on a 1D grid the separate passes are tens of tiny
+// launches per step (the far sums, read by neighbouring tiles too, are cleared
+// at the step's end, step1_end). A CTA owns TILE
 // cells (and their left nodes; the last tile also node nx) and runs every
 // pass in shared memory over its cells plus field1_halo(n_sub) cells around
 // them, which it recomputes: each pass's stencil reaches one cell, so
@@ -1142,113 +1190,139 @@ __device__ __forceinline__ void tile1_substep(const Tile1<T>& t, const FieldCons
 // Bout (neighbouring tiles read Bin's cells), E, Bbar and the packed gather
 // block G at the owned nodes. Same per-element arithmetic as ohm_node /
 // faraday_cell (1D), so FP64 results are those of the separate passes.
-// A chain of 16 dependent passes: in FP64 each instruction holds an SM
-// quarter's pipe for some 64 cycles, so a pass costs its instruction count.
-// 1/n and the pressure term are formed once, B_x and E_x are left out of the
-// stages, and the y and z components go to different warps (8 + 4
-// operations per stage and thread instead of about 70 and a division).
+// A chain of dependent passes (tile1_substep): 1/n and the pressure term are
+// formed once, B_x and E_x are left out of the stages, the y and z components
+// go to different warps, and a thread keeps its node's terms in registers.
 // TILE 32 while that leaves SMs free (tile and halo fill two warps a
-// component), 64 beyond (less halo to recompute).
-__host__ __device__ inline int field1_halo(int n_sub) { return 4 * n_sub + 2; }
+// component), 64 beyond (less halo to recompute). 512 cells FP64 21.5 us
+// before.
+__host__ __device__ constexpr int field1_halo(int n_sub) { return 4 * n_sub + 2; }
 constexpr int kF1 = 64, kF1Small = 32;
-// threads of a component: the nodes of a TILE with the halo of two substeps
-constexpr int field1_threads(int tile) { return 2 * ((tile + 2 * 10 + 1 + 31) / 32 * 32); }
-constexpr int kF1Threads = field1_threads(kF1);
+constexpr int kF1MaxSub = 16;
+constexpr int field1_threads(int tile, int n_sub) {
+  return tile1_threads(tile + 2 * field1_halo(n_sub));
+}
 inline int field1_tile(int nx) { return nx <= 152 * kF1 ? kF1Small : kF1; }
 template <typename T>
 inline size_t field1_smem(int n_sub, int tile) {
   const size_t L = tile + 2 * (size_t)field1_halo(n_sub);
-  return sizeof(T) * (7 * L + 8 * (L + 1));
+  return sizeof(T) * (tile1_words(L, sizeof(T)) + 6 * (L + 1));
 }
 
 // Tile blk of the 1D field advance (the body of k_field_step1); smem is the
-// block's dynamic shared memory (field1_smem(n_sub, TILE) bytes).
+// block's dynamic shared memory (field1_smem(n_sub, TILE) bytes); at least
+// field1_threads(TILE, n_sub) threads.
 template <typename T, int TILE>
-__device__ __forceinline__ void field_step1_body(const T* __restrict__ Bin, T* __restrict__ Bout,
-                                                 const T* __restrict__ nN,
-                                                 const T* __restrict__ uN, T* __restrict__ Eo,
-                                                 T* __restrict__ Bbo, T* __restrict__ G,
-                                                 const Geo& g, const FieldConst<T>& fc,
-                                                 int n_sub, int blk, unsigned char* smem) {
+__device__ __forceinline__ void field_step1_body(const DevPtrs<T>& d, const Geo& g, T n_floor,
+                                                 const FieldConst<T>& fc, int n_sub, int blk,
+                                                 unsigned char* smem) {
   const int nx = g.nx, nxn = g.nxn, t0 = threadIdx.x, nt = blockDim.x;
   const int H = field1_halo(n_sub);
   const int c0 = blk * TILE, c1 = min(nx, c0 + TILE);
   const int lo = max(0, c0 - H), L = min(nx, c1 + H) - lo, Ln = L + 1;
+  auto owns_node = [&](int i) { return i >= c0 && (i < c1 || (i == nx && c1 == nx)); };
   Tile1<T> t;
   t.L = L;
-  t.half = nt / 2;
-  t.comp = t0 >= t.half;
-  t.l0 = t0 - t.comp * t.half;
-  t.Bx = (T*)smem;
-  t.B = t.Bx + L;
-  t.Bs = t.B + 2 * L;
-  t.K = t.Bs + 2 * L;
-  t.E = t.K + 2 * L;
-  t.inv = t.E + 2 * Ln;
-  t.bbx = t.inv + Ln;
-  t.u = t.bbx + Ln;
-  T* pg = t.u + 3 * Ln;  // the pressure term -(T_e dn/dx)
-  T* sn = t.E;           // the density, until the first stage writes E
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-    for (int a = t0; a < L; a += nt) t.Bx[c * L + a] = Bin[c * nx + lo + a];
-  for (int a = t0; a < Ln; a += nt) {
-    sn[a] = nN[lo + a];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) t.u[c * Ln + a] = uN[c * nxn + lo + a];
+  t.half = blockDim.x / 2;
+  t.comp = (int)threadIdx.x >= t.half;
+  const int a = t.a = threadIdx.x - t.comp * t.half;
+  t.S = (T*)smem;
+  t.E = t.S + 2 * L;
+  T* sn = t.S + tile1_words(L, sizeof(T));  // [Ln] n
+  T* sinv = sn + Ln;                        // [Ln] 1/n
+  T* spg = sinv + Ln;                       // [Ln] the pressure term -(T_e dn/dx)
+  T* su = spg + Ln;                         // [3][Ln] J, then u
+  const int gi = lo + a;                    // this thread's cell and node
+  T bxm = (T)0, bxc = (T)0, bxp = (T)0;
+  t.b = (T)0;
+  if (a < L) {
+    t.b = d.B[(t.comp + 1) * nx + gi];
+    t.S[t.comp * L + a] = t.b;
+    bxp = d.B[lo + min(a + 1, L - 1)];
   }
-  __syncthreads();
-  for (int a = t.l0; a < Ln; a += t.half) {
-    if (t.comp == 0) {
-      t.inv[a] = (T)1 / sn[a];
+  if (a < Ln) {
+    bxm = d.B[lo + max(a - 1, 0)];
+    bxc = d.B[lo + min(a, L - 1)];
+  }
+  for (int k = t0; k < 4 * Ln; k += nt) {
+    const int c = k / Ln, i = k - c * Ln;
+    const T v = moment1<T>(d, g, lo + i, c);
+    if (c == 0) {
+      const T n = v < n_floor ? n_floor : v;
+      sn[i] = n;
+      if (owns_node(lo + i)) d.n[lo + i] = n;
     } else {
-      const int gi = lo + a;
-      const int xp = ((gi + 1 > nx) ? 2 * nx - (gi + 1) : gi + 1) - lo;
-      const int xm = ((gi - 1 < 0) ? -(gi - 1) : gi - 1) - lo;
-      const T dnx = (sn[min(max(xp, 0), L)] - sn[min(max(xm, 0), L)]) * fc.hdx;
-      pg[a] = -(fc.te * dnx);
-      t.bbx[a] = (T)0.5 * (t.Bx[max(a - 1, 0)] + t.Bx[min(a, L - 1)]);
+      su[k - Ln] = v;
+      if (owns_node(lo + i)) d.J[(c - 1) * nxn + lo + i] = v;
     }
   }
   __syncthreads();
+  for (int k = t0; k < 5 * Ln; k += nt) {
+    const int c = k / Ln, i = k - c * Ln;
+    if (c < 4) {  // u = J / n, then 1/n
+      const T v = (c < 3 ? su[k] : (T)1) / sn[i];
+      if (c == 3) {
+        sinv[i] = v;
+      } else {
+        su[k] = v;
+        if (owns_node(lo + i)) d.u[c * nxn + lo + i] = v;
+      }
+    } else {
+      const int q = lo + i;
+      const int xp = ((q + 1 > nx) ? 2 * nx - (q + 1) : q + 1) - lo;
+      const int xm = ((q - 1 < 0) ? -(q - 1) : q - 1) - lo;
+      const T dnx = (sn[min(max(xp, 0), L)] - sn[min(max(xm, 0), L)]) * fc.hdx;
+      spg[i] = -(fc.te * dnx);
+    }
+  }
+  __syncthreads();
+  auto node = [&](int i, T bm, T bp) {
+    return Node1<T>{sinv[i], (T)0.5 * (bm + bp), su[i], su[Ln + i], su[2 * Ln + i]};
+  };
+  if (a < Ln) t.n0 = node(a, bxm, bxc);
+  if (sizeof(T) == 4 && a < L) t.n1 = node(a + 1, bxc, bxp);
   for (int sub = 0; sub < n_sub; ++sub) tile1_substep<T>(t, fc, nullptr);
-  for (int a = t0; a < Ln; a += nt) {
-    const int gi = lo + a;
-    if (gi < c0 || (gi >= c1 && !(gi == nx && c1 == nx))) continue;
-    const int im = max(a - 1, 0), ip = min(a, L - 1);
-    const T bmy = t.B[im], bpy = t.B[ip], bmz = t.B[L + im], bpz = t.B[L + ip];
-    const T bby = (T)0.5 * (bmy + bpy), bbz = (T)0.5 * (bmz + bpz);
-    const T dby = (bpy - bmy) * fc.idx, dbz = (bpz - bmz) * fc.idx;
-    T ex, ey, ez;
-    ohm_e<T>((T)0, -dbz, dby, t.bbx[a], bby, bbz, t.inv[a], pg[a], -(fc.te * (T)0), t.u[a],
-             t.u[Ln + a], t.u[2 * Ln + a], fc.jcr, fc.eta, fc.resist != 0, ex, ey, ez);
-    const T v[8] = {ex, ey, ez, t.bbx[a], bby, bbz, (T)0, (T)0};
+  if (t.comp == 0 && a < Ln && owns_node(gi)) {
+    T E[3], Bb[3];
+    tile1_ohm<T>(t.S, L, max(a - 1, 0), min(a, L - 1), t.n0, spg[a], fc, E, Bb);
+    const T v[8] = {E[0], E[1], E[2], Bb[0], Bb[1], Bb[2], (T)0, (T)0};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      Eo[c * nxn + gi] = v[c];
-      Bbo[c * nxn + gi] = v[3 + c];
+      d.E[c * nxn + gi] = E[c];
+      d.Bb[c * nxn + gi] = Bb[c];
     }
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      G[(size_t)gi * 8 + c] = v[c];                  // row 0
-      G[((size_t)(nx + 1) + gi) * 8 + c] = v[c];     // its ghost copy (row ny = 1)
+      d.G[(size_t)gi * 8 + c] = v[c];                  // row 0
+      d.G[((size_t)(nx + 1) + gi) * 8 + c] = v[c];     // its ghost copy (row ny = 1)
     }
   }
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-    for (int a = t0; a < L; a += nt) {
-      const int gi = lo + a;
-      if (gi >= c0 && gi < c1) Bout[c * nx + gi] = t.Bx[c * L + a];
-    }
+  if (a < L && gi >= c0 && gi < c1) {
+    d.Bs[(t.comp + 1) * nx + gi] = t.b;
+    if (t.comp == 0) d.Bs[gi] = bxc;
+  }
 }
 
 template <typename T, int TILE>
-__global__ void __launch_bounds__(field1_threads(TILE))
-    k_field_step1(const T* __restrict__ Bin, T* __restrict__ Bout, const T* __restrict__ nN,
-                  const T* __restrict__ uN, T* __restrict__ Eo, T* __restrict__ Bbo,
-                  T* __restrict__ G, Geo g, FieldConst<T> fc, int n_sub) {
+__global__ void __launch_bounds__(field1_threads(TILE, kF1MaxSub))
+    k_field_step1(DevPtrs<T> d, Geo g, T n_floor, FieldConst<T> fc, int n_sub) {
   extern __shared__ __align__(16) unsigned char smem[];
-  field_step1_body<T, TILE>(Bin, Bout, nN, uN, Eo, Bbo, G, g, fc, n_sub, blockIdx.x, smem);
+  field_step1_body<T, TILE>(d, g, n_floor, fc, n_sub, blockIdx.x, smem);
+}
+
+// The end of a 1D step whose field advance was field_step1: the new B back
+// from the stage buffer, the far sums cleared for the next step, the counters.
+template <typename T>
+__device__ __forceinline__ void step1_end(const DevPtrs<T>& d, const Geo& g, int blk, int nblk) {
+  using A = typename Num<T>::acc;
+  const int id = blk * blockDim.x + threadIdx.x, n = nblk * blockDim.x;
+  for (int k = id; k < 3 * g.nx; k += n) d.B[k] = d.Bs[k];
+  for (int k = id; k < 4 * g.nxn; k += n) ((A*)d.far)[k] = (A)0;
+  if (id == 0) step_end(d.ctr, d.inj, g);
+}
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_step1_end(DevPtrs<T> d, Geo g) {
+  step1_end<T>(d, g, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------------------------

@@ -71,6 +71,7 @@ struct Geo {
   int na;                   // accumulator nodes per tile: (TX+3)*(TY+3) or TX+3
   int nk;                   // sort keys per tile
   int push_ctas;            // cap on the push's persistent CTAs per SM (0: none)
+  int ninj;                 // records of a step's injected particles (0: no injection)
 };
 
 // Constants derived once on the host from fs_params (FP64; kernels cast).
@@ -89,7 +90,7 @@ struct Phys {
 
 // Byte offsets of every region inside the caller's device buffer.
 struct Layout {
-  size_t part[2][7], mov[7];
+  size_t part[2][7], mov[7], injp[7];
   size_t tile_base, cnt[2], mcnt;
   size_t B, Bs, Bsum, E, Es, Bb, G, n, u, J, pre;
   size_t partial, far, acc, inj, ctr, hist, prof, spec, twiddle;
@@ -99,7 +100,7 @@ struct Layout {
 // Typed device pointers (resolved from the layout).
 template <typename T>
 struct DevPtrs {
-  Parts<T> P[2], M;
+  Parts<T> P[2], M, I;  // buffers, mover list, injected particles
   int* tile_base;
   int* cnt[2];
   int* mcnt;      // movers written by each tile this step
@@ -169,7 +170,8 @@ struct Ops {
   cudaError_t (*ohm_final)(Sim*);
   // ev: NULL, or FS_NPHASES + 1 events recorded at the phase boundaries
   cudaError_t (*step)(Sim*, int in_buf, long long step, cudaEvent_t* ev);
-  cudaError_t (*step_rest)(Sim*, int in_buf, cudaEvent_t* ev);  // all but the push
+  // all but the push; drawn: the injection's draws are under way on the side stream
+  cudaError_t (*step_rest)(Sim*, int in_buf, cudaEvent_t* ev, bool drawn);
   // batched ensembles (k_push_batch)
   size_t (*batch_run_bytes)();
   void (*fill_batch_run)(const Sim*, int in_buf, int ncta, void* dst);
@@ -182,11 +184,13 @@ struct Ops {
   cudaError_t (*batch_setup)(int dim, int rel, int chunk, int txc, size_t smem, int* occ);
   cudaError_t (*push_batch)(int dim, int rel, int chunk, int txc, const void* runs,
                             const int2* cta_map, int ncta, size_t smem, cudaStream_t st);
-  // the rest of a batched step in one launch per kernel over every run (1D
-  // runs with x walls): pre holds three block prefixes over the runs (movers,
-  // moments, field tiles; nruns + 1 entries each), nblk their totals
-  // (the movers on stream side, between events fork and join, beside the
-  // injection, moments and field advance on st)
+  // a batched step of 1D runs with x walls in one launch per kernel over every
+  // run: the injection's draws (before or beside the push) ...
+  cudaError_t (*batch_draw)(const void* runs, int nruns, cudaStream_t st);
+  // ... and the rest: pre holds two block prefixes over the runs (movers, field
+  // tiles; nruns + 1 entries each), nblk their totals (the movers on stream
+  // side, between events fork and join, beside the moments and field advance
+  // on st)
   cudaError_t (*batch_rest)(const void* runs, const int* pre, int nruns, const int* nblk,
                             int n_sub_max, cudaStream_t st, cudaStream_t side,
                             cudaEvent_t fork, cudaEvent_t join);
@@ -232,10 +236,11 @@ struct Sim {
   // one captured step per ping-pong parity (replayed by fs_step)
   cudaGraphExec_t graph[2];
   cudaStream_t cap_stream;
-  // a second stream for the captured step: the movers run on it beside the
-  // injection, moments and field advance (fork / join events)
+  // a second stream for the captured step: the injection's draws run on it
+  // beside the push, the movers beside the moments and field advance (events:
+  // the step's start, the draws done, the push done, the movers done)
   cudaStream_t side;
-  cudaEvent_t ev_fork, ev_join;
+  cudaEvent_t ev_fork, ev_draw, ev_push, ev_join;
   // a third stream: the FP32 2D field substep's wall tile columns beside its
   // interior launch
   cudaStream_t side2;
@@ -265,6 +270,7 @@ inline DevPtrs<T> Sim::ptrs(int) const {
   d.P[0] = parts_at<T>(base, L.part[0]);
   d.P[1] = parts_at<T>(base, L.part[1]);
   d.M = parts_at<T>(base, L.mov);
+  d.I = parts_at<T>(base, L.injp);
   d.tile_base = (int*)(base + L.tile_base);
   d.cnt[0] = (int*)(base + L.cnt[0]);
   d.cnt[1] = (int*)(base + L.cnt[1]);

@@ -250,8 +250,11 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  // 1D boxes with x walls: the whole field advance in one tiled launch
-  // (k_field_step1), the new B written to the stage buffer and copied back.
+  // 1D boxes with x walls: moments and the whole field advance in one tiled
+  // launch (k_field_step1), the new B in the stage buffer until step1_end.
+  static bool one_launch_fields(const Sim* s) {
+    return s->g.dim == 1 && s->g.bc_x != FS_BC_PERIODIC && s->p.n_sub <= kF1MaxSub;
+  }
   template <int TILE>
   static cudaError_t field_step1(Sim* s) {
     DevPtrs<T> d = P(s);
@@ -267,17 +270,16 @@ struct OpsImpl {
       while (smem > cur && !attr.compare_exchange_weak(cur, smem)) {
       }
     }
-    k_field_step1<T, TILE><<<(s->g.nx + TILE - 1) / TILE, field1_threads(TILE), smem, s->stream>>>(
-        d.B, d.Bs, d.n, d.u, d.E, d.Bb, d.G, s->g, field_const<T>(s->ph), s->p.n_sub);
-    return cudaMemcpyAsync(d.B, d.Bs, 3 * sizeof(T) * (size_t)s->g.nx, cudaMemcpyDeviceToDevice,
-                           s->stream);
+    k_field_step1<T, TILE><<<(s->g.nx + TILE - 1) / TILE,
+                             field1_threads(TILE, s->p.n_sub), smem, s->stream>>>(
+        d, s->g, (T)s->ph.n_floor, field_const<T>(s->ph), s->p.n_sub);
+    return cudaGetLastError();
   }
   static cudaError_t fields_tiled1(Sim* s) {
     return field1_tile(s->g.nx) == kF1Small ? field_step1<kF1Small>(s) : field_step1<kF1>(s);
   }
 
   static cudaError_t fields(Sim* s) {
-    if (s->g.dim == 1 && s->g.bc_x != FS_BC_PERIODIC && s->p.n_sub <= 16) return fields_tiled1(s);
     if constexpr (sizeof(T) == 4) {
       if (s->g.dim == 2 && s->g.bc_x != FS_BC_PERIODIC) return fields_tiled(s);
     }
@@ -307,69 +309,90 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  // Everything of a step after the push (movers, injection, moments, field
-  // advance, step counter); ev as in step().
-  static cudaError_t step_rest(Sim* s, int in, cudaEvent_t* ev) {
+  // The draws of the step's injected particles, on st: one block counts and
+  // draws when it has few of them, else a count and a grid of draws.
+  static cudaError_t inject(Sim* s, cudaStream_t st) {
+    DevPtrs<T> d = P(s);
+    const Geo& g = s->g;
+    if (g.ninj <= kBlock) {
+      const int threads = (std::max(g.ninj, g.ny) + 31) / 32 * 32;
+      if (g.dim == 1) k_inject_run<T, 1><<<1, threads, 0, st>>>(d, g, s->ph);
+      else k_inject_run<T, 2><<<1, threads, 0, st>>>(d, g, s->ph);
+      return cudaGetLastError();
+    }
+    const int mult = (s->ph.inject_thermal ? 1 : 0) + (s->ph.cr_enable ? 1 : 0);
+    k_inject_count<<<1, 1024, 0, st>>>(d.acc, d.inj, d.inj + g.ny, g.ny, s->ph.rate, mult);
+    const int blocks = (g.ninj + 63) / 64;  // a draw is one long FP64 chain: spread them
+    if (g.dim == 1) k_inject_draw<T, 1><<<blocks, 64, 0, st>>>(d, g, s->ph);
+    else k_inject_draw<T, 2><<<blocks, 64, 0, st>>>(d, g, s->ph);
+    return cudaGetLastError();
+  }
+  static void movers(Sim* s, int out, int what, cudaStream_t st) {
+    const int tiles = (what & 1) ? (s->g.ntiles + 7) / 8 : 0;
+    const int recs = (what & 2) ? (s->g.ninj + kBlock - 1) / kBlock : 0;
+    const int grid = std::max(1, std::min(std::max(tiles, recs), 152 * 16));
+    if (s->g.dim == 1) k_movers<T, 1><<<grid, kBlock, 0, st>>>(P(s), s->g, out, what);
+    else k_movers<T, 2><<<grid, kBlock, 0, st>>>(P(s), s->g, out, what);
+  }
+
+  // Everything of a step after the push (movers, injection unless `drawn`,
+  // moments, field advance, step counter); ev as in step().
+  static cudaError_t step_rest(Sim* s, int in, cudaEvent_t* ev, bool drawn) {
     DevPtrs<T> d = P(s);
     const int out = 1 - in;
+    cudaError_t e = cudaSuccess;
     auto mark = [&](int k) {
       if (ev) cudaEventRecord(ev[k], s->stream);
     };
-    const int mg = std::min((s->g.ntiles + 7) / 8, 152 * 16);
-    // without phase events, the movers (buckets) run on the side stream
-    // beside the injection, moments and field advance, which read no bucket
-    const bool split = !ev && s->side && s->ev_fork && s->ev_join;
-    cudaStream_t mst = s->stream;
-    if (split) {
-      cudaError_t e0 = cudaEventRecord(s->ev_fork, s->stream);
-      if (e0 == cudaSuccess) e0 = cudaStreamWaitEvent(s->side, s->ev_fork, 0);
-      if (e0 != cudaSuccess) return e0;
-      mst = s->side;
+    if (drawn) {
+      // the movers (buckets) on the side stream, behind the draws and the push,
+      // beside the moments and field advance, which read no bucket; the
+      // moments need the draws' deposit
+      if ((e = cudaEventRecord(s->ev_push, s->stream)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(s->side, s->ev_push, 0)) != cudaSuccess) return e;
+      movers(s, out, s->g.ninj ? 3 : 1, s->side);
+      if ((e = cudaEventRecord(s->ev_join, s->side)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(s->stream, s->ev_draw, 0)) != cudaSuccess) return e;
+    } else {
+      movers(s, out, 1, s->stream);
+      mark(2);
+      if (s->g.ninj) {
+        if ((e = inject(s, s->stream)) != cudaSuccess) return e;
+        movers(s, out, 2, s->stream);
+      }
+      mark(3);
     }
-    if (s->g.dim == 1)
-      k_movers<T, 1><<<mg, kBlock, 0, mst>>>(d, s->g, out);
-    else
-      k_movers<T, 2><<<mg, kBlock, 0, mst>>>(d, s->g, out);
-    if (split) {
-      const cudaError_t e0 = cudaEventRecord(s->ev_join, s->side);
-      if (e0 != cudaSuccess) return e0;
-    }
-    mark(2);
-    if (s->g.bc_x == FS_BC_FAUXSHOCK && (s->ph.inject_thermal || s->ph.cr_enable)) {
-      int* rowcnt = d.inj;
-      int* rowoff = rowcnt + s->g.ny;
-      const int mult = (s->ph.inject_thermal ? 1 : 0) + (s->ph.cr_enable ? 1 : 0);
-      k_inject_count<<<1, 1024, 0, s->stream>>>(d.acc, rowcnt, rowoff, s->g.ny, s->ph.rate, mult);
-      const int maxk = (int)s->ph.rate + 2;
-      const long long nthreads = (long long)s->g.ny * maxk;
-      const int blocks = (int)((nthreads + kBlock - 1) / kBlock);
-      if (s->g.dim == 1)
-        k_inject_gen<T, 1><<<blocks, kBlock, 0, s->stream>>>(d, s->g, s->ph, out, rowcnt, rowoff, maxk);
-      else
-        k_inject_gen<T, 2><<<blocks, kBlock, 0, s->stream>>>(d, s->g, s->ph, out, rowcnt, rowoff, maxk);
-      k_inject_commit<<<1, 32, 0, s->stream>>>(d.ctr, rowoff, s->g.ny);
-    }
-    mark(3);
-    cudaError_t e = moments(s);
-    if (e != cudaSuccess) return e;
+    const bool one = one_launch_fields(s);
+    if (!one && (e = moments(s)) != cudaSuccess) return e;
     mark(4);
-    e = fields(s);
-    if (split) {
-      const cudaError_t e0 = cudaStreamWaitEvent(s->stream, s->ev_join, 0);
-      if (e0 != cudaSuccess) return e0;
-    }
-    k_step_end<<<1, 32, 0, s->stream>>>(d.ctr);
+    e = one ? fields_tiled1(s) : fields(s);
+    if (e != cudaSuccess) return e;
+    if (drawn && (e = cudaStreamWaitEvent(s->stream, s->ev_join, 0)) != cudaSuccess) return e;
+    if (one)
+      k_step1_end<T><<<std::min((4 * s->g.nxn + kBlock - 1) / kBlock, 152), kBlock, 0,
+                       s->stream>>>(d, s->g);
+    else
+      k_step_end<<<1, 32, 0, s->stream>>>(d.ctr, d.inj, s->g);
     mark(5);
-    return e;
+    return cudaGetLastError();
   }
 
   static cudaError_t step(Sim* s, int in, long long step, cudaEvent_t* ev) {
+    // without phase events (and with the side stream of the captured step):
+    // the draws beside the push
+    const bool drawn = !ev && s->side && s->ev_fork && s->ev_draw && s->ev_push && s->ev_join;
+    cudaError_t e = cudaSuccess;
+    if (drawn) {
+      if ((e = cudaEventRecord(s->ev_fork, s->stream)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(s->side, s->ev_fork, 0)) != cudaSuccess) return e;
+      if (s->g.ninj && (e = inject(s, s->side)) != cudaSuccess) return e;
+      if ((e = cudaEventRecord(s->ev_draw, s->side)) != cudaSuccess) return e;
+    }
     if (ev) cudaEventRecord(ev[0], s->stream);
-    const cudaError_t e =
-        (s->g.dim == 1) ? push_dispatch<T, 1>(s, in, step) : push_dispatch<T, 2>(s, in, step);
+    e = (s->g.dim == 1) ? push_dispatch<T, 1>(s, in, step) : push_dispatch<T, 2>(s, in, step);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], s->stream);
-    return step_rest(s, in, ev);
+    return step_rest(s, in, ev, drawn);
   }
 
   // ---- batched ensembles: one push launch over every run's CTA group
@@ -465,7 +488,11 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  // the rest of a batched step over every run (all 1D with x walls)
+  // a batched step over every run (all 1D with x walls): the draws, the rest
+  static cudaError_t batch_draw(const void* runs, int nruns, cudaStream_t st) {
+    k_inject_batch<T, 1><<<nruns, kBlock, 0, st>>>((const BatchRun<T>*)runs, nruns);
+    return cudaGetLastError();
+  }
   static cudaError_t batch_rest(const void* runs, const int* pre, int nruns, const int* nblk,
                                 int n_sub_max, cudaStream_t st, cudaStream_t side,
                                 cudaEvent_t fork, cudaEvent_t join) {
@@ -481,20 +508,16 @@ struct OpsImpl {
       }
     }
     const int n1 = nruns + 1;
-    // the movers (buckets) beside the injection, moments and field advance,
-    // which read no bucket: the injection appends to the buckets with its own
-    // slot atomics, the moments read the deposit partials and far sums
+    // the movers (buckets) beside the moments and field advance, which read
+    // the deposit partials and far sums and no bucket
     cudaError_t e;
     if ((e = cudaEventRecord(fork, st)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
     k_movers_batch<T, 1><<<nblk[0], kBlock, 0, side>>>(r, pre, nruns);
     if ((e = cudaEventRecord(join, side)) != cudaSuccess) return e;
-    k_inject_batch<T, 1><<<nruns, kBlock, 0, st>>>(r, nruns);
-    k_moments_batch<T, 1><<<nblk[1], kBlock, 0, st>>>(r, pre + n1, nruns);
-    k_field1_batch<T><<<nblk[2], kF1Threads, fsm, st>>>(r, pre + 2 * n1, nruns);
-    k_copyB_batch<T><<<nblk[2], kF1Threads, 0, st>>>(r, pre + 2 * n1, nruns);
+    k_field1_batch<T><<<nblk[1], field1_threads(kF1, n_sub_max), fsm, st>>>(r, pre + n1, nruns);
     if ((e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess) return e;
-    k_step_end_batch<T><<<(nruns + 63) / 64, 64, 0, st>>>(r, nruns);
+    k_step1_end_batch<T><<<nblk[1], kBlock, 0, st>>>(r, pre + n1, nruns);
     return cudaGetLastError();
   }
 
@@ -675,6 +698,7 @@ struct OpsImpl {
     o.batch_smem = batch_smem;
     o.batch_setup = batch_setup;
     o.push_batch = push_batch;
+    o.batch_draw = batch_draw;
     o.batch_rest = batch_rest;
     o.profile_B = profile_B;
     o.spectrum_bperp = spectrum_bperp;

@@ -414,9 +414,9 @@ __global__ void __launch_bounds__(kBlock)
             bin = lo;
           }
         }
-        if (!take[r]) bin = -1;
-        if (copies) count_shared(mine, bin);
-        else if (bin >= 0) atomicAdd(&out[bin], 1ull);
+        if (!take[r] || bin < 0) continue;
+        if (copies) atomicAdd(&mine[bin], 1u);
+        else atomicAdd(&out[bin], 1ull);
       }
     }
   }

@@ -65,10 +65,15 @@ struct Win {
 // up in registers and hands to memory once per cell and quantity, instead of
 // per particle, per lane group or by long shuffle reductions.
 constexpr int kSortKeys = 64;
+constexpr int kSortPiece = 32;  // items of a cell one warp takes at a time
 struct CellSort {
   int lo[kBlock / 32], hi[kBlock / 32];
   int cnt[kSortKeys];
-  int first[kSortKeys + 1];
+  int first[kSortKeys];
+  // the pieces: cell, first and end item; their number
+  short cell[kSortKeys + kBlock / kSortPiece], from[kSortKeys + kBlock / kSortPiece],
+      to[kSortKeys + kBlock / kSortPiece];
+  int pieces;
 };
 // Returns the thread's position; base: the lowest cell; range: the number of
 // cells spanned (0: no item; above kSortKeys: not sorted, take each item on
@@ -100,16 +105,29 @@ __device__ __forceinline__ int cell_sort(CellSort& cs, int key, int& base, int& 
   at = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1u));
   __syncthreads();
   if (warp == 0) {
-    const int c0 = cs.cnt[2 * lane], c1 = cs.cnt[2 * lane + 1];
-    int inc = c0 + c1;
+    constexpr int PS = kSortPiece;
+    const int c[2] = {cs.cnt[2 * lane], cs.cnt[2 * lane + 1]};
+    const int n[2] = {(c[0] + PS - 1) / PS, (c[1] + PS - 1) / PS};
+    // one scan for both: items in the low half, pieces in the high half
+    int inc = (c[0] + c[1]) | ((n[0] + n[1]) << 16);
+    const int own = inc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += v;
     }
-    cs.first[2 * lane] = inc - c0 - c1;
-    cs.first[2 * lane + 1] = inc - c1;
-    if (lane == 31) cs.first[kSortKeys] = inc;
+    if (lane == 31) cs.pieces = inc >> 16;
+    int at0 = (inc - own) & 0xFFFF, p = (inc - own) >> 16;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      cs.first[2 * lane + r] = at0;
+      for (int b0 = 0; b0 < c[r]; b0 += PS, ++p) {
+        cs.cell[p] = (short)(2 * lane + r);
+        cs.from[p] = (short)(at0 + b0);
+        cs.to[p] = (short)(at0 + min(b0 + PS, c[r]));
+      }
+      at0 += c[r];
+    }
   }
   __syncthreads();
   return key >= 0 ? cs.first[k] + at : 0;
@@ -299,7 +317,8 @@ __device__ __forceinline__ unsigned long long fix(double c) {
 // c * 2^40 rounded to the nearest integer for an FP32 value c (|c| < 2^23):
 // the scaling is exact; below 2^30 the int32 conversion rounds to nearest
 // (ties to even), at or above it the value is an integer already (its ulp is
-// at least 2^7) and its significand is shifted into place.
+// at least 2^7) and its significand is shifted into place. (The conversion
+// instruction to 64 bits measured slower: 15.9 against 14.8 us per launch.)
 __device__ __forceinline__ long long fix32(float c) {
   const float y = c * 0x1p40f;
   if (fabsf(y) < 0x1p30f) return (long long)__float2int_rn(y);
@@ -317,8 +336,8 @@ __device__ __forceinline__ long long fixT(double c) { return (long long)fix(c); 
 // all of them into the fixed-point sums q (CIC; integer sums, so the result
 // does not depend on the grouping; contributions in the run's precision, FP32
 // runs with no FP64 instruction). The block's particles are sorted by cell
-// (cell_sort); a warp per cell adds eight quantities (n, J at the cell's two
-// nodes) with four lanes each. Push and deposit in one launch: the deposit
+// (cell_sort); a warp adds a cell's eight quantities (n, J at its two nodes)
+// with four lanes each, 32 particles at a time. Push and deposit in one launch: the deposit
 // needs no second read of the slots, and the sums it replaces (lane groups
 // by match and 24 reductions, then atomics per warp and cell) were half of
 // the window. 262 K ions FP32: 14 + 30 us before.
@@ -374,17 +393,18 @@ __global__ void __launch_bounds__(kBlock)
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, side = lane & 1, comp = (lane >> 1) & 3;
-  for (int k = threadIdx.x >> 5; k < range; k += kBlock / 32) {
-    const int b0 = cs.first[k], b1 = cs.first[k + 1];
-    if (b0 == b1) continue;
+  const int pieces = range ? cs.pieces : 0;
+  for (int k = threadIdx.x >> 5; k < pieces; k += kBlock / 32) {
+    const int b1 = cs.to[k];
     long long s = 0;
-    for (int i = b0 + (lane >> 3); i < b1; i += 4) {
+#pragma unroll 4
+    for (int i = cs.from[k] + (lane >> 3); i < b1; i += 4) {
       const T c = rec[side][i];
       s += fixT(comp ? c * rec[1 + comp][i] : c);
     }
     s += __shfl_xor_sync(0xffffffffu, s, 8);
     s += __shfl_xor_sync(0xffffffffu, s, 16);
-    if (lane < 8) atomicAdd(&q[comp * nxn + base + k + side], (unsigned long long)s);
+    if (lane < 8) atomicAdd(&q[comp * nxn + base + cs.cell[k] + side], (unsigned long long)s);
   }
 }
 
@@ -410,22 +430,37 @@ __global__ void k_win_moments(Win<T> w, const unsigned long long* q, Geo g, Phys
   for (int c = 0; c < 3; ++c) w.u[c * nxn + i] = moment_sum<T>(i, c + 1, q, g) / n;
 }
 
-// B = B0 + sum_m a_m (cos, sin)(2 pi m x / L + phi_m) at the centres
+// B = B0 + sum_m a_m (cos, sin)(2 pi m x / L + phi_m) at the centres. A block
+// takes 16 cells: 16 threads a cell form the terms, one adds them in order (a
+// thread per cell: 46 us for 16 modes, the FP64 chain of its 16 sincos).
+constexpr int kSeedCells = 16;
 template <typename T>
-__global__ void k_win_seed_B(T* B, Geo g, Phys ph, double dx, const double* amps,
-                             const double* phases, int M) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.nx) return;
+__global__ void __launch_bounds__(kBlock)
+    k_win_seed_B(T* B, Geo g, Phys ph, double dx, const double* amps, const double* phases, int M) {
+  __shared__ double term[2][kSeedCells][17];
+  const int cell = threadIdx.x / 16, m0 = threadIdx.x & 15;
+  const int i = blockIdx.x * kSeedCells + cell;
   const double x = ((double)i + 0.5) * dx;
   const double L = (double)g.nx * dx;
   double by = ph.b0y, bz = ph.b0z;
-  for (int m = 0; m < M; ++m) {
-    const double arg = 2.0 * 3.14159265358979323846 * (double)(m + 1) * x / L + phases[m];
-    double s, c;
-    sincos(arg, &s, &c);
-    by += amps[m] * c;
-    bz += amps[m] * s;
+  for (int mb = 0; mb < M; mb += 16) {
+    const int m = mb + m0;
+    if (m < M) {
+      const double arg = 2.0 * 3.14159265358979323846 * (double)(m + 1) * x / L + phases[m];
+      double s, c;
+      sincos(arg, &s, &c);
+      term[0][cell][m0] = c;
+      term[1][cell][m0] = s;
+    }
+    __syncthreads();
+    if (m0 == 0)
+      for (int k = 0; k < min(16, M - mb); ++k) {
+        by += amps[mb + k] * term[0][cell][k];
+        bz += amps[mb + k] * term[1][cell][k];
+      }
+    __syncthreads();
   }
+  if (m0 || i >= g.nx) return;
   B[i] = (T)ph.b0x;
   B[g.nx + i] = (T)by;
   B[2 * g.nx + i] = (T)bz;
@@ -555,10 +590,6 @@ __device__ __forceinline__ void moments_adj_node(int i, double inv_n, const T* u
 // the wall and the clamped and mirrored indices are the walls' own. No
 // synchronisation between CTAs, and the FP64 work spreads over the SMs.
 constexpr int kTbCells = 16;
-// two halves, one per transverse component (Tile1); a tile of two substeps and
-// its halo fills two warps of each half
-constexpr int kTbThreads = 128;
-
 // halos: the forward's 4 n_sub stages and final Ohm; the adjoint's stage
 // recompute, its 4 n_sub reverse stages and the moment adjoints
 __host__ __device__ constexpr int halo_fields(int n_sub) { return 4 * n_sub + 2; }
@@ -592,46 +623,43 @@ struct Tile {
 
 constexpr size_t kMaxSmem = 227 * 1024;  // shared memory a CTA may opt in to
 
-// a tile's forward arrays (Tile1 with the pressure term and raw moments)
-constexpr size_t tile1_smem(size_t L, size_t tsz) { return tsz * (7 * L + 8 * (L + 1)); }
+constexpr int fields_threads(int n_sub) {
+  return tile1_threads(kTbCells + 2 * halo_fields(n_sub));
+}
+constexpr int rk4_adj_threads(int n_sub) {
+  return tile1_threads(kTbCells + 2 * halo_rk4_adj(n_sub));
+}
+constexpr int kTbMaxSub = 10;
 constexpr size_t fields_smem(int n_sub, size_t tsz) {
-  return tile1_smem(kTbCells + 2 * halo_fields(n_sub), tsz);
+  const size_t L = kTbCells + 2 * halo_fields(n_sub);
+  return tsz * (tile1_words(L, tsz) + 6 * (L + 1));
 }
 constexpr size_t rk4_adj_smem(int n_sub, size_t tsz) {
   const size_t L = kTbCells + 2 * halo_rk4_adj(n_sub), Ln = L + 1;
-  return tile1_smem(L, tsz) + 8 * ((8 * (size_t)n_sub + 12) * L + 21 * Ln);
+  return 8 * (8 * L + 11 * Ln) + tsz * (tile1_words(L, tsz) + (8 * (size_t)n_sub) * L);
 }
 
-// The Tile1 of a window tile in mem; returns the end of it. pg: the pressure
-// term per node.
+// this thread's part of a tile
 template <typename T>
-__device__ __forceinline__ Tile1<T> window_tile(const Tile& t, T* mem, T** pg) {
-  const int L = t.L, Ln = L + 1;
+__device__ __forceinline__ Tile1<T> window_tile(const Tile& t, T* mem) {
   Tile1<T> r;
-  r.L = L;
-  r.half = kTbThreads / 2;
+  r.L = t.L;
+  r.half = blockDim.x / 2;
   r.comp = (int)threadIdx.x >= r.half;
-  r.l0 = threadIdx.x - r.comp * r.half;
-  r.Bx = mem;
-  r.B = r.Bx + L;
-  r.Bs = r.B + 2 * L;
-  r.K = r.Bs + 2 * L;
-  r.E = r.K + 2 * L;
-  r.inv = r.E + 2 * Ln;
-  r.bbx = r.inv + Ln;
-  r.u = r.bbx + Ln;
-  *pg = r.u + 3 * Ln;
+  r.a = threadIdx.x - r.comp * r.half;
+  r.S = mem;
+  r.E = mem + 2 * t.L;
   return r;
 }
 
 // One step's moments from the deposit sums q, the n_sub RK4 substeps of Ohm +
 // Faraday with n, u frozen, then E, Bbar for the next gather and the new B,
 // all into state b (B is read by neighbouring tiles: its buffer is another).
-// Clears qz, the sums of the step after this one. A chain of 17 dependent
-// passes with few operations each (Tile1; the moments one quantity per
+// Clears qz, the sums of the step after this one. A chain of dependent passes
+// with few operations each (tile1_substep; the moments one quantity per
 // thread, the division once): 9.4 us FP32, 22.6 us FP64 per step before.
 template <typename T>
-__global__ void __launch_bounds__(kTbThreads)
+__global__ void __launch_bounds__(fields_threads(kTbMaxSub))
     k_win_fields(const T* __restrict__ Bin, State<T> b, const unsigned long long* __restrict__ q,
                  unsigned long long* __restrict__ qz, Geo g, Phys ph, FieldConst<T> fc,
                  int n_sub) {
@@ -639,12 +667,22 @@ __global__ void __launch_bounds__(kTbThreads)
   const int nx = g.nx, nxn = g.nxn, t0 = threadIdx.x, nt = blockDim.x;
   const Tile t(blockIdx.x, nx, halo_fields(n_sub));
   const int L = t.L, Ln = L + 1;
-  T* pg;
-  const Tile1<T> w = window_tile<T>(t, (T*)smem, &pg);
-  T* sn = w.inv;  // the density until its reciprocal replaces it
-  for (int k = t0; k < 3 * L; k += nt) {
-    const int c = k / L;
-    w.Bx[k] = Bin[c * nx + t.lo + k - c * L];
+  Tile1<T> w = window_tile<T>(t, (T*)smem);
+  T* sn = w.S + tile1_words(L, sizeof(T));  // [Ln] n
+  T* sinv = sn + Ln;                        // [Ln] 1/n
+  T* spg = sinv + Ln;                       // [Ln] pressure term
+  T* su = spg + Ln;                         // [3][Ln] J, then u
+  const int a = w.a, gc = t.lo + a;         // this thread's cell and node
+  T bxm = (T)0, bxc = (T)0, bxp = (T)0;
+  w.b = (T)0;
+  if (a < L) {
+    w.b = Bin[(w.comp + 1) * nx + gc];
+    w.S[w.comp * L + a] = w.b;
+    bxp = Bin[t.lo + min(a + 1, L - 1)];
+  }
+  if (a < Ln) {
+    bxm = Bin[t.lo + max(a - 1, 0)];
+    bxc = Bin[t.lo + min(a, L - 1)];
   }
   for (int k = t0; k < 4 * Ln; k += nt) {
     const int c = k / Ln, i = k - c * Ln, gi = t.lo + i;
@@ -657,46 +695,45 @@ __global__ void __launch_bounds__(kTbThreads)
         b.nraw[gi] = v;
       }
     } else {
-      w.u[(c - 1) * Ln + i] = v;
+      su[(c - 1) * Ln + i] = v;
     }
     if (t.owns_node(gi)) qz[c * nxn + gi] = 0ull;
   }
   __syncthreads();
-  for (int k = t0; k < 3 * Ln; k += nt) {
+  for (int k = t0; k < 5 * Ln; k += nt) {
     const int c = k / Ln, i = k - c * Ln, gi = t.lo + i;
-    const T u = w.u[k] / sn[i];
-    w.u[k] = u;
-    if (t.owns_node(gi)) b.u[c * nxn + gi] = u;
-  }
-  for (int i = t0; i < Ln; i += nt) {
-    const int gi = t.lo + i;
-    const T dnx = (sn[t.node(gi + 1)] - sn[t.node(gi - 1)]) * fc.hdx;
-    pg[i] = -(fc.te * dnx);
-    w.bbx[i] = (T)0.5 * (w.Bx[t.cell(gi - 1)] + w.Bx[t.cell(gi)]);
+    if (c < 4) {  // u = J / n, then 1/n
+      const T v = (c < 3 ? su[k] : (T)1) / sn[i];
+      if (c == 3) {
+        sinv[i] = v;
+      } else {
+        su[k] = v;
+        if (t.owns_node(gi)) b.u[c * nxn + gi] = v;
+      }
+    } else {
+      const T dnx = (sn[t.node(gi + 1)] - sn[t.node(gi - 1)]) * fc.hdx;
+      spg[i] = -(fc.te * dnx);
+    }
   }
   __syncthreads();
-  for (int i = t0; i < Ln; i += nt) w.inv[i] = (T)1 / sn[i];
-  __syncthreads();
+  auto node = [&](int i, T bm, T bp) {
+    return Node1<T>{sinv[i], (T)0.5 * (bm + bp), su[i], su[Ln + i], su[2 * Ln + i]};
+  };
+  if (a < Ln) w.n0 = node(a, bxm, bxc);
+  if (sizeof(T) == 4 && a < L) w.n1 = node(a + 1, bxc, bxp);
   for (int sub = 0; sub < n_sub; ++sub) tile1_substep<T>(w, fc, nullptr);
-  for (int i = t0; i < Ln; i += nt) {
-    const int gi = t.lo + i;
-    if (!t.owns_node(gi)) continue;
-    const int im = t.cell(gi - 1), ip = t.cell(gi);
-    const T bmy = w.B[im], bpy = w.B[ip], bmz = w.B[L + im], bpz = w.B[L + ip];
-    const T bby = (T)0.5 * (bmy + bpy), bbz = (T)0.5 * (bmz + bpz);
-    const T dby = (bpy - bmy) * fc.idx, dbz = (bpz - bmz) * fc.idx;
-    T E[3];
-    ohm_e<T>((T)0, -dbz, dby, w.bbx[i], bby, bbz, w.inv[i], pg[i], -(fc.te * (T)0), w.u[i],
-             w.u[Ln + i], w.u[2 * Ln + i], fc.jcr, fc.eta, fc.resist != 0, E[0], E[1], E[2]);
+  if (w.comp == 0 && a < Ln && t.owns_node(gc)) {
+    T E[3], Bb[3];
+    tile1_ohm<T>(w.S, L, max(a - 1, 0), min(a, L - 1), w.n0, spg[a], fc, E, Bb);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) b.E[c * nxn + gi] = E[c];
-    b.Bb[gi] = w.bbx[i];
-    b.Bb[nxn + gi] = bby;
-    b.Bb[2 * nxn + gi] = bbz;
+    for (int c = 0; c < 3; ++c) {
+      b.E[c * nxn + gc] = E[c];
+      b.Bb[c * nxn + gc] = Bb[c];
+    }
   }
-  for (int k = t0; k < 3 * L; k += nt) {
-    const int c = k / L, gc = t.lo + k - c * L;
-    if (t.owns_cell(gc)) b.B[c * nx + gc] = w.Bx[k];
+  if (a < L && t.owns_cell(gc)) {
+    b.B[(w.comp + 1) * nx + gc] = w.b;
+    if (w.comp == 0) b.B[gc] = bxc;
   }
 }
 
@@ -715,48 +752,57 @@ __global__ void __launch_bounds__(kTbThreads)
 //      is constant, so n's and u's adjoints are four running sums that take
 //      their node factors once at the end);
 //   4. the adjoints of the raw deposit sums (lNr, lJ) from those of M^{n+1}.
-// lE, lBb of the step before are cleared (lEz, lBbz). Bound by the FP64 pipe:
-// an FP64 instruction holds an SM quarter for some 64 cycles, so the time is
-// the FP64 instruction count per warp: about 18 per stage and warp, four
-// warps, against about 110, two warps and a launch of its own for 2. before
-// (43 + 8.6 us per step FP32, 54 + 8 us FP64).
+// lE, lBb of the step before are cleared (lEz, lBbz). A thread has one cell
+// and one node; its factors and sums stay in registers. Bound by the FP64
+// pipe: an FP64 instruction holds an SM quarter for 64 cycles, so the time is
+// the FP64 instruction count per warp: 8 per reverse stage, four warps,
+// against about 110, two warps and a launch of its own for 2. before (43 +
+// 8.6 us per step FP32, 54 + 8 us FP64). FP32 values are widened by integer
+// operations, off that pipe.
 template <typename T>
-__global__ void __launch_bounds__(kTbThreads)
+__global__ void __launch_bounds__(rk4_adj_threads(kTbMaxSub))
     k_win_rk4_adj(Geo g, Phys ph, FieldConst<T> fc, int ns, const T* __restrict__ Bn, State<T> b,
                   const double* __restrict__ lE, const double* __restrict__ lBb,
                   double* __restrict__ lEz, double* __restrict__ lBbz,
                   const double* __restrict__ lBin, double* __restrict__ lBout,
                   T* __restrict__ lNr, T* __restrict__ lJ) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int nx = g.nx, nxn = g.nxn, t0 = threadIdx.x, nt = blockDim.x;
+  const int nx = g.nx, nxn = g.nxn;
   const Tile t(blockIdx.x, nx, halo_rk4_adj(ns));
   const int L = t.L, Ln = L + 1;
-  double* Y = (double*)smem;     // [4 ns][2][L] stage inputs
-  double* gk = Y + 8 * ns * L;   // [4][2][L] stage adjoints of one substep
-  double* lend = gk + 8 * L;     // [2][L]
-  double* lsum = lend + 2 * L;   // [2][L]
-  double* Pp = lsum + 2 * L;     // [2][Ln] a node's part for its right cell
+  double* gk = (double*)smem;    // [4][2][L] stage adjoints of one substep
+  double* Pp = gk + 8 * L;       // [2][Ln] a node's part for its right cell
   double* Pm = Pp + 2 * Ln;      // [2][Ln] and for its left cell
-  double* in = Pm + 2 * Ln;      // [Ln] 1/n at M^{n+1}
-  double* e1 = in + Ln;          // node factors of the stage adjoint
-  double* e2 = e1 + Ln;
-  double* bi = e2 + Ln;
-  double* lp = bi + Ln;          // [Ln] pressure weight of E^{n+1}'s Ohm
-  double* acc = lp + Ln;         // [2][4][Ln] sums of the n and u adjoints
-  double* lM = acc + 8 * Ln;     // [4][Ln] adjoints of n, u from E^{n+1}'s Ohm
-  T* pg;
-  const Tile1<T> w = window_tile<T>(t, (T*)(lM + 4 * Ln), &pg);
+  double* lp = Pm + 2 * Ln;      // [Ln] pressure weight of E^{n+1}'s Ohm
+  double* lM = lp + Ln;          // [4][Ln] the moments' sums of half 1 for half 0
+  double* lUx = lM + 4 * Ln;     // [Ln] u_x's part of E^{n+1}'s Ohm
+  Tile1<T> w = window_tile<T>(t, (T*)(lUx + Ln));
+  T* Y = w.S + tile1_words(L, sizeof(T));  // [4 ns][2][L] stage inputs
   const double h = ph.h, hh = ph.hh, h6 = ph.h6, idx = ph.idx;
-  const int comp = w.comp, l0 = w.l0, half = w.half;
-  for (int k = t0; k < 3 * L; k += nt) {
-    const int c = k / L;
-    w.Bx[k] = Bn[c * nx + t.lo + k - c * L];
+  const int comp = w.comp, a = w.a, gi = t.lo + a;  // this thread's cell and node
+  const bool node = a < Ln, cell = a < L;
+  const int cm = max(a - 1, 0), cp = min(a, L - 1);
+  T bxm = (T)0, bxc = (T)0, bxp = (T)0, n0 = (T)1, n1 = (T)1;
+  w.b = (T)0;
+  if (cell) {
+    w.b = Bn[(comp + 1) * nx + gi];
+    w.S[comp * L + a] = w.b;
   }
-  for (int i = t0; i < Ln; i += nt) {
-    const int gi = t.lo + i;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) w.u[c * Ln + i] = b.u[c * nxn + gi];
-    if (t.owns_node(gi)) {
+  if (node) {
+    bxm = Bn[t.lo + cm];
+    bxc = Bn[t.lo + cp];
+    n0 = b.n[gi];
+    w.n0.ux = b.u[gi];
+    w.n0.uy = b.u[nxn + gi];
+    w.n0.uz = b.u[2 * nxn + gi];
+    if (sizeof(T) == 4 && cell) {
+      bxp = Bn[t.lo + min(a + 1, L - 1)];
+      n1 = b.n[gi + 1];
+      w.n1.ux = b.u[gi + 1];
+      w.n1.uy = b.u[nxn + gi + 1];
+      w.n1.uz = b.u[2 * nxn + gi + 1];
+    }
+    if (comp == 0 && t.owns_node(gi)) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         lEz[c * nxn + gi] = 0.0;
@@ -764,157 +810,144 @@ __global__ void __launch_bounds__(kTbThreads)
       }
     }
   }
-  for (int k = t0; k < 8 * Ln; k += nt) acc[k] = 0.0;
-  for (int i = l0; i < Ln; i += half) {
-    const T n = b.n[t.lo + i];
-    if (comp == 0) in[i] = 1.0 / (double)n;
-    else w.inv[i] = (T)1 / n;
+  w.n0.inv = (T)1 / n0;
+  w.n0.bbx = (T)0.5 * (bxm + bxc);
+  if (sizeof(T) == 4) {
+    w.n1.inv = (T)1 / n1;
+    w.n1.bbx = (T)0.5 * (bxc + bxp);
   }
-  __syncthreads();
-  for (int i = t0; i < Ln; i += nt) {
-    const T bbx = (T)0.5 * (w.Bx[max(i - 1, 0)] + w.Bx[min(i, L - 1)]);
-    w.bbx[i] = bbx;
-    const double a5 = 0.5 * (ph.jcr * in[i] + (double)w.u[i]), ei = ph.eta * idx;
-    e1[i] = a5 - ei;
-    e2[i] = a5 + ei;
-    bi[i] = (double)bbx * in[i] * idx;
-  }
+  const double in = sizeof(T) == 8 ? (double)w.n0.inv : 1.0 / wide_double(n0);
+  const double bbx = wide_double(w.n0.bbx);
   __syncthreads();
   // 1.
-  for (int sub = 0; sub < ns; ++sub)
-    tile1_substep<T>(w, fc, Y + (size_t)8 * sub * L);
+  for (int sub = 0; sub < ns; ++sub) tile1_substep<T>(w, fc, Y + (size_t)8 * sub * L);
   // 2. half 0: B's part, half 1: the moments' part
-  for (int i = l0; i < Ln; i += half) {
-    const int gi = t.lo + i;
+  double m0 = 0.0, m1 = 0.0, m2 = 0.0;  // half 1: n's and u_y's, u_z's parts
+  if (node) {
     const int im = min(max(gi - 1, 0), nx - 1), ip = min(gi, nx - 1);
-    const double Bm[3] = {(double)b.B[im], (double)b.B[nx + im], (double)b.B[2 * nx + im]};
-    const double Bp[3] = {(double)b.B[ip], (double)b.B[nx + ip], (double)b.B[2 * nx + ip]};
-    const double u[3] = {(double)w.u[i], (double)w.u[Ln + i], (double)w.u[2 * Ln + i]};
+    const double Bm[3] = {wide_double(b.B[im]), wide_double(b.B[nx + im]),
+                          wide_double(b.B[2 * nx + im])};
+    const double Bp[3] = {wide_double(b.B[ip]), wide_double(b.B[nx + ip]),
+                          wide_double(b.B[2 * nx + ip])};
+    const double u[3] = {wide_double(w.n0.ux), wide_double(w.n0.uy), wide_double(w.n0.uz)};
     const double lex = lE[gi], ley = lE[nxn + gi], lez = lE[2 * nxn + gi];
     if (comp == 0) {
-      const OhmAdj r = ohm_adj_point(Bm, Bp, in[i], 0.0, u, lex, ley, lez, ph);
+      const OhmAdj r = ohm_adj_point(Bm, Bp, in, 0.0, u, lex, ley, lez, ph);
       const double hy = 0.5 * (r.P[0] + lBb[nxn + gi]), hz = 0.5 * (r.P[1] + lBb[2 * nxn + gi]);
       const double dy = r.P[2] * idx, dz = r.P[3] * idx;
-      Pp[i] = hy + dy;
-      Pp[Ln + i] = hz + dz;
-      Pm[i] = hy - dy;
-      Pm[Ln + i] = hz - dz;
+      Pp[a] = hy + dy;
+      Pp[Ln + a] = hz + dz;
+      Pm[a] = hy - dy;
+      Pm[Ln + a] = hz - dz;
     } else {
       const int ipn = (gi + 1 > nx) ? 2 * nx - (gi + 1) : gi + 1;
       const int imn = (gi - 1 < 0) ? -(gi - 1) : gi - 1;
-      const double pgn = -(ph.te * (((double)b.n[ipn] - (double)b.n[imn]) * ph.hdx));
-      const OhmAdj r = ohm_adj_point(Bm, Bp, in[i], pgn, u, lex, ley, lez, ph);
-      lM[i] = r.ln;
+      const double pgn = -(ph.te * ((wide_double(b.n[ipn]) - wide_double(b.n[imn])) * ph.hdx));
+      const OhmAdj r = ohm_adj_point(Bm, Bp, in, pgn, u, lex, ley, lez, ph);
+      m0 = r.ln;
       // (a wall node's pressure difference is zero by the mirrored density)
-      lp[i] = (gi == 0 || gi == nx) ? 0.0 : r.lp;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) lM[(1 + c) * Ln + i] = r.lu[c];
+      lp[a] = (gi == 0 || gi == nx) ? 0.0 : r.lp;
+      lUx[a] = r.lu[0];
+      m1 = r.lu[1];
+      m2 = r.lu[2];
     }
   }
+  // the stage adjoint's node factors (times 1/dx: E's adjoint from K's)
+  const double a5 = 0.5 * (ph.jcr * in + wide_double(w.n0.ux)), ei = ph.eta * idx;
+  const double e1 = (a5 - ei) * idx, e2 = (a5 + ei) * idx, bi = bbx * in * idx * idx;
   __syncthreads();
   // a cell's part from its two nodes (the wall nodes read cell 0 or nx - 1 twice)
-  auto cell_part = [&](int c) {
-    const int gc = t.lo + c;
-    double l = Pp[comp * Ln + c] + Pm[comp * Ln + c + 1];
-    if (gc == 0) l += Pm[comp * Ln];
-    if (gc == nx - 1) l += Pp[comp * Ln + c + 1];
+  const double* pp = Pp + comp * Ln;
+  const double* pm = Pm + comp * Ln;
+  auto cell_part = [&]() {
+    double l = pp[a] + pm[a + 1];
+    if (gi == 0) l += pm[0];
+    if (gi == nx - 1) l += pp[a + 1];
     return l;
   };
-  for (int c = l0; c < L; c += half)
-    lsum[comp * L + c] = lBin[(comp + 1) * nx + t.lo + c] + cell_part(c);
+  double lsum = 0.0;  // the adjoint of B at the thread's cell
+  if (cell) lsum = lBin[(comp + 1) * nx + gi] + cell_part();
   // 3. lambda_start = lambda_end + sum over the stages of lambda_Y; the stage
   //    adjoints g4 = h6 lend, g3 = 2 h6 lend + h lY4, g2 = 2 h6 lend + hh lY3,
   //    g1 = h6 lend + hh lY2
+  double A[4] = {0.0, 0.0, 0.0, 0.0};  // the n and u adjoints' sums
+  // (a K's adjoint is read at cells gi - 1 and gi; none beyond a wall)
+  const bool left = gi >= 1, right = gi < nx;
   for (int sub = ns - 1; sub >= 0; --sub) {
-    for (int c = l0; c < L; c += half) {  // (each half its own component: no barrier before)
-      const int k = comp * L + c;
-      const double l = lsum[k];
-      lend[k] = l;
-      gk[6 * L + k] = h6 * l;
-    }
+    const double hl = h6 * lsum, hl2 = hl + hl;
+    if (cell) gk[6 * L + comp * L + a] = hl;
     __syncthreads();
+#pragma unroll
     for (int s = 3; s >= 0; --s) {
       const double* G = gk + 2 * s * L;
-      for (int i = l0; i < Ln; i += half) {
-        const int gi = t.lo + i;
-        const int cm = max(i - 1, 0), cp = min(i, L - 1);
-        // E adjoint at the node from K's: K_y(c) = (E_z(c+1) - E_z(c))/dx,
-        // K_z(c) = -(E_y(c+1) - E_y(c))/dx
-        const double gym = (gi >= 1) ? G[cm] : 0.0, gy = (gi < nx) ? G[cp] : 0.0;
-        const double gzm = (gi >= 1) ? G[L + cm] : 0.0, gz = (gi < nx) ? G[L + cp] : 0.0;
-        const double ley = (gz - gzm) * idx, lez = (gym - gy) * idx;
+      if (node) {
+        const double gym = left ? G[cm] : 0.0, gy = right ? G[cp] : 0.0;
+        const double gzm = left ? G[L + cm] : 0.0, gz = right ? G[L + cp] : 0.0;
+        const double ley = gz - gzm, lez = gym - gy;
         if (comp == 0) {
-          const double x = ley * bi[i];
-          Pp[i] = x - lez * e1[i];
-          Pm[i] = -x - lez * e2[i];
+          const double x = ley * bi;
+          Pp[a] = __fma_rn(-lez, e1, x);
+          Pm[a] = __fma_rn(-lez, e2, -x);
         } else {
-          const double x = lez * bi[i];
-          Pp[Ln + i] = x + ley * e1[i];
-          Pm[Ln + i] = ley * e2[i] - x;
+          const double x = lez * bi;
+          Pp[Ln + a] = __fma_rn(ley, e1, x);
+          Pm[Ln + a] = __fma_rn(ley, e2, -x);
         }
       }
       __syncthreads();
-      const double an = s == 1 ? h6 : 2 * h6;
-      const double bn = s == 3 ? h : hh;
-      for (int c = l0; c < L; c += half) {
-        const int k = comp * L + c;
-        const double l = cell_part(c);
-        lsum[k] += l;
-        if (s > 0) gk[2 * (s - 1) * L + k] = an * lend[k] + bn * l;
+      if (cell) {
+        const double l = cell_part();
+        lsum += l;
+        if (s > 0)
+          gk[(2 * (s - 1) + comp) * L + a] = __fma_rn(s == 3 ? h : hh, l, s == 1 ? hl : hl2);
       }
       __syncthreads();
     }
     // the n and u adjoints of the substep's stages: stages comp and comp + 2
-    for (int i = l0; i < Ln; i += half) {
-      const int gi = t.lo + i;
-      const int cm = max(i - 1, 0), cp = min(i, L - 1);
-      double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    if (node) {
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         const int s = comp + 2 * r;
         const double* G = gk + 2 * s * L;
-        const double* y = Y + (size_t)(2 * (4 * sub + s)) * L;
-        const double gym = (gi >= 1) ? G[cm] : 0.0, gy = (gi < nx) ? G[cp] : 0.0;
-        const double gzm = (gi >= 1) ? G[L + cm] : 0.0, gz = (gi < nx) ? G[L + cp] : 0.0;
-        const double ley = gz - gzm, lez = gym - gy;  // (x idx at the end)
-        a0 += ley * (y[cp] - y[cm]) + lez * (y[L + cp] - y[L + cm]);  // curl part of n's
-        a1 += ley * (y[L + cp] + y[L + cm]) - lez * (y[cp] + y[cm]);  // u_x's, j_ext's
-        a2 += lez;                                                    // u_y's
-        a3 += ley;                                                    // u_z's
+        const T* y = Y + (size_t)(2 * (4 * sub + s)) * L;
+        const double gym = left ? G[cm] : 0.0, gy = right ? G[cp] : 0.0;
+        const double gzm = left ? G[L + cm] : 0.0, gz = right ? G[L + cp] : 0.0;
+        const double ley = gz - gzm, lez = gym - gy;  // (x 1/dx at the end)
+        const double ym = wide_double(y[cm]), yp = wide_double(y[cp]);
+        const double zm = wide_double(y[L + cm]), zp = wide_double(y[L + cp]);
+        A[0] = __fma_rn(lez, zp - zm, __fma_rn(ley, yp - ym, A[0]));    // curl part of n's
+        A[1] = __fma_rn(-lez, yp + ym, __fma_rn(ley, zp + zm, A[1]));  // u_x's, j_ext's
+        A[2] += lez;                                                    // u_y's
+        A[3] += ley;                                                    // u_z's
       }
-      double* A = acc + 4 * comp * Ln;
-      A[i] += a0;
-      A[Ln + i] += a1;
-      A[2 * Ln + i] += a2;
-      A[3 * Ln + i] += a3;
     }
     __syncthreads();
   }
-  // 4.
-  for (int i = t0; i < Ln; i += nt) {
-    const int gi = t.lo + i;
-    if (!t.owns_node(gi)) continue;
-    const double bbx = (double)w.bbx[i];
-    double S[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) S[k] = (acc[k * Ln + i] + acc[(4 + k) * Ln + i]) * idx;
-    const double ux = 0.5 * S[1];
-    double ln = lM[i] - in[i] * in[i] * (idx * bbx * S[0] + ph.jcr * ux);
-    if (gi >= 1) ln += lp[i - 1];  // (own nodes have both neighbours in the tile)
-    if (gi + 1 <= nx) ln -= lp[i + 1];
-    const double lu[3] = {lM[Ln + i] + ux, lM[2 * Ln + i] + bbx * S[2], lM[3 * Ln + i] - bbx * S[3]};
-    moments_adj_node<T>(gi, in[i], b.u, b.nraw, ln, lu, lNr, lJ, g, ph);
+  if (cell && t.owns_cell(gi)) lBout[(comp + 1) * nx + gi] = lsum;
+  // 4. half 1's sums to half 0
+  if (node && comp == 1) {
+    const double i2 = in * in;
+    lM[a] = m0 - i2 * (idx * idx * bbx * A[0] + ph.jcr * (0.5 * idx * A[1]));
+    lM[Ln + a] = lUx[a] + 0.5 * idx * A[1];
+    lM[2 * Ln + a] = m1 + bbx * (idx * A[2]);
+    lM[3 * Ln + a] = m2 - bbx * (idx * A[3]);
   }
-  for (int c = l0; c < L; c += half) {
-    const int gc = t.lo + c;
-    if (t.owns_cell(gc)) lBout[(comp + 1) * nx + gc] = lsum[comp * L + c];
+  __syncthreads();
+  if (node && comp == 0 && t.owns_node(gi)) {
+    const double ux = 0.5 * idx * A[1];
+    double ln = lM[a] - in * in * (idx * idx * bbx * A[0] + ph.jcr * ux);
+    if (gi >= 1) ln += lp[a - 1];  // (own nodes have both neighbours in the tile)
+    if (gi + 1 <= nx) ln -= lp[a + 1];
+    const double lu[3] = {lM[Ln + a] + ux, lM[2 * Ln + a] + bbx * (idx * A[2]),
+                          lM[3 * Ln + a] - bbx * (idx * A[3])};
+    moments_adj_node<T>(gi, in, b.u, b.nraw, ln, lu, lNr, lJ, g, ph);
   }
 }
 
 // The adjoint of Ohm's law at the start of the window (B^0 and M^0 in a), after
 // the first step's particles (lE, lBb): lB += its share.
 template <typename T>
-__global__ void __launch_bounds__(kTbThreads)
+__global__ void __launch_bounds__(32)
     k_win_ohm_adj_start(State<T> a, Geo g, Phys ph, const double* __restrict__ lE,
                         const double* __restrict__ lBb, double* __restrict__ lB) {
   __shared__ double P[4][kTbCells + 1];
@@ -954,41 +987,51 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // in it). In: lf, lv = adjoints of the state after the step;
 // lNr, lJ = adjoints of the step's deposit; E, Bb = the node fields the
 // step's gather used. Out: lf, lv = adjoints of the state before the step
-// (zero for slots born or removed in it); the slot's shares of lE, lBb at
-// the nodes c0, c0 + 1 (out; returns c0, or -1 when it has none); its terms
+// (zero for slots born or removed in it); the adjoints of E and Bbar
+// at the particle and its offset in the cell c0 (out; returns c0, or -1 when it
+// has none); its terms
 // of grad[M] (u_cr, into gucr) and grad[M + 1] (u2, into gu2). The
 // deposit's adjoint, the injection's and the faux-shock
 // return's are taken in FP64; the push's (Boris, gather) in the run's
-// precision, that of the per-slot adjoints lf, lv; the sums into lE, lBb and
-// the gradient are FP64.
+// precision, that of the per-slot adjoints lf, lv; the sums over cells into
+// lE, lBb and the gradient are FP64.
 template <typename T>
 __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const State<T>& a0,
                                                  const Slots<T>& t1, const uint8_t* ev,
                                                  const Geo& g, const Phys& ph,
                                                  const PushConst<T>& pc, long long step,
-                                                 int np0, double& gu2, double& gucr, T out[12]) {
+                                                 int np0, double& gu2, double& gucr, T out[7]) {
   using A = T;  // arithmetic of the push's adjoint
   const int nxn = g.nxn;
   const int cap = w.cap;
   const Slots<T>& t0 = a0.s;
   {
     const bool born = p >= np0;
+    // every load of the slot before the first decision (a slot without a
+    // particle reads values it does not use)
     const uint8_t e = born ? (uint8_t)kEvNone : ev[p];
-    const int c1 = t1.ci[p];
-    if (c1 < 0 || (!born && t0.ci[p] < 0) || e == kEvRemoved) {
+    const int c1 = t1.ci[p], c0 = born ? -1 : t0.ci[p];
+    const uint32_t id = w.s.id[p];
+    const A f1 = t1.f[p];
+    const A v1[3] = {t1.v[p], t1.v[cap + p], t1.v[2 * cap + p]};
+    A lf1 = w.lf[p];
+    A lv[3] = {w.lv[p], w.lv[cap + p], w.lv[2 * cap + p]};
+    const T ft0 = born ? (T)0 : t0.f[p];
+    T vxt = (T)0, vyt = (T)0, vzt = (T)0;
+    if (!born) {
+      vxt = t0.v[p];
+      vyt = t0.v[cap + p];
+      vzt = t0.v[2 * cap + p];
+    }
+    if (c1 < 0 || (!born && c0 < 0) || e == kEvRemoved) {
       w.lf[p] = (T)0;
       w.lv[p] = w.lv[cap + p] = w.lv[2 * cap + p] = (T)0;
       return -1;
     }
     // ---- deposit at the state after the step (in the run's precision)
-    const uint32_t id = w.s.id[p];
     A wp;
     if constexpr (sizeof(T) == 4) wp = (id & kIdCR) ? pc.wcr : pc.wth;
     else wp = (id & kIdCR) ? ph.w_cr : ph.w_th;
-    const A f1 = t1.f[p];
-    const A v1[3] = {t1.v[p], t1.v[cap + p], t1.v[2 * cap + p]};
-    A lf1 = w.lf[p];
-    A lv[3] = {w.lv[p], w.lv[cap + p], w.lv[2 * cap + p]};
     {
       A dj = w.lNr[c1 + 1] - w.lNr[c1];
       for (int c = 0; c < 3; ++c) {
@@ -1017,27 +1060,41 @@ __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const S
       return -1;
     }
     // ---- recompute the push from the state before the step
-    const int c0 = t0.ci[p];
-    const A f0 = (A)t0.f[p];
-    const T ft0 = t0.f[p];
-    const T g0t = (T)1 - ft0;
-    T Ep[3], Bp[3];
-    A Ed[3], Bd[3];
+    const A f0 = (A)ft0;
+    const A v0[3] = {vxt, vyt, vzt};
+    // (E at the particle as E0 + f (E1 - E0): the adjoint needs the difference too)
+    A Ep[3], Bp[3], Ed[3], Bd[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      Ep[c] = fmaT(ft0, a0.E[c * nxn + c0 + 1], g0t * a0.E[c * nxn + c0]);
-      Bp[c] = fmaT(ft0, a0.Bb[c * nxn + c0 + 1], g0t * a0.Bb[c * nxn + c0]);
-      Ed[c] = (A)a0.E[c * nxn + c0 + 1] - (A)a0.E[c * nxn + c0];
-      Bd[c] = (A)a0.Bb[c * nxn + c0 + 1] - (A)a0.Bb[c * nxn + c0];
+      const A e0 = a0.E[c * nxn + c0], b0 = a0.Bb[c * nxn + c0];
+      Ed[c] = a0.E[c * nxn + c0 + 1] - e0;
+      Bd[c] = a0.Bb[c * nxn + c0 + 1] - b0;
+      Ep[c] = fmaT(f0, Ed[c], e0);
+      Bp[c] = fmaT(f0, Bd[c], b0);
     }
-    const A v0[3] = {(A)t0.v[p], (A)t0.v[cap + p], (A)t0.v[2 * cap + p]};
-    T vxt = t0.v[p], vyt = t0.v[cap + p], vzt = t0.v[2 * cap + p];
-    boris<T>(vxt, vyt, vzt, Ep, Bp, pc.hdt);
-    const A vp[3] = {(A)vxt, (A)vyt, (A)vzt};  // before the return
+    // ---- Boris: v+ = q + em, q = vm + p x s, p = vm + vm x t,
+    //      s = (2 / (1 + t.t)) t, t = hdt B, vm = v + em, em = hdt E
+    const A hdt = pc.hdt;
+    A em[3], vm[3], t[3], sv[3], pp[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      em[c] = hdt * Ep[c];
+      vm[c] = v0[c] + em[c];
+      t[c] = hdt * Bp[c];
+    }
+    const A fct = (A)2 * rcpT((A)1 + fmaT(t[2], t[2], fmaT(t[1], t[1], t[0] * t[0])));
+    for (int c = 0; c < 3; ++c) sv[c] = fct * t[c];
+    pp[0] = fmaT(vm[1], t[2], fmaT(-vm[2], t[1], vm[0]));
+    pp[1] = fmaT(vm[2], t[0], fmaT(-vm[0], t[2], vm[1]));
+    pp[2] = fmaT(vm[0], t[1], fmaT(-vm[1], t[0], vm[2]));
     A lvp[3];  // adjoint of vp
     A lf0;
     if (e == kEvReturned) {
-      // vnew = R(vp; u2), f1 = clamp(gf * vnew_x * dtdx), gf = Xn/(Xn - Xo)
+      // vnew = R(vp; u2), f1 = clamp(gf * vnew_x * dtdx), gf = Xn/(Xn - Xo);
+      // vp: the velocity before the return
+      const A vp[3] = {fmaT(pp[1], sv[2], fmaT(-pp[2], sv[1], vm[0])) + em[0],
+                       fmaT(pp[2], sv[0], fmaT(-pp[0], sv[2], vm[1])) + em[1],
+                       fmaT(pp[0], sv[1], fmaT(-pp[1], sv[0], vm[2])) + em[2]};
       const Philox4 r = draw4(ph.seed, id & kIdMask, step, kPurposeFS);
       const double s1 = sqrt(u01(r.x[1]));
       double cs, sn2;
@@ -1081,21 +1138,7 @@ __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const S
       lvp[2] = lv[2];
       lf0 = lf1;
     }
-    // ---- Boris adjoint: v+ = q + em, q = vm + p x s, p = vm + vm x t,
-    //      s = (2 / (1 + t.t)) t, t = hdt B, vm = v + em, em = hdt E
-    const A hdt = pc.hdt;
-    A em[3], vm[3], t[3], sv[3], pp[3];
-    for (int c = 0; c < 3; ++c) {
-      em[c] = hdt * (A)Ep[c];
-      vm[c] = v0[c] + em[c];
-      t[c] = hdt * (A)Bp[c];
-    }
-    const A tt = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
-    const A fct = (A)2 / ((A)1 + tt);
-    for (int c = 0; c < 3; ++c) sv[c] = fct * t[c];
-    pp[0] = vm[0] + (vm[1] * t[2] - vm[2] * t[1]);
-    pp[1] = vm[1] + (vm[2] * t[0] - vm[0] * t[2]);
-    pp[2] = vm[2] + (vm[0] * t[1] - vm[1] * t[0]);
+    // ---- Boris adjoint
     const A* Lq = lvp;
     A Lem[3] = {lvp[0], lvp[1], lvp[2]};
     A Lvm[3] = {Lq[0], Lq[1], Lq[2]};
@@ -1119,15 +1162,15 @@ __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const S
     }
     const A LE[3] = {hdt * Lem[0], hdt * Lem[1], hdt * Lem[2]};
     const A LB[3] = {hdt * Lt[0], hdt * Lt[1], hdt * Lt[2]};
-    // ---- gather adjoint at the state before the step: the shares of the
-    //      nodes c0, c0 + 1 in lE, lBb go to the caller
+    // ---- gather adjoint at the state before the step: the adjoints of E and
+    //      Bbar at the particle and its offset go to the caller, which
+    //      shares them out to the nodes c0, c0 + 1
     for (int c = 0; c < 3; ++c) {
-      out[4 * c] = ((A)1 - f0) * LE[c];
-      out[4 * c + 1] = f0 * LE[c];
-      out[4 * c + 2] = ((A)1 - f0) * LB[c];
-      out[4 * c + 3] = f0 * LB[c];
-      lf0 += LE[c] * Ed[c] + LB[c] * Bd[c];
+      out[c] = LE[c];
+      out[3 + c] = LB[c];
+      lf0 = fmaT(LE[c], Ed[c], fmaT(LB[c], Bd[c], lf0));
     }
+    out[6] = f0;
     w.lf[p] = (T)lf0;
     w.lv[p] = (T)Lvm[0];
     w.lv[cap + p] = (T)Lvm[1];
@@ -1149,39 +1192,44 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 4 : 2)
                        double* lBb, Geo g, Phys ph, PushConst<T> pc, long long step, int np0,
                        int np1, int M) {
   __shared__ CellSort cs;
-  __shared__ T rec[kBlock][12];
+  __shared__ T rec[kBlock][8];  // adjoints of E, Bbar; the node weights 1 - f, f
   const int nxn = g.nxn;
   const int lane = threadIdx.x & 31;
   double gu2 = 0.0, gucr = 0.0;
   const int blk = (blockIdx.x & 1) ? gridDim.x - 1 - blockIdx.x / 2 : blockIdx.x / 2;
   const int p = blk * kBlock + threadIdx.x;
-  T a[12];
+  T a[7];
   const int c0 =
       (p < np1) ? particle_adj_slot<T>(p, w, a0, t1, ev, g, ph, pc, step, np0, gu2, gucr, a) : -1;
-  // value k of a cell's 12: E or Bbar (k & 2), component k / 4, node k & 1
+  // value k of a cell's 12: component k / 2 (E, then Bbar), node k & 1
   auto target = [&](int k, int c) {
-    return ((k & 2) ? lBb : lE) + (k >> 2) * nxn + c + (k & 1);
+    return (k < 6 ? lE + (k >> 1) * nxn : lBb + ((k >> 1) - 3) * nxn) + c + (k & 1);
   };
   int base, range;
   const int pos = cell_sort(cs, c0, base, range);
   if (range > kSortKeys) {
     if (c0 >= 0)
 #pragma unroll
-      for (int k = 0; k < 12; ++k) atomicAdd(target(k, c0), wide_double(a[k]));
+      for (int k = 0; k < 12; ++k)
+        atomicAdd(target(k, c0), wide_double(a[k >> 1] * ((k & 1) ? a[6] : (T)1 - a[6])));
   } else {
-    if (c0 >= 0)
+    if (c0 >= 0) {
 #pragma unroll
-      for (int k = 0; k < 12; ++k) rec[pos][k] = a[k];
+      for (int k = 0; k < 6; ++k) rec[pos][k] = a[k];
+      rec[pos][6] = (T)1 - a[6];
+      rec[pos][7] = a[6];
+    }
     __syncthreads();
-    const int k = lane & 15;
-    for (int c = threadIdx.x >> 5; c < range; c += kBlock / 32) {
-      const int b0 = cs.first[c], b1 = cs.first[c + 1];
-      if (b0 == b1) continue;
+    const int k = lane & 15, pieces = range ? cs.pieces : 0;
+    for (int c = threadIdx.x >> 5; c < pieces; c += kBlock / 32) {
+      const int b1 = cs.to[c];
       T s = (T)0;
       if (k < 12)
-        for (int i = b0 + (lane >> 4); i < b1; i += 2) s += rec[i][k];
+#pragma unroll 4
+        for (int i = cs.from[c] + (lane >> 4); i < b1; i += 2)
+          s = fmaT(rec[i][k >> 1], rec[i][6 + (k & 1)], s);
       s += __shfl_xor_sync(0xffffffffu, s, 16);
-      if (lane < 12) atomicAdd(target(k, base + c), wide_double(s));
+      if (lane < 12) atomicAdd(target(k, base + cs.cell[c]), wide_double(s));
     }
   }
   // only slots that were returned or injected add to these: most warps have
@@ -1197,28 +1245,23 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 4 : 2)
   }
 }
 
-// d loss / d a_m = sum_c lB_y(c) cos(arg) + lB_z(c) sin(arg), one CTA per mode
+// d loss / d a_m = sum_c lB_y(c) cos(arg) + lB_z(c) sin(arg), a CTA per mode
+// and 256 cells (grad is zero before)
 __global__ void k_win_mode_grad(const double* lB, double* grad, const double* phases, Geo g,
                                 double dx) {
   const int m = blockIdx.x;
   const double L = (double)g.nx * dx;
   double s = 0.0;
-  for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
+  const int i = blockIdx.y * blockDim.x + threadIdx.x;
+  if (i < g.nx) {
     const double x = ((double)i + 0.5) * dx;
     const double arg = 2.0 * 3.14159265358979323846 * (double)(m + 1) * x / L + phases[m];
     double sn, cs;
     sincos(arg, &sn, &cs);
-    s += lB[g.nx + i] * cs + lB[2 * g.nx + i] * sn;
+    s = lB[g.nx + i] * cs + lB[2 * g.nx + i] * sn;
   }
-  __shared__ double red[32];
   s = warp_sum_d(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double r = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-    r = warp_sum_d(r);
-    if (threadIdx.x == 0) grad[m] = r;
-  }
+  if ((threadIdx.x & 31) == 0) atomicAdd(&grad[m], s);
 }
 
 }  // namespace win
@@ -1448,7 +1491,7 @@ void forward_step(fs_window* w, const Win<T>& r, int n, const State<T>& a, const
   if (np1 > 0)
     k_win_push_deposit<T><<<blocks(np1), kBlock, 0, w->st>>>(r, a, b.s, drawn, ev, q, w->g, w->ph,
                                                              push_const<T>(w->ph), n, np, np1);
-  k_win_fields<T><<<tiles(w->g.nx), kTbThreads, fields_smem(w->p.n_sub, sizeof(T)), w->st>>>(
+  k_win_fields<T><<<tiles(w->g.nx), fields_threads(w->p.n_sub), fields_smem(w->p.n_sub, sizeof(T)), w->st>>>(
       a.B, b, q, qz, w->g, w->ph, field_const<T>(w->ph), w->p.n_sub);
   w->qsel ^= 1;
 }
@@ -1492,7 +1535,7 @@ int do_forward(fs_window* w, const double* theta, double* loss) {
   if (nborn > 0)
     k_win_draw<T><<<blocks(nborn), kBlock, 0, w->st>>>(r, w->g, w->ph,
                                                        (const int*)(w->base + w->o_sched), w->steps);
-  k_win_seed_B<T><<<blocks(w->g.nx), kBlock, 0, w->st>>>(r.B[0], w->g, w->ph, w->p.dx, amps,
+  k_win_seed_B<T><<<(w->g.nx + kSeedCells - 1) / kSeedCells, kBlock, 0, w->st>>>(r.B[0], w->g, w->ph, w->p.dx, amps,
                                                           amps + M, M);
   const size_t qb = 8 * 4 * (size_t)w->g.nxn;
   cudaMemsetAsync(r.q[0], 0, qb, w->st);
@@ -1555,7 +1598,7 @@ int do_backward(fs_window* w, double dloss, double* grad) {
       const State<T> a = at(k), b = at(k + 1);
       // the step's field update and moments in reverse, with the Ohm's law
       // that followed it
-      k_win_rk4_adj<T><<<tiles(nx), kTbThreads, rk4_adj_smem(w->p.n_sub, sizeof(T)), w->st>>>(
+      k_win_rk4_adj<T><<<tiles(nx), rk4_adj_threads(w->p.n_sub), rk4_adj_smem(w->p.n_sub, sizeof(T)), w->st>>>(
           w->g, w->ph, field_const<T>(w->ph), w->p.n_sub, a.B, b, r.lE[esel], r.lBb[esel],
           r.lE[1 - esel], r.lBb[1 - esel], r.lB, r.lBx, r.lNr, r.lJ);
       std::swap(r.lB, r.lBx);
@@ -1567,11 +1610,11 @@ int do_backward(fs_window* w, double dloss, double* grad) {
             npa, npb, M);
     }
     if (seg == 0)
-      k_win_ohm_adj_start<T><<<tiles(nx), kTbThreads, 0, w->st>>>(first, w->g, w->ph, r.lE[esel],
+      k_win_ohm_adj_start<T><<<tiles(nx), 32, 0, w->st>>>(first, w->g, w->ph, r.lE[esel],
                                                                   r.lBb[esel], r.lB);
   }
   double* phases = (double*)(w->base + w->o_params) + M;
-  if (M > 0) k_win_mode_grad<<<M, kBlock, 0, w->st>>>(r.lB, r.grad, phases, w->g, w->p.dx);
+  if (M > 0) k_win_mode_grad<<<dim3(M, blocks(nx)), kBlock, 0, w->st>>>(r.lB, r.grad, phases, w->g, w->p.dx);
   if (cudaMemcpyAsync(grad, r.grad, 8 * (M + 2), cudaMemcpyDeviceToHost, w->st) != cudaSuccess ||
       cudaStreamSynchronize(w->st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
     return FS_ECUDA;
