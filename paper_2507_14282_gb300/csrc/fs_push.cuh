@@ -12,8 +12,9 @@
 //      of the tile) or REMOVED; lanes with the same key take consecutive
 //      ranks after one shared atomic per key; then deposit the PREVIOUS
 //      chunk, in pieces (a key's particles, at most kPiece) that the warps
-//      claim from a shared counter, each piece a corner x split team
-//      reduction, so that warps which finished their push early take more;
+//      claim from a shared counter two at a time, each piece a half-warp's
+//      corner x split team reduction, so that warps which finished their push
+//      early take more;
 //   3. (barrier) each warp scans the key counts; every thread copies its
 //      particles into the key-sorted buffer;
 //   4. (barrier) the stage is refilled with a later chunk; coalesced writes
@@ -112,6 +113,7 @@ struct StepArgs {
 
 // ---------------------------------------------------------------- layout
 constexpr int kMaxStages = 4;
+constexpr int kPiece = 80;  // particles of a deposit piece at most (a half-warp's)
 constexpr int kWarps = kBlock / 32;
 
 template <typename T, int DIM>
@@ -120,7 +122,7 @@ struct PushLayout {
   // stage 0's regions; stage b sits b * bstride bytes further
   size_t F[1], cell[1], ox[1], oy[1], vx[1], vy[1], vz[1], id[1];
   size_t sW, sV, sF, scell, sid;  // key-sorted buffer
-  size_t acc, kc, wk, e2k, k2e, desc, bar, pf, tally, pst, dq, bytes;
+  size_t acc, kc, wk, e2k, k2e, desc, bar, pf, tally, pcs, dq, bytes;
   size_t bstride;  // distance between two chunk buffers
   __host__ __device__ static size_t take(size_t& o, size_t n) {
     o = (o + 15) / 16 * 16;
@@ -171,12 +173,19 @@ struct PushLayout {
     tally = take(o, sizeof(unsigned long long) * 4 + sizeof(double) * 2);
     acc = take(o, sizeof(typename Num<T>::acc) * 2 * 4 * NA);  // two tiles in flight
     kc = take(o, sizeof(int) * 2 * NK);                         // two chunks in flight
-    wk = take(o, sizeof(int) * kWarps * (NK + 1));              // key offsets per warp
-    pst = take(o, sizeof(int) * (NK + 1));  // first deposit piece of each key
-    dq = take(o, sizeof(int) * 2);          // deposit piece counters, two chunks
+    // key offsets per warp (16 bits: a 5 x 5-cell tile then fits four CTAs per SM)
+    wk = take(o, sizeof(uint16_t) * kWarps * (NK + 1));
+    pcs = take(o, sizeof(int) * (max_pieces() + 1));  // deposit pieces, their number
+    dq = take(o, sizeof(int) * 2);                    // deposit piece counters, two chunks
     e2k = take(o, sizeof(uint16_t) * NE);
     k2e = take(o, sizeof(int) * NE);
     bytes = (o + 127) / 128 * 128;
+  }
+  // deposit pieces of a chunk at most: one per key and one per full kPiece, and
+  // no more than its particles
+  __host__ __device__ int max_pieces() const {
+    const int a = NE + CH / kPiece;
+    return a < CH ? a : CH;
   }
   // bytes one chunk of m particles brings in
   __host__ __device__ uint32_t chunk_bytes(int m) const {
@@ -187,7 +196,7 @@ struct PushLayout {
 };
 
 // exclusive scan of n ints by one warp (lanes of warp w); out[n] = total
-__device__ __forceinline__ void warp_scan_excl(const int* in, int* out, int n,
+__device__ __forceinline__ void warp_scan_excl(const int* in, uint16_t* out, int n,
                                                int lane) {
   if (n <= 32) {  // one value per lane
     const int s = lane < n ? in[lane] : 0;
@@ -197,8 +206,8 @@ __device__ __forceinline__ void warp_scan_excl(const int* in, int* out, int n,
       const int v = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += v;
     }
-    if (lane < n) out[lane] = inc - s;
-    if (lane == 31) out[n] = inc;
+    if (lane < n) out[lane] = (uint16_t)(inc - s);
+    if (lane == 31) out[n] = (uint16_t)inc;
     return;
   }
   const int per = (n + 31) / 32;
@@ -213,10 +222,10 @@ __device__ __forceinline__ void warp_scan_excl(const int* in, int* out, int n,
   }
   int run = inc - s;
   for (int k = b; k < e; ++k) {
-    out[k] = run;
+    out[k] = (uint16_t)run;
     run += in[k];
   }
-  if (lane == 31) out[n] = inc;
+  if (lane == 31) out[n] = (uint16_t)inc;
 }
 
 // The chunk after c = {tile, first particle, count, tile count} for a CTA
@@ -313,7 +322,7 @@ __device__ __forceinline__ int push_one(const T* __restrict__ F, int NFX, int& c
                                         int EX, int EY, int NE, const uint16_t* e2k,
                                         const Geo& g, const Phys& ph, T dtdx, T dtdy,
                                         T hdt, T c2inv_t, long long step, PushTally* tl,
-                                        int& status, bool inner) {
+                                        int& status, bool inner, T& ig_out) {
   const int i = cell & 0xFFFF, j = cell >> 16;
   const int lx = i - i0, ly = j - j0;
   if ((unsigned)lx >= (unsigned)TX || (unsigned)ly >= (unsigned)TY) {
@@ -406,6 +415,7 @@ __device__ __forceinline__ int push_one(const T* __restrict__ F, int NFX, int& c
     mvx = vx * ig;
     mvy = vy * ig;
   }
+  ig_out = ig;  // 1/gamma of the stored state
   const T fxr = fmaT(mvx, dtdx, fx);
   T fyr = fy;
   if (DIM == 2) fyr = fmaT(mvy, dtdy, fy);
@@ -529,6 +539,7 @@ __device__ __forceinline__ int push_one(const T* __restrict__ F, int NFX, int& c
       vx = (T)ux;
       vy = (T)uy;
       vz = (T)uz;
+      if (c2inv > (T)0) ig_out = inv_gamma_u(vx, vy, vz, c2inv);
       id |= kIdReturned;
     } else {
       atomicAdd(&tl->tr, 1ull);
@@ -584,14 +595,14 @@ __device__ __forceinline__ void issue_chunk(unsigned char* sm, const PushLayout<
 }
 
 
-// CIC deposit of one key's particles, which sit contiguously in [b0, b1) of
-// the key-sorted chunk (W: corner weights, V: {vx, vy, vz, 1/gamma}). The warp
-// works as NC corners x SPL splits: lane (corner c, split s) sums corner c's
-// four quantities (weight, weight * v) over particles b0 + s, b0 + s + SPL,
-// ...; a transpose reduction over the splits then leaves each quantity's
-// total in one lane, which adds it to the tile's node accumulator. Each
-// contribution is formed as in the per-particle scheme, so in fixed point
-// the sums do not depend on the order.
+// CIC deposit of one piece per half-warp: a key's particles, which sit
+// contiguously in [b0, b1) of the key-sorted chunk (W: corner weights, V: {vx,
+// vy, vz, 1/gamma}). A half-warp works as NC corners x SPL splits: lane (corner
+// c, split s) sums corner c's four quantities (weight, weight * v) over
+// particles b0 + s, b0 + s + SPL, ...; a transpose reduction over the splits
+// then leaves each quantity's total in one lane, which adds it to the tile's
+// node accumulator. Each contribution is formed as in the per-particle scheme,
+// so in fixed point the sums do not depend on the order.
 template <typename T, int DIM, bool REL>
 __device__ __forceinline__ void team_add(typename Num<T>::acc (&acc)[4], const T* W,
                                          const T* V, const T* Fo, const uint32_t* ID,
@@ -633,8 +644,8 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
                                              int lane) {
   using A_t = typename Num<T>::acc;
   constexpr int NC = (DIM == 2) ? 4 : 2;
-  constexpr int SPL = 32 / NC;
-  const int s = lane % SPL, c = lane / SPL;
+  constexpr int SPL = 16 / NC;
+  const int s = lane % SPL, c = (lane & 15) / SPL;
   A_t acc[4] = {(A_t)0, (A_t)0, (A_t)0, (A_t)0};
   int i = b0 + s;
   for (; i + SPL < b1; i += 2 * SPL) {  // two particles in flight per lane
@@ -642,6 +653,7 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
     team_add<T, DIM, REL>(acc, W, V, Fo, ID, wth, wcr, i + SPL, c);
   }
   if (i < b1) team_add<T, DIM, REL>(acc, W, V, Fo, ID, wth, wcr, i, c);
+  __syncwarp();
   // two halving levels leave one quantity per lane, the rest add pairs
   {
     const bool up = (s & (SPL / 2)) != 0;
@@ -660,7 +672,7 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
   }
 #pragma unroll
   for (int off = SPL / 8; off >= 1; off >>= 1) acc[0] = acc[0] + shfl_xor(acc[0], off);
-  if ((s & (SPL / 4 - 1)) == 0) {
+  if (b0 < b1 && (s & (SPL / 4 - 1)) == 0) {
     const int q = ((s & (SPL / 2)) ? 2 : 0) + ((s & (SPL / 4)) ? 1 : 0);
     const int a00 = (le & 0xFFFF) + (le >> 16) * AX;
     const int an = a00 + (c & 1) + ((DIM == 2) ? (c >> 1) * AX : 0);
@@ -668,49 +680,43 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
   }
 }
 
-// Deposit of a key-sorted chunk in pieces: key k's particles [wk[k], wk[k+1])
-// form ceil(n / kPiece) pieces of at most kPiece, numbered from pst[k]. Warp
-// w > 0 takes piece w - 1, then (and warp 0 from the start) the next
-// unclaimed piece from the counter *q until none is left, so that warps which
-// reach the deposit early take more of it. A piece is one team reduction:
-// whole keys (cells) where they are not large, since the reduction, not the
-// particle count, sets most of a piece's cost. Each particle's contributions
-// are formed as in the per-particle scheme, so in fixed point (FP64) the sums
-// do not depend on which warp takes which piece.
-constexpr int kPiece = 160;
+// Deposit of a key-sorted chunk in pieces of at most kPiece particles of one
+// key (list pcs: key << 10 | first particle; pcs[npmax] their number). Warps
+// claim pairs of pieces: warp w > 0 takes pair w - 1 first, then (and warp 0,
+// which issues the bulk copies, from the start) the next unclaimed pair from
+// the counter *q until none is left, so that warps which reach the deposit
+// early take more of it. A pair is two pieces two apart (4 m + r and 4 m + r +
+// 2), one per half-warp: neighbouring cells share nodes, whose shared-memory
+// adds (a compare-and-swap loop in FP32) would retry against each other. A
+// piece's team reduction, not its particle count, sets most of its cost: with
+// a whole warp per piece, found by a search over the keys, the 49 keys of a
+// 5 x 5-cell tile at 20 particles per cell made the push 27.3 warp
+// instructions per particle (17.0 on 4 x 2 cells at 64). Each particle's
+// contributions are formed as in the per-particle scheme, so in fixed point
+// (FP64) the sums do not depend on which warp takes which piece.
 template <typename T, int DIM, bool REL>
-__device__ __forceinline__ void deposit_pieces(typename Num<T>::acc* ACC, int NA, int AX, int NE,
-                                               const int* wk, const int* pst, const int* k2e,
-                                               const T* W, const T* V, const T* Fo,
-                                               const uint32_t* ID, T wth, T wcr, int* q,
-                                               int warp, int lane) {
-  constexpr int PS = kPiece;
-  const int np = pst[NE];
-  // warp 0 (which issues the bulk copies) claims from the start; warp w > 0
-  // takes piece w - 1 first
-  int gi;
+__device__ __forceinline__ void deposit_pieces(typename Num<T>::acc* ACC, int NA, int AX,
+                                               const uint16_t* wk, const int* pcs, int npmax,
+                                               const int* k2e, const T* W, const T* V,
+                                               const T* Fo, const uint32_t* ID, T wth, T wcr,
+                                               int* q, int warp, int lane) {
+  const int np = pcs[npmax];
+  int gi = warp - 1;
   if (warp == 0) {
     int nx = 0;
     if (lane == 0) nx = atomicAdd(q, 1);
     gi = kWarps - 1 + __shfl_sync(0xffffffffu, nx, 0);
-  } else {
-    gi = warp - 1;
   }
-  while (gi < np) {
-    int k = -1;
-    for (int kb = 0; kb < NE; kb += 32) {
-      const int kk = kb + lane;
-      const unsigned h =
-          __ballot_sync(0xffffffffu, kk < NE && pst[kk] <= gi && gi < pst[kk + 1]);
-      if (h) {
-        k = kb + __ffs(h) - 1;
-        break;
-      }
+  while ((gi >> 1) * 4 + (gi & 1) < np) {
+    const int at = (gi >> 1) * 4 + (gi & 1) + ((lane >> 4) << 1);
+    int b0 = 0, b1 = 0, le = 0;
+    if (at < np) {
+      const int pc = pcs[at], k = pc >> 10;
+      b0 = pc & 1023;
+      b1 = min(b0 + kPiece, (int)wk[k + 1]);
+      le = k2e[k];
     }
-    if (k < 0) break;
-    const int b0 = wk[k] + (gi - pst[k]) * PS;
-    const int b1 = min(b0 + PS, wk[k + 1]);
-    team_deposit<T, DIM, REL>(ACC, NA, AX, k2e[k], b0, b1, W, V, Fo, ID, wth, wcr, lane);
+    team_deposit<T, DIM, REL>(ACC, NA, AX, le, b0, b1, W, V, Fo, ID, wth, wcr, lane);
     int nx = 0;
     if (lane == 0) nx = atomicAdd(q, 1);
     gi = kWarps - 1 + __shfl_sync(0xffffffffu, nx, 0);
@@ -748,7 +754,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
   int* pf = (int*)(sm + L.pf);
   PushTally* tl = (PushTally*)(sm + L.tally);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int* wk = (int*)(sm + L.wk) + warp * (NK + 1);
+  uint16_t* wk = (uint16_t*)(sm + L.wk) + warp * (NK + 1);
   const int* cnt_in = d.cnt[in];
   const Parts<T> PI = d.P[in];
   const Parts<T> PO = d.P[out];
@@ -778,7 +784,8 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
   }
   for (int k = tid; k < 2 * 4 * NA; k += kBlock) ACC0[k] = (A)0;
   for (int k = tid; k < 2 * NK; k += kBlock) kc0[k] = 0;
-  int* pst = (int*)(sm + L.pst);
+  int* pcs = (int*)(sm + L.pcs);
+  const int npmax = L.max_pieces();
   int* dq = (int*)(sm + L.dq);
   if (tid < 2) dq[tid] = 0;
 
@@ -824,7 +831,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
     if (c.x >= g.ntiles) {
       // the last chunk's deposit
       if (dpar >= 0)
-        deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, NE, wk, pst, k2e, oW, oV,
+        deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, wk, pcs, npmax, k2e, oW, oV,
                                     oF, oid, wth, wcr, dq + ((ci - 1) & 1), warp, lane);
       break;
     }
@@ -856,7 +863,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
     int ky[PPT], rk[PPT];
     int rc_[PPT];
     uint32_t rid_[PPT];
-    T rfx_[PPT], rfy_[PPT], rvx_[PPT], rvy_[PPT], rvz_[PPT];
+    T rfx_[PPT], rfy_[PPT], rvx_[PPT], rvy_[PPT], rvz_[PPT], rig_[PPT];
 #pragma unroll
     for (int r = 0; r < PPT; ++r) {
       const int p = tid + r * kBlock;
@@ -870,9 +877,10 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
         T fy = (DIM == 2) ? sy[p] : (T)0;
         T vx = svx[p], vy = svy[p], vz = svz[p];
         uint32_t id = sid[p];
+        T ig;
         key = push_one<T, DIM, REL>(F, L.NFX, cell, fx, fy, vx, vy, vz, id, i0, j0, TX, TY, EX,
                                EY, NE, e2k, g, ph, dtdx, dtdy, hdt, c2inv, step, tl,
-                               status, inner);
+                               status, inner, ig);
         if (key == NE) {  // far mover: straight to the global far sums
           T dvx, dvy, dvz;  // the current uses the velocity
           velocity_of<T>(vx, vy, vz, c2inv, dvx, dvy, dvz);
@@ -886,6 +894,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
           rvx_[r] = vx;
           rvy_[r] = vy;
           rvz_[r] = vz;
+          rig_[r] = ig;
           rid_[r] = id;
         } else {
           sc[p] = cell;
@@ -909,7 +918,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
     // ---- the previous chunk's deposit, after this chunk's push: warps that
     //      finished their push early take more of it
     if (dpar >= 0)
-      deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, NE, wk, pst, k2e, oW, oV, oF,
+      deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, wk, pcs, npmax, k2e, oW, oV, oF,
                                   oid, wth, wcr, dq + ((ci - 1) & 1), warp, lane);
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
@@ -935,23 +944,30 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
     // ---- key offsets (each warp its own copy); copy into key order
     warp_scan_excl(kc, wk, NK, lane);
     __syncwarp();
-    if (warp == kWarps - 1) {  // the deposit's pieces per key
-      constexpr int PS = kPiece;
+    if (warp == kWarps - 1) {  // the deposit's pieces, by key
       int carry = 0;
       for (int kb = 0; kb < NE; kb += 32) {
         const int kk = kb + lane;
-        const int n = kk < NE ? wk[kk + 1] - wk[kk] : 0;
-        const int pc = (n + PS - 1) / PS;
-        int inc = pc;
+        const int b0 = kk < NE ? wk[kk] : 0, n = kk < NE ? wk[kk + 1] - b0 : 0;
+        const unsigned any = __ballot_sync(0xffffffffu, n > 0);
+        const unsigned more = __ballot_sync(0xffffffffu, n > kPiece);
+        int at = carry + __popc(any & ((1u << lane) - 1u));
+        carry += __popc(any);
+        if (more) {  // keys of several pieces
+          const int x = n > kPiece ? (n - 1) / kPiece : 0;
+          int inc = x;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += v;
+          for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+          }
+          at += inc - x;
+          carry += __shfl_sync(0xffffffffu, inc, 31);
+          for (int r = 1; r <= x; ++r) pcs[at + r] = (kk << 10) | (b0 + r * kPiece);
         }
-        if (kk < NE) pst[kk] = carry + inc - pc;
-        carry += __shfl_sync(0xffffffffu, inc, 31);
+        if (n > 0) pcs[at] = (kk << 10) | b0;
       }
-      if (lane == 0) pst[NE] = carry;
+      if (lane == 0) pcs[npmax] = carry;
     }
 #pragma unroll
     for (int r = 0; r < PPT; ++r) {
@@ -970,11 +986,15 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
       oc[pos] = inreg ? rc_[r] : sc[p];
       oid[pos] = id;
       st2(oF + 2 * pos, fx, fy);
-      // {u} of the state, and 1/gamma (the current uses v = u / gamma)
+      // {u} of the state, and 1/gamma (the current uses v = u / gamma; FP64
+      // keeps the push's, a square root and a division on its narrow pipe)
       // (FP32 without relativistic terms: the particle weight, which the
       // deposit lanes use to form their corner weights)
       st4(oV + 4 * pos, ux, uy, uz,
-          (sizeof(T) == 4 && !REL) ? wp : (rel ? inv_gamma_u(ux, uy, uz, c2inv) : (T)1));
+          (sizeof(T) == 4 && !REL) ? wp
+          : !rel                   ? (T)1
+          : inreg                  ? rig_[r]
+                                   : inv_gamma_u(ux, uy, uz, c2inv));
       // corner weights: wp * (gx * gy), corners (0,0) (1,0) (0,1) (1,1)
       // (FP32: formed in the deposit)
       if constexpr (sizeof(T) == 8) {
