@@ -388,17 +388,17 @@ int grid_blocks(long long n) {
 // Kernels one step launches: push, movers, injection (1, or 2 with many rows),
 // moments, the field advance, step end. Moments and field advance are one
 // tiled launch in 1D boxes with x walls; else the field advance is one launch
-// per substep in FP32 2D boxes with x walls, or [FP64: Ohm density terms],
-// 2 x 4 x n_sub stage passes and the final Ohm (the same choice as the field
-// launcher makes).
+// per substep in FP32 2D boxes, Ohm and one per RK4 stage in FP64 2D boxes, and
+// in 1D [FP64: Ohm density terms], 2 x 4 x n_sub stage passes and the final Ohm
+// (the same choice as the field launcher makes).
 long long launches_per_step(const Sim* s) {
   const long long inj = s->g.ninj == 0 ? 0 : s->g.ninj <= 256 ? 1 : 2;
   const bool walls = s->g.bc_x != FS_BC_PERIODIC;
   long long fields;
   if (s->g.dim == 1 && walls && s->p.n_sub <= 16)
     fields = 0;  // with the moments
-  else if (s->p.precision == FS_FP32 && s->g.dim == 2 && walls)
-    fields = s->p.n_sub;
+  else if (s->g.dim == 2)
+    fields = s->p.precision == FS_FP32 ? s->p.n_sub : 1 + 4LL * s->p.n_sub;
   else
     fields = (s->p.precision == FS_FP64 ? 1 : 0) + 8LL * s->p.n_sub + 1;
   return 1 + 1 + inj + 1 + fields + 1;
@@ -413,11 +413,6 @@ int build_graphs(Sim* s) {
   for (cudaEvent_t* ev : {&s->ev_fork, &s->ev_draw, &s->ev_push, &s->ev_join})
     if (!*ev && cudaEventCreateWithFlags(ev, cudaEventDisableTiming) != cudaSuccess)
       return FS_ECUDA;
-  if (!s->side2 && cudaStreamCreateWithFlags(&s->side2, cudaStreamNonBlocking) != cudaSuccess)
-    return FS_ECUDA;
-  if ((!s->ev_fork2 && cudaEventCreateWithFlags(&s->ev_fork2, cudaEventDisableTiming) != cudaSuccess) ||
-      (!s->ev_join2 && cudaEventCreateWithFlags(&s->ev_join2, cudaEventDisableTiming) != cudaSuccess))
-    return FS_ECUDA;
   // the captured work must follow everything already queued on the caller's stream
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return FS_ECUDA;
   cudaStream_t user = s->stream;
@@ -464,18 +459,6 @@ void release_graphs(Sim* s) {
       cudaEventDestroy(*ev);
       *ev = nullptr;
     }
-  if (s->side2) {
-    cudaStreamDestroy(s->side2);
-    s->side2 = nullptr;
-  }
-  if (s->ev_fork2) {
-    cudaEventDestroy(s->ev_fork2);
-    s->ev_fork2 = nullptr;
-  }
-  if (s->ev_join2) {
-    cudaEventDestroy(s->ev_join2);
-    s->ev_join2 = nullptr;
-  }
   s->graphs_ready = false;
 }
 

@@ -865,7 +865,7 @@ __device__ __forceinline__ void rk4_stage(int stage, T K, T& bsum, T& bs, T& b, 
 template <typename T, int DIM>
 __device__ __forceinline__ void ohm_node(int q, const T* Bc, const T* nN, const T* uN,
                                          const T* pre, T* Eo, T* Bbo, T* G, const Geo& g,
-                                         const Phys& ph) {
+                                         const Phys& ph, T* preo = nullptr) {
   const int nx = g.nx, ny = g.ny, nxn = g.nxn;
   const int nc = nx * ny, nn = nxn * ny;
   const T hdx = (T)ph.hdx, hdy = (T)ph.hdy, idx = (T)ph.idx;
@@ -919,6 +919,11 @@ __device__ __forceinline__ void ohm_node(int q, const T* Bc, const T* nN, const 
       pgy = pre[2 * nn + q];
     } else {
       density_terms<T, DIM>(nN, i, j, g, ph, inv_n, pgx, pgy);
+      if (preo) {
+        preo[q] = inv_n;
+        preo[nn + q] = pgx;
+        preo[2 * nn + q] = pgy;
+      }
     }
     T ex, ey, ez;
     ohm_e<T>(cxv, cyv, czv, bbx, bby, bbz, inv_n, pgx, pgy, uN[q], uN[nn + q], uN[2 * nn + q],
@@ -1028,6 +1033,389 @@ template <typename T>
 __device__ __forceinline__ FieldConst<T> field_const_dev(const Phys& ph) {
   return FieldConst<T>{(T)ph.idx, (T)ph.hdx, (T)ph.hdy, (T)ph.te, (T)ph.jcr,
                        (T)ph.eta, (T)ph.h,   (T)ph.hh,  (T)ph.h6, ph.eta != 0.0 ? 1 : 0};
+}
+
+// Ohm's law from B at every node with the density terms formed here and kept in
+// preo ([1/n][-(T_e dn/dx)][-(T_e dn/dy)]) for the stages that follow: the
+// start of the 2D field advance.
+template <typename T, int DIM>
+__global__ void k_ohm_start(const T* __restrict__ Bc, const T* __restrict__ nN,
+                            const T* __restrict__ uN, T* __restrict__ Eo, T* __restrict__ preo,
+                            Geo g, Phys ph) {
+  const int nn = g.nxn * g.ny;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nn; q += gridDim.x * blockDim.x)
+    ohm_node<T, DIM>(q, Bc, nN, uN, nullptr, Eo, nullptr, nullptr, g, ph, preo);
+}
+
+// ------------------------------------------------------------------------
+// One RK4 stage of the 2D field advance in one pass: Faraday from Ei and the
+// stage update of B (stages 1-3: the stage field, kept in registers; stage 4:
+// the new B, into Bnew), then Ohm's E of that field at the nodes into Eo; with
+// FIN also Bbar and the packed gather block G. A warp marches down the rows
+// of a strip of 32 columns (lane = column i: its node and the cell to its
+// right): a row's E, B, RK4 sum, u and density terms are read once, the
+// neighbour columns come by shuffles, the previous row's sums stay in
+// registers, and nothing is shared between warps. Cell i needs node i + 1 (the
+// lane above), node i needs cell i - 1 (the lane below), so lanes 1 .. 30 are
+// the strip's own 30 columns; the cell row above the chunk is formed again.
+// Same expressions as ohm_node and faraday_cell. Used in FP64, where the narrow
+// FP64 pipe binds (82 % busy): against a pass per operator the row and column
+// sums that neighbours share are formed once, 53 operations per node and stage
+// instead of 65, and the stage field never goes to memory. 4096 x 256 cells,
+// two substeps: 1345 -> 1176 us. (In FP32, 8192 x 512 cells: 612 us against
+// k_field_substep's 340.)
+// One warp per block: the marches are few and long, so that blocks of several
+// would leave SMs uneven.
+constexpr int kMarchCols = 30;
+template <typename T, int STAGE, bool FIN>
+__global__ void __launch_bounds__(32)
+    k_field_march(const T* __restrict__ Ei, T* __restrict__ Eo, const T* __restrict__ B,
+                  T* __restrict__ Bsum, T* __restrict__ Bnew, const T* __restrict__ uN,
+                  const T* __restrict__ pre, T* __restrict__ Bbo, T* __restrict__ G, Geo g,
+                  FieldConst<T> fc, int rows, int strips) {
+  const int nx = g.nx, ny = g.ny, nxn = g.nxn;
+  const int nc = nx * ny, nn = nxn * ny;
+  const int lane = threadIdx.x & 31;
+  const int strip = blockIdx.x % strips, j0 = (blockIdx.x / strips) * rows;
+  const int j1 = min(ny, j0 + rows);
+  const bool per = g.bc_x == FS_BC_PERIODIC;
+  const int i = strip * kMarchCols - 1 + lane;
+  // this lane's node and cell columns (clamped or wrapped into the box)
+  const int ni = per ? wrap(i, nx) : min(max(i, 0), nx);
+  const int ci = per ? ni : min(max(i, 0), nx - 1);
+  const bool own = lane >= 1 && lane <= kMarchCols;
+  const bool own_node = own && i < nxn, own_cell = own && i < nx;
+  const bool wall0 = !per && i == 0, wall1 = !per && i == nx;
+  const T hdx = fc.hdx, hdy = fc.hdy;
+  const unsigned full = 0xffffffffu;
+  struct Row {  // what a row needs from memory; e: the node row below it
+    T e[3], b[3], s[3], u[3], p[3];
+  };
+  auto load = [&](int j, bool node, Row& r) {
+    const int jp = j + 1 == ny ? 0 : j + 1;
+    const int qe = jp * nxn + ni, qc = j * nx + ci, qn = j * nxn + ni;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      r.e[c] = Ei[c * nn + qe];
+      r.b[c] = B[c * nc + qc];
+      if (STAGE != 1) r.s[c] = Bsum[c * nc + qc];
+      if (node) {
+        r.u[c] = uN[c * nn + qn];
+        r.p[c] = pre[c * nn + qn];
+      }
+    }
+  };
+  T ea[3];        // E of the node row of the current cell row
+  T rx, rz;       // its sums of Ex, Ez over a cell's two nodes
+  T bs[3], bp[3]; // stage field of the current and the previous cell row
+  T pp[3];        // the previous row's sums over a node's two cells
+  auto right_sum = [&](T v) { return v + __shfl_down_sync(full, v, 1); };
+  // the stage field of a cell row from its loads; st: store the cell's values
+  auto cell_row = [&](int j, const Row& r, bool st) {
+    const T cy = ea[1] + r.e[1], cz = ea[2] + r.e[2];
+    const T dxey = (__shfl_down_sync(full, cy, 1) - cy) * hdx;
+    const T dxez = (__shfl_down_sync(full, cz, 1) - cz) * hdx;
+    const T nx_ = right_sum(r.e[0]), nz_ = right_sum(r.e[2]);
+    const T dyex = (nx_ - rx) * hdy;
+    const T dyez = (nz_ - rz) * hdy;
+    rx = nx_;
+    rz = nz_;
+    const T K[3] = {-dyez, dxez, dyex - dxey};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      T sum = STAGE != 1 ? r.s[c] : (T)0, b = r.b[c];
+      rk4_stage<T>(STAGE, K[c], sum, bs[c], b, fc.h, fc.hh, fc.h6);
+      if (STAGE == 4) bs[c] = b;
+      if (st) {
+        const size_t k = (size_t)c * nc + (size_t)j * nx + i;
+        if (STAGE == 4) Bnew[k] = b;
+        else Bsum[k] = sum;
+      }
+      ea[c] = r.e[c];
+    }
+  };
+  // a node's two cells of the current row: lb the left one
+  auto pair_sums = [&](T (&p)[3], T (&lb)[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      lb[c] = __shfl_up_sync(full, bs[c], 1);
+      if (wall1) bs[c] = lb[c];
+      if (wall0) lb[c] = bs[c];
+      p[c] = lb[c] + bs[c];
+    }
+  };
+  {
+    const int jm = j0 == 0 ? ny - 1 : j0 - 1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ea[c] = Ei[c * nn + jm * nxn + ni];
+    rx = right_sum(ea[0]);
+    rz = right_sum(ea[2]);
+    Row r;
+    load(jm, false, r);
+    cell_row(jm, r, false);
+    T lb[3];
+    pair_sums(pp, lb);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) bp[c] = bs[c];
+  }
+  Row cur;
+  load(j0, true, cur);
+  for (int j = j0; j < j1; ++j) {
+    Row nxt;
+    if (j + 1 < j1) load(j + 1, true, nxt);  // in flight while this row is worked on
+    cell_row(j, cur, own_cell);
+    T p[3], lb[3];
+    pair_sums(p, lb);
+    T bb[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) bb[c] = (T)0.25 * (pp[c] + p[c]);
+    const T cy = bs[1] + bp[1], cz = bs[2] + bp[2];  // right column's sums
+    T ly = __shfl_up_sync(full, cy, 1), lz = __shfl_up_sync(full, cz, 1);
+    if (wall0) {
+      ly = cy;
+      lz = cz;
+    }
+    const T dxby = (cy - ly) * hdx, dxbz = (cz - lz) * hdx;
+    const T dybx = (p[0] - pp[0]) * hdy, dybz = (p[2] - pp[2]) * hdy;
+    T E[3];
+    ohm_e<T>(dybz, -dxbz, dxby - dybx, bb[0], bb[1], bb[2], cur.p[0], cur.p[1], cur.p[2], cur.u[0],
+             cur.u[1], cur.u[2], fc.jcr, fc.eta, fc.resist != 0, E[0], E[1], E[2]);
+    if (own_node) {
+      const size_t q = (size_t)j * nxn + i;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) Eo[(size_t)c * nn + q] = E[c];
+      if (FIN) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Bbo[(size_t)c * nn + q] = bb[c];
+        const T v[8] = {E[0], E[1], E[2], bb[0], bb[1], bb[2], (T)0, (T)0};
+        auto put = [&](int gi, int gj) {
+          T* dst = G + ((size_t)gj * (nx + 1) + gi) * 8;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) dst[c] = v[c];
+        };
+        put(i, j);
+        if (j == 0) put(i, ny);
+        if (per && i == 0) {
+          put(nx, j);
+          if (j == 0) put(nx, ny);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      pp[c] = p[c];
+      bp[c] = bs[c];
+    }
+    cur = nxt;
+  }
+}
+
+// ------------------------------------------------------------------------
+// One RK4 substep of the 2D FP32 field advance in one launch: the four stages
+// follow each other down the rows of a warp's strip of columns (lane = column),
+// each a row behind the one before. At row t the warp reads B, n and u of the
+// row once; Ohm's E of B at node row t, stage 1 at cell row t - 1, its E at node
+// row t - 1, stage 2 at cell row t - 2, ... stage 4 (the new B) at cell row
+// t - 4; with FIN also E, Bbar and the packed gather block G of the new B. What
+// a stage needs of earlier rows (B, the RK4 sum, node terms, E and sums of the
+// previous row) is kept in registers, neighbour columns come by shuffles: no
+// shared memory and no barrier. Each stage spoils one column at either end of
+// the warp, the density differences one more at the right: 23 of 32 lanes are
+// the strip's own (22 with FIN), and a march starts 4 (5) rows early. At an x
+// wall the wall's node reads its one cell on both sides and the density is
+// mirrored; y wraps. Same expressions as ohm_node and faraday_cell.
+// Bound by instruction issue: about 420 per row of 23 columns. The tiles of
+// 32 x 16 cells before recomputed a halo of 4 to 5 cells, 2.1 times their
+// cells, through shared memory and 8 barriers: 8192 x 512 cells, two substeps,
+// 571 -> 340 us; 3000 x 250 172 -> 90; 256 x 64 59 -> 34; 512 x 512 periodic
+// (a pass per operator before) 141 -> 51.
+template <typename T>
+struct NodeRow {  // 1/n, the pressure terms and u at a node
+  T inv, pgx, pgy, ux, uy, uz;
+};
+template <typename T>
+struct CellSums {  // of the previous cell row: a node's two-cell sums, B_y, B_z
+  T p[3], by, bz;
+};
+template <typename T>
+struct NodeSums {  // of the previous node row: E, a cell's two-node sums of Ex, Ez
+  T e[3], rx, rz;
+};
+template <typename T, bool FIN>
+__global__ void __launch_bounds__(32)
+    k_field_substep(const T* __restrict__ B, T* __restrict__ Bn, const T* __restrict__ nN,
+                    const T* __restrict__ uN, T* __restrict__ Eo, T* __restrict__ Bbo,
+                    T* __restrict__ G, Geo g, FieldConst<T> fc, int rows, int strips) {
+  constexpr int OFF = FIN ? 5 : 4, COLS = FIN ? 22 : 23;
+  const int nx = g.nx, ny = g.ny, nxn = g.nxn;
+  const int nc = nx * ny, nn = nxn * ny;
+  const int lane = threadIdx.x;
+  const int strip = blockIdx.x % strips, j0 = (blockIdx.x / strips) * rows;
+  const int j1 = min(ny, j0 + rows);
+  const bool per = g.bc_x == FS_BC_PERIODIC;
+  const int i = strip * COLS - OFF + lane;
+  const int ni = per ? wrap(i, nx) : min(max(i, 0), nx);
+  const int ci = per ? ni : min(max(i, 0), nx - 1);
+  const bool own = lane >= OFF && lane < OFF + COLS;
+  const bool own_node = own && i < nxn, own_cell = own && i < nx;
+  const bool wall0 = !per && i == 0, wall1 = !per && i == nx;
+  const bool edge = __any_sync(0xffffffffu, wall0 || wall1);
+  const T hdx = fc.hdx, hdy = fc.hdy, te = fc.te;
+  const unsigned full = 0xffffffffu;
+  auto up1 = [&](T v) { return __shfl_up_sync(full, v, 1); };
+  auto down1 = [&](T v) { return __shfl_down_sync(full, v, 1); };
+  // Ohm's law at a node row from the cell row f below it and the sums of the
+  // cell row above (kept up to date)
+  auto ohm_row = [&](CellSums<T>& s, T (&f)[3], const NodeRow<T>& d, T (&E)[3], T (&bb)[3]) {
+    T lb[3], p[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lb[c] = up1(f[c]);
+    if (edge) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (wall1) f[c] = lb[c];
+        if (wall0) lb[c] = f[c];
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      p[c] = lb[c] + f[c];
+      bb[c] = (T)0.25 * (s.p[c] + p[c]);
+    }
+    const T cy = f[1] + s.by, cz = f[2] + s.bz;
+    T ly = up1(cy), lz = up1(cz);
+    if (edge && wall0) {
+      ly = cy;
+      lz = cz;
+    }
+    const T dxby = (cy - ly) * hdx, dxbz = (cz - lz) * hdx;
+    const T dybx = (p[0] - s.p[0]) * hdy, dybz = (p[2] - s.p[2]) * hdy;
+    ohm_e<T>(dybz, -dxbz, dxby - dybx, bb[0], bb[1], bb[2], d.inv, d.pgx, d.pgy, d.ux, d.uy, d.uz,
+             fc.jcr, fc.eta, fc.resist != 0, E[0], E[1], E[2]);
+    s = CellSums<T>{{p[0], p[1], p[2]}, f[1], f[2]};
+  };
+  // K = -curl E at the cell row between the node row in s and the row E
+  auto faraday_row = [&](NodeSums<T>& s, const T (&E)[3], T (&K)[3]) {
+    const T cy = s.e[1] + E[1], cz = s.e[2] + E[2];
+    const T dxey = (down1(cy) - cy) * hdx, dxez = (down1(cz) - cz) * hdx;
+    const T rx = E[0] + down1(E[0]), rz = E[2] + down1(E[2]);
+    const T dyex = (rx - s.rx) * hdy, dyez = (rz - s.rz) * hdy;
+    K[0] = -dyez;
+    K[1] = dxez;
+    K[2] = dyex - dxey;
+    s = NodeSums<T>{{E[0], E[1], E[2]}, rx, rz};
+  };
+  CellSums<T> cs[5] = {};
+  NodeSums<T> ns[4] = {};
+  NodeRow<T> nd[5] = {};  // node rows t, t - 1, ...
+  T bq[4][3] = {};        // B of cell rows t - 1, t - 2, ...
+  T sq[3][3] = {};        // RK4 sums of cell rows t - 2, t - 3, t - 4
+  int t = j0 - OFF;
+  int r = wrap(t, ny);  // row t in the box
+  T nm = nN[wrap(t - 1, ny) * nxn + ni], n0 = nN[r * nxn + ni];
+  struct In {
+    T b[3], u[3], np;
+  };
+  auto load = [&](int row, In& x) {
+    const int rp = row + 1 == ny ? 0 : row + 1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      x.b[c] = B[c * nc + row * nx + ci];
+      x.u[c] = uN[c * nn + row * nxn + ni];
+    }
+    x.np = nN[rp * nxn + ni];
+  };
+  In cur;
+  load(r, cur);
+  for (; t < j1 + 4; ++t) {
+    In nxt;
+    r = r + 1 == ny ? 0 : r + 1;
+    load(r, nxt);  // in flight while this row is worked on
+    {
+      T nl = up1(n0), nr = down1(n0);
+      if (edge) {
+        if (wall0) nl = nr;
+        if (wall1) nr = nl;
+      }
+      const T dnx = (nr - nl) * hdx, dny = (cur.np - nm) * hdy;
+      nd[0] = NodeRow<T>{(T)1 / n0, -(te * dnx), -(te * dny), cur.u[0], cur.u[1], cur.u[2]};
+      nm = n0;
+      n0 = cur.np;
+    }
+    T E[3], bb[3], K[3], f[3], s1[3], s2[3], s3[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f[c] = cur.b[c];
+    ohm_row(cs[0], f, nd[0], E, bb);
+    faraday_row(ns[0], E, K);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      T b = bq[0][c];
+      rk4_stage<T>(1, K[c], s1[c], f[c], b, fc.h, fc.hh, fc.h6);
+    }
+    ohm_row(cs[1], f, nd[1], E, bb);
+    faraday_row(ns[1], E, K);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      T b = bq[1][c];
+      s2[c] = sq[0][c];
+      rk4_stage<T>(2, K[c], s2[c], f[c], b, fc.h, fc.hh, fc.h6);
+    }
+    ohm_row(cs[2], f, nd[2], E, bb);
+    faraday_row(ns[2], E, K);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      T b = bq[2][c];
+      s3[c] = sq[1][c];
+      rk4_stage<T>(3, K[c], s3[c], f[c], b, fc.h, fc.hh, fc.h6);
+    }
+    ohm_row(cs[3], f, nd[3], E, bb);
+    faraday_row(ns[3], E, K);
+    const int j = t - 4;
+    const bool mine = j >= j0;  // (the rows before are the march's start)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      T b = bq[3][c], sum = sq[2][c], none;
+      rk4_stage<T>(4, K[c], sum, none, b, fc.h, fc.hh, fc.h6);
+      f[c] = b;
+      if (mine && own_cell) Bn[(size_t)c * nc + (size_t)j * nx + i] = b;
+    }
+    if (FIN) {
+      ohm_row(cs[4], f, nd[4], E, bb);
+      if (mine && own_node) {
+        const size_t q = (size_t)j * nxn + i;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          Eo[(size_t)c * nn + q] = E[c];
+          Bbo[(size_t)c * nn + q] = bb[c];
+        }
+        auto put = [&](int gi, int gj) {
+          float4* dst = (float4*)(G + ((size_t)gj * (nx + 1) + gi) * 8);
+          dst[0] = make_float4(E[0], E[1], E[2], bb[0]);
+          dst[1] = make_float4(bb[1], bb[2], 0.0f, 0.0f);
+        };
+        put(i, j);
+        if (j == 0) put(i, ny);
+        if (per && i == 0) {
+          put(nx, j);
+          if (j == 0) put(nx, ny);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 3; k > 0; --k)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) bq[k][c] = bq[k - 1][c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      bq[0][c] = cur.b[c];
+      sq[2][c] = s3[c];
+      sq[1][c] = s2[c];
+      sq[0][c] = s1[c];
+    }
+#pragma unroll
+    for (int k = 4; k > 0; --k) nd[k] = nd[k - 1];
+    cur = nxt;
+  }
 }
 
 // Quantity c (n, Jx, Jy, Jz) at node i of a 1D box with x walls: the far sum,
@@ -1323,229 +1711,6 @@ __device__ __forceinline__ void step1_end(const DevPtrs<T>& d, const Geo& g, int
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_step1_end(DevPtrs<T> d, Geo g) {
   step1_end<T>(d, g, blockIdx.x, gridDim.x);
-}
-
-// ------------------------------------------------------------------------
-// One RK4 substep of the 2D field advance by tiles, for boxes with x walls
-// (as separate passes it is memory-bound in FP32: each stage's Ohm and
-// Faraday re-read and re-write the grid). A CTA owns kFTX x kFTY cells (and
-// their lower-left nodes; the last tile in x also the wall nodes nx) and
-// runs the four stages in shared memory over its cells plus a halo of 4
-// cells (5 when it also forms E), which it recomputes: a stage's stencils reach one cell (node (i, j) reads
-// cells i-1..i, j-1..j and n at i±1, j±1; cell (i, j) reads nodes i..i+1,
-// j..j+1), so values made wrong at a tile's inner edges (read there with
-// indices clamped to the tile) move in by one cell per pass and stay outside
-// the owned cells. At an x wall the tile ends at the wall, where the clamped
-// indices are the wall's zero-gradient ghost cells and the density is
-// mirrored as in density_terms; y is periodic (rows wrap when loaded).
-// Reads B from Bin and writes the new B to Bout (neighbouring tiles read
-// Bin's cells). With `fin`, also Ohm's E and Bbar at the owned nodes from
-// the new B (Eo, Bbo, and the packed gather block G with its ghost row), as
-// the step's final k_ohm does. Same per-element arithmetic as ohm_node /
-// faraday_cell (2D). Boxes that are a whole number of tiles (x and y) run
-// the interior tile columns 1 .. gx - 2 (full tiles whose halo lies inside
-// the box) as one launch with the tile's local sizes compiled in, and the
-// two wall columns as a second launch of the general form.
-constexpr int kFTX = 32, kFTY = 16, kFH = 5;  // owned cells; halo of the last substep
-constexpr int kFLX = kFTX + 2 * kFH, kFLY = kFTY + 2 * kFH;
-constexpr int kFNPT = ((kFLX + 1) * (kFLY + 1) + kBlock - 1) / kBlock;  // nodes per thread
-// (the density, needed only for the density terms at the start, shares the
-// first E plane)
-template <typename T>
-constexpr size_t field_tile_smem() {
-  return sizeof(T) * (9 * (size_t)kFLX * kFLY + 3 * (size_t)(kFLX + 1) * (kFLY + 1));
-}
-
-// Walks the elements k = t0, t0 + kBlock, ... of an nx-by-ny local array,
-// keeping (a, b) = (k mod nx, k div nx) by increments.
-struct TileWalk {
-  int k, a, b, da, db, n, w;
-  __device__ __forceinline__ TileWalk(int t0, int w_, int h_) : k(t0), n(w_ * h_), w(w_) {
-    b = t0 / w_;
-    a = t0 - b * w_;
-    db = kBlock / w_;
-    da = kBlock - db * w_;
-  }
-  __device__ __forceinline__ void next() {
-    k += kBlock;
-    a += da;
-    b += db;
-    if (a >= w) {
-      a -= w;
-      ++b;
-    }
-  }
-};
-
-// FINC: -1 / -2 (fin from the argument) or the compile-time fin of an interior
-// tile launch (a full tile whose halo lies inside the box: its local sizes
-// are constants); bx0: the first tile column of the launch (blockIdx.x + bx0)
-template <typename T, int FINC>
-__global__ void __launch_bounds__(kBlock, (FINC >= 0 ? 4 : 1))
-    k_field_substep2(const T* __restrict__ Bin, T* __restrict__ Bout, const T* __restrict__ nN,
-                     const T* __restrict__ uN, T* __restrict__ Eo, T* __restrict__ Bbo,
-                     T* __restrict__ G, Geo g, Phys ph, FieldConst<T> fc, int fin_arg, int bx0,
-                     int bx_last) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int fin = FINC >= 0 ? FINC : fin_arg;
-  const int nx = g.nx, ny = g.ny, nxn = g.nxn;
-  const int nc = nx * ny, nn = nxn * ny;
-  const int H = fin ? kFH : kFH - 1;  // four stages need 4 cells, the final Ohm one more
-  // interior launch: columns bx0 ..; edge launch (FINC -1): columns 0 and
-  // bx_last; FINC -2: every column, general sizes
-  const int bx = (FINC >= 0) ? (int)blockIdx.x + bx0
-                 : (FINC == -1 ? (blockIdx.x == 0 ? 0 : bx_last) : (int)blockIdx.x);
-  const int cx0 = bx * kFTX, cx1 = (FINC >= 0) ? cx0 + kFTX : min(nx, cx0 + kFTX);
-  const int cy0 = blockIdx.y * kFTY, cy1 = (FINC >= 0) ? cy0 + kFTY : min(ny, cy0 + kFTY);
-  const int lx0 = (FINC >= 0) ? cx0 - H : max(0, cx0 - H);
-  const int LX = (FINC >= 0) ? kFTX + 2 * H : min(nx, cx1 + H) - lx0;  // local cell columns
-  const int ly0 = cy0 - H, LY = (cy1 - cy0) + 2 * H;             // local rows (unwrapped)
-  const int NX = LX + 1, NC = LX * LY, NN = NX * (LY + 1);        // nodes: NX x (LY + 1)
-  T* sB = (T*)smem;
-  T* sBs = sB + 3 * NC;
-  T* sK = sBs + 3 * NC;
-  T* sE = sK + 3 * NC;  // [3][NN]
-  T* sn = sE;           // [NN], read only before the first stage writes sE
-  const int t0 = threadIdx.x;
-  auto row = [&](int b) { return wrap(ly0 + b, ny); };
-  // (unrolled so that a thread's loads are in flight together)
-#pragma unroll 8
-  for (TileWalk w(t0, LX, 3 * LY); w.k < 3 * NC; w.next()) {
-    const int c = w.b / LY, b = w.b - c * LY;
-    sB[w.k] = Bin[(size_t)c * nc + (size_t)row(b) * nx + lx0 + w.a];
-  }
-  // this thread's nodes: u and (after the barrier) the density terms, fixed
-  // for the substep, stay in registers
-  T u[kFNPT][3], inv_n[kFNPT], pgx[kFNPT], pgy[kFNPT];
-  {
-    TileWalk w(t0, NX, LY + 1);
-#pragma unroll
-    for (int r = 0; r < kFNPT; ++r, w.next()) {
-      if (w.k < NN) {
-        const size_t q = (size_t)row(w.b) * nxn + lx0 + w.a;
-        sn[w.k] = nN[q];
-        u[r][0] = uN[q];
-        u[r][1] = uN[nn + q];
-        u[r][2] = uN[2 * nn + q];
-      }
-    }
-  }
-  __syncthreads();
-  const T hdx = fc.hdx, hdy = fc.hdy, te = fc.te, jcr = fc.jcr, eta = fc.eta;
-  const T h = fc.h, hh = fc.hh, h6 = fc.h6;
-  const bool resist = fc.resist != 0;
-  {
-    TileWalk w(t0, NX, LY + 1);
-#pragma unroll
-    for (int r = 0; r < kFNPT; ++r, w.next()) {
-      if (w.k < NN) {
-        // x neighbours mirrored at the walls, y neighbours in the tile
-        const int gx = lx0 + w.a;
-        const int xp = ((gx + 1 > nx) ? 2 * nx - (gx + 1) : gx + 1) - lx0;
-        const int xm = ((gx - 1 < 0) ? -(gx - 1) : gx - 1) - lx0;
-        const int rb = w.b * NX;
-        const T dnx = (sn[rb + min(max(xp, 0), LX)] - sn[rb + min(max(xm, 0), LX)]) * hdx;
-        const T dny = (sn[min(w.b + 1, LY) * NX + w.a] - sn[max(w.b - 1, 0) * NX + w.a]) * hdy;
-        inv_n[r] = (T)1 / sn[w.k];
-        pgx[r] = -(te * dnx);
-        pgy[r] = -(te * dny);
-      }
-    }
-  }
-  __syncthreads();  // the density terms are read before sE (which holds sn) is written
-  // Ohm at local node (a, b), the r-th of this thread, from the centre field Bc
-  auto ohm = [&](const T* Bc, int a, int b, int r, T E[3], T Bb[3]) {
-    const int im = min(max(a - 1, 0), LX - 1), ip = min(a, LX - 1);
-    const int jm = min(max(b - 1, 0), LY - 1), jp = min(b, LY - 1);
-    const int cmm = jm * LX + im, cpm = jm * LX + ip, cmp = jp * LX + im, cpp = jp * LX + ip;
-    T v[3][4];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      v[c][0] = Bc[c * NC + cmm];
-      v[c][1] = Bc[c * NC + cpm];
-      v[c][2] = Bc[c * NC + cmp];
-      v[c][3] = Bc[c * NC + cpp];
-    }
-    Bb[0] = (T)0.25 * ((v[0][0] + v[0][1]) + (v[0][2] + v[0][3]));
-    Bb[1] = (T)0.25 * ((v[1][0] + v[1][1]) + (v[1][2] + v[1][3]));
-    Bb[2] = (T)0.25 * ((v[2][0] + v[2][1]) + (v[2][2] + v[2][3]));
-    const T dxby = ((v[1][3] + v[1][1]) - (v[1][2] + v[1][0])) * hdx;
-    const T dxbz = ((v[2][3] + v[2][1]) - (v[2][2] + v[2][0])) * hdx;
-    const T dybx = ((v[0][3] + v[0][2]) - (v[0][1] + v[0][0])) * hdy;
-    const T dybz = ((v[2][3] + v[2][2]) - (v[2][1] + v[2][0])) * hdy;
-    ohm_e<T>(dybz, -dxbz, dxby - dybx, Bb[0], Bb[1], Bb[2], inv_n[r], pgx[r], pgy[r], u[r][0],
-             u[r][1], u[r][2], jcr, eta, resist, E[0], E[1], E[2]);
-  };
-  for (int stage = 1; stage <= 4; ++stage) {
-    const T* Bc = (stage == 1) ? sB : sBs;
-    {
-      TileWalk w(t0, NX, LY + 1);
-#pragma unroll
-      for (int r = 0; r < kFNPT; ++r, w.next()) {
-        if (w.k < NN) {
-          T E[3], Bb[3];
-          ohm(Bc, w.a, w.b, r, E, Bb);
-          sE[w.k] = E[0];
-          sE[NN + w.k] = E[1];
-          sE[2 * NN + w.k] = E[2];
-        }
-      }
-    }
-    __syncthreads();
-    for (TileWalk w(t0, LX, LY); w.k < NC; w.next()) {
-      const int k = w.k;
-      const int q00 = w.b * NX + w.a, q10 = q00 + 1, q01 = q00 + NX, q11 = q01 + 1;
-      const T dxey = ((sE[NN + q10] + sE[NN + q11]) - (sE[NN + q00] + sE[NN + q01])) * hdx;
-      const T dxez =
-          ((sE[2 * NN + q10] + sE[2 * NN + q11]) - (sE[2 * NN + q00] + sE[2 * NN + q01])) * hdx;
-      const T dyex = ((sE[q01] + sE[q11]) - (sE[q00] + sE[q10])) * hdy;
-      const T dyez =
-          ((sE[2 * NN + q01] + sE[2 * NN + q11]) - (sE[2 * NN + q00] + sE[2 * NN + q10])) * hdy;
-      const T K[3] = {-dyez, dxez, dyex - dxey};
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        rk4_stage<T>(stage, K[c], sK[c * NC + k], sBs[c * NC + k], sB[c * NC + k], h, hh, h6);
-    }
-    __syncthreads();
-  }
-  // owned cells: the new B
-  const int oa0 = cx0 - lx0, ob0 = H;
-  const int ow = cx1 - cx0, oh = cy1 - cy0;
-  for (TileWalk w(t0, ow, 3 * oh); w.k < 3 * ow * oh; w.next()) {
-    const int c = w.b / oh, y = w.b - c * oh;
-    Bout[(size_t)c * nc + (size_t)(cy0 + y) * nx + cx0 + w.a] =
-        sB[c * NC + (ob0 + y) * LX + oa0 + w.a];
-  }
-  if (!fin) return;
-  // owned nodes (and the wall nodes nx in the last tile): E, Bbar, G; each
-  // thread takes the owned nodes among its own (their density terms and u
-  // are in its registers)
-  const int ox1 = cx1 + (cx1 == nx ? 1 : 0);
-  TileWalk w(t0, NX, LY + 1);
-#pragma unroll
-  for (int r = 0; r < kFNPT; ++r, w.next()) {
-    if (w.k >= NN) continue;
-    const int i = lx0 + w.a, y = w.b - ob0;
-    if (i < cx0 || i >= ox1 || y < 0 || y >= oh) continue;
-    const int j = cy0 + y;
-    T E[3], Bb[3];
-    ohm(sB, w.a, w.b, r, E, Bb);
-    const size_t q = (size_t)j * nxn + i;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      Eo[(size_t)c * nn + q] = E[c];
-      Bbo[(size_t)c * nn + q] = Bb[c];
-    }
-    const T v[8] = {E[0], E[1], E[2], Bb[0], Bb[1], Bb[2], (T)0, (T)0};
-    T* dst = G + ((size_t)j * (nx + 1) + i) * 8;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) dst[c] = v[c];
-    if (j == 0) {
-      T* gh = G + ((size_t)ny * (nx + 1) + i) * 8;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) gh[c] = v[c];
-    }
-  }
 }
 
 // ------------------------------------------------------------------------

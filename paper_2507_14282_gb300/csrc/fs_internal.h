@@ -241,10 +241,6 @@ struct Sim {
   // the step's start, the draws done, the push done, the movers done)
   cudaStream_t side;
   cudaEvent_t ev_fork, ev_draw, ev_push, ev_join;
-  // a third stream: the FP32 2D field substep's wall tile columns beside its
-  // interior launch
-  cudaStream_t side2;
-  cudaEvent_t ev_fork2, ev_join2;
   bool graphs_ready;
   int steps_direct;    // steps launched directly (graphs are captured after one)
   template <typename T>

@@ -149,104 +149,20 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  // pre: the per-step density terms (k_ohm_pre), or nullptr to form them here
+  // Ohm's law at every node, one thread per node (pre: the per-step density
+  // terms of k_ohm_pre, or nullptr to form them here)
+  template <int DIM>
   static void ohm(Sim* s, const T* Bc, T* Eo, T* Bbo, T* G, const T* pre = nullptr) {
     DevPtrs<T> d = P(s);
     const long long nn = (long long)s->g.nxn * s->g.ny;
-    if (s->g.dim == 1)
-      k_ohm<T, 1><<<grid_for(nn), kBlock, 0, s->stream>>>(Bc, d.n, d.u, pre, Eo, Bbo, G, s->g,
+    k_ohm<T, DIM><<<grid_for(nn), kBlock, 0, s->stream>>>(Bc, d.n, d.u, pre, Eo, Bbo, G, s->g,
                                                           s->ph);
-    else
-      k_ohm<T, 2><<<grid_for(nn), kBlock, 0, s->stream>>>(Bc, d.n, d.u, pre, Eo, Bbo, G, s->g,
-                                                          s->ph);
-  }
-
-  static void faraday(Sim* s, int stage) {
-    DevPtrs<T> d = P(s);
-    const long long nc = (long long)s->g.nx * s->g.ny;
-    if (s->g.dim == 1)
-      k_faraday<T, 1><<<grid_for(nc), kBlock, 0, s->stream>>>(d.Es, d.B, d.Bs, d.Bsum, stage, s->g, s->ph);
-    else
-      k_faraday<T, 2><<<grid_for(nc), kBlock, 0, s->stream>>>(d.Es, d.B, d.Bs, d.Bsum, stage, s->g, s->ph);
   }
 
   static cudaError_t ohm_final(Sim* s) {
     DevPtrs<T> d = P(s);
-    ohm(s, d.B, d.E, d.Bb, d.G);
-    return cudaGetLastError();
-  }
-
-  // FP32 2D boxes with x walls: each RK4 substep in one tiled launch
-  // (k_field_substep2); B alternates with the stage buffer Bs, which that
-  // path does not otherwise use.
-  static cudaError_t fields_tiled(Sim* s) {
-    static_assert(sizeof(T) == 4, "the tiled field advance is the FP32 path");
-    DevPtrs<T> d = P(s);
-    constexpr size_t smem = field_tile_smem<T>();
-    static std::atomic<bool> attr(false);  // set once per process; setting it twice is harmless
-    if (!attr.load()) {
-      for (auto k : {k_field_substep2<T, -2>, k_field_substep2<T, -1>, k_field_substep2<T, 0>,
-                     k_field_substep2<T, 1>}) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-      }
-      attr.store(true);
-    }
-    const int gx = (s->g.nx + kFTX - 1) / kFTX, gy = (s->g.ny + kFTY - 1) / kFTY;
-    // interior tile columns (full, halo inside the box): 1 .. gx - 2 when the
-    // box is a whole number of tiles and rows; the rest take the general form
-    const bool split = gx >= 3 && s->g.nx % kFTX == 0 && s->g.ny % kFTY == 0 &&
-                       kFTX >= kFH;
-    T* src = d.B;
-    T* dst = d.Bs;
-    const FieldConst<T> fc = field_const<T>(s->ph);
-    for (int sub = 0; sub < s->p.n_sub; ++sub) {
-      const int fin = (sub + 1 == s->p.n_sub) ? 1 : 0;
-      if (split) {
-        const dim3 gi(gx - 2, gy), ge(2, gy);
-        // the two wall columns (few CTAs) on the third stream beside the
-        // interior launch, joined before the next substep
-        const bool side = s->side2 && s->ev_fork2 && s->ev_join2;
-        cudaStream_t es = s->stream;
-        if (side) {
-          cudaError_t e0 = cudaEventRecord(s->ev_fork2, s->stream);
-          if (e0 == cudaSuccess) e0 = cudaStreamWaitEvent(s->side2, s->ev_fork2, 0);
-          if (e0 != cudaSuccess) return e0;
-          es = s->side2;
-        }
-        k_field_substep2<T, -1><<<ge, kBlock, smem, es>>>(src, dst, d.n, d.u, d.E, d.Bb, d.G,
-                                                          s->g, s->ph, fc, fin, 0, gx - 1);
-        if (side) {
-          const cudaError_t e0 = cudaEventRecord(s->ev_join2, s->side2);
-          if (e0 != cudaSuccess) return e0;
-        }
-        // the substeps before the last need a halo of kFH - 1 cells only: their
-        // smaller shared memory lets four CTAs share an SM
-        constexpr size_t smem0 =
-            sizeof(T) * (9 * (size_t)(kFTX + 2 * (kFH - 1)) * (kFTY + 2 * (kFH - 1)) +
-                         3 * (size_t)(kFTX + 2 * (kFH - 1) + 1) * (kFTY + 2 * (kFH - 1) + 1));
-        if (fin)
-          k_field_substep2<T, 1><<<gi, kBlock, smem, s->stream>>>(src, dst, d.n, d.u, d.E, d.Bb,
-                                                                d.G, s->g, s->ph, fc, fin, 1, 0);
-        else
-          k_field_substep2<T, 0><<<gi, kBlock, smem0, s->stream>>>(src, dst, d.n, d.u, d.E, d.Bb,
-                                                                 d.G, s->g, s->ph, fc, fin, 1, 0);
-        if (side) {
-          const cudaError_t e0 = cudaStreamWaitEvent(s->stream, s->ev_join2, 0);
-          if (e0 != cudaSuccess) return e0;
-        }
-      } else {
-        const dim3 grid(gx, gy);
-        // every column: the general form
-        k_field_substep2<T, -2><<<grid, kBlock, smem, s->stream>>>(src, dst, d.n, d.u, d.E, d.Bb,
-                                                                 d.G, s->g, s->ph, fc, fin, 0, 0);
-      }
-      std::swap(src, dst);
-    }
-    if (src != d.B)  // odd n_sub: the field ended in the stage buffer
-      return cudaMemcpyAsync(d.B, src, 3 * sizeof(T) * (size_t)s->g.nx * s->g.ny,
-                             cudaMemcpyDeviceToDevice, s->stream);
+    if (s->g.dim == 1) ohm<1>(s, d.B, d.E, d.Bb, d.G);
+    else ohm<2>(s, d.B, d.E, d.Bb, d.G);
     return cudaGetLastError();
   }
 
@@ -279,33 +195,104 @@ struct OpsImpl {
     return field1_tile(s->g.nx) == kF1Small ? field_step1<kF1Small>(s) : field_step1<kF1>(s);
   }
 
+  // Rows of a warp's march over ny rows in `strips` strips, each march
+  // re-forming `extra` rows: the least work on the fullest SM, among the lengths
+  // that give an SM at least `lo` warps (where there are that many rows) and
+  // at most the `hi` it holds at once.
+  static int march_rows(int strips, int ny, int extra, int lo, int hi) {
+    int rows = 1;
+    long long best = -1;
+    for (int r = 1; r <= 128 && r <= ny; ++r) {
+      const long long per_sm = ((long long)strips * ((ny + r - 1) / r) + 151) / 152;
+      if (best >= 0 && per_sm < lo) break;
+      const long long cost = per_sm * (r + extra);
+      if (best >= 0 && cost >= best && per_sm <= hi) continue;
+      best = per_sm > hi ? -1 : cost;
+      rows = r;
+    }
+    return rows;
+  }
+
+  // FP32 2D: one launch per substep (k_field_substep), B alternating with the
+  // stage buffer Bs.
+  static cudaError_t fields_substeps(Sim* s) {
+    DevPtrs<T> d = P(s);
+    const Geo& g = s->g;
+    const FieldConst<T> fc = field_const<T>(s->ph);
+    T *b = d.B, *bn = d.Bs;
+    for (int sub = 0; sub < s->p.n_sub; ++sub) {
+      const bool fin = sub + 1 == s->p.n_sub;
+      const int strips = fin ? (g.nxn + 21) / 22 : (g.nxn + 22) / 23;
+      const int rows = march_rows(strips, g.ny, fin ? 10 : 9, 8, 16);
+      const int grid = strips * ((g.ny + rows - 1) / rows);
+      if (fin)
+        k_field_substep<T, true><<<grid, 32, 0, s->stream>>>(b, bn, d.n, d.u, d.E, d.Bb, d.G, g, fc,
+                                                             rows, strips);
+      else
+        k_field_substep<T, false><<<grid, 32, 0, s->stream>>>(b, bn, d.n, d.u, d.E, d.Bb, d.G, g,
+                                                              fc, rows, strips);
+      std::swap(b, bn);
+    }
+    if (b != d.B)  // odd n_sub: the field ended in the stage buffer
+      return cudaMemcpyAsync(d.B, b, 3 * sizeof(T) * (size_t)g.nx * g.ny,
+                             cudaMemcpyDeviceToDevice, s->stream);
+    return cudaGetLastError();
+  }
+
+  // FP64 2D: Ohm's E of B, then a marching pass per RK4 stage (k_field_march); E
+  // alternates with Es, B with Bs from one substep to the next.
+  static cudaError_t fields_march(Sim* s) {
+    DevPtrs<T> d = P(s);
+    const Geo& g = s->g;
+    const FieldConst<T> fc = field_const<T>(s->ph);
+    k_ohm_start<T, 2><<<grid_for((long long)g.nxn * g.ny), kBlock, 0, s->stream>>>(
+        d.B, d.n, d.u, d.E, d.pre, g, s->ph);
+    const int strips = (g.nxn + kMarchCols - 1) / kMarchCols;
+    const int rows = march_rows(strips, g.ny, 2, 11, 16);
+    const int grid = strips * ((g.ny + rows - 1) / rows);
+    T *b = d.B, *bn = d.Bs;
+    auto pass = [&](auto kern, const T* ei, T* eo) {
+      kern<<<grid, 32, 0, s->stream>>>(ei, eo, b, d.Bsum, bn, d.u, d.pre, d.Bb, d.G, g,
+                                                  fc, rows, strips);
+    };
+    for (int sub = 0; sub < s->p.n_sub; ++sub) {
+      pass(k_field_march<T, 1, false>, d.E, d.Es);
+      pass(k_field_march<T, 2, false>, d.Es, d.E);
+      pass(k_field_march<T, 3, false>, d.E, d.Es);
+      if (sub + 1 == s->p.n_sub) pass(k_field_march<T, 4, true>, d.Es, d.E);
+      else pass(k_field_march<T, 4, false>, d.Es, d.E);
+      std::swap(b, bn);
+    }
+    if (b != d.B)  // odd n_sub: the field ended in the stage buffer
+      return cudaMemcpyAsync(d.B, b, 3 * sizeof(T) * (size_t)g.nx * g.ny,
+                             cudaMemcpyDeviceToDevice, s->stream);
+    return cudaGetLastError();
+  }
+
+  // The field advance of boxes that k_field_step1 does not take: 2D, and 1D
+  // periodic ones, whose passes stay one launch each.
   static cudaError_t fields(Sim* s) {
-    if constexpr (sizeof(T) == 4) {
-      if (s->g.dim == 2 && s->g.bc_x != FS_BC_PERIODIC) return fields_tiled(s);
+    if (s->g.dim == 2) {
+      if constexpr (sizeof(T) == 4) return fields_substeps(s);
+      else return fields_march(s);
     }
     DevPtrs<T> d = P(s);
-    // FP64 (bound by the FP64 pipe): 1/n and the pressure terms once per
-    // step; FP32 (bound by memory) forms them in every stage instead
+    // FP64 (bound by the FP64 pipe): 1/n and the pressure terms once per step
     const T* pre = nullptr;
     if (sizeof(T) == 8) {
-      const long long nn = (long long)s->g.nxn * s->g.ny;
-      if (s->g.dim == 1)
-        k_ohm_pre<T, 1><<<grid_for(nn), kBlock, 0, s->stream>>>(d.n, d.pre, s->g, s->ph);
-      else
-        k_ohm_pre<T, 2><<<grid_for(nn), kBlock, 0, s->stream>>>(d.n, d.pre, s->g, s->ph);
+      k_ohm_pre<T, 1><<<grid_for(s->g.nxn), kBlock, 0, s->stream>>>(d.n, d.pre, s->g, s->ph);
       pre = d.pre;
     }
-    for (int sub = 0; sub < s->p.n_sub; ++sub) {
-      ohm(s, d.B, d.Es, nullptr, nullptr, pre);
-      faraday(s, 1);
-      ohm(s, d.Bs, d.Es, nullptr, nullptr, pre);
-      faraday(s, 2);
-      ohm(s, d.Bs, d.Es, nullptr, nullptr, pre);
-      faraday(s, 3);
-      ohm(s, d.Bs, d.Es, nullptr, nullptr, pre);
-      faraday(s, 4);
-    }
-    ohm(s, d.B, d.E, d.Bb, d.G, pre);
+    auto faraday = [&](int stage) {
+      k_faraday<T, 1><<<grid_for(s->g.nx), kBlock, 0, s->stream>>>(d.Es, d.B, d.Bs, d.Bsum, stage,
+                                                                   s->g, s->ph);
+    };
+    for (int sub = 0; sub < s->p.n_sub; ++sub)
+      for (int stage = 1; stage <= 4; ++stage) {
+        ohm<1>(s, stage == 1 ? d.B : d.Bs, d.Es, nullptr, nullptr, pre);
+        faraday(stage);
+      }
+    ohm<1>(s, d.B, d.E, d.Bb, d.G, pre);
     return cudaGetLastError();
   }
 
