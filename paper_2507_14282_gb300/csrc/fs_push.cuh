@@ -113,7 +113,7 @@ struct StepArgs {
 
 // ---------------------------------------------------------------- layout
 constexpr int kMaxStages = 4;
-constexpr int kPiece = 80;  // particles of a deposit piece at most (a half-warp's)
+constexpr int kPiece = 160;  // particles of a deposit piece at most (a half-warp's)
 constexpr int kWarps = kBlock / 32;
 
 template <typename T, int DIM>
@@ -828,16 +828,11 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
   int b = 0;
   for (int ci = 0;; ++ci, b = (b + 1 == NS) ? 0 : b + 1) {
     const int4 c = desc[2 * b];
-    if (c.x >= g.ntiles) {
-      // the last chunk's deposit
-      if (dpar >= 0)
-        deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, wk, pcs, npmax, k2e, oW, oV,
-                                    oF, oid, wth, wcr, dq + ((ci - 1) & 1), warp, lane);
-      break;
-    }
+    // past the last chunk: no particles, only its deposit is due
+    const bool done = c.x >= g.ntiles;
     const int i0 = desc[2 * b + 1].x, j0 = desc[2 * b + 1].y;
     const bool inner = desc[2 * b + 1].z != 0;
-    const int t = c.x, m = c.z;
+    const int t = c.x, m = done ? 0 : c.z;
     if (c.y == 0) tpar = (tiles_seen++) & 1;
     bool ok = true;
     if (m > 0) {
@@ -920,6 +915,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
     if (dpar >= 0)
       deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, wk, pcs, npmax, k2e, oW, oV, oF,
                                   oid, wth, wcr, dq + ((ci - 1) & 1), warp, lane);
+    if (done) break;
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         atomicOr(&d.ctr->status, kStatusTimeout);
