@@ -2053,6 +2053,7 @@ __global__ void __launch_bounds__(kBlock)
       }
 #pragma unroll
       for (int r = 0; r < U; ++r) {
+        if (!__any_sync(0xffffffffu, take[r])) continue;
         const int i = cell[r] & 0xFFFF;
         const float tx = fmaf((float)(i - i0) + near_float(ox[r]), fsx, fx0);
         const float tp = (near_float(vx[r]) - pmin) * fsp;

@@ -619,9 +619,10 @@ struct OpsImpl {
     const int copies = (long long)np * kWarpsPerBlock <= kSpecShared ? kWarpsPerBlock
                        : np <= kSpecShared                           ? 1
                                                                      : 0;
-    // the FP32 bin: log2 of u.u is within about 1e-5 of the exact value
+    // the FP32 bin: half the log2 of u.u is within about 1e-5 of the exact value
+    // (|log2| <= 100: two units in the last place of the fast logarithm)
     const double per = (double)np / log2(s->p.spec_pmax / s->p.spec_pmin);
-    const double eps = 1e-5 * per * (1.0 + 0.05 * fabs(log2(s->p.spec_pmin))) + 1e-6 * np;
+    const double eps = 2e-5 * per * (1.0 + 0.05 * fabs(log2(s->p.spec_pmin))) + 1e-6 * np;
     const size_t smem = sizeof(unsigned) * (size_t)np * copies;
     k_spectrum_p<T><<<tile_warps_grid(s), kBlock, smem, s->stream>>>(
         P(s), s->g, buf, species, np, copies, (float)log2(s->p.spec_pmin), (float)per,

@@ -395,9 +395,10 @@ __global__ void __launch_bounds__(kBlock)
       }
 #pragma unroll
       for (int r = 0; r < U; ++r) {
+        if (!__any_sync(0xffffffffu, take[r])) continue;
         const float fx = near_float(vx[r]), fy = near_float(vy[r]), fz = near_float(vz[r]);
         const float p2 = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
-        const float tb = (0.5f * log2f(p2) - l2min) * per;
+        const float tb = (0.5f * __log2f(p2) - l2min) * per;
         const float fb = floorf(tb), fr = tb - fb;
         int bin = -1;
         if (p2 > 1e-30f && p2 < 1e30f && fr > eps && fr < 1.0f - eps) {

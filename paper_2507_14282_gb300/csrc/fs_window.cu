@@ -1296,6 +1296,10 @@ struct fs_window {
   // slot schedule: slots at the start of step n (n = 0..steps; also on the
   // device); a slot born in the window has its slot number as id
   std::vector<int> np_at;
+  // the recompute of a segment beside the reversal of the one after it: its
+  // stream and events (made by the first backward), indexed by tape
+  cudaStream_t side = nullptr;
+  cudaEvent_t ready = nullptr, taped[2] = {nullptr, nullptr}, reversed[2] = {nullptr, nullptr};
   bool have_forward = false;
   int qsel = 0;  // which of the two deposit sums the next step uses
   long long counts[5] = {0, 0, 0, 0, 0};  // of the last forward
@@ -1352,11 +1356,14 @@ int window_sizes(const fs_params* p, int steps, int ckpt, long long n_init, int 
   off[0] = o; o += slot_bytes(*cap, tsz);                                  // state
   off[1] = o;                                                               // checkpoints
   o += (size_t)nseg * (slot_bytes(*cap, tsz) + al(3 * tsz * nx) + mom_bytes(nxn, tsz));
-  off[2] = o; o += (size_t)K * tape_slot_bytes(*cap, tsz);                 // particle tape
-  off[3] = o; o += (size_t)K * al((size_t)*cap);                           // events
-  off[4] = o; o += (size_t)K * al(3 * tsz * nx);                           // B tape
-  off[5] = o; o += (size_t)K * mom_bytes(nxn, tsz);                        // moments tape
-  off[11] = o; o += (size_t)K * 2 * al(3 * tsz * nxn);                     // E, Bbar tape
+  // the tape of a segment; two of them, when there are two segments: one is
+  // recomputed while the other is reversed
+  const size_t KT = (size_t)K * (nseg > 1 ? 2 : 1);
+  off[2] = o; o += KT * tape_slot_bytes(*cap, tsz);                        // particles
+  off[3] = o; o += KT * al((size_t)*cap);                                  // events
+  off[4] = o; o += KT * al(3 * tsz * nx);                                  // B
+  off[5] = o; o += KT * mom_bytes(nxn, tsz);                               // moments
+  off[11] = o; o += (KT + 2) * 2 * al(3 * tsz * nxn);                      // E, Bbar
   off[6] = o; o += 2 * al(3 * tsz * nxn) + 2 * al(3 * tsz * nx) + mom_bytes(nxn, tsz);
   off[7] = o; o += 2 * al(8 * 4 * (size_t)nxn);                            // fixed-point sums
   off[8] = o; o += al(8 * 8);                                              // counters
@@ -1445,35 +1452,43 @@ void mom_ptrs(char* b, int nxn, T** n, T** u, T** r) {
   *u = (T*)(b + al(sizeof(T) * nxn));
   *r = (T*)(b + 4 * al(sizeof(T) * nxn));
 }
-uint8_t* ev_at(fs_window* w, int k) {
-  return (uint8_t*)(w->base + w->o_ev) + (size_t)k * al(w->cap);
+// entry k of tape t
+size_t tape_entry(const fs_window* w, int t, int k) {
+  return (size_t)t * std::min(w->ckpt, w->steps) + k;
+}
+uint8_t* ev_at(fs_window* w, int t, int k) {
+  return (uint8_t*)(w->base + w->o_ev) + tape_entry(w, t, k) * al(w->cap);
+}
+// E, Bbar entry e (2 per tape besides the steps' own: 0 and 1 hold the tapes' first)
+template <typename T>
+void tape_E(fs_window* w, size_t e, State<T>* a) {
+  const size_t b = al(3 * sizeof(T) * w->g.nxn);
+  a->E = (T*)(w->base + w->o_tapeE + e * 2 * b);
+  a->Bb = (T*)((char*)a->E + b);
 }
 
-// the state at the start of a segment: its checkpoint, with E, Bbar formed
-// from it into r's
+// the state at the start of segment c, for tape t: its checkpoint, with E, Bbar
+// formed from it
 template <typename T>
-State<T> ckpt_state(fs_window* w, const Win<T>& r, int c) {
+State<T> ckpt_state(fs_window* w, int c, int t) {
   const Ck ck = ckpt_at(w, c);
   State<T> a;
   a.s = slots_at<T>(ck.slots, w->cap, false);
   a.B = (T*)ck.B;
   mom_ptrs<T>(ck.mom, w->g.nxn, &a.n, &a.u, &a.nraw);
-  a.E = r.E;
-  a.Bb = r.Bb;
+  tape_E<T>(w, t, &a);
   return a;
 }
-// state k >= 1 of a recomputed segment (on the tape)
+// state k >= 1 of a recomputed segment (on tape t)
 template <typename T>
-State<T> tape_state(fs_window* w, int k) {
-  const size_t nxn = w->g.nxn, e = al(3 * sizeof(T) * nxn);
+State<T> tape_state(fs_window* w, int t, int k) {
+  const size_t e = tape_entry(w, t, k - 1);
   State<T> a;
-  a.s = slots_at<T>(w->base + w->o_tape + (size_t)(k - 1) * tape_slot_bytes(w->cap, w->tsz),
-                    w->cap, false);
-  a.B = (T*)(w->base + w->o_tapeB + (size_t)(k - 1) * al(3 * sizeof(T) * w->g.nx));
-  mom_ptrs<T>(w->base + w->o_tapeM + (size_t)(k - 1) * mom_bytes(w->g.nxn, w->tsz), w->g.nxn,
-              &a.n, &a.u, &a.nraw);
-  a.E = (T*)(w->base + w->o_tapeE + (size_t)(k - 1) * 2 * e);
-  a.Bb = (T*)((char*)a.E + e);
+  a.s = slots_at<T>(w->base + w->o_tape + e * tape_slot_bytes(w->cap, w->tsz), w->cap, false);
+  a.B = (T*)(w->base + w->o_tapeB + e * al(3 * sizeof(T) * w->g.nx));
+  mom_ptrs<T>(w->base + w->o_tapeM + e * mom_bytes(w->g.nxn, w->tsz), w->g.nxn, &a.n, &a.u,
+              &a.nraw);
+  tape_E<T>(w, 2 + e, &a);
   return a;
 }
 
@@ -1485,13 +1500,13 @@ void cpy(void* d, const void* s, size_t n, cudaStream_t st) {
 // ions born in it; ev: where the step's events go (or nullptr)
 template <typename T>
 void forward_step(fs_window* w, const Win<T>& r, int n, const State<T>& a, const State<T>& b,
-                  const Slots<T>& drawn, uint8_t* ev) {
+                  const Slots<T>& drawn, uint8_t* ev, cudaStream_t st) {
   const int np = w->np_at[n], np1 = w->np_at[n + 1];
   unsigned long long *q = r.q[w->qsel], *qz = r.q[1 - w->qsel];
   if (np1 > 0)
-    k_win_push_deposit<T><<<blocks(np1), kBlock, 0, w->st>>>(r, a, b.s, drawn, ev, q, w->g, w->ph,
+    k_win_push_deposit<T><<<blocks(np1), kBlock, 0, st>>>(r, a, b.s, drawn, ev, q, w->g, w->ph,
                                                              push_const<T>(w->ph), n, np, np1);
-  k_win_fields<T><<<tiles(w->g.nx), fields_threads(w->p.n_sub), fields_smem(w->p.n_sub, sizeof(T)), w->st>>>(
+  k_win_fields<T><<<tiles(w->g.nx), fields_threads(w->p.n_sub), fields_smem(w->p.n_sub, sizeof(T)), st>>>(
       a.B, b, q, qz, w->g, w->ph, field_const<T>(w->ph), w->p.n_sub);
   w->qsel ^= 1;
 }
@@ -1509,8 +1524,8 @@ void save_ckpt(fs_window* w, const State<T>& a, int c) {
 }
 
 template <typename T>
-void ohm_of(fs_window* w, const State<T>& a) {
-  k_ohm<T, 1><<<blocks(w->g.nxn), kBlock, 0, w->st>>>(a.B, a.n, a.u, nullptr, a.E, a.Bb, nullptr,
+void ohm_of(fs_window* w, const State<T>& a, cudaStream_t st) {
+  k_ohm<T, 1><<<blocks(w->g.nxn), kBlock, 0, st>>>(a.B, a.n, a.u, nullptr, a.E, a.Bb, nullptr,
                                                        w->g, w->ph);
 }
 
@@ -1546,13 +1561,13 @@ int do_forward(fs_window* w, const double* theta, double* loss) {
     k_win_push_deposit<T><<<blocks(np0), kBlock, 0, w->st>>>(
         r, a, r.s, r.s, nullptr, r.q[1], w->g, w->ph, push_const<T>(w->ph), 0, 0, np0);
   k_win_moments<T><<<blocks(w->g.nxn), kBlock, 0, w->st>>>(r, r.q[1], w->g, w->ph);
-  ohm_of<T>(w, a);
+  ohm_of<T>(w, a, w->st);
   w->qsel = 0;  // (the first step clears the other sums)
   for (int n = 0; n < w->steps; ++n) {
     if (n % w->ckpt == 0) save_ckpt<T>(w, a, n / w->ckpt);
     State<T> b = a;
     b.B = a.B == r.B[0] ? r.B[1] : r.B[0];
-    forward_step<T>(w, r, n, a, b, r.s, nullptr);
+    forward_step<T>(w, r, n, a, b, r.s, nullptr, w->st);
     a = b;
   }
   double* dl = r.lBx;  // scratch for the loss (free outside the backward)
@@ -1569,9 +1584,21 @@ int do_forward(fs_window* w, const double* theta, double* loss) {
   return FS_OK;
 }
 
+// the side stream and its events; false if one cannot be made
+bool make_side(fs_window* w) {
+  if (!w->side && cudaStreamCreateWithFlags(&w->side, cudaStreamNonBlocking) != cudaSuccess)
+    return false;
+  for (cudaEvent_t* e : {&w->ready, &w->taped[0], &w->taped[1], &w->reversed[0], &w->reversed[1]})
+    if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return false;
+  return true;
+}
+
 template <typename T>
 int do_backward(fs_window* w, double dloss, double* grad) {
   if (!w->have_forward) return FS_EINVAL;
+  if (!make_side(w)) return FS_ECUDA;
+  // the recompute overwrites the forward's sums: a new forward is due
+  w->have_forward = false;
   Win<T> r = win_ptrs<T>(w);
   const int nx = w->g.nx, nxn = w->g.nxn, M = w->M;
   const size_t fb = 8 * 3 * (size_t)(nx + nxn);
@@ -1584,15 +1611,34 @@ int do_backward(fs_window* w, double dloss, double* grad) {
   // d loss / d B at the end (the final field after the forward)
   k_win_loss<T><<<1, kBlock, 0, w->st>>>(r.B[w->steps & 1], w->g, w->ph, w->loss_i0, w->p.dx,
                                                   nullptr, r.lB, dloss);
-  for (int seg = w->nseg - 1; seg >= 0; --seg) {
-    const int n0 = seg * w->ckpt;
-    const int n1 = std::min(w->steps, n0 + w->ckpt);
-    // recompute the segment, keeping every state
-    const State<T> first = ckpt_state<T>(w, r, seg);
-    auto at = [&](int k) { return k == 0 ? first : tape_state<T>(w, k); };
-    ohm_of<T>(w, first);
+  // Segment by segment from the end: recompute it, keeping every state, then
+  // reverse it. The recompute of segment seg - 1 (its own tape; it needs only
+  // its checkpoint) runs on the side stream while segment seg is reversed:
+  // both are chains of short kernels that leave most of the GPU idle.
+  auto wait = [](cudaStream_t st, cudaEvent_t e) {
+    return cudaStreamWaitEvent(st, e, 0) == cudaSuccess;
+  };
+  auto recompute = [&](int seg) {
+    const int t = seg & 1, n0 = seg * w->ckpt, n1 = std::min(w->steps, n0 + w->ckpt);
+    const State<T> first = ckpt_state<T>(w, seg, t);
+    auto at = [&](int k) { return k == 0 ? first : tape_state<T>(w, t, k); };
+    ohm_of<T>(w, first, w->side);
     for (int n = n0; n < n1; ++n)
-      forward_step<T>(w, r, n, at(n - n0), at(n - n0 + 1), first.s, ev_at(w, n - n0));
+      forward_step<T>(w, r, n, at(n - n0), at(n - n0 + 1), first.s, ev_at(w, t, n - n0), w->side);
+    return cudaEventRecord(w->taped[t], w->side) == cudaSuccess;
+  };
+  if (cudaEventRecord(w->ready, w->st) != cudaSuccess || !wait(w->side, w->ready) ||
+      !recompute(w->nseg - 1))
+    return FS_ECUDA;
+  for (int seg = w->nseg - 1; seg >= 0; --seg) {
+    const int t = seg & 1, n0 = seg * w->ckpt, n1 = std::min(w->steps, n0 + w->ckpt);
+    if (seg > 0) {  // (the other tape: free once segment seg + 1 is reversed)
+      if (seg + 1 < w->nseg && !wait(w->side, w->reversed[1 - t])) return FS_ECUDA;
+      if (!recompute(seg - 1)) return FS_ECUDA;
+    }
+    if (!wait(w->st, w->taped[t])) return FS_ECUDA;
+    const State<T> first = ckpt_state<T>(w, seg, t);
+    auto at = [&](int k) { return k == 0 ? first : tape_state<T>(w, t, k); };
     for (int n = n1 - 1; n >= n0; --n) {
       const int k = n - n0;
       const State<T> a = at(k), b = at(k + 1);
@@ -1606,9 +1652,10 @@ int do_backward(fs_window* w, double dloss, double* grad) {
       const int npa = w->np_at[n], npb = w->np_at[n + 1];
       if (npb > 0)
         k_win_particle_adj<T><<<blocks(npb), kBlock, 0, w->st>>>(
-            r, a, b.s, ev_at(w, k), r.lE[esel], r.lBb[esel], w->g, w->ph, push_const<T>(w->ph), n,
+            r, a, b.s, ev_at(w, t, k), r.lE[esel], r.lBb[esel], w->g, w->ph, push_const<T>(w->ph), n,
             npa, npb, M);
     }
+    if (cudaEventRecord(w->reversed[t], w->st) != cudaSuccess) return FS_ECUDA;
     if (seg == 0)
       k_win_ohm_adj_start<T><<<tiles(nx), 32, 0, w->st>>>(first, w->g, w->ph, r.lE[esel],
                                                                   r.lBb[esel], r.lB);
@@ -1618,8 +1665,6 @@ int do_backward(fs_window* w, double dloss, double* grad) {
   if (cudaMemcpyAsync(grad, r.grad, 8 * (M + 2), cudaMemcpyDeviceToHost, w->st) != cudaSuccess ||
       cudaStreamSynchronize(w->st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
     return FS_ECUDA;
-  // the recompute overwrote the forward's sums: a new forward is due
-  w->have_forward = false;
   return FS_OK;
 }
 
@@ -1754,6 +1799,13 @@ int fs_window_counts(fs_window* w, long long* out5) {
 
 int fs_window_destroy(fs_window* w) {
   FS_GUARD_BEGIN
+  if (!w) return FS_OK;
+  if (w->side) {
+    cudaStreamSynchronize(w->side);
+    cudaStreamDestroy(w->side);
+  }
+  for (cudaEvent_t e : {w->ready, w->taped[0], w->taped[1], w->reversed[0], w->reversed[1]})
+    if (e) cudaEventDestroy(e);
   delete w;
   return FS_OK;
   FS_GUARD_END
