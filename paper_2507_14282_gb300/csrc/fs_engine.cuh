@@ -702,29 +702,29 @@ __global__ void k_moments(DevPtrs<T> d, Geo g, Phys ph) {
   moments_body<T, DIM>(d, g, ph, blockIdx.x, gridDim.x);
 }
 
-// The same sums for a 2D box with x walls whose tile shape TXC x TYC is
-// compiled in (and whose rows hold more than one tile's accumulator rows and
-// more tile rows than cover a node): the candidate tiles of a node are a
-// fixed, small set (MX columns by MY rows), so every load is issued without a
-// data-dependent loop; rows are taken in increasing wrapped order, columns
-// in increasing order, as in moments_body.
-template <typename T, int TXC, int TYC>
+// The same sums for a 2D box with x walls (whose rows hold more than one tile's
+// accumulator rows and more tile rows than cover a node): the candidate tiles
+// of a node are a fixed, small set (MX columns by MY rows), so every load is
+// issued without a data-dependent loop; rows are taken in increasing wrapped
+// order, columns in increasing order, as in moments_body. The tile shape is
+// compiled in (TXC x TYC) or the run's (0).
+template <typename T, int TXC, int TYC, int MX, int MY>
 __global__ void k_moments_ct(DevPtrs<T> d, Geo g, Phys ph) {
   using A = typename Num<T>::acc;
-  constexpr int AX = TXC + 3, AY = TYC + 3, NA = AX * AY;
-  constexpr int MX = (AX + TXC - 1) / TXC, MY = (AY + TYC - 1) / TYC;
+  const int TX = TXC ? TXC : g.TX, TY = TYC ? TYC : g.TY;
+  const int AX = TX + 3, AY = TY + 3, NA = AX * AY;
   const int nn = g.nxn * g.ny;
   const A* far = (const A*)d.far;
   const A* partial = (const A*)d.partial;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nn; q += gridDim.x * blockDim.x) {
     const int i = q % g.nxn, j = q / g.nxn;
-    // candidate rows: ty with 0 <= j - (ty TYC - 1) < AY, wrapped, ascending
+    // candidate rows: ty with 0 <= j - (ty TY - 1) < AY, wrapped, ascending
     int tyw[MY], ayv[MY];
-    const int tyh = (j + 1) / TYC;
+    const int tyh = (j + 1) / TY;
 #pragma unroll
     for (int u = 0; u < MY; ++u) {
       const int ty = tyh - (MY - 1) + u;
-      const int ay = j - (ty * TYC - 1);
+      const int ay = j - (ty * TY - 1);
       const bool ok = ay >= 0 && ay < AY;
       tyw[u] = ok ? (ty < 0 ? ty + g.nty : (ty >= g.nty ? ty - g.nty : ty)) : 0x7fffffff;
       ayv[u] = ay;
@@ -741,14 +741,14 @@ __global__ void k_moments_ct(DevPtrs<T> d, Geo g, Phys ph) {
     A s[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) s[c] = far[(size_t)c * nn + q];
-    const int txh = (i + 1) / TXC;
+    const int txh = (i + 1) / TX;
 #pragma unroll
     for (int u = 0; u < MY; ++u) {
       if (tyw[u] == 0x7fffffff) continue;
 #pragma unroll
       for (int x = 0; x < MX; ++x) {
         const int tx = txh - (MX - 1) + x;
-        const int ax = i - (tx * TXC - 1);
+        const int ax = i - (tx * TX - 1);
         if (tx < 0 || tx >= g.ntx || ax < 0 || ax >= AX) continue;
         const A* part = partial + (size_t)(tyw[u] * g.ntx + tx) * 4 * NA + ax + ayv[u] * AX;
 #pragma unroll

@@ -134,18 +134,25 @@ struct OpsImpl {
   static cudaError_t moments(Sim* s) {
     const long long nn = (long long)s->g.nxn * s->g.ny;
     const Geo& g = s->g;
-    // the tile shapes the library picks for the 2D workloads (FP32 4 x 2 at
-    // 64 ppc, FP64 8 x 4 at 16 ppc), compiled in, for boxes with x walls that
-    // are more than a tile's accumulator high and more than three tile rows
+    // boxes with x walls that are more than a tile's accumulator high and more
+    // than three tile rows: a fixed set of candidate tiles per node; the shapes
+    // the library picks for the benchmark's 2D workloads (FP32 4 x 2 at 64 ppc,
+    // FP64 8 x 4 at 16 ppc) compiled in
     const bool ct = g.dim == 2 && g.bc_x != FS_BC_PERIODIC && g.ny >= 2 * (g.TY + 3) && g.nty > 3;
-    if (g.dim == 1)
-      k_moments<T, 1><<<grid_for(nn), kBlock, 0, s->stream>>>(P(s), g, s->ph);
-    else if (ct && g.TX == 4 && g.TY == 2)
-      k_moments_ct<T, 4, 2><<<grid_for(nn), kBlock, 0, s->stream>>>(P(s), g, s->ph);
-    else if (ct && g.TX == 8 && g.TY == 4)
-      k_moments_ct<T, 8, 4><<<grid_for(nn), kBlock, 0, s->stream>>>(P(s), g, s->ph);
-    else
-      k_moments<T, 2><<<grid_for(nn), kBlock, 0, s->stream>>>(P(s), g, s->ph);
+    auto run = [&](auto kern) {
+      kern<<<grid_for(nn), kBlock, 0, s->stream>>>(P(s), g, s->ph);
+    };
+    if (g.dim == 1) run(k_moments<T, 1>);
+    else if (!ct) run(k_moments<T, 2>);
+    else if (g.TX == 4 && g.TY == 2) run(k_moments_ct<T, 4, 2, 2, 3>);
+    else if (g.TX == 8 && g.TY == 4) run(k_moments_ct<T, 8, 4, 2, 2>);
+    // tiles that can cover a node: (TX + 3) / TX columns rounded up, rows alike
+    else if (g.TX == 2 && g.TY == 1) run(k_moments_ct<T, 0, 0, 3, 4>);
+    else if (g.TX == 2 && g.TY == 2) run(k_moments_ct<T, 0, 0, 3, 3>);
+    else if (g.TX == 2) run(k_moments_ct<T, 0, 0, 3, 2>);
+    else if (g.TY == 1) run(k_moments_ct<T, 0, 0, 2, 4>);
+    else if (g.TY == 2) run(k_moments_ct<T, 0, 0, 2, 3>);
+    else run(k_moments_ct<T, 0, 0, 2, 2>);
     return cudaGetLastError();
   }
 

@@ -1062,15 +1062,22 @@ __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const S
     // ---- recompute the push from the state before the step
     const A f0 = (A)ft0;
     const A v0[3] = {vxt, vyt, vzt};
-    // (E at the particle as E0 + f (E1 - E0): the adjoint needs the difference too)
+    // (FP32: E at the particle rounded as in the forward, so that the gradient is
+    // that of the trajectory it took; FP64: E0 + f (E1 - E0), the difference is
+    // needed anyway)
     A Ep[3], Bp[3], Ed[3], Bd[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const A e0 = a0.E[c * nxn + c0], b0 = a0.Bb[c * nxn + c0];
       Ed[c] = a0.E[c * nxn + c0 + 1] - e0;
       Bd[c] = a0.Bb[c * nxn + c0 + 1] - b0;
-      Ep[c] = fmaT(f0, Ed[c], e0);
-      Bp[c] = fmaT(f0, Bd[c], b0);
+      if constexpr (sizeof(T) == 4) {
+        Ep[c] = fmaT(f0, a0.E[c * nxn + c0 + 1], ((A)1 - f0) * e0);
+        Bp[c] = fmaT(f0, a0.Bb[c * nxn + c0 + 1], ((A)1 - f0) * b0);
+      } else {
+        Ep[c] = fmaT(f0, Ed[c], e0);
+        Bp[c] = fmaT(f0, Bd[c], b0);
+      }
     }
     // ---- Boris: v+ = q + em, q = vm + p x s, p = vm + vm x t,
     //      s = (2 / (1 + t.t)) t, t = hdt B, vm = v + em, em = hdt E
@@ -1084,9 +1091,9 @@ __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const S
     }
     const A fct = (A)2 * rcpT((A)1 + fmaT(t[2], t[2], fmaT(t[1], t[1], t[0] * t[0])));
     for (int c = 0; c < 3; ++c) sv[c] = fct * t[c];
-    pp[0] = fmaT(vm[1], t[2], fmaT(-vm[2], t[1], vm[0]));
-    pp[1] = fmaT(vm[2], t[0], fmaT(-vm[0], t[2], vm[1]));
-    pp[2] = fmaT(vm[0], t[1], fmaT(-vm[1], t[0], vm[2]));
+    pp[0] = vm[0] + fmaT(vm[1], t[2], -(vm[2] * t[1]));
+    pp[1] = vm[1] + fmaT(vm[2], t[0], -(vm[0] * t[2]));
+    pp[2] = vm[2] + fmaT(vm[0], t[1], -(vm[1] * t[0]));
     A lvp[3];  // adjoint of vp
     A lf0;
     if (e == kEvReturned) {
@@ -1165,11 +1172,13 @@ __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const S
     // ---- gather adjoint at the state before the step: the adjoints of E and
     //      Bbar at the particle and its offset go to the caller, which
     //      shares them out to the nodes c0, c0 + 1
+    A dlf = (A)0;  // summed on its own: one rounding at the size of lf0 a step
     for (int c = 0; c < 3; ++c) {
       out[c] = LE[c];
       out[3 + c] = LB[c];
-      lf0 = fmaT(LE[c], Ed[c], fmaT(LB[c], Bd[c], lf0));
+      dlf = fmaT(LE[c], Ed[c], fmaT(LB[c], Bd[c], dlf));
     }
+    lf0 += dlf;
     out[6] = f0;
     w.lf[p] = (T)lf0;
     w.lv[p] = (T)Lvm[0];

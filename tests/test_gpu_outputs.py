@@ -131,3 +131,19 @@ def test_particles_round_trip_in_chunks(fs, dim, nx, ny, prec):
     sim.load_fields(B)
     np.testing.assert_array_equal(sim.grid(fs.FS_B), B)
     sim.close()
+
+
+@pytest.mark.parametrize("tx,ty", [(2, 1), (2, 2), (2, 5), (3, 1), (5, 2), (3, 3), (5, 5), (10, 3)])
+def test_moments_of_any_tile_shape_equal_the_oracle(fs, tx, ty):
+    """The node sums with each count of candidate tiles, next to the walls and
+    across the periodic rows: FP64 bit for bit, after two steps."""
+    kw = dict(dim=2, nx=30, ny=30, ppc=5, dt=0.005, mach_a=12.0, theta_bn_deg=20.0, cr_enable=1,
+              p_iso=40.0, seed=7)
+    gpu = fs.FauxShock(tile_x=tx, tile_y=ty, **kw)
+    ref = O.Oracle(**kw)
+    gpu.step(2)
+    ref.step(2)
+    for what, name in ((fs.FS_N, O.GRID_N), (fs.FS_J, O.GRID_J), (fs.FS_B, O.GRID_B)):
+        np.testing.assert_array_equal(gpu.grid(what), ref.grid(name))
+    gpu.close()
+    ref.close()
