@@ -290,7 +290,7 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   // FP64 only: per-step Ohm's-law terms that depend on n alone
   L->pre = take(p->precision == FS_FP64 ? 3 * T * nn : 0);
   L->partial = take(A * 4 * (size_t)g->na * g->ntiles);
-  L->far = take(A * 4 * nn);
+  L->far = take(A * 4 * nn * (p->dim == 1 ? 2 : 1));  // (1D: two steps', Sim::swaps_fields)
   L->acc = take(8 * (size_t)p->ny);
   L->inj = take(4 * (2 * (size_t)p->ny + 2));
   L->ctr = take(sizeof(Counters));
@@ -386,8 +386,8 @@ int grid_blocks(long long n) {
 // Capture one step for each ping-pong parity on a private stream (the legacy
 // default stream cannot be captured); the graphs replay on the caller's stream.
 // Kernels one step launches: push, movers, injection (1, or 2 with many rows),
-// moments, the field advance, step end. Moments and field advance are one
-// tiled launch in 1D boxes with x walls; else the field advance is one launch
+// moments, the field advance, step end. The last three are one tiled launch in
+// 1D boxes with x walls; else the field advance is one launch
 // per substep in FP32 2D boxes, Ohm and one per RK4 stage in FP64 2D boxes, and
 // in 1D [FP64: Ohm density terms], 2 x 4 x n_sub stage passes and the final Ohm
 // (the same choice as the field launcher makes).
@@ -396,7 +396,7 @@ long long launches_per_step(const Sim* s) {
   const bool walls = s->g.bc_x != FS_BC_PERIODIC;
   long long fields;
   if (s->g.dim == 1 && walls && s->p.n_sub <= 16)
-    fields = 0;  // with the moments
+    fields = -1;  // moments, fields and step end in one
   else if (s->g.dim == 2)
     fields = s->p.precision == FS_FP32 ? s->p.n_sub : 1 + 4LL * s->p.n_sub;
   else
@@ -464,8 +464,7 @@ void release_graphs(Sim* s) {
 
 int redeposit(Sim* s) {
   cudaError_t e = cudaMemsetAsync(s->base + s->L.far, 0,
-                                  (s->p.precision == FS_FP64 ? 8 : 4) * 4 *
-                                      (size_t)s->g.nxn * s->g.ny,
+                                  s->L.acc - s->L.far,
                                   s->stream);
   if (e != cudaSuccess) return FS_ECUDA;
   if ((e = s->ops->deposit_all(s, s->cur)) != cudaSuccess) return FS_ECUDA;

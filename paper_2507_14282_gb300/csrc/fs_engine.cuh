@@ -1566,8 +1566,9 @@ __device__ __forceinline__ void tile1_ohm(const T* y, int L, int m, int p, const
 // The moments and the whole field advance of a 1D step with x walls (n, J, u
 // from the deposit, n_sub RK4 substeps, then Ohm's E and Bbar for the next
 // gather) in one launch: on a 1D grid the separate passes are tens of tiny
-// launches per step (the far sums, read by neighbouring tiles too, are cleared
-// at the step's end, step1_end). A CTA owns TILE
+// launches per step (the far sums are read by neighbouring tiles too: the
+// next step's, of the step before, are cleared here). The first block also
+// ends the step. A CTA owns TILE
 // cells (and their left nodes; the last tile also node nx) and runs every
 // pass in shared memory over its cells plus field1_halo(n_sub) cells around
 // them, which it recomputes: each pass's stencil reaches one cell, so
@@ -1635,6 +1636,7 @@ __device__ __forceinline__ void field_step1_body(const DevPtrs<T>& d, const Geo&
   for (int k = t0; k < 4 * Ln; k += nt) {
     const int c = k / Ln, i = k - c * Ln;
     const T v = moment1<T>(d, g, lo + i, c);
+    if (owns_node(lo + i)) ((typename Num<T>::acc*)d.far_next)[c * nxn + lo + i] = 0;
     if (c == 0) {
       const T n = v < n_floor ? n_floor : v;
       sn[i] = n;
@@ -1689,6 +1691,7 @@ __device__ __forceinline__ void field_step1_body(const DevPtrs<T>& d, const Geo&
     d.Bs[(t.comp + 1) * nx + gi] = t.b;
     if (t.comp == 0) d.Bs[gi] = bxc;
   }
+  if (blk == 0 && t0 == 0) step_end(d.ctr, d.inj, g);
 }
 
 template <typename T, int TILE>
@@ -1696,21 +1699,6 @@ __global__ void __launch_bounds__(field1_threads(TILE, kF1MaxSub))
     k_field_step1(DevPtrs<T> d, Geo g, T n_floor, FieldConst<T> fc, int n_sub) {
   extern __shared__ __align__(16) unsigned char smem[];
   field_step1_body<T, TILE>(d, g, n_floor, fc, n_sub, blockIdx.x, smem);
-}
-
-// The end of a 1D step whose field advance was field_step1: the new B back
-// from the stage buffer, the far sums cleared for the next step, the counters.
-template <typename T>
-__device__ __forceinline__ void step1_end(const DevPtrs<T>& d, const Geo& g, int blk, int nblk) {
-  using A = typename Num<T>::acc;
-  const int id = blk * blockDim.x + threadIdx.x, n = nblk * blockDim.x;
-  for (int k = id; k < 3 * g.nx; k += n) d.B[k] = d.Bs[k];
-  for (int k = id; k < 4 * g.nxn; k += n) ((A*)d.far)[k] = (A)0;
-  if (id == 0) step_end(d.ctr, d.inj, g);
-}
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_step1_end(DevPtrs<T> d, Geo g) {
-  step1_end<T>(d, g, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------------------------

@@ -108,6 +108,7 @@ struct DevPtrs {
   T* pre;          // FP64: 1/n and the two pressure terms per node, per step
   void* partial;   // float accumulators (FP32) or int64 fixed point (FP64)
   void* far;
+  void* far_next;  // the next step's far sums (1D, see Sim::swaps_fields), cleared in this step
   double* acc;
   int* inj;        // injection row counts [ny] and offsets [ny + 1]
   Counters* ctr;
@@ -243,8 +244,15 @@ struct Sim {
   cudaEvent_t ev_fork, ev_draw, ev_push, ev_join;
   bool graphs_ready;
   int steps_direct;    // steps launched directly (graphs are captured after one)
+  // 1D boxes with x walls form moments and fields in one launch that reads B and
+  // the far sums of one step and writes those of the next: two of each, by the
+  // parity of the particle buffer, so that a step ends with that launch.
+  bool swaps_fields() const {
+    return g.dim == 1 && g.bc_x != FS_BC_PERIODIC && p.n_sub <= 16;
+  }
+  // par: the particle buffer of the step (-1: the current one)
   template <typename T>
-  DevPtrs<T> ptrs(int dummy = 0) const;
+  DevPtrs<T> ptrs(int par = -1) const;
 };
 
 template <typename T>
@@ -261,7 +269,7 @@ inline Parts<T> parts_at(char* base, const size_t off[7]) {
 }
 
 template <typename T>
-inline DevPtrs<T> Sim::ptrs(int) const {
+inline DevPtrs<T> Sim::ptrs(int par) const {
   DevPtrs<T> d;
   d.P[0] = parts_at<T>(base, L.part[0]);
   d.P[1] = parts_at<T>(base, L.part[1]);
@@ -283,7 +291,18 @@ inline DevPtrs<T> Sim::ptrs(int) const {
   d.J = (T*)(base + L.J);
   d.pre = (T*)(base + L.pre);
   d.partial = (void*)(base + L.partial);
-  d.far = (void*)(base + L.far);
+  d.far = d.far_next = (void*)(base + L.far);
+  if (swaps_fields()) {
+    char* other = base + L.far + sizeof(T) * 4 * (size_t)g.nxn;
+    if (par < 0 ? cur : par) {
+      T* t = d.B;
+      d.B = d.Bs;
+      d.Bs = t;
+      d.far = other;
+    } else {
+      d.far_next = other;
+    }
+  }
   d.acc = (double*)(base + L.acc);
   d.inj = (int*)(base + L.inj);
   d.ctr = (Counters*)(base + L.ctr);

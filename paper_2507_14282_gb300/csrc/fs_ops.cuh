@@ -66,7 +66,7 @@ cudaError_t launch_push(Sim* s, int in, long long step) {
   const long long want = (long long)n_sm * per_sm;
   const int grid = (int)std::min<long long>(want, s->g.ntiles);
   k_push<T, DIM, CH, NS, REL, TXC, TYC><<<grid, kBlock, L.bytes, s->stream>>>(
-      s->ptrs<T>(), a, push_const<T>(s->ph));
+      s->ptrs<T>(in), a, push_const<T>(s->ph));
   return cudaGetLastError();
 }
 
@@ -173,14 +173,12 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  // 1D boxes with x walls: moments and the whole field advance in one tiled
-  // launch (k_field_step1), the new B in the stage buffer until step1_end.
-  static bool one_launch_fields(const Sim* s) {
-    return s->g.dim == 1 && s->g.bc_x != FS_BC_PERIODIC && s->p.n_sub <= kF1MaxSub;
-  }
+  // 1D boxes with x walls: moments, the whole field advance and the step's end
+  // in one tiled launch (k_field_step1).
+  static_assert(kF1MaxSub == 16, "Sim::swaps_fields");
   template <int TILE>
-  static cudaError_t field_step1(Sim* s) {
-    DevPtrs<T> d = P(s);
+  static cudaError_t field_step1(Sim* s, int in) {
+    DevPtrs<T> d = s->ptrs<T>(in);
     const size_t smem = field1_smem<T>(s->p.n_sub, TILE);
     // the largest size enabled so far; a raise races harmlessly (each caller
     // sets at least its own size before it launches)
@@ -198,8 +196,9 @@ struct OpsImpl {
         d, s->g, (T)s->ph.n_floor, field_const<T>(s->ph), s->p.n_sub);
     return cudaGetLastError();
   }
-  static cudaError_t fields_tiled1(Sim* s) {
-    return field1_tile(s->g.nx) == kF1Small ? field_step1<kF1Small>(s) : field_step1<kF1>(s);
+  static cudaError_t fields_tiled1(Sim* s, int in) {
+    return field1_tile(s->g.nx) == kF1Small ? field_step1<kF1Small>(s, in)
+                                            : field_step1<kF1>(s, in);
   }
 
   // Rows of a warp's march over ny rows in `strips` strips, each march
@@ -305,8 +304,8 @@ struct OpsImpl {
 
   // The draws of the step's injected particles, on st: one block counts and
   // draws when it has few of them, else a count and a grid of draws.
-  static cudaError_t inject(Sim* s, cudaStream_t st) {
-    DevPtrs<T> d = P(s);
+  static cudaError_t inject(Sim* s, int in, cudaStream_t st) {
+    DevPtrs<T> d = s->ptrs<T>(in);
     const Geo& g = s->g;
     if (g.ninj <= kBlock) {
       const int threads = (std::max(g.ninj, g.ny) + 31) / 32 * 32;
@@ -332,7 +331,7 @@ struct OpsImpl {
   // Everything of a step after the push (movers, injection unless `drawn`,
   // moments, field advance, step counter); ev as in step().
   static cudaError_t step_rest(Sim* s, int in, cudaEvent_t* ev, bool drawn) {
-    DevPtrs<T> d = P(s);
+    DevPtrs<T> d = s->ptrs<T>(in);
     const int out = 1 - in;
     cudaError_t e = cudaSuccess;
     auto mark = [&](int k) {
@@ -351,22 +350,18 @@ struct OpsImpl {
       movers(s, out, 1, s->stream);
       mark(2);
       if (s->g.ninj) {
-        if ((e = inject(s, s->stream)) != cudaSuccess) return e;
+        if ((e = inject(s, in, s->stream)) != cudaSuccess) return e;
         movers(s, out, 2, s->stream);
       }
       mark(3);
     }
-    const bool one = one_launch_fields(s);
+    const bool one = s->swaps_fields();  // (ends the step, too)
     if (!one && (e = moments(s)) != cudaSuccess) return e;
     mark(4);
-    e = one ? fields_tiled1(s) : fields(s);
+    e = one ? fields_tiled1(s, in) : fields(s);
     if (e != cudaSuccess) return e;
     if (drawn && (e = cudaStreamWaitEvent(s->stream, s->ev_join, 0)) != cudaSuccess) return e;
-    if (one)
-      k_step1_end<T><<<std::min((4 * s->g.nxn + kBlock - 1) / kBlock, 152), kBlock, 0,
-                       s->stream>>>(d, s->g);
-    else
-      k_step_end<<<1, 32, 0, s->stream>>>(d.ctr, d.inj, s->g);
+    if (!one) k_step_end<<<1, 32, 0, s->stream>>>(d.ctr, d.inj, s->g);
     mark(5);
     return cudaGetLastError();
   }
@@ -379,7 +374,7 @@ struct OpsImpl {
     if (drawn) {
       if ((e = cudaEventRecord(s->ev_fork, s->stream)) != cudaSuccess) return e;
       if ((e = cudaStreamWaitEvent(s->side, s->ev_fork, 0)) != cudaSuccess) return e;
-      if (s->g.ninj && (e = inject(s, s->side)) != cudaSuccess) return e;
+      if (s->g.ninj && (e = inject(s, in, s->side)) != cudaSuccess) return e;
       if ((e = cudaEventRecord(s->ev_draw, s->side)) != cudaSuccess) return e;
     }
     if (ev) cudaEventRecord(ev[0], s->stream);
@@ -393,7 +388,7 @@ struct OpsImpl {
   static size_t batch_run_bytes() { return sizeof(BatchRun<T>); }
   static void fill_batch_run(const Sim* s, int in, int ncta, void* dst) {
     BatchRun<T> r;
-    r.d = const_cast<Sim*>(s)->ptrs<T>();
+    r.d = s->ptrs<T>(in);
     r.g = s->g;
     r.ph = s->ph;
     r.pc = push_const<T>(s->ph);
@@ -511,7 +506,6 @@ struct OpsImpl {
     if ((e = cudaEventRecord(join, side)) != cudaSuccess) return e;
     k_field1_batch<T><<<nblk[1], field1_threads(kF1, n_sub_max), fsm, st>>>(r, pre + n1, nruns);
     if ((e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess) return e;
-    k_step1_end_batch<T><<<nblk[1], kBlock, 0, st>>>(r, pre + n1, nruns);
     return cudaGetLastError();
   }
 

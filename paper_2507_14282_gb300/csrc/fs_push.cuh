@@ -1117,8 +1117,8 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 ? 3 : 2))
 
 // ---------------------------------------------------------------- batched step tail
 // A batched step besides the push (injection draws, movers, moments with the 1D
-// tiled field advance, step end) as one launch per kernel over every run of the
-// batch: block b belongs to the run r with pre[r] <= b < pre[r + 1] and works
+// tiled field advance and the step's end) as one launch per kernel over every
+// run of the batch: block b belongs to the run r with pre[r] <= b < pre[r + 1] and works
 // as block b - pre[r] of that run's own launch; the run's record is copied
 // into shared memory first. Same bodies, so the same results, as the per-run
 // kernels.
@@ -1172,16 +1172,6 @@ __global__ void __launch_bounds__(field1_threads(kF1, kF1MaxSub))
   const int r = load_batch_run<T>(runs, pre, nruns, R);
   const FieldConst<T> fc = field_const_dev<T>(R.ph);
   field_step1_body<T, kF1>(R.d, R.g, (T)R.ph.n_floor, fc, R.n_sub, blockIdx.x - pre[r], smem);
-}
-
-// each run's step1_end by its field tiles' blocks
-template <typename T>
-__global__ void __launch_bounds__(kBlock)
-    k_step1_end_batch(const BatchRun<T>* __restrict__ runs, const int* __restrict__ pre,
-                      int nruns) {
-  __shared__ __align__(16) BatchRun<T> R;
-  const int r = load_batch_run<T>(runs, pre, nruns, R);
-  step1_end<T>(R.d, R.g, blockIdx.x - pre[r], pre[r + 1] - pre[r]);
 }
 
 }  // namespace fsx
