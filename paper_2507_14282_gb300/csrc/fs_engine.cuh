@@ -58,12 +58,13 @@ struct Num<double> {
 // worked out on the bit pattern with integer shifts: the value is
 // mant * 2^(e - 1075); the bits shifted out decide the rounding. Exact for
 // every double; it keeps the addition off GB300's narrow FP64 pipe.
-__device__ __forceinline__ float to_acc(float c) { return c; }
-__device__ __forceinline__ unsigned long long to_acc(double c) {
+__device__ __forceinline__ float to_acc(float c, int = 0) { return c; }
+// (exp: of c 2^exp)
+__device__ __forceinline__ unsigned long long to_acc(double c, int exp = 0) {
   const long long b = __double_as_longlong(c);
   const int e = (int)((b >> 52) & 0x7FF);
   const long long mant = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
-  const int sh = 1075 - e;  // right shift of the 53-bit significand
+  const int sh = 1075 - exp - e;  // right shift of the 53-bit significand
   long long r;
   if (e == 0 || sh > 53) {
     r = 0;  // zero, subnormal, or |c| < 1/2
@@ -81,11 +82,12 @@ __device__ __forceinline__ unsigned long long to_acc(double c) {
 // the nearest integer (fma with 1.5 * 2^52), as the written scheme states.
 // (An all-integer version with the 106-bit product measured 3 % slower in the
 // push: the fused multiply-add is worth its FP64 pipe slot here.)
-__device__ __forceinline__ float to_acc_prod(float a, float b) { return a * b; }
-__device__ __forceinline__ unsigned long long to_acc_prod(double a, double b) {
-  const double m = __fma_rn(a, b, 0x1.8p52);
-  return (unsigned long long)(__double_as_longlong(m) -
-                              __double_as_longlong(0x1.8p52));
+// (magic: 1.5 * 2^(52 - exp), for the product times 2^exp)
+__device__ __forceinline__ float to_acc_prod(float a, float b, float = 0.0f) { return a * b; }
+__device__ __forceinline__ unsigned long long to_acc_prod(double a, double b,
+                                                          double magic = 0x1.8p52) {
+  const double m = __fma_rn(a, b, magic);
+  return (unsigned long long)(__double_as_longlong(m) - __double_as_longlong(magic));
 }
 __device__ __forceinline__ float fmaT(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmaT(double a, double b, double c) { return __fma_rn(a, b, c); }

@@ -1,6 +1,8 @@
 // fs_internal.h -- host-side state shared by the C ABI (fs_api.cu) and the
 // per-precision kernel translation units (fs_f32.cu, fs_f64.cu).
 #pragma once
+#include <math.h>
+
 #include <new>
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -139,12 +141,28 @@ struct PushConst {
   T dtdx, dtdy, hdt;  // dt/dx, dt/dy, dt/2
   T wth, wcr;         // deposit weights (x 2^40 in FP64: the fixed-point scale)
   T c2inv;            // 1/c^2 (0: non-relativistic)
+  // FP64: what a deposit contribution still lacks of the weight, a power of two
+  // 2^acc_exp, goes into its rounding to fixed point (exact, and free: no
+  // multiplication on the narrow FP64 pipe); acc_th, acc_cr are the rest per
+  // species. With a thermal weight that is no power of two: exponent 0, the
+  // weights themselves.
+  T acc_th, acc_cr;
+  T acc_magic;  // 1.5 * 2^(52 - acc_exp): adding it rounds to multiples of 2^-acc_exp
+  int acc_exp;
 };
 template <typename T>
 inline PushConst<T> push_const(const Phys& ph) {
   const double ws = sizeof(T) == 8 ? 0x1p40 : 1.0;
-  return PushConst<T>{(T)ph.dtdx, (T)ph.dtdy, (T)ph.hdt, (T)(ph.w_th * ws), (T)(ph.w_cr * ws),
-                      (T)ph.c2inv};
+  PushConst<T> c{(T)ph.dtdx, (T)ph.dtdy, (T)ph.hdt, (T)(ph.w_th * ws), (T)(ph.w_cr * ws),
+                 (T)ph.c2inv, (T)(ph.w_th * ws), (T)(ph.w_cr * ws), (T)0x1.8p52, 0};
+  int e = 0;
+  if (sizeof(T) == 8 && frexp(ph.w_th, &e) == 0.5) {  // w_th = 2^(e - 1)
+    c.acc_exp = 40 + e - 1;
+    c.acc_th = (T)1;
+    c.acc_cr = (T)ldexp(ph.w_cr * ws, -c.acc_exp);
+    c.acc_magic = (T)ldexp(1.5, 52 - c.acc_exp);
+  }
+  return c;
 }
 
 template <typename T>

@@ -606,7 +606,7 @@ __device__ __forceinline__ void issue_chunk(unsigned char* sm, const PushLayout<
 template <typename T, int DIM, bool REL>
 __device__ __forceinline__ void team_add(typename Num<T>::acc (&acc)[4], const T* W,
                                          const T* V, const T* Fo, const uint32_t* ID,
-                                         T wth, T wcr, int i, int c) {
+                                         const PushConst<T>& pc, int i, int c) {
   T cw;
   T v[4];
   ld4(V + 4 * i, v);
@@ -614,7 +614,7 @@ __device__ __forceinline__ void team_add(typename Num<T>::acc (&acc)[4], const T
     T f[2];
     ld2(Fo + 2 * i, f);
     // the particle weight: in V's fourth slot without relativistic terms
-    const T wp = REL ? ((ID[i] & kIdCR) ? wcr : wth) : v[3];
+    const T wp = REL ? ((ID[i] & kIdCR) ? pc.wcr : pc.wth) : v[3];
     // gx = fx or 1 - fx by one fused multiply-add (the same rounded value)
     const T gx = fmaT((c & 1) ? (T)1 : (T)-1, f[0], (c & 1) ? (T)0 : (T)1);
     if (DIM == 2) {
@@ -631,17 +631,17 @@ __device__ __forceinline__ void team_add(typename Num<T>::acc (&acc)[4], const T
     v[1] = v[1] * v[3];
     v[2] = v[2] * v[3];
   }
-  acc[0] = acc[0] + to_acc(cw);
-  acc[1] = acc[1] + to_acc_prod(cw, v[0]);
-  acc[2] = acc[2] + to_acc_prod(cw, v[1]);
-  acc[3] = acc[3] + to_acc_prod(cw, v[2]);
+  acc[0] = acc[0] + to_acc(cw, pc.acc_exp);
+  acc[1] = acc[1] + to_acc_prod(cw, v[0], pc.acc_magic);
+  acc[2] = acc[2] + to_acc_prod(cw, v[1], pc.acc_magic);
+  acc[3] = acc[3] + to_acc_prod(cw, v[2], pc.acc_magic);
 }
 
 template <typename T, int DIM, bool REL>
 __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, int AX,
                                              int le, int b0, int b1, const T* W, const T* V,
-                                             const T* Fo, const uint32_t* ID, T wth, T wcr,
-                                             int lane) {
+                                             const T* Fo, const uint32_t* ID,
+                                             const PushConst<T>& pc, int lane) {
   using A_t = typename Num<T>::acc;
   constexpr int NC = (DIM == 2) ? 4 : 2;
   constexpr int SPL = 16 / NC;
@@ -649,10 +649,10 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
   A_t acc[4] = {(A_t)0, (A_t)0, (A_t)0, (A_t)0};
   int i = b0 + s;
   for (; i + SPL < b1; i += 2 * SPL) {  // two particles in flight per lane
-    team_add<T, DIM, REL>(acc, W, V, Fo, ID, wth, wcr, i, c);
-    team_add<T, DIM, REL>(acc, W, V, Fo, ID, wth, wcr, i + SPL, c);
+    team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
+    team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i + SPL, c);
   }
-  if (i < b1) team_add<T, DIM, REL>(acc, W, V, Fo, ID, wth, wcr, i, c);
+  if (i < b1) team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
   __syncwarp();
   // two halving levels leave one quantity per lane, the rest add pairs
   {
@@ -698,8 +698,9 @@ template <typename T, int DIM, bool REL>
 __device__ __forceinline__ void deposit_pieces(typename Num<T>::acc* ACC, int NA, int AX,
                                                const uint16_t* wk, const int* pcs, int npmax,
                                                const int* k2e, const T* W, const T* V,
-                                               const T* Fo, const uint32_t* ID, T wth, T wcr,
-                                               int* q, int warp, int lane) {
+                                               const T* Fo, const uint32_t* ID,
+                                               const PushConst<T>& cst, int* q, int warp,
+                                               int lane) {
   const int np = pcs[npmax];
   int gi = warp - 1;
   if (warp == 0) {
@@ -716,7 +717,7 @@ __device__ __forceinline__ void deposit_pieces(typename Num<T>::acc* ACC, int NA
       b1 = min(b0 + kPiece, (int)wk[k + 1]);
       le = k2e[k];
     }
-    team_deposit<T, DIM, REL>(ACC, NA, AX, le, b0, b1, W, V, Fo, ID, wth, wcr, lane);
+    team_deposit<T, DIM, REL>(ACC, NA, AX, le, b0, b1, W, V, Fo, ID, cst, lane);
     int nx = 0;
     if (lane == 0) nx = atomicAdd(q, 1);
     gi = kWarps - 1 + __shfl_sync(0xffffffffu, nx, 0);
@@ -914,7 +915,7 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
     //      finished their push early take more of it
     if (dpar >= 0)
       deposit_pieces<T, DIM, REL>(ACC0 + dpar * 4 * NA, NA, AX, wk, pcs, npmax, k2e, oW, oV, oF,
-                                  oid, wth, wcr, dq + ((ci - 1) & 1), warp, lane);
+                                  oid, pc, dq + ((ci - 1) & 1), warp, lane);
     if (done) break;
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
@@ -991,16 +992,29 @@ __device__ __forceinline__ void push_run(const DevPtrs<T>& d, const Geo& g, cons
           : !rel                   ? (T)1
           : inreg                  ? rig_[r]
                                    : inv_gamma_u(ux, uy, uz, c2inv));
-      // corner weights: wp * (gx * gy), corners (0,0) (1,0) (0,1) (1,1)
+      // corner weights: wp * (gx * gy) but for the power of two that the
+      // deposit's rounding takes, corners (0,0) (1,0) (0,1) (1,1)
       // (FP32: formed in the deposit)
       if constexpr (sizeof(T) == 8) {
         const T gx0 = (T)1 - fx;
+        const T wr = (id & kIdCR) ? pc.acc_cr : pc.acc_th;  // (1: none left to multiply)
+        T w[4];
         if (DIM == 2) {
           const T gy0 = (T)1 - fy;
-          st4(oW + 4 * pos, wp * (gx0 * gy0), wp * (fx * gy0), wp * (gx0 * fy), wp * (fx * fy));
+          w[0] = gx0 * gy0;
+          w[1] = fx * gy0;
+          w[2] = gx0 * fy;
+          w[3] = fx * fy;
         } else {
-          st4(oW + 4 * pos, wp * gx0, wp * fx, (T)0, (T)0);
+          w[0] = gx0;
+          w[1] = fx;
+          w[2] = w[3] = (T)0;
         }
+        if (__double_as_longlong(wr) != kKeyOne) {
+#pragma unroll
+          for (int c = 0; c < (DIM == 2 ? 4 : 2); ++c) w[c] = wr * w[c];
+        }
+        st4(oW + 4 * pos, w[0], w[1], w[2], w[3]);
       }
     }
     __syncthreads();
