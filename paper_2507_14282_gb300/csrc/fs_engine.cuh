@@ -1980,7 +1980,8 @@ __global__ void k_diag_field(DevPtrs<T> d, Geo g, Phys ph) {
   atomicMax(&zblk, __reduce_max_sync(0xffffffffu, __float_as_uint(zf)));
   __syncthreads();
   const float lim = __uint_as_float(zblk);
-  const float from = (lim < 1e30f && lim > 1e-30f) ? lim * (1.0f - 1e-4f) : -1.0f;
+  // (below 1e-6 the squares of what makes up z may leave FP32's normal range)
+  const float from = (lim < 1e30f && lim > 1e-6f) ? lim * (1.0f - 1e-4f) : -1.0f;
   double zmax = 0.0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nn;
        c += gridDim.x * blockDim.x) {

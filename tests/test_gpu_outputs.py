@@ -147,3 +147,21 @@ def test_moments_of_any_tile_shape_equal_the_oracle(fs, tx, ty):
         np.testing.assert_array_equal(gpu.grid(what), ref.grid(name))
     gpu.close()
     ref.close()
+
+
+@pytest.mark.parametrize("scale,seed", [(1.0, 3), (1e-6, 3), (3e-23, 1), (2.5e-23, 8), (1e-25, 3)])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_stability_number_at_any_field_strength(fs, prec, scale, seed):
+    """The largest node's z, from the run's own node fields, also where the
+    squares of B and u are below FP32's range: the written FP64 expression, so
+    equal to rounding (a few operations of 1e-16 each)."""
+    nx, ny, dt = 60, 40, 0.005
+    sim = fs.FauxShock(dim=2, nx=nx, ny=ny, ppc=4, dt=dt, dx=0.5, dy=0.5, precision=prec,
+                       init_plasma=0, bc_x=O.BC_PERIODIC, mach_a=0.0, beta_i=0.0, beta_e=0.0)
+    rng = np.random.default_rng(seed)
+    sim.load_fields(scale * rng.normal(size=(ny, nx, 3)))
+    bb, n, u = sim.grid(fs.FS_BBAR), sim.grid(fs.FS_N), sim.grid(fs.FS_U)
+    z = 0.5 * dt * (8.0 / 0.25 * np.sqrt((bb ** 2).sum(-1)) / n +
+                    8.0 * np.sqrt((u ** 2).sum(-1)))
+    assert sim.diag()["max_z"] == pytest.approx(z.max(), rel=1e-12, abs=0)
+    sim.close()
