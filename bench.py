@@ -62,9 +62,9 @@ def particle_bytes(prec_bytes: int, dim: int) -> int:
 GRID_WORDS_PER_CELL = 23
 # FP64-pipe operations of the FP64 push per particle-step in 2D, from ncu
 # (sm__thread_inst_executed_pipe_fp64_pred_on.sum over the particles of one
-# launch of the 1024 x 256-cell case: 408.2 M / 4 194 771; DADD + DMUL + DFMA
-# alone give 96.9); an FMA is one pipe operation, like the denominator.
-FP64_OPS_PER_PARTICLE_STEP = 97.3
+# launch of the 1024 x 256-cell case: 391.4 M / 4 194 771); an FMA is one pipe
+# operation, like the denominator.
+FP64_OPS_PER_PARTICLE_STEP = 93.3
 FP64_OPS_SOURCE = ("ncu sm__thread_inst_executed_pipe_fp64_pred_on.sum / particles, "
                    "1024x256-cell case of the FP64 workload")
 PHASE_TIMING = ("value: the product path (graph replay, no phase events); phases and "
@@ -81,13 +81,13 @@ FP64_PEAK_OPS = 0.625e12
 # + dram__bytes_write.sum) on a 1024 x 256-cell case of the same kernel, scaled
 # by the particles of a launch; valid only while the kernel sources are the
 # ones the counters were taken on (their hash below), else reported as null.
-PUSH_TRAFFIC = {"fp32": (506.448128e6 + 448.124416e6) / 16779950,
-                "fp64": (224.050944e6 + 175.183872e6) / 4194771}
+PUSH_TRAFFIC = {"fp32": (506.231552e6 + 447.919616e6) / 16779950,
+                "fp64": (224.007424e6 + 175.378944e6) / 4194771}
 PUSH_SOURCES = ("paper_2507_14282_gb300/csrc/fs_push.cuh",
                 "paper_2507_14282_gb300/csrc/fs_engine.cuh")
 # hash of PUSH_SOURCES when each precision's counters were taken
-PUSH_SOURCES_SHA1 = {"fp32": "f2d64bea1b9ff0cea678960c8fe9e907546835bf",
-                     "fp64": "f2d64bea1b9ff0cea678960c8fe9e907546835bf"}
+PUSH_SOURCES_SHA1 = {"fp32": "bfeae8b0189b491409c359215ccef68131edc52f",
+                     "fp64": "bfeae8b0189b491409c359215ccef68131edc52f"}
 
 
 def push_sources_sha1() -> str:

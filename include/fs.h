@@ -356,10 +356,10 @@ int fs_field_advance_noalloc(const fs_params* p, const double* B_in,
    of CTAs about proportional to its particles (a (run, tile) work list, each
    run's pointers, geometry and physics read from a device table). When every run
    is 1D with x walls (the one-launch field advance), the rest of the step --
-   movers, injection, moments, field advance, step counter -- is one launch
-   per kernel over all runs too (each block works for one run, found from
-   per-run block prefixes in the table): about seven launches per step
-   whatever the number of runs. Otherwise each run's remaining kernels run in
+   injection draws, movers, moments with field advance and step counter -- is
+   one launch per kernel over all runs too (each block works for one run,
+   found from per-run block prefixes in the table), three launches besides
+   the pushes whatever the number of runs. Otherwise each run's remaining kernels run in
    parallel branches. Either way the step is captured as a CUDA graph. The
    push's launch shape is the runs' push_chunk and push_ctas_per_sm when all
    runs agree on them, else the library's choice. Each

@@ -709,7 +709,8 @@ __global__ void k_moments(DevPtrs<T> d, Geo g, Phys ph) {
 // of a node are a fixed, small set (MX columns by MY rows), so every load is
 // issued without a data-dependent loop; rows are taken in increasing wrapped
 // order, columns in increasing order, as in moments_body. The tile shape is
-// compiled in (TXC x TYC) or the run's (0).
+// compiled in (TXC x TYC) or the run's (0). Bound by the loads in flight:
+// 3000 x 250 cells, FP32, 39 -> 25 us against moments_body's loops.
 template <typename T, int TXC, int TYC, int MX, int MY>
 __global__ void k_moments_ct(DevPtrs<T> d, Geo g, Phys ph) {
   using A = typename Num<T>::acc;
@@ -1064,7 +1065,7 @@ __global__ void k_ohm_start(const T* __restrict__ Bc, const T* __restrict__ nN,
 // FP64 pipe binds (82 % busy): against a pass per operator the row and column
 // sums that neighbours share are formed once, 53 operations per node and stage
 // instead of 65, and the stage field never goes to memory. 4096 x 256 cells,
-// two substeps: 1345 -> 1176 us. (In FP32, 8192 x 512 cells: 612 us against
+// two substeps: 1345 -> 1175 us. (In FP32, 8192 x 512 cells: 612 us against
 // k_field_substep's 340.)
 // One warp per block: the marches are few and long, so that blocks of several
 // would leave SMs uneven.
@@ -1568,11 +1569,12 @@ __device__ __forceinline__ void tile1_ohm(const T* y, int L, int m, int p, const
 // The moments and the whole field advance of a 1D step with x walls (n, J, u
 // from the deposit, n_sub RK4 substeps, then Ohm's E and Bbar for the next
 // gather) in one launch: on a 1D grid the separate passes are tens of tiny
-// launches per step (the far sums are read by neighbouring tiles too: the
-// next step's, of the step before, are cleared here). The first block also
-// ends the step. A CTA owns TILE
-// cells (and their left nodes; the last tile also node nx) and runs every
-// pass in shared memory over its cells plus field1_halo(n_sub) cells around
+// launches per step. Neighbouring tiles read the same B and far sums, so the
+// new B goes to the other buffer and the other far sums, of the step before,
+// are cleared for the next (Sim::swaps_fields); the first block counts the
+// step. (With a launch of its own for that, ten steps of 512 cells: 758 us
+// FP64, 524 FP32; now 726 and 509.) A CTA owns TILE cells (and their left
+// nodes; the last tile also node nx) and runs every pass in shared memory over its cells plus field1_halo(n_sub) cells around
 // them, which it recomputes: each pass's stencil reaches one cell, so
 // values made wrong at a tile's inner edges (read with indices clamped to
 // the tile) move in by one cell per pass and stay outside the owned cells;
@@ -1585,8 +1587,8 @@ __device__ __forceinline__ void tile1_ohm(const T* y, int L, int m, int p, const
 // formed once, B_x and E_x are left out of the stages, the y and z components
 // go to different warps, and a thread keeps its node's terms in registers.
 // TILE 32 while that leaves SMs free (tile and halo fill two warps a
-// component), 64 beyond (less halo to recompute). 512 cells FP64 21.5 us
-// before.
+// component), 64 beyond (less halo to recompute). 512 cells FP64: 14.4 us with
+// the moments, which took 8.6 us beside the fields' 21.5 before.
 __host__ __device__ constexpr int field1_halo(int n_sub) { return 4 * n_sub + 2; }
 constexpr int kF1 = 64, kF1Small = 32;
 constexpr int kF1MaxSub = 16;
@@ -1895,7 +1897,7 @@ __device__ __forceinline__ void count_shared(unsigned* cnt, int k) {
 // operations per particle without relativistic terms (its weight and the cell
 // volume come as one factor), against 19 and a block reduction per tile
 // before; one set of sums for both species (two, chosen per lane, ran both
-// sides of the choice: 449 us). 17.8 M particles FP64: 990 us before.
+// sides of the choice: 449 us). 17.8 M particles FP64: 990 -> 290 us.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kBlock) k_diag_particles(DevPtrs<T> d, Geo g, Phys ph, int buf) {
   const Parts<T> P = d.P[buf];
@@ -2003,7 +2005,7 @@ __global__ void k_diag_field(DevPtrs<T> d, Geo g, Phys ph) {
 // global memory) and added to the histogram once. The bins are formed in FP32
 // relative to the CTA's first cell; only values within eps of a bin edge
 // take the written FP64 expressions (GB300's FP64 pipe is narrow).
-// 17.8 M particles FP64: 505 us before.
+// 17.8 M particles FP64: 505 -> 91 us.
 constexpr int kHistShared = 8192;  // counters
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kBlock)
@@ -2094,7 +2096,7 @@ __global__ void k_import_B(T* B, const double* src, int nc, int q0, int n) {
 // (off: the tiles' first numbers), as contiguous FP64 columns: one warp per
 // tile. Bound by HBM; it replaces seven small device-to-host copies per tile
 // (1 M particles in 2458 tiles: the checkpoint's read-back, 138 ms in all
-// with its restart, was almost all of them).
+// with its restart, was almost all of them): 61 us.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kBlock)
     k_pack_columns(DevPtrs<T> d, Geo g, int buf, const int* __restrict__ off, int k0, int m,

@@ -145,7 +145,7 @@ struct PushConst {
   // 2^acc_exp, goes into its rounding to fixed point (exact, and free: no
   // multiplication on the narrow FP64 pipe); acc_th, acc_cr are the rest per
   // species. With a thermal weight that is no power of two: exponent 0, the
-  // weights themselves.
+  // weights themselves. (Push of 4096 x 256 cells, 16 ppc: 3418 -> 3393 us.)
   T acc_th, acc_cr;
   T acc_magic;  // 1.5 * 2^(52 - acc_exp): adding it rounds to multiples of 2^-acc_exp
   int acc_exp;

@@ -691,7 +691,8 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
 // piece's team reduction, not its particle count, sets most of its cost: with
 // a whole warp per piece, found by a search over the keys, the 49 keys of a
 // 5 x 5-cell tile at 20 particles per cell made the push 27.3 warp
-// instructions per particle (17.0 on 4 x 2 cells at 64). Each particle's
+// instructions per particle (17.0 on 4 x 2 cells at 64); now 22.5 (16.2): the
+// push 532 -> 404 us at 3000 x 250 cells, 5.26 -> 5.08 ms at 8192 x 512. Each particle's
 // contributions are formed as in the per-particle scheme, so in fixed point
 // (FP64) the sums do not depend on which warp takes which piece.
 template <typename T, int DIM, bool REL>
