@@ -147,3 +147,71 @@ def test_window_slots_in_any_order_match_the_oracle(fs, ckpt):
     assert g[16] == pytest.approx(g0[16], rel=1e-5)
     assert g[17] == pytest.approx(g0[17], rel=1e-6)
     w.close()
+
+
+def march_rows(strips, ny, extra, lo, hi):
+    """Rows of a warp's march, as the launcher chooses them for 152 SMs."""
+    rows, best = 1, -1
+    for r in range(1, min(128, ny) + 1):
+        per_sm = (strips * -(-ny // r) + 151) // 152
+        if best >= 0 and per_sm < lo:
+            break
+        cost = per_sm * (r + extra)
+        if best >= 0 and cost >= best and per_sm <= hi:
+            continue
+        best = -1 if per_sm > hi else cost
+        rows = r
+    return rows
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("nx,ny,n_sub", [(1002, 152, 1), (1002, 152, 2), (1024, 256, 3)])
+@pytest.mark.parametrize("bc", ["walls", "periodic"])
+def test_field_march_of_several_rows(fs, prec, nx, ny, n_sub, bc):
+    """Marches that carry a row's sums to the next, with a short last march."""
+    for cols, extra, lo in ((23, 9, 8), (22, 10, 8)) if prec else ((30, 2, 11),):
+        rows = march_rows(-(-(nx + (bc == "walls")) // cols), ny, extra, lo, 16)
+        assert rows > 1 and ny % rows
+    cfg = W.scaled(W.CONFIG_2D_FP32 if prec else W.CONFIG_2D, nx=nx, ny=ny, ppc=2, n_sub=n_sub,
+                   theta_bn_deg=30.0)
+    if bc == "periodic":
+        cfg.update(bc_x=O.BC_PERIODIC, mach_a=1.0, j_cr_ext=0.2)
+    gpu, ref = pair(fs, prec, **cfg)
+    gpu.step(1)
+    ref.step(1)
+    compare(fs, gpu, ref, not prec)
+    gpu.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("first", [1, 3])
+def test_runs_changed_after_an_odd_number_of_batched_steps(fs, first):
+    """Particles put in and fields loaded between odd numbers of batched steps act
+    on the buffers of the step that comes next."""
+    cfgs = [W.scaled(W.CONFIG_1D, nx=nx, ppc=8, seed=nx, capacity_factor=16.0) for nx in (64, 96, 256)]
+    runs = [pair(fs, 0, **c) for c in cfgs]
+    batch = fs.FsBatch([g for g, _ in runs])
+    for steps in (first, 2, 1):
+        batch.step(steps)
+        for k, (gpu, ref) in enumerate(runs):
+            ref.step(steps)
+            compare(fs, gpu, ref, True)
+            new = W.random_particles(np.random.default_rng(steps + k), 5, cfgs[k]["nx"], 1)
+            gpu.inject(*new)
+            ref.inject(*new)
+            compare(fs, gpu, ref, True)
+        batch.step(1)
+        for gpu, ref in runs:
+            ref.step(1)
+            compare(fs, gpu, ref, True)
+            B = ref.grid(O.GRID_B) * 1.01
+            gpu.load_fields(B)
+            ref.set_B(B)
+    batch.step(2)
+    for gpu, ref in runs:
+        ref.step(2)
+        compare(fs, gpu, ref, True)
+    batch.close()
+    for gpu, ref in runs:
+        gpu.close()
+        ref.close()
