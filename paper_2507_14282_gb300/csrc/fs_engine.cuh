@@ -1956,23 +1956,29 @@ __global__ void k_diag_field(DevPtrs<T> d, Geo g, Phys ph) {
   // maximum over nodes in sums[5] (non-negative doubles order like their
   // bit patterns).
   // Two square roots and a division per node in FP64 would bind this kernel to
-  // the FP64 pipe, so a node's z is first formed in FP32 and only nodes
-  // within 1e-4 of the block's largest take the FP64 expression.
+  // the FP64 pipe, so a node's z is first bounded in FP32 and only nodes whose
+  // upper bound reaches the block's largest lower bound take the FP64 expression.
   const double kk = 16.0 * (ph.hdx * ph.hdx + ph.hdy * ph.hdy);
   const double ka = 4.0 * (ph.hdx + ph.hdy);
   const int nn = g.nxn * g.ny;
   const float kkf = (float)kk, kaf = (float)ka;
-  auto approx = [&](int c) {
+  // side -1: a lower, 1: an upper bound of z / h but for rounding (below 1e-5):
+  // what the squares of B or u lose below FP32's normal range is far less than
+  // the 1e-30 that is taken off or added, which changes |B| or |u| by 1e-15 at
+  // most (from 1e-12 on by less than 1e-6 of it)
+  auto bound = [&](int c, float side) {
     const float bx = near_float(d.Bb[c]), by = near_float(d.Bb[nn + c]),
                 bz = near_float(d.Bb[2 * nn + c]);
     const float ux = near_float(d.u[c]), uy = near_float(d.u[nn + c]),
                 uz = near_float(d.u[2 * nn + c]);
-    return kkf * sqrtf(bx * bx + by * by + bz * bz) / near_float(d.n[c]) +
-           kaf * sqrtf(ux * ux + uy * uy + uz * uz);
+    const float b2 = bx * bx + by * by + bz * bz + side * 1e-30f;
+    const float u2 = ux * ux + uy * uy + uz * uz + side * 1e-30f;
+    return kkf * sqrtf(b2 < 0.0f ? 0.0f : b2) / near_float(d.n[c]) +
+           kaf * sqrtf(u2 < 0.0f ? 0.0f : u2);  // (NaN stays NaN)
   };
   float zf = 0.0f;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nn; c += gridDim.x * blockDim.x) {
-    const float z = approx(c);
+    const float z = bound(c, -1.0f);
     // beyond FP32's range (or NaN): every node takes the FP64 expression
     zf = (z < 1e30f) ? fmaxf(zf, z) : INFINITY;
   }
@@ -1982,12 +1988,16 @@ __global__ void k_diag_field(DevPtrs<T> d, Geo g, Phys ph) {
   atomicMax(&zblk, __reduce_max_sync(0xffffffffu, __float_as_uint(zf)));
   __syncthreads();
   const float lim = __uint_as_float(zblk);
-  // (below 1e-6 the squares of what makes up z may leave FP32's normal range)
-  const float from = (lim < 1e30f && lim > 1e-6f) ? lim * (1.0f - 1e-4f) : -1.0f;
+  // the bounds hold while their factors' products stay in FP32's normal range:
+  // factors and densities within 1e-15 .. 1e15 (n >= n_floor), and a largest z
+  // to which a product below that range adds nothing
+  const bool plain = kkf > 1e-15f && kkf < 1e15f && kaf > 1e-15f && kaf < 1e15f &&
+                     ph.n_floor > 1e-15;
+  const float from = (plain && lim < 1e30f && lim > 1e-6f) ? lim * (1.0f - 1e-4f) : -1.0f;
   double zmax = 0.0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nn;
        c += gridDim.x * blockDim.x) {
-    if (from >= 0.0f && !(approx(c) >= from)) continue;
+    if (from >= 0.0f && !(bound(c, 1.0f) >= from)) continue;
     const double bx = d.Bb[c], by = d.Bb[nn + c], bz = d.Bb[2 * nn + c];
     const double ux = d.u[c], uy = d.u[nn + c], uz = d.u[2 * nn + c];
     const double b = sqrt(bx * bx + by * by + bz * bz);

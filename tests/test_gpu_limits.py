@@ -1,0 +1,70 @@
+"""Values at the ends of the types' ranges, runs with an error pending, and
+several live handles of one kernel: each against the written expressions, or
+against the same calls made alone."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from tests import window_inputs as WI
+from tests import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fs():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2507_14282_gb300 import build
+    build.build()
+    from paper_2507_14282_gb300 import fs as m
+    return m
+
+
+@pytest.mark.parametrize("scale,seed,n_floor,dx,n_part", [
+    (3e-23, 1, 1e-20, 0.5, 0), (2.5e-23, 8, 1e-18, 0.5, 0), (1e-22, 3, 1e-20, 0.5, 0),
+    (3e-23, 4, 0.05, 1e-8, 0), (2e-23, 6, 0.05, 1e-9, 600), (1e-20, 5, 1e-30, 0.5, 0),
+    (1.0, 2, 1e-25, 0.5, 600), (1e-15, 7, 1e-12, 1e-3, 600)])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_stability_number_of_thin_plasma_and_small_cells(fs, prec, scale, seed, n_floor, dx, n_part):
+    """The largest node's z where it is not small although the squares of B (or
+    u) are below FP32's range, by 1/n or 1/dx^2: the written FP64 expression on
+    the run's own node fields, so equal to rounding."""
+    nx, ny, dt = 60, 40, 0.005
+    sim = fs.FauxShock(dim=2, nx=nx, ny=ny, ppc=4, dt=dt, dx=dx, dy=dx, precision=prec,
+                       init_plasma=0, bc_x=O.BC_PERIODIC, mach_a=0.0, beta_i=0.0, beta_e=0.0,
+                       n_floor=n_floor)
+    rng = np.random.default_rng(seed)
+    if n_part:
+        p = list(W.random_particles(rng, n_part, nx, ny))
+        sim.inject(*p[:4], *[scale * v for v in p[4:]])
+    sim.load_fields(scale * rng.normal(size=(ny, nx, 3)))
+    bb, n, u = sim.grid(fs.FS_BBAR), sim.grid(fs.FS_N), sim.grid(fs.FS_U)
+    z = 0.5 * dt * (8.0 / dx ** 2 * np.sqrt((bb ** 2).sum(-1)) / n +
+                    4.0 / dx * np.sqrt((u ** 2).sum(-1)))
+    assert sim.diag()["max_z"] == pytest.approx(z.max(), rel=1e-12, abs=0)
+    sim.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_stability_number_passes_over_nan_nodes(fs, prec):
+    """A node without a z (NaN field) next to fast plasma: the largest of the rest."""
+    nx, ny = 60, 40
+    sim = fs.FauxShock(dim=2, nx=nx, ny=ny, ppc=4, precision=prec, init_plasma=0,
+                       bc_x=O.BC_PERIODIC, mach_a=0.0, beta_i=0.0, beta_e=0.0)
+    rng = np.random.default_rng(9)
+    p = list(W.random_particles(rng, 600, nx, ny))
+    p[4][:50] += 1e4
+    p[0][:50], p[1][:50] = 10, 10
+    sim.inject(*p)
+    B = rng.normal(size=(ny, nx, 3))
+    B[8:13, 8:13] = np.nan
+    sim.load_fields(B)
+    bb, n, u = sim.grid(fs.FS_BBAR), sim.grid(fs.FS_N), sim.grid(fs.FS_U)
+    z = 0.0025 * (32.0 * np.sqrt((bb ** 2).sum(-1)) / n + 8.0 * np.sqrt((u ** 2).sum(-1)))
+    assert np.isnan(z[10, 10]) and u[10, 10, 0] > 100 * np.nanmax(z)
+    assert sim.diag()["max_z"] == pytest.approx(np.nanmax(z), rel=1e-12, abs=0)
+    sim.close()
