@@ -1861,13 +1861,17 @@ __device__ __forceinline__ float near_float(double x) {
   return __uint_as_float((hi & 0x80000000u) | m);
 }
 // An FP32 value as FP64 (exact) by integer operations, for the same reason;
-// zero and subnormals give zero, infinities and NaN stay so.
+// subnormals are brought into the normal range first (x 2^64, exact);
+// infinities and NaN stay so.
 __device__ __forceinline__ double wide_double(double x) { return x; }
 __device__ __forceinline__ double wide_double(float x) {
-  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xFFu;
+  const bool low = fabsf(x) < 0x1p-126f;
+  const unsigned b = __float_as_uint(low ? x * 0x1p64f : x), e = (b >> 23) & 0xFFu;
   const unsigned hi = (b & 0x80000000u) |
-                      (e == 0 ? 0u : (((e == 0xFFu ? 0x7FFu : e + 896u) << 20) | ((b & 0x7FFFFFu) >> 3)));
-  return __hiloint2double((int)hi, e == 0 ? 0 : (int)((b & 7u) << 29));
+                      (e == 0 ? 0u
+                              : (((e == 0xFFu ? 0x7FFu : e + (low ? 832u : 896u)) << 20) |
+                                 ((b & 0x7FFFFFu) >> 3)));
+  return __hiloint2double((int)hi, (int)((b & 7u) << 29));
 }
 
 constexpr int kWarpsPerBlock = kBlock / 32;

@@ -68,3 +68,22 @@ def test_stability_number_passes_over_nan_nodes(fs, prec):
     assert np.isnan(z[10, 10]) and u[10, 10, 0] > 100 * np.nanmax(z)
     assert sim.diag()["max_z"] == pytest.approx(np.nanmax(z), rel=1e-12, abs=0)
     sim.close()
+
+
+def test_energy_and_momentum_of_subnormal_velocities(fs):
+    """FP32 velocities below the normal range count in the sums with their exact
+    values (FP64 sums of some hundred terms)."""
+    nx, n = 32, 300
+    sim = fs.FauxShock(dim=1, nx=nx, ppc=4, precision=1, init_plasma=0, bc_x=O.BC_PERIODIC,
+                       mach_a=0.0, beta_i=0.0, beta_e=0.0, capacity_factor=16.0)
+    rng = np.random.default_rng(1)
+    v = rng.choice([1e-45, 3e-42, 1e-40, 1.1e-38, 2e-38, 0.0], (3, n)) * rng.choice([-1, 1], (3, n))
+    sim.inject(rng.integers(0, nx, n), np.zeros(n), rng.random(n), np.zeros(n), *v)
+    p, d = sim.particles(), sim.diag()
+    w = 0.25 * 0.5
+    for k in ("vx", "vy", "vz"):
+        assert np.abs(p[k]).min() < 1e-44 < np.abs(p[k]).max()
+        assert d["p" + k[1]] == pytest.approx((w * p[k]).sum(), rel=1e-9, abs=0)
+    e = (0.5 * w * (p["vx"] ** 2 + p["vy"] ** 2 + p["vz"] ** 2)).sum()
+    assert d["kinetic"] == pytest.approx(e, rel=1e-12, abs=0)
+    sim.close()
