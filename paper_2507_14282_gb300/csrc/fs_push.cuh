@@ -648,11 +648,24 @@ __device__ __forceinline__ void team_deposit(typename Num<T>::acc* ACC, int NA, 
   const int s = lane % SPL, c = (lane & 15) / SPL;
   A_t acc[4] = {(A_t)0, (A_t)0, (A_t)0, (A_t)0};
   int i = b0 + s;
-  for (; i + SPL < b1; i += 2 * SPL) {  // two particles in flight per lane
-    team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
-    team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i + SPL, c);
+  if constexpr (sizeof(T) == 4) {
+    // a sum for each of the two particles in flight: a chain of FP32 additions
+    // is then as short as with a whole warp per piece
+    A_t second[4] = {(A_t)0, (A_t)0, (A_t)0, (A_t)0};
+    for (; i + SPL < b1; i += 2 * SPL) {
+      team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
+      team_add<T, DIM, REL>(second, W, V, Fo, ID, pc, i + SPL, c);
+    }
+    if (i < b1) team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = acc[q] + second[q];
+  } else {
+    for (; i + SPL < b1; i += 2 * SPL) {  // two particles in flight per lane
+      team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
+      team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i + SPL, c);
+    }
+    if (i < b1) team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
   }
-  if (i < b1) team_add<T, DIM, REL>(acc, W, V, Fo, ID, pc, i, c);
   __syncwarp();
   // two halving levels leave one quantity per lane, the rest add pairs
   {

@@ -87,3 +87,30 @@ def test_energy_and_momentum_of_subnormal_velocities(fs):
     e = (0.5 * w * (p["vx"] ** 2 + p["vy"] ** 2 + p["vz"] ** 2)).sum()
     assert d["kinetic"] == pytest.approx(e, rel=1e-12, abs=0)
     sim.close()
+
+
+@pytest.mark.parametrize("dim,chain", [(1, 10), (2, 20)])
+def test_fp32_deposit_adds_short_chains(fs, dim, chain):
+    """160 equal particles at rest in one cell: their FP32 sum errs no more than
+    sums of `chain` terms, added in pairs (exact, the sums being equal), would.
+    With these offsets a chain of twice that errs at least twice as much."""
+    f = 0.5 - 7.0 * 2.0 ** -24
+    n, cell = 160, 3
+    sim = fs.FauxShock(dim=dim, nx=8, ny=4 if dim == 2 else 1, ppc=64, precision=1, init_plasma=0,
+                       bc_x=O.BC_PERIODIC, mach_a=0.0, beta_i=0.0, beta_e=0.0, n_floor=1e-6,
+                       tile_x=2, capacity_factor=8.0)
+    z = np.zeros(n)
+    sim.inject(np.full(n, cell), z, np.full(n, f), z, z, z, z)
+    sim.step(1)
+    got = sim.grid(fs.FS_N)[0]
+
+    def err(x, terms):
+        s = np.float32(0)
+        for _ in range(terms):
+            s = np.float32(s + np.float32(x))
+        return abs(float(s) / (terms * float(np.float32(x))) - 1)
+    for node, x in ((cell, 1.0 - f), (cell + 1, f)):
+        allowed = err(x, chain)
+        assert err(x, 2 * chain) > 2 * allowed
+        assert abs(got[node] / (n / 64 * x) - 1) <= allowed * (1 + 1e-6)
+    sim.close()
