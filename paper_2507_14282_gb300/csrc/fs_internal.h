@@ -3,6 +3,7 @@
 #pragma once
 #include <math.h>
 
+#include <mutex>
 #include <new>
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -98,6 +99,21 @@ struct Layout {
   size_t partial, far, acc, inj, ctr, hist, prof, spec, twiddle;
   size_t total;
 };
+
+// Raises kernel Kern's dynamic shared memory limit to at least `bytes`. The limit
+// is the kernel's, whatever handle or thread launches it, so it never falls and
+// is read and set under one lock.
+template <auto Kern>
+inline cudaError_t raise_smem(size_t bytes) {
+  static std::mutex mu;
+  static size_t limit = 0;
+  std::lock_guard<std::mutex> lock(mu);
+  if (bytes <= limit) return cudaSuccess;
+  const cudaError_t e =
+      cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) limit = bytes;
+  return e;
+}
 
 // Typed device pointers (resolved from the layout).
 template <typename T>

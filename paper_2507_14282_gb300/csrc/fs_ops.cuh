@@ -3,7 +3,6 @@
 // fs_f64.cu (the latter compiled with -fmad=false).
 #pragma once
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include <mutex>
 
@@ -24,22 +23,16 @@ inline int grid_for(long long n, int block = kBlock) {
 template <typename T, int DIM, int CH, int NS, bool REL, int TXC = 0, int TYC = 0>
 cudaError_t launch_push(Sim* s, int in, long long step) {
   const PushLayout<T, DIM> L(s->g.TX, s->g.TY, CH, NS);
-  // per kernel instance: the largest dynamic shared memory enabled so far and
-  // the occupancy at the last size asked for (host threads may share them)
+  // per kernel instance: the occupancy at the last size asked for (host threads
+  // may share it)
   static std::mutex mu;
-  static size_t attr_bytes = 0;
   static size_t occ_bytes = 0;
   static int occ_blocks_c = 1, n_sm_c = 0;
   int occ_blocks, n_sm;
   {
     std::lock_guard<std::mutex> lock(mu);
-    if (L.bytes > attr_bytes) {
-      cudaError_t e = cudaFuncSetAttribute(k_push<T, DIM, CH, NS, REL, TXC, TYC>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)L.bytes);
-      if (e != cudaSuccess) return e;
-      attr_bytes = L.bytes;
-    }
+    const cudaError_t er = raise_smem<k_push<T, DIM, CH, NS, REL, TXC, TYC>>(L.bytes);
+    if (er != cudaSuccess) return er;
     if (L.bytes != occ_bytes) {
       int dev = 0, nsm = 0, occ = 0;
       cudaError_t e = cudaGetDevice(&dev);
@@ -180,17 +173,8 @@ struct OpsImpl {
   static cudaError_t field_step1(Sim* s, int in) {
     DevPtrs<T> d = s->ptrs<T>(in);
     const size_t smem = field1_smem<T>(s->p.n_sub, TILE);
-    // the largest size enabled so far; a raise races harmlessly (each caller
-    // sets at least its own size before it launches)
-    static std::atomic<size_t> attr(0);
-    if (smem > attr.load()) {
-      cudaError_t e = cudaFuncSetAttribute(k_field_step1<T, TILE>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      size_t cur = attr.load();
-      while (smem > cur && !attr.compare_exchange_weak(cur, smem)) {
-      }
-    }
+    const cudaError_t e = raise_smem<k_field_step1<T, TILE>>(smem);
+    if (e != cudaSuccess) return e;
     k_field_step1<T, TILE><<<(s->g.nx + TILE - 1) / TILE,
                              field1_threads(TILE, s->p.n_sub), smem, s->stream>>>(
         d, s->g, (T)s->ph.n_floor, field_const<T>(s->ph), s->p.n_sub);
@@ -413,11 +397,10 @@ struct OpsImpl {
   }
   template <int DIM, int CH, int NS, bool REL, int TXC = 0>
   static cudaError_t batch_kernel_setup(size_t smem, int* occ) {
-    auto kern = k_push_batch<T, DIM, CH, NS, REL, TXC>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = raise_smem<k_push_batch<T, DIM, CH, NS, REL, TXC>>(smem);
     if (e == cudaSuccess && occ)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, kBlock, smem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          occ, k_push_batch<T, DIM, CH, NS, REL, TXC>, kBlock, smem);
     return e;
   }
   template <int CH, int NS>
@@ -487,19 +470,11 @@ struct OpsImpl {
                                 cudaEvent_t fork, cudaEvent_t join) {
     const BatchRun<T>* r = (const BatchRun<T>*)runs;
     const size_t fsm = field1_smem<T>(n_sub_max, kF1);
-    static std::atomic<size_t> attr(0);  // the largest size enabled so far
-    if (fsm > attr.load()) {
-      cudaError_t e = cudaFuncSetAttribute(k_field1_batch<T>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
-      if (e != cudaSuccess) return e;
-      size_t cur = attr.load();
-      while (fsm > cur && !attr.compare_exchange_weak(cur, fsm)) {
-      }
-    }
+    cudaError_t e = raise_smem<k_field1_batch<T>>(fsm);
+    if (e != cudaSuccess) return e;
     const int n1 = nruns + 1;
     // the movers (buckets) beside the moments and field advance, which read
     // the deposit partials and far sums and no bucket
-    cudaError_t e;
     if ((e = cudaEventRecord(fork, st)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
     k_movers_batch<T, 1><<<nblk[0], kBlock, 0, side>>>(r, pre, nruns);

@@ -1437,11 +1437,8 @@ Win<T> win_ptrs(fs_window* w) {
 // dynamic shared memory of the blocked field kernels beyond the default 48 KB
 template <typename T>
 bool smem_opt_in(int n_sub) {
-  const int f = (int)fields_smem(n_sub, sizeof(T)), a = (int)rk4_adj_smem(n_sub, sizeof(T));
-  return cudaFuncSetAttribute(k_win_fields<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, f) ==
-             cudaSuccess &&
-         cudaFuncSetAttribute(k_win_rk4_adj<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, a) ==
-             cudaSuccess;
+  return raise_smem<k_win_fields<T>>(fields_smem(n_sub, sizeof(T))) == cudaSuccess &&
+         raise_smem<k_win_rk4_adj<T>>(rk4_adj_smem(n_sub, sizeof(T))) == cudaSuccess;
 }
 
 // checkpoint c: slots, B, moments

@@ -114,3 +114,55 @@ def test_fp32_deposit_adds_short_chains(fs, dim, chain):
         assert err(x, 2 * chain) > 2 * allowed
         assert abs(got[node] / (n / 64 * x) - 1) <= allowed * (1 + 1e-6)
     sim.close()
+
+
+def window(fs, prec, n_sub, steps, ckpt, nx=64):
+    from paper_2507_14282_gb300 import window as m
+    X, V = WI.plasma(nx, 8)
+    amps, ph = WI.modes()
+    w = m.FauxShockWindow(X, V, ph, steps=steps, ckpt=ckpt, nx=nx, ny=1, ppc=8, n_sub=n_sub,
+                          precision=prec, cr_enable=1, fs_mode_thermal=1, p_iso=100.0,
+                          n_cr_ratio=0.01, **WI.COMMON)
+    return w, WI.theta(amps)
+
+
+# A window run twice: the forward's sums are fixed point, so the loss repeats
+# exactly; the backward adds in FP64 in any order, and an FP32 adjoint rounds
+# what came out, at some 1e-7 of its size.
+GRAD_REPEATS = {0: 1e-11, 1: 1e-5}
+
+
+@pytest.mark.parametrize("prec,n_sub", [(0, 9), (1, 10)])
+def test_window_runs_on_after_one_of_fewer_substeps(fs, prec, n_sub):
+    """A live window keeps its kernels' shared memory when a later one needs less."""
+    first, th = window(fs, prec, n_sub, 6, 3)
+    L, g = first.loss_and_grad(th)
+    second, _ = window(fs, prec, 2, 6, 3)
+    second.loss_and_grad(th)
+    again = first.loss_and_grad(th)
+    assert again[0] == L
+    np.testing.assert_allclose(again[1], g, rtol=0, atol=GRAD_REPEATS[prec] * np.abs(g).max())
+    first.close()
+    second.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_batch_runs_on_after_one_of_narrower_tiles(fs, prec):
+    """The same for the batched push: the second batch's tiles need less."""
+    kw = dict(dim=1, nx=256, ppc=8, precision=prec, mach_a=10.0, dt=0.005, capacity_factor=8.0)
+    alone = fs.FauxShock(tile_x=64, **kw)
+    wide = [fs.FauxShock(tile_x=64, **kw) for _ in range(2)]
+    narrow = [fs.FauxShock(tile_x=2, **kw) for _ in range(2)]
+    batches = [fs.FsBatch(wide), fs.FsBatch(narrow)]
+    alone.step(3)
+    for b in batches[::-1]:
+        b.step(1)
+        b.step(2)
+    for s in wide:
+        assert s.diag()["step"] == 3
+        np.testing.assert_allclose(s.grid(fs.FS_B), alone.grid(fs.FS_B), rtol=0,
+                                   atol=1e-4 if prec else 0)
+    for b in batches:
+        b.close()
+    for s in [alone] + wide + narrow:
+        s.close()
