@@ -346,6 +346,18 @@ int sync_and_check(Sim* s) {
   Counters c;
   return read_counters(s, &c);
 }
+// Copies a result in the run's buffer to its destination, once everything on
+// the stream is known to have gone well (else the destination stays as it is).
+int copy_out(Sim* s, void* dst, const void* src, size_t bytes, int dst_on_device) {
+  const int r = sync_and_check(s);
+  if (r) return r;
+  if (cudaMemcpyAsync(dst, src, bytes,
+                      dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                      s->stream) != cudaSuccess ||
+      cudaStreamSynchronize(s->stream) != cudaSuccess)
+    return s->sticky = FS_ECUDA;
+  return FS_OK;
+}
 
 // Device scratch of the host transfers: the particle buffer that holds no
 // current particles (the next step's output, which the push overwrites).
@@ -833,9 +845,14 @@ int fs_moments(fs_handle* h, int what, void* dst, size_t dst_bytes, int dst_on_d
   Sim* s = &h->sim;
   if (s->sticky) return s->sticky;
   const Geo& g = s->g;
+  // an error of the run comes before one of the call
+  auto refused = [&] {
+    const int r = sync_and_check(s);
+    return r ? r : FS_EINVAL;
+  };
   if (what == FS_STATE) {
     const size_t need = sizeof(fs_run_state) + 8 * (size_t)g.ny;
-    if (dst_bytes < need) return FS_EINVAL;
+    if (dst_bytes < need) return refused();
     Counters c;
     std::vector<char> blob(need);
     if (cudaMemcpyAsync(blob.data() + sizeof(fs_run_state), s->base + s->L.acc,
@@ -867,60 +884,44 @@ int fs_moments(fs_handle* h, int what, void* dst, size_t dst_bytes, int dst_on_d
   }
   if (what == FS_HIST_XPX || what == FS_HIST_XPX_CR) {
     const size_t need = 8 * (size_t)s->ph.hist_nx * s->ph.hist_np;
-    if (dst_bytes < need) return FS_EINVAL;
+    if (dst_bytes < need) return refused();
     if (s->ops->hist(s, s->cur, what == FS_HIST_XPX ? -1 : 1) != cudaSuccess)
       return s->sticky = FS_ECUDA;
-    if (cudaMemcpyAsync(dst, s->base + s->L.hist, need,
-                        dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                        s->stream) != cudaSuccess)
-      return s->sticky = FS_ECUDA;
-    return sync_and_check(s);
+    return copy_out(s, dst, s->base + s->L.hist, need, dst_on_device);
   }
   if (what == FS_PROFILE_N || what == FS_PROFILE_DB2) {
     const size_t cnt = (what == FS_PROFILE_N) ? g.nxn : g.nx;
-    if (dst_bytes < 8 * cnt) return FS_EINVAL;
+    if (dst_bytes < 8 * cnt) return refused();
     if (s->ops->profiles(s, what) != cudaSuccess) return s->sticky = FS_ECUDA;
     const size_t off = s->L.prof + (what == FS_PROFILE_N ? 0 : 8 * (size_t)g.nxn);
-    if (cudaMemcpyAsync(dst, s->base + off, 8 * cnt,
-                        dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                        s->stream) != cudaSuccess)
-      return s->sticky = FS_ECUDA;
-    return sync_and_check(s);
+    return copy_out(s, dst, s->base + off, 8 * cnt, dst_on_device);
   }
   if (what == FS_SPECTRUM_P_CR || what == FS_SPECTRUM_P_ALL) {
     const size_t np = (size_t)s->p.spec_np;
-    if (dst_bytes < 8 * np) return FS_EINVAL;
+    if (dst_bytes < 8 * np) return refused();
     if (s->ops->spectrum_p(s, s->cur, what == FS_SPECTRUM_P_CR ? 1 : -1) != cudaSuccess)
       return s->sticky = FS_ECUDA;
-    if (cudaMemcpyAsync(dst, s->base + s->L.spec + 8 * (np + 1), 8 * np,
-                        dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                        s->stream) != cudaSuccess)
-      return s->sticky = FS_ECUDA;
-    return sync_and_check(s);
+    return copy_out(s, dst, s->base + s->L.spec + 8 * (np + 1), 8 * np, dst_on_device);
   }
   if (what == FS_PROFILE_B || what == FS_SPECTRUM_BPERP) {
     const bool spec = (what == FS_SPECTRUM_BPERP);
     const size_t cnt = spec ? (size_t)g.nx / 2 + 1 : 3 * (size_t)g.nx;
-    if (dst_bytes < 8 * cnt) return FS_EINVAL;
+    if (dst_bytes < 8 * cnt) return refused();
     const cudaError_t e = spec ? s->ops->spectrum_bperp(s) : s->ops->profile_B(s);
     if (e != cudaSuccess) return s->sticky = FS_ECUDA;
     const size_t off = s->L.prof + 8 * ((size_t)g.nxn + g.nx + (spec ? 3 * (size_t)g.nx : 0));
-    if (cudaMemcpyAsync(dst, s->base + off, 8 * cnt,
-                        dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                        s->stream) != cudaSuccess)
-      return s->sticky = FS_ECUDA;
-    return sync_and_check(s);
+    return copy_out(s, dst, s->base + off, 8 * cnt, dst_on_device);
   }
   size_t planes = 3, cols = g.nxn;
   switch (what) {
     case FS_B: cols = g.nx; break;
     case FS_N: planes = 1; break;
     case FS_E: case FS_BBAR: case FS_J: case FS_U: break;
-    default: return FS_EINVAL;
+    default: return refused();
   }
   const long long npts = (long long)cols * g.ny;
-  if (dst_bytes < 8 * planes * (size_t)npts) return FS_EINVAL;
-  if (dst_on_device) {
+  if (dst_bytes < 8 * planes * (size_t)npts) return refused();
+  if (dst_on_device) {  // (writes nothing when the run has an error)
     if (s->ops->export_grid(s, what, 0, (int)npts, (double*)dst) != cudaSuccess)
       return s->sticky = FS_ECUDA;
     return sync_and_check(s);
@@ -930,12 +931,12 @@ int fs_moments(fs_handle* h, int what, void* dst, size_t dst_bytes, int dst_on_d
   const long long chunk = std::min<long long>(npts, (long long)(scr.bytes / (8 * planes)));
   for (long long q0 = 0; q0 < npts; q0 += chunk) {
     const int m = (int)std::min(chunk, npts - q0);
-    if (s->ops->export_grid(s, what, (int)q0, m, (double*)scr.p) != cudaSuccess ||
-        cudaMemcpyAsync((double*)dst + planes * q0, scr.p, 8 * planes * (size_t)m,
-                        cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+    if (s->ops->export_grid(s, what, (int)q0, m, (double*)scr.p) != cudaSuccess)
       return s->sticky = FS_ECUDA;
+    const int r = copy_out(s, (double*)dst + planes * q0, scr.p, 8 * planes * (size_t)m, 0);
+    if (r) return r;
   }
-  return sync_and_check(s);
+  return FS_OK;
   FS_GUARD_END
 }
 

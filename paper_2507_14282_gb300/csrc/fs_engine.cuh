@@ -2090,9 +2090,12 @@ __global__ void __launch_bounds__(kBlock)
 }
 
 // Grid export / import in FP64 host layout ([row][col][component]), points
-// q0 .. q0 + n - 1 of a grid of npts.
+// q0 .. q0 + n - 1 of a grid of npts; nothing is exported from a run with an
+// error.
 template <typename T>
-__global__ void k_export_grid(const T* src, int planes, int npts, int q0, int n, double* dst) {
+__global__ void k_export_grid(const T* src, int planes, int npts, int q0, int n, double* dst,
+                              const Counters* ctr) {
+  if (ctr->status) return;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += gridDim.x * blockDim.x)
     for (int c = 0; c < planes; ++c)

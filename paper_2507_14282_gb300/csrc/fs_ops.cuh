@@ -631,7 +631,8 @@ struct OpsImpl {
       case FS_U: src = d.u; break;
       default: return cudaErrorInvalidValue;
     }
-    k_export_grid<T><<<grid_for(n), kBlock, 0, s->stream>>>(src, planes, cols * s->g.ny, q0, n, dst);
+    k_export_grid<T><<<grid_for(n), kBlock, 0, s->stream>>>(src, planes, cols * s->g.ny, q0, n, dst,
+                                                           d.ctr);
     return cudaGetLastError();
   }
 

@@ -166,3 +166,29 @@ def test_batch_runs_on_after_one_of_narrower_tiles(fs, prec):
         b.close()
     for s in [alone] + wide + narrow:
         s.close()
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("what", ["B", "N", "PROFILE_N", "PROFILE_DB2", "PROFILE_B",
+                                  "SPECTRUM_BPERP", "SPECTRUM_P_ALL", "HIST_XPX", "STATE"])
+@pytest.mark.parametrize("on_device", [0, 1])
+def test_reads_of_a_run_with_an_error_pending_leave_their_destination(fs, dim, what, on_device):
+    """A non-finite motion that only the device knows of yet: its code comes back,
+    also from a read that is refused for its size, and nothing is written."""
+    import torch
+    cfg = W.scaled(W.CONFIG_2D if dim == 2 else W.CONFIG_1D, nx=64, ppc=8,
+                   **(dict(ny=16) if dim == 2 else {}))
+    for size in (1 << 20, 4):
+        sim = fs.FauxShock(precision=0, **cfg)
+        B = sim.grid(fs.FS_B)
+        B[0, 20, 1] = np.nan
+        sim.load_fields(B)
+        sim.step(1)
+        dst = torch.full((1 << 20,), 7, dtype=torch.uint8, device="cuda" if on_device else "cpu")
+        torch.cuda.synchronize()
+        rc = fs.lib().fs_moments(sim._h, getattr(fs, "FS_" + what), C.c_void_p(dst.data_ptr()),
+                                 C.c_size_t(size), on_device)
+        torch.cuda.synchronize()
+        assert rc == fs.FS_ENAN
+        assert bool((dst == 7).all())
+        sim.close()
