@@ -1307,9 +1307,10 @@ struct fs_window {
   // device); a slot born in the window has its slot number as id
   std::vector<int> np_at;
   // the recompute of a segment beside the reversal of the one after it: its
-  // stream and events (made by the first backward), indexed by tape
+  // stream and events (made by the first backward): a segment recomputed, and how
+  // far the reversal is
   cudaStream_t side = nullptr;
-  cudaEvent_t ready = nullptr, taped[2] = {nullptr, nullptr}, reversed[2] = {nullptr, nullptr};
+  cudaEvent_t taped = nullptr, reversed = nullptr;
   bool have_forward = false;
   int qsel = 0;  // which of the two deposit sums the next step uses
   long long counts[5] = {0, 0, 0, 0, 0};  // of the last forward
@@ -1339,6 +1340,11 @@ void injection_schedule(const Phys& ph, int steps, std::vector<int>* ninj) {
   }
 }
 
+// Entries of the tape for segments of up to K steps. A segment is recomputed while
+// the one after it is reversed, into the entries that this has done with: the two
+// run through the tape in opposite directions (tape_entry), one entry apart.
+int tape_entries(int K, int nseg) { return K + (nseg > 1 ? 1 : 0); }
+
 int window_sizes(const fs_params* p, int steps, int ckpt, long long n_init, int M, Geo* g,
                  Phys* ph, int* cap, size_t* total, size_t off[13]) {
   if (!p || steps < 1 || ckpt < 1 || n_init < 0 || M < 0 || M > 4096) return FS_EINVAL;
@@ -1366,14 +1372,13 @@ int window_sizes(const fs_params* p, int steps, int ckpt, long long n_init, int 
   off[0] = o; o += slot_bytes(*cap, tsz);                                  // state
   off[1] = o;                                                               // checkpoints
   o += (size_t)nseg * (slot_bytes(*cap, tsz) + al(3 * tsz * nx) + mom_bytes(nxn, tsz));
-  // the tape of a segment; two of them, when there are two segments: one is
-  // recomputed while the other is reversed
-  const size_t KT = (size_t)K * (nseg > 1 ? 2 : 1);
+  const size_t KT = (size_t)tape_entries(K, nseg);                         // tape:
   off[2] = o; o += KT * tape_slot_bytes(*cap, tsz);                        // particles
   off[3] = o; o += KT * al((size_t)*cap);                                  // events
   off[4] = o; o += KT * al(3 * tsz * nx);                                  // B
   off[5] = o; o += KT * mom_bytes(nxn, tsz);                               // moments
-  off[11] = o; o += (KT + 2) * 2 * al(3 * tsz * nxn);                      // E, Bbar
+  off[11] = o; o += (KT + 2) * 2 * al(3 * tsz * nxn);                      // E, Bbar (and of
+                                                                            // two checkpoints)
   off[6] = o; o += 2 * al(3 * tsz * nxn) + 2 * al(3 * tsz * nx) + mom_bytes(nxn, tsz);
   off[7] = o; o += 2 * al(8 * 4 * (size_t)nxn);                            // fixed-point sums
   off[8] = o; o += al(8 * 8);                                              // counters
@@ -1459,14 +1464,14 @@ void mom_ptrs(char* b, int nxn, T** n, T** u, T** r) {
   *u = (T*)(b + al(sizeof(T) * nxn));
   *r = (T*)(b + 4 * al(sizeof(T) * nxn));
 }
-// entry k of tape t
+// where step k of a segment of parity t keeps its events and the state after it
 size_t tape_entry(const fs_window* w, int t, int k) {
-  return (size_t)t * std::min(w->ckpt, w->steps) + k;
+  return t ? tape_entries(std::min(w->ckpt, w->steps), w->nseg) - 1 - k : k;
 }
 uint8_t* ev_at(fs_window* w, int t, int k) {
   return (uint8_t*)(w->base + w->o_ev) + tape_entry(w, t, k) * al(w->cap);
 }
-// E, Bbar entry e (2 per tape besides the steps' own: 0 and 1 hold the tapes' first)
+// E, Bbar entry e (0 and 1: of the checkpoints of segments of either parity)
 template <typename T>
 void tape_E(fs_window* w, size_t e, State<T>* a) {
   const size_t b = al(3 * sizeof(T) * w->g.nxn);
@@ -1474,22 +1479,22 @@ void tape_E(fs_window* w, size_t e, State<T>* a) {
   a->Bb = (T*)((char*)a->E + b);
 }
 
-// the state at the start of segment c, for tape t: its checkpoint, with E, Bbar
-// formed from it
+// the state at the start of segment c: its checkpoint, with E, Bbar formed from it
 template <typename T>
-State<T> ckpt_state(fs_window* w, int c, int t) {
+State<T> ckpt_state(fs_window* w, int c) {
   const Ck ck = ckpt_at(w, c);
   State<T> a;
   a.s = slots_at<T>(ck.slots, w->cap, false);
   a.B = (T*)ck.B;
   mom_ptrs<T>(ck.mom, w->g.nxn, &a.n, &a.u, &a.nraw);
-  tape_E<T>(w, t, &a);
+  tape_E<T>(w, c & 1, &a);
   return a;
 }
-// state k >= 1 of a recomputed segment (on tape t)
+// state k of segment c (k >= 1: recomputed)
 template <typename T>
-State<T> tape_state(fs_window* w, int t, int k) {
-  const size_t e = tape_entry(w, t, k - 1);
+State<T> seg_state(fs_window* w, int c, int k) {
+  if (k == 0) return ckpt_state<T>(w, c);
+  const size_t e = tape_entry(w, c & 1, k - 1);
   State<T> a;
   a.s = slots_at<T>(w->base + w->o_tape + e * tape_slot_bytes(w->cap, w->tsz), w->cap, false);
   a.B = (T*)(w->base + w->o_tapeB + e * al(3 * sizeof(T) * w->g.nx));
@@ -1595,7 +1600,7 @@ int do_forward(fs_window* w, const double* theta, double* loss) {
 bool make_side(fs_window* w) {
   if (!w->side && cudaStreamCreateWithFlags(&w->side, cudaStreamNonBlocking) != cudaSuccess)
     return false;
-  for (cudaEvent_t* e : {&w->ready, &w->taped[0], &w->taped[1], &w->reversed[0], &w->reversed[1]})
+  for (cudaEvent_t* e : {&w->taped, &w->reversed})
     if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return false;
   return true;
 }
@@ -1619,36 +1624,32 @@ int do_backward(fs_window* w, double dloss, double* grad) {
   k_win_loss<T><<<1, kBlock, 0, w->st>>>(r.B[w->steps & 1], w->g, w->ph, w->loss_i0, w->p.dx,
                                                   nullptr, r.lB, dloss);
   // Segment by segment from the end: recompute it, keeping every state, then
-  // reverse it. The recompute of segment seg - 1 (its own tape; it needs only
-  // its checkpoint) runs on the side stream while segment seg is reversed:
-  // both are chains of short kernels that leave most of the GPU idle.
-  auto wait = [](cudaStream_t st, cudaEvent_t e) {
-    return cudaStreamWaitEvent(st, e, 0) == cudaSuccess;
+  // reverse it. The recompute of segment seg - 1 (it needs only its checkpoint)
+  // runs on the side stream while segment seg is reversed: both are chains of
+  // short kernels that leave most of the GPU idle. Its step k takes the tape
+  // entry of step K - k of segment seg, so it follows the reversal of that step.
+  const int K = std::min(w->ckpt, w->steps);
+  auto follow = [](cudaEvent_t e, cudaStream_t from, cudaStream_t to) {
+    return cudaEventRecord(e, from) == cudaSuccess && cudaStreamWaitEvent(to, e, 0) == cudaSuccess;
   };
-  auto recompute = [&](int seg) {
-    const int t = seg & 1, n0 = seg * w->ckpt, n1 = std::min(w->steps, n0 + w->ckpt);
-    const State<T> first = ckpt_state<T>(w, seg, t);
-    auto at = [&](int k) { return k == 0 ? first : tape_state<T>(w, t, k); };
-    ohm_of<T>(w, first, w->side);
-    for (int n = n0; n < n1; ++n)
-      forward_step<T>(w, r, n, at(n - n0), at(n - n0 + 1), first.s, ev_at(w, t, n - n0), w->side);
-    return cudaEventRecord(w->taped[t], w->side) == cudaSuccess;
+  auto recompute = [&](int seg, int k) {
+    const State<T> first = ckpt_state<T>(w, seg);
+    if (k == 0) ohm_of<T>(w, first, w->side);
+    forward_step<T>(w, r, seg * w->ckpt + k, seg_state<T>(w, seg, k), seg_state<T>(w, seg, k + 1),
+                    first.s, ev_at(w, seg & 1, k), w->side);
   };
-  if (cudaEventRecord(w->ready, w->st) != cudaSuccess || !wait(w->side, w->ready) ||
-      !recompute(w->nseg - 1))
-    return FS_ECUDA;
+  if (!follow(w->reversed, w->st, w->side)) return FS_ECUDA;
+  for (int k = 0; k < w->steps - (w->nseg - 1) * w->ckpt; ++k) recompute(w->nseg - 1, k);
   for (int seg = w->nseg - 1; seg >= 0; --seg) {
-    const int t = seg & 1, n0 = seg * w->ckpt, n1 = std::min(w->steps, n0 + w->ckpt);
-    if (seg > 0) {  // (the other tape: free once segment seg + 1 is reversed)
-      if (seg + 1 < w->nseg && !wait(w->side, w->reversed[1 - t])) return FS_ECUDA;
-      if (!recompute(seg - 1)) return FS_ECUDA;
-    }
-    if (!wait(w->st, w->taped[t])) return FS_ECUDA;
-    const State<T> first = ckpt_state<T>(w, seg, t);
-    auto at = [&](int k) { return k == 0 ? first : tape_state<T>(w, t, k); };
+    const int n0 = seg * w->ckpt, n1 = std::min(w->steps, n0 + w->ckpt);
+    // (st: after the segment's recompute; side: after the reversal of the segment
+    // after it, which had the first entries and the checkpoint's E, Bbar)
+    if (!follow(w->taped, w->side, w->st)) return FS_ECUDA;
+    if (seg > 0)
+      for (int k = 0; K - k >= n1 - n0; ++k) recompute(seg - 1, k);
     for (int n = n1 - 1; n >= n0; --n) {
       const int k = n - n0;
-      const State<T> a = at(k), b = at(k + 1);
+      const State<T> a = seg_state<T>(w, seg, k), b = seg_state<T>(w, seg, k + 1);
       // the step's field update and moments in reverse, with the Ohm's law
       // that followed it
       k_win_rk4_adj<T><<<tiles(nx), rk4_adj_threads(w->p.n_sub), rk4_adj_smem(w->p.n_sub, sizeof(T)), w->st>>>(
@@ -1659,12 +1660,15 @@ int do_backward(fs_window* w, double dloss, double* grad) {
       const int npa = w->np_at[n], npb = w->np_at[n + 1];
       if (npb > 0)
         k_win_particle_adj<T><<<blocks(npb), kBlock, 0, w->st>>>(
-            r, a, b.s, ev_at(w, t, k), r.lE[esel], r.lBb[esel], w->g, w->ph, push_const<T>(w->ph), n,
-            npa, npb, M);
+            r, a, b.s, ev_at(w, seg & 1, k), r.lE[esel], r.lBb[esel], w->g, w->ph,
+            push_const<T>(w->ph), n, npa, npb, M);
+      if (seg > 0) {
+        if (!follow(w->reversed, w->st, w->side)) return FS_ECUDA;
+        if (k > 0) recompute(seg - 1, K - k);
+      }
     }
-    if (cudaEventRecord(w->reversed[t], w->st) != cudaSuccess) return FS_ECUDA;
     if (seg == 0)
-      k_win_ohm_adj_start<T><<<tiles(nx), 32, 0, w->st>>>(first, w->g, w->ph, r.lE[esel],
+      k_win_ohm_adj_start<T><<<tiles(nx), 32, 0, w->st>>>(ckpt_state<T>(w, 0), w->g, w->ph, r.lE[esel],
                                                                   r.lBb[esel], r.lB);
   }
   double* phases = (double*)(w->base + w->o_params) + M;
@@ -1811,7 +1815,7 @@ int fs_window_destroy(fs_window* w) {
     cudaStreamSynchronize(w->side);
     cudaStreamDestroy(w->side);
   }
-  for (cudaEvent_t e : {w->ready, w->taped[0], w->taped[1], w->reversed[0], w->reversed[1]})
+  for (cudaEvent_t e : {w->taped, w->reversed})
     if (e) cudaEventDestroy(e);
   delete w;
   return FS_OK;

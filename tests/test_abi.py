@@ -147,3 +147,20 @@ def test_query_accepts_push_launch_shapes(fs):
         s = fs.query(dim=2, nx=256, ny=64, ppc=64, precision=prec, push_chunk=chunk,
                      push_ctas_per_sm=2)
         assert s.device_bytes > 0
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_window_memory_falls_with_its_segments(fs, prec):
+    # every segment has a checkpoint of about a step's state, and one tape of a
+    # segment's steps serves them all
+    import ctypes as C
+
+    def need(steps, ckpt):
+        p = fs.make_params(dim=1, nx=2048, ppc=128, dt=0.0025, precision=prec, inject_thermal=0)
+        b = C.c_size_t()
+        assert fs.lib().fs_window_query(C.byref(p), steps, ckpt, 262144, 16, C.byref(b)) == 0
+        return b.value
+
+    state = need(201, 201) - need(200, 200)  # one more step of tape
+    assert need(200, 100) < need(200, 200) - 90 * state
+    assert need(200, 20) < need(200, 40) - 10 * state

@@ -192,3 +192,20 @@ def test_reads_of_a_run_with_an_error_pending_leave_their_destination(fs, dim, w
         assert rc == fs.FS_ENAN
         assert bool((dst == 7).all())
         sim.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("steps,ckpts", [(23, (1, 2, 5, 8, 22)), (24, (3, 12))])
+def test_window_segments_of_any_length_give_one_gradient(fs, prec, steps, ckpts):
+    """One tape for all segments, a segment written into it while the one after it
+    is read back: against the same window in one segment."""
+    whole, th = window(fs, prec, 2, steps, steps)
+    L, g = whole.loss_and_grad(th)
+    for ckpt in ckpts:
+        w, _ = window(fs, prec, 2, steps, ckpt)
+        for _ in range(3):
+            L1, g1 = w.loss_and_grad(th)
+            assert L1 == L
+            np.testing.assert_allclose(g1, g, rtol=0, atol=GRAD_REPEATS[prec] * np.abs(g).max())
+        w.close()
+    whole.close()
