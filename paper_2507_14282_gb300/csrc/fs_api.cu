@@ -84,13 +84,22 @@ void choose_full_tile(const fs_params* p, int* tx, int* ty, long long* ref) {
   *ref = (long long)bx * by;
 }
 
+// Slots of a tile with `ref` cells' worth of them.
+long long tile_slots(const fs_params* p, long long ref) {
+  const double want = ceil(p->capacity_factor * (double)(ref * p->ppc)) + 64;
+  return want > 0x1p40 ? 1LL << 40 : ((long long)want + 31) / 32 * 32;
+}
+
 // The tile of a run: the caller's, else the full tile; in a box whose full
 // tiles occupy at most half of the GPU's SMs, tiles cut into equal parts of at
 // least 128 particles on average until there is one per SM (a CTA works on one tile at a
 // time: 512 cells of 32 particles in 32 tiles left 120 SMs idle and gave each
 // of the rest two rounds of particles, FP64 push 24 us per step). A cut tile
-// keeps the slots of the full one (*ref cells' worth), so that a density peak
-// that fitted before still does.
+// keeps the slots of the full one (*ref cells' worth), and as many of the mover
+// list, so that a density peak that fitted before still does: up to four times
+// the particle memory. Beyond kCutSlots slots in all (0.3 GB in FP64; a
+// capacity factor of some 13) the memory counts for more and tiles stay whole.
+constexpr long long kCutSlots = 1LL << 21;
 void choose_tile(const fs_params* p, int* tx, int* ty, long long* ref) {
   if (p->tile_x > 0 && (p->dim == 1 || p->tile_y > 0)) {
     *tx = p->tile_x;
@@ -115,6 +124,7 @@ void choose_tile(const fs_params* p, int* tx, int* ty, long long* ref) {
       if (squarer || (had ? (enough && c > best) : c < best)) { best = c; bx = cx; by = cy; }
     }
   }
+  if (cells / best * tile_slots(p, *ref) > kCutSlots) return;
   *tx = bx;
   *ty = by;
 }
@@ -179,8 +189,7 @@ int derive(const fs_params* p, Geo* g, Phys* ph, Layout* L) {
   g->nty = p->ny / ty;
   g->ntiles = g->ntx * g->nty;
   const long long cells_per_tile = (long long)tx * ty;
-  long long cap = (long long)ceil(p->capacity_factor * (double)(ref * p->ppc)) + 64;
-  cap = (cap + 31) / 32 * 32;
+  const long long cap = tile_slots(p, ref);
   if (cap > (1LL << 30)) return FS_EINVAL;
   g->tile_cap = (int)cap;
   g->cap_total = cap * g->ntiles;

@@ -164,3 +164,23 @@ def test_window_memory_falls_with_its_segments(fs, prec):
     state = need(201, 201) - need(200, 200)  # one more step of tape
     assert need(200, 100) < need(200, 200) - 90 * state
     assert need(200, 20) < need(200, 40) - 10 * state
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("box", [dict(dim=1, nx=512, ppc=32), dict(dim=2, nx=64, ny=32, ppc=16)])
+def test_small_boxes_take_any_capacity(fs, prec, box):
+    # a box cut into a tile per SM gives every tile the slots of an uncut one:
+    # at most 2^21 slots in all, beyond which the tiles stay whole
+    tile = dict(dim1=(16, 1), dim2=(8, 4))["dim%d" % box["dim"]]
+    whole = dict(tile_x=tile[0], tile_y=tile[1])
+    cells = box["nx"] * box.get("ny", 1)
+    cut = fs.query(precision=prec, **box)
+    assert cut.tiles > cells // (tile[0] * tile[1])
+    for factor in (1.0, 3.0, 10.0, 50.0, 1e3, 3e4):
+        got = fs.query(precision=prec, capacity_factor=factor, **box)
+        full = fs.query(precision=prec, capacity_factor=factor, **box, **whole)
+        assert got.particle_capacity <= max(1 << 21, full.particle_capacity)
+        if factor <= 3.0:
+            assert got.tiles == cut.tiles
+        if got.tiles == full.tiles:
+            assert got.device_bytes == full.device_bytes
