@@ -445,7 +445,7 @@ int build_graphs(Sim* s) {
       rc = FS_ECUDA;
       break;
     }
-    const cudaError_t e = s->ops->step(s, par, 0, nullptr);
+    const cudaError_t e = s->ops->step(s, par, nullptr);
     const cudaError_t e2 = cudaStreamEndCapture(s->stream, &gr);
     if (e != cudaSuccess || e2 != cudaSuccess || !gr) {
       rc = FS_ECUDA;
@@ -752,7 +752,7 @@ int fs_step(fs_handle* h, int nsteps) {
       ev = &h->events[h->used * kSet];
       h->used++;
     }
-    if (s->ops->step(s, s->cur, s->step, ev) != cudaSuccess) return s->sticky = FS_ECUDA;
+    if (s->ops->step(s, s->cur, ev) != cudaSuccess) return s->sticky = FS_ECUDA;
     s->cur = 1 - s->cur;
     s->step++;
     s->launches += per_step;

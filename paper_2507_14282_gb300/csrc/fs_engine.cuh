@@ -1487,7 +1487,6 @@ struct Tile1 {
   T* E;  // FP64 only: E_y, E_z [2][L + 1]
   Node1<T> n0, n1;  // the thread's node a, and (FP32) node a + 1
   T b, k;           // B of the thread's component at cell a, the RK4 sum
-  __device__ __forceinline__ T* field() { return S; }  // [2][L] between substeps
 };
 // values of T a tile keeps in shared memory
 __host__ __device__ constexpr size_t tile1_words(size_t L, size_t tsz) {

@@ -204,7 +204,7 @@ struct Ops {
   cudaError_t (*moments)(Sim*);
   cudaError_t (*ohm_final)(Sim*);
   // ev: NULL, or FS_NPHASES + 1 events recorded at the phase boundaries
-  cudaError_t (*step)(Sim*, int in_buf, long long step, cudaEvent_t* ev);
+  cudaError_t (*step)(Sim*, int in_buf, cudaEvent_t* ev);
   // all but the push; drawn: the injection's draws are under way on the side stream
   cudaError_t (*step_rest)(Sim*, int in_buf, cudaEvent_t* ev, bool drawn);
   // batched ensembles (k_push_batch)
@@ -229,7 +229,6 @@ struct Ops {
   cudaError_t (*batch_rest)(const void* runs, const int* pre, int nruns, const int* nblk,
                             int n_sub_max, cudaStream_t st, cudaStream_t side,
                             cudaEvent_t fork, cudaEvent_t join);
-  cudaError_t (*fields)(Sim*);
   // ids NULL: first, first + 1, ...
   cudaError_t (*insert_columns)(Sim*, int buf, const Columns& src, int n, const uint32_t* ids,
                                 unsigned long long first);

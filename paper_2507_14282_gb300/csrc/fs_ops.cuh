@@ -21,7 +21,7 @@ inline int grid_for(long long n, int block = kBlock) {
 }
 
 template <typename T, int DIM, int CH, int NS, bool REL, int TXC = 0, int TYC = 0>
-cudaError_t launch_push(Sim* s, int in, long long step) {
+cudaError_t launch_push(Sim* s, int in) {
   const PushLayout<T, DIM> L(s->g.TX, s->g.TY, CH, NS);
   // per kernel instance: the occupancy at the last size asked for (host threads
   // may share it)
@@ -54,7 +54,6 @@ cudaError_t launch_push(Sim* s, int in, long long step) {
   a.ph = s->ph;
   a.in = in;
   a.out = 1 - in;
-  a.step = step;
   const int per_sm = s->g.push_ctas > 0 ? std::min(occ_blocks, s->g.push_ctas) : occ_blocks;
   const long long want = (long long)n_sm * per_sm;
   const int grid = (int)std::min<long long>(want, s->g.ntiles);
@@ -78,25 +77,25 @@ struct PushShape<double> {
 };
 
 template <typename T, int DIM>
-cudaError_t push_dispatch(Sim* s, int in, long long step) {
+cudaError_t push_dispatch(Sim* s, int in) {
   using S = PushShape<T>;
   // the relativistic terms are compiled in only for runs with a finite c
   if (s->ph.c2inv > 0.0) {
     if (s->g.chunk == S::kChunkSmall)
-      return launch_push<T, DIM, S::kChunkSmall, S::kStagesSmall, true>(s, in, step);
-    return launch_push<T, DIM, S::kChunkLarge, S::kStagesLarge, true>(s, in, step);
+      return launch_push<T, DIM, S::kChunkSmall, S::kStagesSmall, true>(s, in);
+    return launch_push<T, DIM, S::kChunkLarge, S::kStagesLarge, true>(s, in);
   }
   if (s->g.chunk == S::kChunkSmall)
-    return launch_push<T, DIM, S::kChunkSmall, S::kStagesSmall, false>(s, in, step);
+    return launch_push<T, DIM, S::kChunkSmall, S::kStagesSmall, false>(s, in);
   // The 2D FP32 tile shape the library picks at 64 ppc (4 x 2 cells), compiled
   // in: every layout offset and tile constant of the push becomes an
   // immediate (7.11 -> 6.67 ms on the 268 M-particle precision form; the
   // FP64 push, bound by its FP64 pipe, gains nothing from the same).
   if constexpr (DIM == 2 && sizeof(T) == 4) {
     if (s->g.TX == 4 && s->g.TY == 2)
-      return launch_push<T, DIM, S::kChunkLarge, S::kStagesLarge, false, 4, 2>(s, in, step);
+      return launch_push<T, DIM, S::kChunkLarge, S::kStagesLarge, false, 4, 2>(s, in);
   }
-  return launch_push<T, DIM, S::kChunkLarge, S::kStagesLarge, false>(s, in, step);
+  return launch_push<T, DIM, S::kChunkLarge, S::kStagesLarge, false>(s, in);
 }
 
 template <typename T>
@@ -350,7 +349,7 @@ struct OpsImpl {
     return cudaGetLastError();
   }
 
-  static cudaError_t step(Sim* s, int in, long long step, cudaEvent_t* ev) {
+  static cudaError_t step(Sim* s, int in, cudaEvent_t* ev) {
     // without phase events (and with the side stream of the captured step):
     // the draws beside the push
     const bool drawn = !ev && s->side && s->ev_fork && s->ev_draw && s->ev_push && s->ev_join;
@@ -362,7 +361,7 @@ struct OpsImpl {
       if ((e = cudaEventRecord(s->ev_draw, s->side)) != cudaSuccess) return e;
     }
     if (ev) cudaEventRecord(ev[0], s->stream);
-    e = (s->g.dim == 1) ? push_dispatch<T, 1>(s, in, step) : push_dispatch<T, 2>(s, in, step);
+    e = (s->g.dim == 1) ? push_dispatch<T, 1>(s, in) : push_dispatch<T, 2>(s, in);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], s->stream);
     return step_rest(s, in, ev, drawn);
@@ -648,7 +647,6 @@ struct OpsImpl {
     o.moments = moments;
     o.ohm_final = ohm_final;
     o.step = step;
-    o.fields = fields;
     o.insert_columns = insert_columns;
     o.scan_counts = scan_counts;
     o.pack_columns = pack_columns;

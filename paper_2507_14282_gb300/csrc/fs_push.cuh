@@ -23,8 +23,8 @@
 // A tile's node accumulator is written out as its deposit partial after the
 // first barrier of the chunk that follows the tile's last chunk (whose
 // deposit is done by then); two accumulators alternate between tiles. Each
-// chunk costs two block-wide barriers; the CTA's last chunk is deposited
-// after the loop.
+// chunk costs two block-wide barriers; the CTA's last chunk is deposited in
+// a last turn of the loop, which has no particles.
 #pragma once
 #include "fs_engine.cuh"
 
@@ -108,7 +108,6 @@ struct StepArgs {
   Geo g;
   Phys ph;
   int in, out;
-  long long step;
 };
 
 // ---------------------------------------------------------------- layout

@@ -605,11 +605,6 @@ struct Tile {
     lo = max(0, c0 - halo);
     L = min(nx, c1 + halo) - lo;
   }
-  // global cell (clamped at the walls) -> local cell (clamped to the tile)
-  __device__ __forceinline__ int cell(int c) const {
-    c = min(max(c, 0), nx - 1);
-    return min(max(c - lo, 0), L - 1);
-  }
   // global node (mirrored at the walls) -> local node (clamped to the tile)
   __device__ __forceinline__ int node(int i) const {
     i = (i < 0) ? -i : ((i > nx) ? 2 * nx - i : i);
