@@ -100,18 +100,22 @@ struct Layout {
   size_t total;
 };
 
-// Raises kernel Kern's dynamic shared memory limit to at least `bytes`. The limit
-// is the kernel's, whatever handle or thread launches it, so it never falls and
-// is read and set under one lock.
+// Raises kernel Kern's dynamic shared memory limit on the current device to at
+// least `bytes`. The limit is the kernel's, whatever handle or thread launches
+// it, so it never falls and is read and set under one lock.
 template <auto Kern>
 inline cudaError_t raise_smem(size_t bytes) {
+  constexpr int kDevices = 64;
   static std::mutex mu;
-  static size_t limit = 0;
+  static size_t limit[kDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= kDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
-  if (bytes <= limit) return cudaSuccess;
-  const cudaError_t e =
-      cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) limit = bytes;
+  if (bytes <= limit[dev]) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) limit[dev] = bytes;
   return e;
 }
 
