@@ -293,7 +293,9 @@ int fs_diag(fs_handle* h, fs_diag_t* out);
 /* Per-phase timing of fs_step with CUDA events on the handle's stream
    (tracing). Phases: FS_PHASE_PUSH (fused gather/push/faux shock/sort/
    deposit kernel), FS_PHASE_MOVERS, FS_PHASE_INJECT, FS_PHASE_MOMENTS,
-   FS_PHASE_FIELDS (RK4 Ohm + Faraday and the node packing).
+   FS_PHASE_FIELDS (RK4 Ohm + Faraday and the node packing). In 1D boxes
+   with x walls and up to 16 substeps, moments, fields and the step's end are
+   one launch: FS_PHASE_FIELDS holds all of it, FS_PHASE_MOMENTS about zero.
    fs_profile(h, 1) starts recording (events are created on the host, no
    device memory); fs_profile_read() synchronises and writes, per phase, the
    summed milliseconds ms[k] and the number of steps timed counts[k] since the

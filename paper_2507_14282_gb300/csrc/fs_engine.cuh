@@ -1062,7 +1062,7 @@ __global__ void k_ohm_start(const T* __restrict__ Bc, const T* __restrict__ nN,
 // lane above), node i needs cell i - 1 (the lane below), so lanes 1 .. 30 are
 // the strip's own 30 columns; the cell row above the chunk is formed again.
 // Same expressions as ohm_node and faraday_cell. Used in FP64, where the narrow
-// FP64 pipe binds (82 % busy): against a pass per operator the row and column
+// FP64 pipe binds (80 % busy): against a pass per operator the row and column
 // sums that neighbours share are formed once, 53 operations per node and stage
 // instead of 65, and the stage field never goes to memory. 4096 x 256 cells,
 // two substeps: 1345 -> 1175 us. (In FP32, 8192 x 512 cells: 612 us against
@@ -1227,7 +1227,7 @@ __global__ void __launch_bounds__(32)
 // the strip's own (22 with FIN), and a march starts 4 (5) rows early. At an x
 // wall the wall's node reads its one cell on both sides and the density is
 // mirrored; y wraps. Same expressions as ohm_node and faraday_cell.
-// Bound by instruction issue: about 420 per row of 23 columns. The tiles of
+// Bound by instruction issue: 465 per row of 23 columns (556 of 22 with FIN). The tiles of
 // 32 x 16 cells before recomputed a halo of 4 to 5 cells, 2.1 times their
 // cells, through shared memory and 8 barriers: 8192 x 512 cells, two substeps,
 // 571 -> 340 us; 3000 x 250 172 -> 90; 256 x 64 59 -> 34; 512 x 512 periodic
@@ -1571,9 +1571,10 @@ __device__ __forceinline__ void tile1_ohm(const T* y, int L, int m, int p, const
 // launches per step. Neighbouring tiles read the same B and far sums, so the
 // new B goes to the other buffer and the other far sums, of the step before,
 // are cleared for the next (Sim::swaps_fields); the first block counts the
-// step. (With a launch of its own for that, ten steps of 512 cells: 758 us
-// FP64, 524 FP32; now 726 and 509.) A CTA owns TILE cells (and their left
-// nodes; the last tile also node nx) and runs every pass in shared memory over its cells plus field1_halo(n_sub) cells around
+// step. (With a launch of its own for that, twenty FP64 steps of 512 cells 758
+// us, ten FP32 steps of 8100 cells 524; now 719 and 509.) A CTA owns TILE cells
+// (and their left nodes; the last tile also node nx) and runs every pass in
+// shared memory over its cells plus field1_halo(n_sub) cells around
 // them, which it recomputes: each pass's stencil reaches one cell, so
 // values made wrong at a tile's inner edges (read with indices clamped to
 // the tile) move in by one cell per pass and stay outside the owned cells;

@@ -986,11 +986,11 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // (zero for slots born or removed in it); the adjoints of E and Bbar
 // at the particle and its offset in the cell c0 (out; returns c0, or -1 when it
 // has none); its terms
-// of grad[M] (u_cr, into gucr) and grad[M + 1] (u2, into gu2). The
-// deposit's adjoint, the injection's and the faux-shock
-// return's are taken in FP64; the push's (Boris, gather) in the run's
-// precision, that of the per-slot adjoints lf, lv; the sums over cells into
-// lE, lBb and the gradient are FP64.
+// of grad[M] (u_cr, into gucr) and grad[M + 1] (u2, into gu2). The injection's
+// and the faux-shock return's adjoints are taken in FP64; those of the deposit
+// and the push (Boris, gather) in the run's precision, that of the per-slot
+// adjoints lf, lv and of lNr, lJ. The caller sums E's and Bbar's over a piece of
+// a cell's slots in the run's precision, pieces and the gradient in FP64.
 template <typename T>
 __device__ __forceinline__ int particle_adj_slot(int p, const Win<T>& w, const State<T>& a0,
                                                  const Slots<T>& t1, const uint8_t* ev,
